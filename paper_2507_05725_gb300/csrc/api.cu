@@ -831,6 +831,18 @@ fthms_status fthms_densities_dev(fthms_req* req, int arc, int m, int q, double* 
   if (cap < n) return fail(FTHMS_EINVAL, "fthms_densities_dev: output buffer too small");
   TRY(ensure_device(req->ctx->device));
   const Plan& p = req->plan;
+  // Device (or managed) memory of this device: one kernel gathers the rank's frequencies.  Any other pointer
+  // goes through the runtime's copies, which check it.
+  cudaPointerAttributes at{};
+  const cudaError_t pe = cudaPointerGetAttributes(&at, out_dev);
+  if (pe != cudaSuccess) cudaGetLastError();
+  const bool own = pe == cudaSuccess && (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) &&
+                   at.device == req->ctx->device && reinterpret_cast<size_t>(out_dev) % sizeof(double) == 0;
+  if (own) {
+    CK(launch_gather_density(req->J.sys + (size_t)arc * (p.L - 1) + p.lb - 1, p.le - p.lb, base, p.Q, q, out_dev,
+                             req->stream));
+    return FTHMS_OK;
+  }
   size_t o = 0;
   for (int l = p.lb; l < p.le; ++l) {
     const SysDesc& s = p.sys[(size_t)arc * (p.L - 1) + l - 1];

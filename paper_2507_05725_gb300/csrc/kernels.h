@@ -155,6 +155,9 @@ cudaError_t launch_synth_fwd(const DevJob& J, cudaStream_t st, int* launches);
 // Frequency-partitioned jobs: the partial synthesis into J.ginc, then (after the ranks' sum) the rest.
 cudaError_t launch_synth_partial(const DevJob& J, cudaStream_t st, int* launches);
 cudaError_t launch_fwd_after_sum(const DevJob& J, cudaStream_t st, int* launches);
+// One window of the densities of n consecutive systems (vec: the [q][i] blocks of every system) as one array.
+cudaError_t launch_gather_density(const SysDesc* sys, int n, const double2* vec, int Q, int q, double* out,
+                                  cudaStream_t st);
 cudaError_t launch_traces(const DevJob& J, cudaStream_t st, int* launches);
 
 }  // namespace fthms
