@@ -396,7 +396,7 @@ fthms_status fthms_assemble_self(const fthms_curve* curve, const fthms_arc* arc,
  * process running under a fixed memory cap, or a latency-bound pipeline that cannot accept the
  * device-wide synchronisation that cudaFree implies.  It computes the same matrix (same kernels, same
  * layout: A[i + l*N], interleaved complex, 2*N*N doubles in A_dev) but keeps its temporary device
- * data in a fixed ~534 KB static device array of the library instead of allocating: every GPU that
+ * data in a fixed ~13 KB static device array of the library instead of allocating: every GPU that
  * loads the library holds that array until the process exits.  The caller still provides A_dev.
  *  - Arguments are checked as in fthms_assemble_self, except that N must lie in [2, 256] (the
  *    array's capacity); N outside that range returns FTHMS_EINVAL.

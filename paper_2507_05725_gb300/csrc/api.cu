@@ -17,6 +17,7 @@
 
 #include "fthms.h"
 #include "kernels.h"
+#include "self_one.h"
 #include "plan.h"
 
 using namespace fthms;
@@ -1120,41 +1121,23 @@ fthms_status fthms_assemble_self(const fthms_curve* curve, const fthms_arc* arc,
   c.by.assign(curve->by, curve->by + curve->degree + 1);
   std::vector<double> t, x, y, sp;
   arc_nodes(c, arc->theta_a, arc->theta_b, N, t, x, y, sp);
+  std::vector<unsigned char> host(self_one_copy_bytes(N));
+  self_one_pack(host.data(), N, kappa);
+  const size_t nb = (size_t)N * sizeof(double);
+  std::memcpy(host.data() + kSelfOneNodes, t.data(), nb);
+  std::memcpy(host.data() + kSelfOneNodes + nb, x.data(), nb);
+  std::memcpy(host.data() + kSelfOneNodes + 2 * nb, y.data(), nb);
+  std::memcpy(host.data() + kSelfOneNodes + 3 * nb, sp.data(), nb);
   fthms_req tmp;
   tmp.stream = st;
-  DevJob& J = tmp.J;
-  std::vector<SysDesc> sys(1);
-  // One system in a band of length 1 at frequency index 1 with step h = kappa: the band kernel's
-  // kappa = l h, ln l = 0 and the recurrence step h R all refer to this kappa.
-  sys[0].arc = 0; sys[0].l = 1; sys[0].N = N; sys[0].panel = 0; sys[0].mat_off = 0; sys[0].vec_off = 0;
-  sys[0].piv_off = 0; sys[0].rlog_off = 0; sys[0].kappa = kappa;
-  std::vector<Panel> panels(1, Panel{0, N, 0});
-  std::vector<int> rlogN(1, N);
-  std::vector<long long> rlog_off(1, 0);
-  std::vector<SelfTile> tiles;
-  int nt = (N + kSelfTile - 1) / kSelfTile;
-  for (int a = 0; a < nt; ++a)
-    for (int b = a; b < nt; ++b) tiles.push_back(SelfTile{0, 1, a, b});
-  fthms_status s = FTHMS_OK;
-  if (s == FTHMS_OK) s = dev_upload(&tmp, sys, &J.sys);
-  if (s == FTHMS_OK) s = dev_upload(&tmp, panels, &J.panels);
-  if (s == FTHMS_OK) s = dev_upload(&tmp, t, &J.node_t);
-  if (s == FTHMS_OK) s = dev_upload(&tmp, x, &J.node_x);
-  if (s == FTHMS_OK) s = dev_upload(&tmp, y, &J.node_y);
-  if (s == FTHMS_OK) s = dev_upload(&tmp, sp, &J.node_sp);
-  if (s == FTHMS_OK) s = dev_upload(&tmp, rlogN, &J.rlogN);
-  if (s == FTHMS_OK) s = dev_upload(&tmp, rlog_off, &J.rlog_off_N);
-  if (s == FTHMS_OK) s = dev_upload(&tmp, tiles, &J.tiles);
-  if (s == FTHMS_OK) s = dev_alloc(&tmp, (size_t)N * N, &J.rlog);
+  unsigned char* base = nullptr;
+  fthms_status s = dev_alloc(&tmp, self_one_bytes(N), &base);
   if (s == FTHMS_OK) {
-    J.A = reinterpret_cast<double2*>(A_dev);
-    J.h = kappa;
-    J.n_rlogN = 1;
-    J.n_tiles = (int)tiles.size();
-    J.max_n = N;
-    J.K = 16;  // unused FFT tables are not launched below
+    DevJob& J = tmp.J;
+    self_one_bind(J, base, N, kappa, A_dev);
     int nl = 0;
-    cudaError_t e = launch_tables_rlog_only(J, st, &nl);
+    cudaError_t e = cudaMemcpyAsync(base, host.data(), host.size(), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = launch_tables_rlog_only(J, st, &nl);
     if (e == cudaSuccess) e = launch_assemble_self(J, st, &nl);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) s = cuda_fail(e, "fthms_assemble_self");

@@ -13,7 +13,7 @@ struct SysDesc {
   long long mat_off;  // complex offset of the N x N matrix / LU factor (column-major)
   long long vec_off;  // complex offset of the Q x N data / density block ([q][i])
   long long piv_off;  // int offset of the N pivots
-  long long rlog_off; // double offset of the N x N self log-weight table
+  long long rlog_off; // double offset of the N + 1 cosine sums of the self log weights
   double kappa;
 };
 

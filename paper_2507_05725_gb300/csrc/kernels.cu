@@ -101,31 +101,50 @@ __global__ void k_freq_tw(DevJob J) {
   J.fwd_tw[idx] = make_double2(J.dt * c, J.dt * s);
 }
 
-// Self log weights Rlog_il = -(pi/N) [ln 2 + F(|i-l|) + F(i+l+1)], F(m) = sum_{n=1}^{N-1} cos(n m pi/N)/n
-// (the product-to-sum form of -(pi/N)[ln 2 + 2 sum_n T_n(t_i) T_n(t_l)/n]).
-__global__ void k_rlog(DevJob J) {
+// Cosine sums F(m) = sum_{n=1}^{N-1} cos(n m pi/N)/n, m = 0..N, of the self log weights
+//   Rlog_il = -(pi/N) [ln 2 + F(|i-l|) + F(i+l+1)],  F(2N - m) = F(m)
+// (the product-to-sum form of -(pi/N)[ln 2 + 2 sum_n T_n(t_i) T_n(t_l)/n]); the assembly adds the two F values
+// itself (rlog_at), so no N x N table is written or read.  Grid: (distinct N, blocks of kRlogRows values m), eight
+// lanes per m.  Bound by the FP64 pipe (N DFMA a value plus the cosine table of each block); one block per N
+// that also wrote the N x N table took 1.1 ms at N = 777, this split 0.02 ms.
+constexpr int kRlogRows = 32;
+__global__ void __launch_bounds__(8 * kRlogRows) k_rlog(DevJob J) {
   extern __shared__ double sh[];
-  const int N = J.rlogN[blockIdx.x];
-  double* cosr = sh;           // 2N
-  double* F = sh + 2 * N;      // 2N
-  double* invn = sh + 4 * N;   // N
-  for (int r = threadIdx.x; r < 2 * N; r += blockDim.x) cosr[r] = cospi((double)r / N);
+  const int N = J.rlogN[blockIdx.x], m0 = blockIdx.y * kRlogRows;
+  if (m0 > N) return;
+  double* cosr = sh;           // 2N: cos(r pi/N), the first quadrant evaluated, the rest by symmetry
+  double* invn = sh + 2 * N;   // N
+  for (int r = threadIdx.x; 2 * r <= N; r += blockDim.x) {
+    const double c = cospi((double)r / N);
+    cosr[r] = c;
+    cosr[N - r] = -c;
+    if (r) {
+      cosr[2 * N - r] = c;
+      cosr[N + r] = -c;
+    }
+  }
   for (int n = threadIdx.x; n < N; n += blockDim.x) invn[n] = n ? 1.0 / n : 0.0;
   __syncthreads();
-  for (int m = threadIdx.x; m < 2 * N; m += blockDim.x) {
-    double acc = 0.0;
-    for (int n = 1; n < N; ++n) acc = fma(cosr[(n * m) % (2 * N)], invn[n], acc);
-    F[m] = acc;
+  const int m = m0 + (threadIdx.x >> 3), sub = threadIdx.x & 7;
+  double acc = 0.0;
+  if (m <= N) {
+    const int mod = 2 * N, step = (8 * m) % mod;
+    int idx = ((1 + sub) * m) % mod;
+    for (int n = 1 + sub; n < N; n += 8) {
+      acc = fma(cosr[idx], invn[n], acc);
+      idx += step;
+      if (idx >= mod) idx -= mod;
+    }
   }
-  __syncthreads();
-  double* out = J.rlog + J.rlog_off_N[blockIdx.x];
+  for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (sub == 0 && m <= N) J.rlog[J.rlog_off_N[blockIdx.x] + m] = acc;
+}
+
+// Rlog_il from the cosine sums F of its N.
+__device__ __forceinline__ double rlog_at(const double* __restrict__ F, int N, int i, int l) {
   const double ln2 = 0.69314718055994530941723212145817657;
-  const double sc = -kPiD / N;
-  for (int e = threadIdx.x; e < N * N; e += blockDim.x) {
-    int i = e / N, l = e % N;
-    int d = i > l ? i - l : l - i;
-    out[e] = sc * (ln2 + F[d] + F[i + l + 1]);
-  }
+  const int d = i > l ? i - l : l - i, s = i + l + 1 <= N ? i + l + 1 : 2 * N - (i + l + 1);
+  return (-kPiD / N) * (ln2 + __ldg(&F[d]) + __ldg(&F[s]));
 }
 
 // Transposed restriction tables RT[x][i] = l_x(t_i): the Lagrange basis of the first-kind grid of
@@ -317,7 +336,7 @@ __global__ void __launch_bounds__(256) k_assemble_self(DevJob J) {
   if (i >= N || c >= N) return;
   if (tile.ti == tile.tl && i > c) return;
   const Panel pn = J.panels[s0.panel];
-  const double rl = J.rlog[s0.rlog_off + (long long)i * N + c];
+  const double rl = rlog_at(J.rlog + s0.rlog_off, N, i, c);
   const double w = kPiD / N;
   const long long e1 = (long long)c * N + i, e2 = (long long)i * N + c;
   if (i == c) {
@@ -722,7 +741,7 @@ __device__ void assemble_one(const DevJob& J, int sidx) {
     while ((long long)(c + 1) * (c + 2) / 2 <= t) ++c;
     while ((long long)c * (c + 1) / 2 > t) --c;
     const int i = (int)(t - (long long)c * (c + 1) / 2);
-    const double rl = J.rlog[s.rlog_off + (long long)i * N + c];
+    const double rl = rlog_at(J.rlog + s.rlog_off, N, i, c);
     const long long e1 = (long long)c * N + i, e2 = (long long)i * N + c;
     double2 v;
     if (i == c) {
@@ -2424,10 +2443,8 @@ cudaError_t launch_tables(const DevJob& J, cudaStream_t st, int* launches) {
   k_freq_tw<<<cdiv((long long)J.Q * J.L, 256), 256, 0, st>>>(J);
   *launches += 2;
   if (J.n_rlogN > 0) {
-    size_t sh = (size_t)5 * J.max_n * sizeof(double);
-    cudaFuncSetAttribute(k_rlog, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
-    k_rlog<<<J.n_rlogN, 256, sh, st>>>(J);
-    *launches += 1;
+    cudaError_t e = launch_tables_rlog_only(J, st, launches);
+    if (e != cudaSuccess) return e;
   }
   if (J.n_restr > 0) {
     const size_t sh = (size_t)3 * (J.max_n + J.max_nmax) * sizeof(double);   // <= 38 KB
@@ -2438,10 +2455,10 @@ cudaError_t launch_tables(const DevJob& J, cudaStream_t st, int* launches) {
 }
 
 cudaError_t launch_tables_rlog_only(const DevJob& J, cudaStream_t st, int* launches) {
-  size_t sh = (size_t)5 * J.max_n * sizeof(double);
+  const size_t sh = (size_t)3 * J.max_n * sizeof(double);
   cudaError_t e = cudaFuncSetAttribute(k_rlog, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
   if (e != cudaSuccess) return e;
-  k_rlog<<<J.n_rlogN, 256, sh, st>>>(J);
+  k_rlog<<<dim3(J.n_rlogN, cdiv(J.max_n + 1, kRlogRows)), 8 * kRlogRows, sh, st>>>(J);
   *launches += 1;
   return cudaGetLastError();
 }

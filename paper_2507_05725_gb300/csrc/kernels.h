@@ -36,7 +36,7 @@ struct DevJob {
   const double *node_t, *node_x, *node_y, *node_sp;
   const int* rlogN;
   const long long* rlog_off_N;
-  double* rlog;
+  double* rlog;              // cosine sums F(0..N) of the self log weights, per distinct N
   const int* restr_N;        // [n_restr][2] (N, Nmax)
   const long long* restr_off;
   double* restr;             // transposed tables RT[x][i]

@@ -1,5 +1,5 @@
 // fthms_assemble_self_noalloc: the self-matrix assembly of fthms_assemble_self without any device
-// allocation.  Its temporary device data (node coordinates, the log-weight table, the tile and system
+// allocation.  Its temporary device data (node coordinates, the log weights' cosine sums, the tile and system
 // descriptors) live in one file-scope device array that every GPU loading the library holds until the
 // process exits.
 #include <cuda_runtime.h>
@@ -11,26 +11,14 @@
 
 #include "fthms.h"
 #include "kernels.h"
+#include "self_one.h"
 
 namespace {
 
 using namespace fthms;
 
 constexpr int kNoallocMaxN = 256;                       // largest N accepted
-constexpr int kNoallocMaxTiles = 136;                   // (16 * 17) / 2 tiles at N = 256
-constexpr size_t kAlign = 256;
-
-constexpr size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
-
-// Scratch layout (byte offsets inside the array).
-constexpr size_t kOffNodes = 0;                                                   // 4 x N doubles
-constexpr size_t kOffRlog = align_up(kOffNodes + 4 * kNoallocMaxN * sizeof(double));  // N x N doubles
-constexpr size_t kOffSys = align_up(kOffRlog + (size_t)kNoallocMaxN * kNoallocMaxN * sizeof(double));
-constexpr size_t kOffPanel = align_up(kOffSys + sizeof(SysDesc));
-constexpr size_t kOffRlogN = align_up(kOffPanel + sizeof(Panel));
-constexpr size_t kOffRlogOff = align_up(kOffRlogN + sizeof(int));
-constexpr size_t kOffTiles = align_up(kOffRlogOff + sizeof(long long));
-constexpr size_t kScratchBytes = align_up(kOffTiles + kNoallocMaxTiles * sizeof(SelfTile));   // ~534 KB
+constexpr size_t kScratchBytes = self_one_bytes(kNoallocMaxN);   // ~13 KB
 
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
@@ -95,9 +83,12 @@ extern "C" fthms_status fthms_assemble_self_noalloc(const fthms_curve* curve, co
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
 
   // Host-side tables on the stack (no heap, no device allocation).  A copy from pageable host memory
-  // has been staged by the time cudaMemcpyAsync returns, so these buffers may go out of scope after
-  // the loop below; the kernels stay queued on the stream.
-  double nodes[4 * kNoallocMaxN];
+  // has been staged by the time cudaMemcpyAsync returns, so this buffer may go out of scope; the kernels stay
+  // queued on the stream.  Every byte that the kernels read is overwritten here or by k_rlog and every
+  // entry of A is written, so nothing carried over from an earlier call is used and nothing needs clearing.
+  alignas(16) unsigned char host[self_one_copy_bytes(kNoallocMaxN)];
+  self_one_pack(host, N, kappa);
+  double* nodes = reinterpret_cast<double*>(host + kSelfOneNodes);
   const double tc = 0.5 * (arc->theta_a + arc->theta_b), half = 0.5 * (arc->theta_b - arc->theta_a);
   for (int i = 0; i < N; ++i) {
     const double t = std::cos((2.0 * i + 1.0) * 3.14159265358979323846 / (2.0 * N));
@@ -108,45 +99,10 @@ extern "C" fthms_status fthms_assemble_self_noalloc(const fthms_curve* curve, co
     nodes[2 * N + i] = y;
     nodes[3 * N + i] = std::hypot(dx, dy) * half;
   }
-  SysDesc sys{};
-  sys.arc = 0; sys.l = 1; sys.N = N; sys.panel = 0; sys.mat_off = 0; sys.vec_off = 0; sys.piv_off = 0;
-  sys.rlog_off = 0; sys.kappa = kappa;
-  Panel pn{0, N, 0};
-  int rlogN = N;
-  long long rlog_off = 0;
-  SelfTile tiles[kNoallocMaxTiles];
-  int nt = (N + kSelfTile - 1) / kSelfTile, ntile = 0;
-  for (int a = 0; a < nt; ++a)
-    for (int b = a; b < nt; ++b) tiles[ntile++] = SelfTile{0, 1, a, b};
-
-  // Every region the kernels read is overwritten here and every entry of A is written by the
-  // kernel, so nothing carried over from an earlier call is used and nothing needs clearing.
-  const struct { size_t off; const void* src; size_t n; } ups[] = {
-      {kOffNodes, nodes, 4 * (size_t)N * sizeof(double)}, {kOffSys, &sys, sizeof sys},
-      {kOffPanel, &pn, sizeof pn}, {kOffRlogN, &rlogN, sizeof rlogN}, {kOffRlogOff, &rlog_off, sizeof rlog_off},
-      {kOffTiles, tiles, ntile * sizeof(SelfTile)}};
-  for (const auto& u : ups) {
-    e = cudaMemcpyAsync(base + u.off, u.src, u.n, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return cuda_msg(e, "cudaMemcpyAsync(no-alloc scratch)");
-  }
+  e = cudaMemcpyAsync(base, host, self_one_copy_bytes(N), cudaMemcpyHostToDevice, st);
+  if (e != cudaSuccess) return cuda_msg(e, "cudaMemcpyAsync(no-alloc scratch)");
   DevJob J{};
-  const double* nd = reinterpret_cast<const double*>(base + kOffNodes);
-  J.node_t = nd;
-  J.node_x = nd + N;
-  J.node_y = nd + 2 * N;
-  J.node_sp = nd + 3 * N;
-  J.rlog = reinterpret_cast<double*>(base + kOffRlog);
-  J.sys = reinterpret_cast<const SysDesc*>(base + kOffSys);
-  J.panels = reinterpret_cast<const Panel*>(base + kOffPanel);
-  J.rlogN = reinterpret_cast<const int*>(base + kOffRlogN);
-  J.rlog_off_N = reinterpret_cast<const long long*>(base + kOffRlogOff);
-  J.tiles = reinterpret_cast<const SelfTile*>(base + kOffTiles);
-  J.A = reinterpret_cast<double2*>(A_dev);
-  J.h = kappa;
-  J.n_rlogN = 1;
-  J.n_tiles = ntile;
-  J.max_n = N;
-  J.K = 16;
+  self_one_bind(J, base, N, kappa, A_dev);
   int nl = 0;
   e = launch_tables_rlog_only(J, st, &nl);
   if (e == cudaSuccess) e = launch_assemble_self(J, st, &nl);

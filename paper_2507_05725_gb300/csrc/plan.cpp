@@ -457,7 +457,7 @@ int build_plan(const fthms_curve* curves, int ncurves, const fthms_arc* arcs, in
     kv.second = p.rlog_total;
     p.rlogN.push_back(kv.first);
     p.rlog_off_N.push_back(p.rlog_total);
-    p.rlog_total += (long long)kv.first * kv.first;
+    p.rlog_total += kv.first + 1;
   }
   for (auto& s : p.sys)
     if (p.own(s.l)) s.rlog_off = rlog_map[s.N];
@@ -691,7 +691,7 @@ size_t plan_device_bytes(const Plan& p) {
          p.sys.size() * (24 + 32) + (size_t)p.piv_total * 8 + p.rchunks.size() * sizeof(ResidChunk);
   b += p.sig_f.size() * 8;                       // samples of a sampled signal
   b += (size_t)p.piv_total * 4;                  // pivots
-  b += (size_t)p.rlog_total * 8;                 // self log tables
+  b += (size_t)p.rlog_total * 8;                 // cosine sums of the self log weights
   b += (size_t)p.vec_total * 16 * 3;             // G, phi (current), phi sum
   if (p.opt.keep_densities) b += (size_t)p.vec_total * 16 * p.M;
   b += (size_t)p.spec_total * 16 * 2;            // W and Gt on transfer meshes

@@ -42,6 +42,29 @@ def _rel(job, ref, problem):
     return math.sqrt(num / den)
 
 
+@pytest.mark.parametrize("N", [2, 3, 31, 32, 33, 64, 65, 1023, 1024])
+def test_log_weights_at_block_edges(F, N):
+    """The cosine sums F(0..N) come in blocks of 32 values; the matrix takes F(|i-l|) and F(i+l+1), folded at N.
+    1e-13 of the largest entry: the bar of the self-matrix parity test."""
+    curve, arc, kappa = wl.kite(0.1, 0.2), (-1.3, 1.1), 0.21 * N + 0.7
+    A = torch.empty(2 * N * N, dtype=torch.float64, device="cuda")
+    F.fthms_assemble_self(curve, arc, N, kappa, A.data_ptr())
+    got = A.cpu().numpy().reshape(N, N, 2)
+    got = (got[..., 0] + 1j * got[..., 1]).T
+    # The oracle's own weights carry cos(k arccos t_i) with a rounding error that grows with k (1e-12 of the
+    # largest entry at N = 1024), so they are replaced by the same sums with the phase k m pi/N reduced in integers.
+    t, n = geo.cheb_nodes(N), np.arange(1, N)
+    arc_ = geo.Arc(0, 0, curve, *arc)
+    cosr = np.cos(np.arange(2 * N) * (np.pi / N))
+    Fm = np.array([np.sum(cosr[(n * m) % (2 * N)] / n) for m in range(2 * N)])
+    i = np.arange(N)
+    rlog = -(np.pi / N) * (math.log(2.0) + Fm[np.abs(i[:, None] - i)] + Fm[i[:, None] + i + 1])
+    X = arc_.point(t)[0]
+    R = np.linalg.norm(X[:, None] - X[None], axis=-1)
+    ref = oker.self_matrix(arc_, N, kappa) - special.j0(kappa * R) / (2.0 * np.pi) * (rlog - oker.rlog_self(N))
+    assert np.max(np.abs(got - ref)) <= 1e-13 * np.max(np.abs(ref))
+
+
 @pytest.mark.parametrize("shift", [0, 1])
 def test_densities_on_the_device_equal_the_host_copy(F, ctx, shift):
     """Byte for byte, also into a buffer that is only 8-byte aligned, for uneven N and several windows."""
