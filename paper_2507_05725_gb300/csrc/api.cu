@@ -350,6 +350,29 @@ fthms_status upload_job(fthms_req* r) {
   }
   TRY(dev_alloc(r, (size_t)p.vec_total, &J.G));
   TRY(dev_alloc(r, (size_t)p.vec_total, &J.phi));
+  // Point-source data by interpolation in the distance from the source: when the points are at most half the
+  // active nodes (their rows plus the interpolation then cost less than a row per node) and the samples and the
+  // basis fit the densities' memory, which nothing reads before the first solve writes it.
+  J.inc_m = 0;
+  J.inc_u = J.inc_basis = nullptr;
+  if (incident_recurrent(J) && !p.act_idx.empty()) {
+    double r0 = 1e300, r1 = 0.0;
+    for (size_t a = 0; a < p.act_idx.size(); ++a) {
+      const long long o = p.panels[p.tpanel[p.act_arc[a]]].off + p.act_idx[a];
+      const double d = std::hypot(p.node_x[o] - J.z0x, p.node_y[o] - J.z0y);
+      r0 = std::min(r0, d);
+      r1 = std::max(r1, d);
+    }
+    const size_t m = (size_t)incident_points(r0, r1, J.carrier, J.width);
+    if (m > 0 && 2 * m <= p.act_idx.size() &&
+        m * ((size_t)p.NT + p.act_idx.size()) <= 2 * (size_t)p.vec_total) {
+      J.inc_m = (int)m;
+      J.inc_mid = 0.5 * (r0 + r1);
+      J.inc_half = 0.5 * (r1 - r0);
+      J.inc_u = reinterpret_cast<double*>(J.phi);
+      J.inc_basis = J.inc_u + m * (size_t)p.NT;
+    }
+  }
   J.phi_df = nullptr;
   if (J.mixed) TRY(dev_alloc(r, (size_t)p.vec_total, &J.phi_df));
   TRY(dev_alloc(r, (size_t)p.vec_total, &J.phi_sum));

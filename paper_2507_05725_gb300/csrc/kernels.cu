@@ -2188,40 +2188,68 @@ __device__ double incident_u(const DevJob& J, double X, double Y, double t) {
 }
 
 // Incident time samples g[a][n] = sign chi_k u^i(x, t_n) at the active transfer nodes, t_n = -H + n dt.
-// One thread per run of kIncRun consecutive samples.  Point source with the analytic signal: the
-// trapezoid rule in v on the run's common range [v_lo(t_first), v_hi(t_last)] (it contains every sample's
-// own range, outside of which f < e^{-64}) with the step of the run's largest rate, and each term of the
-// sum advanced from sample to sample by an exact recurrence: with rho = r cosh v and d = t - centre - rho,
-// T(t) = e^{i carrier (t - rho)} e^{-(d/width)^2} (so f = amp Im T) satisfies
-//   T(t_{j+1}) = T(t_j) u g_j,  u = e^{i carrier dt} e^{-(dt^2 + 2 dt d_0)/width^2},  g_j = e^{-2 j dt^2/width^2}
-// from the run's first sample (d_0 = t_first - centre - rho; |d_0| <= 10 width keeps u within e^{+-3}),
-// so a term costs one seed (sincos, exp) per run and a complex product per sample.  Runs whose Gaussian
-// factor could change by more than e^{-64} within the run (dt kIncRun > 2 width) and sampled signals
-// evaluate every sample directly (incident_u).
+//
+// Point source with the analytic signal (k_incident_ps): the trapezoid rule in v for a run of kIncRun consecutive
+// samples on the run's common range [v_lo(t_first), v_hi(t_last)] (it contains every sample's own range, outside
+// of which f < e^{-64}) with the step of the run's largest rate.  With rho = r cosh v, t_c the run's middle
+// sample, d = t_c - centre - rho and delta = dt, the signal at t_c + j delta is
+//   f = amp Im(e^{i carrier (t_c - rho)} e^{-(d/width)^2} b^j Gamma_j),   b = e^{-2 delta d/width^2},
+//   Gamma_j = e^{i carrier j delta} e^{-(j delta/width)^2},
+// so a term costs one seed (cosh, sincos, two exp) per run and three FP64 operations per sample (b^j by repeated
+// multiplication from the middle outwards, at most kIncRun / 2 of them), Gamma_j entering after the sum.  One warp
+// per (row, run), the terms split over its lanes: a row's runs are few in a small job, and one thread per run left
+// the GPU empty (45 nodes, 256 samples: 1.45 ms; 0.1 ms so).  Runs whose Gaussian factor could change by more
+// than e^{-64} within the run (dt kIncRun > 2 width) and sampled signals evaluate every sample directly.
+//
+// Rows are the active nodes, or (J.inc_m > 0) inc_m first-kind Chebyshev points of the interval of distances
+// r = |x - z0| that the active nodes span: u^i depends on the node through r alone and is analytic in it, so its
+// interpolant in r gives every node's samples (k_inc_interp, one small FP64 product) to below rounding; the number of
+// points follows from the signal's growth on a Bernstein ellipse (incident_points).  12-arc cavity with 2 500
+// active nodes: 76 rows instead of 2 500.
 constexpr int kIncRun = 16;
 constexpr int kIncThreads = 128;
 
+__device__ __forceinline__ double inc_point(const DevJob& J, int i) {
+  return fma(J.inc_half, cospi((2.0 * i + 1.0) / (2.0 * J.inc_m)), J.inc_mid);
+}
+
+// Direct form: one thread per sample.
 __global__ void __launch_bounds__(kIncThreads) k_incident_u(DevJob J) {
   const int a = blockIdx.x;
-  const int n0 = (blockIdx.y * kIncThreads + threadIdx.x) * kIncRun;
-  if (n0 >= J.NT) return;
-  const int nr = min(kIncRun, J.NT - n0);
+  const int n = blockIdx.y * kIncThreads + threadIdx.x;
+  if (n >= J.NT) return;
   const int k = J.act_arc[a], x = J.act_idx[a];
   const Panel pn = J.panels[J.tpanel[k]];
-  const double X = J.node_x[pn.off + x], Y = J.node_y[pn.off + x];
   const double pref = J.sign * J.chi[J.tr_off[k] + x];
-  double* g = J.ginc + (long long)a * J.NT + n0;
-  const bool rec = J.sig_kind == 0 && J.sig_nt == 0 && J.dt * kIncRun <= 2.0 * J.width;
-  if (!rec) {
-    for (int j = 0; j < nr; ++j) g[j] = pref * incident_u(J, X, Y, -J.H + (n0 + j) * J.dt);
-    return;
+  J.ginc[(long long)a * J.NT + n] =
+      pref * incident_u(J, J.node_x[pn.off + x], J.node_y[pn.off + x], -J.H + n * J.dt);
+}
+
+__global__ void __launch_bounds__(kIncThreads) k_incident_ps(DevJob J) {
+  const int row = blockIdx.x, lane = threadIdx.x & 31;
+  const int n0 = (blockIdx.y * (kIncThreads / 32) + (threadIdx.x >> 5)) * kIncRun;
+  if (n0 >= J.NT) return;
+  const int nr = min(kIncRun, J.NT - n0);
+  double r, pref, *out;
+  if (J.inc_m > 0) {
+    r = inc_point(J, row);
+    pref = 1.0;
+    out = J.inc_u;
+  } else {
+    const int k = J.act_arc[row], x = J.act_idx[row];
+    const Panel pn = J.panels[J.tpanel[k]];
+    const double dx = J.node_x[pn.off + x] - J.z0x, dy = J.node_y[pn.off + x] - J.z0y;
+    r = sqrt(fma(dx, dx, dy * dy));
+    pref = J.sign * J.chi[J.tr_off[k] + x];
+    out = J.ginc;
   }
-  const double dx = X - J.z0x, dy = Y - J.z0y;
-  const double r = sqrt(fma(dx, dx, dy * dy));
+  out += (long long)row * J.NT + n0;
+  constexpr int kMid = kIncRun / 2;
   const double t_first = -J.H + n0 * J.dt, t_last = -J.H + (n0 + nr - 1) * J.dt;
-  double acc[kIncRun];
+  double v[2 * kIncRun];   // [2 j] real, [2 j + 1] imaginary part of sum_k T_k b_k^(j - kMid)
 #pragma unroll
-  for (int j = 0; j < kIncRun; ++j) acc[j] = 0.0;
+  for (int j = 0; j < 2 * kIncRun; ++j) v[j] = 0.0;
+  double sc = 0.0;
   const double tau_hi = t_last - J.centre + 8.0 * J.width;
   const double tau_lo = fmax(r, t_first - J.centre - 8.0 * J.width);
   if (tau_hi > r && tau_lo < tau_hi) {
@@ -2230,32 +2258,123 @@ __global__ void __launch_bounds__(kIncThreads) k_incident_u(DevJob J) {
     const int n = (int)ceil((v_hi - v_lo) * (1.25 * rate + 24.0) / (2.0 * kPiD) * 2.0) + 16;
     const double dv = (v_hi - v_lo) / n;
     const double iw2 = 1.0 / (J.width * J.width);
-    double sa, ca;
-    sincos(J.carrier * J.dt, &sa, &ca);
-    const double gam = exp(-2.0 * J.dt * J.dt * iw2);
-    for (int kk = 0; kk <= n; ++kk) {
+    const double t_c = -J.H + (n0 + kMid) * J.dt;
+    for (int kk = lane; kk <= n; kk += 32) {
       const double rho = r * cosh(fma((double)kk, dv, v_lo));
       const double wgt = (kk == 0 || kk == n) ? 0.5 : 1.0;
-      const double d0 = t_first - J.centre - rho;
+      const double d = t_c - J.centre - rho;
       double sp, cp;
-      sincos(J.carrier * (t_first - rho), &sp, &cp);
-      const double e0 = wgt * exp(-d0 * d0 * iw2);
-      double2 z = make_double2(e0 * cp, e0 * sp);
-      const double b = exp(-(J.dt * J.dt + 2.0 * J.dt * d0) * iw2);
-      const double2 u = make_double2(ca * b, sa * b);
-      double gj = 1.0;
+      sincos(J.carrier * (t_c - rho), &sp, &cp);
+      const double e0 = wgt * exp(-d * d * iw2), x = 2.0 * J.dt * d * iw2;
+      const double b = exp(-x), ib = exp(x);
+      cp *= e0;
+      sp *= e0;
+      v[2 * kMid] += cp;
+      v[2 * kMid + 1] += sp;
+      double p = b, m = ib;
 #pragma unroll
-      for (int j = 0; j < kIncRun; ++j) {
-        acc[j] += z.y;
-        z = cmul(z, make_double2(u.x * gj, u.y * gj));
-        gj *= gam;
+      for (int j = 1; j <= kMid; ++j) {
+        if (kMid + j < kIncRun) {
+          v[2 * (kMid + j)] = fma(p, cp, v[2 * (kMid + j)]);
+          v[2 * (kMid + j) + 1] = fma(p, sp, v[2 * (kMid + j) + 1]);
+          p *= b;
+        }
+        v[2 * (kMid - j)] = fma(m, cp, v[2 * (kMid - j)]);
+        v[2 * (kMid - j) + 1] = fma(m, sp, v[2 * (kMid - j) + 1]);
+        m *= ib;
       }
     }
-    const double sc = pref * J.amp * dv * (0.5 * kInvPi);
-#pragma unroll
-    for (int j = 0; j < kIncRun; ++j) acc[j] *= sc;
+    sc = pref * J.amp * dv * (0.5 * kInvPi);
   }
-  for (int j = 0; j < nr; ++j) g[j] = acc[j];
+  // sum over the lanes: each step keeps half of the values, so lane e ends with value e (j = e / 2)
+#pragma unroll
+  for (int w = kIncRun; w >= 1; w >>= 1) {
+    const bool up = (lane & w) != 0;
+#pragma unroll
+    for (int e = 0; e < w; ++e) {
+      const double keep = up ? v[e + w] : v[e], give = up ? v[e] : v[e + w];
+      v[e] = keep + __shfl_xor_sync(0xffffffffu, give, w);
+    }
+  }
+  const double im = __shfl_down_sync(0xffffffffu, v[0], 1);
+  const int j = lane >> 1;
+  if ((lane & 1) == 0 && j < nr) {
+    const double y = (j - kMid) * J.dt, g = exp(-(y / J.width) * (y / J.width));
+    double s, c;
+    sincos(J.carrier * y, &s, &c);
+    out[j] = sc * g * fma(s, v[0], c * im);
+  }
+}
+
+// Lagrange basis of the inc_m Chebyshev points at every active node's distance, times sign chi_k (barycentric
+// form, weights (-1)^i sin((2i+1) pi/(2m))); one warp per node.
+__global__ void __launch_bounds__(kIncThreads) k_inc_basis(DevJob J) {
+  const int a = blockIdx.x * (kIncThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (a >= J.n_act) return;
+  const int k = J.act_arc[a], x = J.act_idx[a], m = J.inc_m;
+  const Panel pn = J.panels[J.tpanel[k]];
+  const double dx = J.node_x[pn.off + x] - J.z0x, dy = J.node_y[pn.off + x] - J.z0y;
+  const double r = sqrt(fma(dx, dx, dy * dy));
+  const double pref = J.sign * J.chi[J.tr_off[k] + x];
+  double* L = J.inc_basis + (long long)a * m;
+  double den = 0.0;
+  int hit = -1;
+  for (int i = lane; i < m; i += 32) {
+    double s, c;
+    sincospi((2.0 * i + 1.0) / (2.0 * m), &s, &c);
+    const double d = r - fma(J.inc_half, c, J.inc_mid);
+    if (d == 0.0) hit = i;
+    const double q = ((i & 1) ? -s : s) / (d == 0.0 ? 1.0 : d);
+    L[i] = q;
+    den += q;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    den += __shfl_xor_sync(0xffffffffu, den, o);
+    hit = max(hit, __shfl_xor_sync(0xffffffffu, hit, o));
+  }
+  const double sc = pref / den;
+  for (int i = lane; i < m; i += 32) L[i] = hit >= 0 ? (i == hit ? pref : 0.0) : L[i] * sc;
+}
+
+// ginc[a][n] = sum_i basis[a][i] u[i][n]: 64 x 64 tiles, 4 x 4 values a thread, 16 points staged at a time.  FP64-pipe
+// bound (2 n_act m NT flops: 2.3 GFLOP, 2 ms, for the 12-arc cavity with four windows).
+constexpr int kItpTile = 64, kItpK = 16;
+__global__ void __launch_bounds__(256) k_inc_interp(DevJob J) {
+  __shared__ double As[kItpK][kItpTile + 1], Bs[kItpK][kItpTile];
+  const int a0 = blockIdx.y * kItpTile, n0 = blockIdx.x * kItpTile, m = J.inc_m;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  double acc[4][4] = {};
+  for (int k0 = 0; k0 < m; k0 += kItpK) {
+    for (int e = threadIdx.x; e < kItpK * kItpTile; e += 256) {
+      const int ka = e % kItpK, a = e / kItpK, kb = e / kItpTile, n = e % kItpTile;
+      As[ka][a] = a0 + a < J.n_act && k0 + ka < m ? J.inc_basis[(long long)(a0 + a) * m + k0 + ka] : 0.0;
+      Bs[kb][n] = n0 + n < J.NT && k0 + kb < m ? J.inc_u[(long long)(k0 + kb) * J.NT + n0 + n] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int k = 0; k < kItpK; ++k) {
+      double av[4], bv[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        av[i] = As[k][ty + 16 * i];
+        bv[i] = Bs[k][tx + 16 * i];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int a = a0 + ty + 16 * i;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int n = n0 + tx + 16 * j;
+      if (a < J.n_act && n < J.NT) J.ginc[(long long)a * J.NT + n] = acc[i][j];
+    }
+  }
 }
 
 // Slow transforms of the incident samples of one active transfer node (eq. Fourierk per window).
@@ -2555,10 +2674,25 @@ cudaError_t launch_cross_assemble(const DevJob& J, cudaStream_t st, int* launche
 
 static size_t time_smem(const DevJob& J) { return (size_t)J.K * sizeof(double2) + (size_t)J.NT * sizeof(double); }
 
+bool incident_recurrent(const DevJob& J) {
+  return J.sig_kind == 0 && J.sig_nt == 0 && J.dt * kIncRun <= 2.0 * J.width;
+}
+
 cudaError_t launch_incident(const DevJob& J, cudaStream_t st, int* launches) {
   if (J.n_act == 0) return cudaSuccess;
-  const int runs = (J.NT + kIncRun - 1) / kIncRun;
-  k_incident_u<<<dim3(J.n_act, (runs + kIncThreads - 1) / kIncThreads), kIncThreads, 0, st>>>(J);
+  if (incident_recurrent(J)) {
+    const int runs = cdiv(J.NT, kIncRun), rows = J.inc_m > 0 ? J.inc_m : J.n_act;
+    k_incident_ps<<<dim3(rows, cdiv(runs, kIncThreads / 32)), kIncThreads, 0, st>>>(J);
+    *launches += 1;
+    if (J.inc_m > 0) {
+      k_inc_basis<<<cdiv(J.n_act, kIncThreads / 32), kIncThreads, 0, st>>>(J);
+      k_inc_interp<<<dim3(cdiv(J.NT, kItpTile), cdiv(J.n_act, kItpTile)), 256, 0, st>>>(J);
+      *launches += 2;
+    }
+  } else {
+    k_incident_u<<<dim3(J.n_act, cdiv(J.NT, kIncThreads)), kIncThreads, 0, st>>>(J);
+    *launches += 1;
+  }
   size_t sh = time_smem(J);
   const int nt = J.shape_time > 0 ? J.shape_time : kTimeThreads;
   const bool df = J.mixed && !J.fp64keep;   // double-float FFT butterflies
@@ -2567,7 +2701,7 @@ cudaError_t launch_incident(const DevJob& J, cudaStream_t st, int* launches) {
   if (e != cudaSuccess) return e;
   if (df) k_incident<true><<<J.n_act, nt, sh, st>>>(J);
   else k_incident<false><<<J.n_act, nt, sh, st>>>(J);
-  *launches += 2;
+  *launches += 1;
   return cudaGetLastError();
 }
 

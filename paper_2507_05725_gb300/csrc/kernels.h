@@ -24,6 +24,12 @@ struct DevJob {
   int sig_nt;                    // > 0: sampled signal f[0..sig_nt) at sig_t0 + i sig_dt
   double sig_t0, sig_dt, sig_band;
   const double* sig_f;
+  // point source, analytic signal: u^i(r, t) sampled at inc_m Chebyshev points of [inc_mid -+ inc_half] and
+  // interpolated to the active nodes' distances (0: evaluated at every active node)
+  int inc_m;
+  double inc_mid, inc_half;
+  double* inc_u;              // [inc_m][NT], in the densities' memory (written by the first solve only later)
+  double* inc_basis;          // [n_act][inc_m], after inc_u
   // tables
   const SysDesc* sys;
   const int* sys_order;       // systems by decreasing N (launch order of the solves and restriction)
@@ -141,6 +147,8 @@ size_t lu_big_panel_smem(int maxN);
 cudaError_t launch_fused_asf(const DevJob& J, int* counter, cudaStream_t st, int* launches);
 cudaError_t launch_cross_assemble(const DevJob& J, cudaStream_t st, int* launches);
 cudaError_t launch_incident(const DevJob& J, cudaStream_t st, int* launches);
+// Point source with an analytic signal that the runs of kIncRun samples resolve (else every sample directly).
+bool incident_recurrent(const DevJob& J);
 cudaError_t launch_restrict(const DevJob& J, cudaStream_t st, int* launches);
 cudaError_t launch_solve(const DevJob& J, int m, cudaStream_t st, int* launches);
 // Mixed forms, the same step piece by piece: launch_msolve(pass 0), then for pass = 1 .. refine_passes(J)

@@ -671,6 +671,24 @@ int build_plan(const fthms_curve* curves, int ncurves, const fthms_arc* arcs, in
   return FTHMS_OK;
 }
 
+// u^i(r, t) = (1/(2 pi)) int f(t - r cosh v) dv is a superposition of outgoing waves H0^(1)(omega r) weighted with
+// F(omega), analytic in r away from r = 0.  On the Bernstein ellipse of [r0, r1] with parameter rho (semi-minor
+// axis b = (r1 - r0)(rho - 1/rho)/4, kept clear of r = 0) a wave grows by at most e^{omega b}, and the signal's Gaussian
+// spectrum then by e^{carrier b + (b/width)^2}; the degree m - 1 interpolant's error is below about
+// 4 e^{carrier b + (b/width)^2} rho^{-m}.  The smallest m over rho with that below e^{-40} (4e-18).
+int incident_points(double r0, double r1, double carrier, double width) {
+  if (!(r0 > 0.0) || !(r1 > r0)) return 0;
+  const double c = (r1 + r0) / (r1 - r0), far = c + std::sqrt(c * c - 1.0);   // the ellipse through r = 0
+  int best = 0;
+  for (double f = 0.30; f <= 0.901; f += 0.05) {
+    const double rho = 1.0 + f * (far - 1.0);
+    const double b = 0.25 * (r1 - r0) * (rho - 1.0 / rho);
+    const double m = (std::fabs(carrier) * b + (b / width) * (b / width) + 40.0 + std::log(4.0)) / std::log(rho);
+    if (m < 100000.0 && (best == 0 || (int)m + 2 < best)) best = (int)m + 2;
+  }
+  return best;
+}
+
 void arc_nodes(const Curve& c, double theta_a, double theta_b, int N, std::vector<double>& t,
                std::vector<double>& x, std::vector<double>& y, std::vector<double>& sp) {
   const double tc = 0.5 * (theta_a + theta_b), half = 0.5 * (theta_b - theta_a);

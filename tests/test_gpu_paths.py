@@ -1,4 +1,5 @@
 """Sizes at which the kernels' tiles and dispatch rules can go wrong, against the oracle or the general path."""
+import copy
 import math
 
 import numpy as np
@@ -84,3 +85,30 @@ def test_densities_on_the_device_equal_the_host_copy(F, ctx, shift):
                 got = buf.cpu().numpy()
                 assert np.array_equal(got[shift:shift + want.size], want)
                 assert got[shift + want.size] == 7.0 and (shift == 0 or got[0] == 7.0)
+
+
+@pytest.mark.parametrize("case", ["interpolated", "near-source", "few-nodes", "steep", "partitioned"])
+def test_point_source_rows(F, ctx, case):
+    """Incident data by interpolation in the distance from the source (many active nodes), node by node (source
+    close to an arc, or few nodes) and sample by sample (a signal shorter than a run of samples)."""
+    p = wl.config1(L=41, M=1, N=24 if case == "few-nodes" else 72)
+    p["options"].update(H=4.0, n_period=256, W=16.0)
+    if case == "near-source":
+        p["signal"]["z0"] = [1.004, 0.0]
+    if case == "steep":
+        p["signal"].update(width=0.02, centre=1.5)
+        p["options"]["n_period"] = 128
+    ref = run_oracle(p)
+    if case == "partitioned":
+        p = copy.deepcopy(p)
+        p["options"].update(omega_rank=1, omega_ranks=2)
+        job = F.Job(ctx, p)
+        job.set_allreduce(lambda buf, n, stream: None)
+        job.run().wait()
+        for j in range(3):
+            for l, v in job.densities(j, 1, 0).items():
+                assert np.linalg.norm(v - ref.phi[(1, j, l)][0]) <= 1e-11 * max(
+                    np.linalg.norm(ref.phi[(1, j, k)][0]) for k in range(1, 41))
+        return
+    job = F.Job(ctx, p).run().wait()
+    assert _rel(job, ref, p) < 1e-11
