@@ -109,7 +109,7 @@ typedef struct {
  *  precision : 0 = FP64 throughout.  1 = mixed form: FP32 LU factors; solutions refined against the
  *              matrix kept as double-float (two floats, ~48 bits) until the relative error estimated
  *              to remain (last correction x estimated contraction factor) is below refine_tol, at most
- *              refine_max steps; self and cross entries (Taylor range and far-field recurrence), the
+ *              refine_max steps; self and cross entries (Taylor range, far field), the
  *              refinement residuals, the FFT butterflies of the time transforms, the restriction and the
  *              cross apply in double-float on the FP32 pipe; diagonal self entries, per-pair setup,
  *              phase-seed reduction, log-singular corrections, transform folds and phase factors stay

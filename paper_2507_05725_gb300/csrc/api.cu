@@ -10,6 +10,7 @@
 #include <functional>
 #include <map>
 #include <mutex>
+#include <numeric>
 #include <set>
 #include <string>
 #include <thread>
@@ -299,6 +300,9 @@ fthms_status upload_job(fthms_req* r) {
     TRY(dev_upload(r, p.otf_res_off, &J.otf_res_off));
     TRY(dev_alloc(r, (size_t)p.wn_total, &J.wn));
     J.n_otf = (int)p.otf.size();
+    // launch order: about a golden-section stride, made coprime to the task count
+    J.otf_stride = std::max(1LL, (long long)(0.6180339887 * J.n_otf));
+    while (std::gcd(J.otf_stride, (long long)std::max(1, J.n_otf)) != 1) ++J.otf_stride;
   }
   apply_shapes(r, p.opt.shapes);       // launch shapes and LU split (fthms_options.shapes; 0 = default)
   TRY(dev_upload(r, p.tpanel, &J.tpanel));
@@ -386,6 +390,12 @@ fthms_status upload_job(fthms_req* r) {
   TRY(dev_alloc(r, (size_t)std::max(1, p.n_obs * p.Q * p.L), &J.Vobs));
   TRY(dev_alloc(r, (size_t)std::max(1, p.n_obs * p.n_tout), &J.traces));
   TRY(dev_alloc(r, (size_t)p.K / 2, &J.fft_tw));
+  J.freq_df = nullptr;
+  if (J.mixed) {
+    unsigned char* fd = nullptr;
+    TRY(dev_alloc(r, (size_t)p.L * kFreqDfBytes, &fd));
+    J.freq_df = reinterpret_cast<FreqDf*>(fd);
+  }
   J.fft_tw_df = nullptr;
   if (J.mixed) TRY(dev_alloc(r, (size_t)p.K / 2, &J.fft_tw_df));
   TRY(dev_alloc(r, (size_t)p.Q * p.L, &J.syn_tw));

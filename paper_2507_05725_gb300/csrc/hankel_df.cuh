@@ -1,0 +1,301 @@
+// The Hankel kernel of one (target, source) pair along a run of frequencies l, in double-float on the FP32 pipe
+// (mixed forms).  With T = h R/(2 pi) the pair's turns per frequency index, z = 2 pi l T and w = 1/z:
+//   z < 20 : J0 and Yhat0 from Taylor expansions about the centres of 160 intervals of width 1/8 (the expansions of
+//            bessel_taylor.cuh shifted on the host), the terms n <= 4 in double-float, n = 5..8 in FP32 (|d| <= 1/16,
+//            so they lie below 2^-26 of the sum);
+//   z >= 20: modulus and phase, H0^(1)(z) = sqrt(2/(pi z)) m(w) e^{i(z - pi/4 + phi(w))}.  The phase z/(2 pi) = l T mod 1
+//            is an exact 64-bit integer multiple of T's fraction, so no recurrence, no re-seeding and no FP64
+//            reduction: -w/8 and its cubic correction join it as integers, the top 9 bits pick (cos, sin) from a
+//            table of 512 angles and the rest (|x| <= pi/512) needs three Taylor terms.
+//            phi = -(w/8)(1 - s (25/48 - s rho(s))), m = 1 - s/16 + s^2 kappa(s), s = w^2 (the leading terms of
+//            DLMF 10.18.17-18), rho and kappa polynomials fitted to the exact modulus and phase on s <= 1/400 at 60
+//            digits (their fit errors enter below 2^-54 and 2^-47 of the result).
+// About 125 FP32-pipe instructions an entry above z = 20 against ~225 of the rotated P + iQ recurrence this
+// replaces, and the set-up per pair needs no sine or cosine, so short bands cost no more per entry than long ones.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <cmath>
+
+#include "bessel.cuh"
+#include "df64.cuh"
+#include "kernels.h"
+
+namespace fthms {
+
+constexpr int kAngles = 512;            // (cos, sin)(2 pi k/512)
+constexpr int kTayFine = 160;           // Taylor intervals of width 1/8 on [0, 20)
+__device__ float4 c_angle_df[kAngles];          // cos hi, lo, sin hi, lo
+__device__ float4 c_tayfine_df[kTayFine][7];    // J0: c8..c5 | c4 c3 | c2 c1 (pairs) | c0, Yhat0: see tayfine_pack
+__device__ float4 c_log_df[128];                // reciprocal rc (9 bits) of the 128th's centre, -ln rc (hi, lo)
+
+// Per-frequency constants as double-float (two float4 a frequency, then ln l in FP64): 2 pi l, 1/(2 pi l);
+// 1/sqrt(l), ln l + ln pi + gamma (so that ln(z/2) + gamma = ln T + it).
+struct FreqDf {
+  float4 a, b;
+  double lnl, pad;
+};
+static_assert(sizeof(FreqDf) == kFreqDfBytes, "size of the per-frequency constants");
+
+// One pair: everything that its frequencies share.
+struct PairTurns {
+  unsigned long long v;   // fraction of T in units of 2^-64 turns
+  df T, iu, aw;           // T, 1/T, (w/(4 pi)) / sqrt(T)
+};
+
+__device__ __forceinline__ double f2d_bits(float f) {       // exact for normal f (zero gives 2^-127-ish)
+  const unsigned u = __float_as_uint(f);
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ float d2f_trunc(double d) {      // a non-negative double in FP32's normal range, truncated
+  return __uint_as_float((((unsigned)__double2hiint(d) - 0x38000000u) << 3) | ((unsigned)__double2loint(d) >> 29));
+}
+
+// Distance in FP64 without the library's square root: the FP32 reciprocal root and two Newton steps on r^2 = R2
+// (relative error 2^-22 -> 2^-45 -> below 2^-53).
+__device__ __forceinline__ double dist_f64(double R2) {
+  const float y = rsqrtf(d2f_trunc(R2));
+  const double yd = f2d_bits(y), hy = f2d_bits(0.5f * y);
+  double r = R2 * yd;
+  r = fma(fma(-r, r, R2), hy, r);
+  return fma(fma(-r, r, R2), hy, r);
+}
+
+// hi + lo ~ a to 2^-47 by integer operations and selects alone (split_f64_bits without its FP64 branch, whose
+// instructions occupy the FP64 pipe even when no lane takes them): below FP32's normal range zero, above it NaN.
+__device__ __forceinline__ df df_split_bits(double a) {
+  const unsigned uh = (unsigned)__double2hiint(a), ul = (unsigned)__double2loint(a);
+  const int e = (int)((uh >> 20) & 0x7FFu);
+  const unsigned sign = uh & 0x80000000u, rem = ul & 0x1FFFFFFFu;
+  const float h = __uint_as_float(sign | ((unsigned)(e - 896) << 23) | (__funnelshift_l(ul, uh, 3) & 0x007FFFFFu));
+  const float r = __uint_as_float(__float_as_uint(__uint2float_rn(rem)) + ((unsigned)(e - 1075) << 23));
+  const bool lo_ok = rem != 0u && e > 1023 - 70;
+  df v;
+  v.hi = e < 1023 - 126 ? 0.f : e > 1023 + 127 ? __uint_as_float(0x7FFFFFFFu) : h;
+  v.lo = lo_ok ? __uint_as_float(__float_as_uint(r) | sign) : 0.f;
+  return v;
+}
+
+__device__ __forceinline__ unsigned long long turn_fraction(double T) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(T);
+  const int s = (int)((u >> 52) & 0x7FF) - 1011;            // T = m 2^(e - 1075), m the 53-bit significand
+  const unsigned long long m = (u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+  return s >= 0 ? (s < 64 ? m << s : 0ull) : (s > -64 ? m >> -s : 0ull);
+}
+
+// a b without the final renormalisation (|low word| a few ulp of the high one)
+__device__ __forceinline__ df df_mulq(df a, df b) {
+  const float p = __fmul_rn(a.hi, b.hi);
+  float e = fmaf(a.hi, b.hi, -p);
+  e = fmaf(a.hi, b.lo, e);
+  return df{p, fmaf(a.lo, b.hi, e)};
+}
+
+__device__ __forceinline__ PairTurns pair_turns(double T, df camp4) {   // camp4 = w/(4 pi)
+  PairTurns p;
+  p.v = turn_fraction(T);
+  p.T = df_split_bits(T);
+  // 1/sqrt(T): y = rsqrt(T) (2^-22), then y (1 + e/2 + 3 e^2/8) with e = 1 - T y^2 in double-float
+  const float y = rsqrtf(p.T.hi);
+  const float q = __fmul_rn(y, y), qe = fmaf(y, y, -q);
+  const float t = __fmul_rn(p.T.hi, q);
+  const float te = fmaf(p.T.lo, q, fmaf(p.T.hi, qe, fmaf(p.T.hi, q, -t)));
+  const float e = __fsub_rn(__fsub_rn(1.f, t), te);
+  df r;
+  quick_two_sum(y, __fmul_rn(y, __fmul_rn(e, fmaf(0.375f, e, 0.5f))), r.hi, r.lo);
+  p.iu = df_mul(r, r);
+  p.aw = df_mul(r, camp4);
+  return p;
+}
+
+// ln T for T > 0 (a normal float range): T = 2^e m, r = m rc - 1 (|r| < 0.006), the series of ln(1 + r) with its first
+// two terms in double-float.  Error about 2^-47.
+__device__ __forceinline__ df df_log(df T) {
+  const unsigned u = __float_as_uint(T.hi);
+  const int ex = (int)(u >> 23) - 127;
+  const float mh = __uint_as_float((u & 0x7FFFFFu) | 0x3F800000u);
+  const float ml = __fmul_rn(T.lo, __uint_as_float((unsigned)(127 - ex) << 23));
+  const float4 tb = __ldg(&c_log_df[(u >> 16) & 127u]);
+  const float p = __fmul_rn(mh, tb.x);
+  float rl = fmaf(ml, tb.x, fmaf(mh, tb.x, -p));
+  float rh = __fsub_rn(p, 1.f);                               // exact
+  quick_two_sum(rh, rl, rh, rl);
+  const float h = __fmul_rn(rh, rh), hl = fmaf(2.f * rh, rl, fmaf(rh, rh, -h));
+  const float c = __fmul_rn(__fmul_rn(h, rh), fmaf(rh, fmaf(rh, fmaf(rh, -1.f / 6.f, 0.2f), -0.25f), 1.f / 3.f));
+  df v;
+  quick_two_sum(rh, -0.5f * h, v.hi, v.lo);
+  v.lo = __fadd_rn(v.lo, __fadd_rn(fmaf(-0.5f, hl, rl), c));
+  constexpr float kLn2Hi = 0x1.62e4p-1f;                      // 15 bits: ex kLn2Hi is exact
+  constexpr double kLn2Rest = 0.69314718055994530941723212145817657 - 0.693145751953125;
+  constexpr df kLn2Lo = df_const(kLn2Rest);
+  const float fe = (float)ex;
+  df s, t;
+  two_sum(__fmul_rn(fe, kLn2Hi), tb.y, s.hi, s.lo);
+  s.lo = __fadd_rn(s.lo, tb.z);
+  two_sum(s.hi, v.hi, t.hi, t.lo);
+  t.lo = __fadd_rn(t.lo, __fadd_rn(s.lo, v.lo));
+  const float k = __fmul_rn(fe, kLn2Lo.hi);
+  two_sum(t.hi, k, s.hi, s.lo);
+  s.lo = __fadd_rn(__fadd_rn(s.lo, t.lo), fmaf(fe, kLn2Lo.lo, fmaf(fe, kLn2Lo.hi, -k)));
+  df r;
+  quick_two_sum(s.hi, s.lo, r.hi, r.lo);
+  if (!(T.hi > 0.f)) r = df{__uint_as_float(0xFF800000u), 0.f};
+  return r;
+}
+
+// J0 and Yhat0 at 0 <= z < 20.
+__device__ __forceinline__ df tayfine_eval(const float4 f, df c4, df c3, df c2, df c1, df c0, df d) {
+  const float t = fmaf(fmaf(fmaf(f.x, d.hi, f.y), d.hi, f.z), d.hi, f.w);   // c8..c5
+  df s = df_add_fast(df{__fmul_rn(t, d.hi), 0.f}, c4);
+  s = df_add_fast(df_mulq(s, d), c3);
+  s = df_add_fast(df_mulq(s, d), c2);
+  s = df_add_fast(df_mulq(s, d), c1);
+  return df_add_fast(df_mulq(s, d), c0);
+}
+__device__ __forceinline__ void bessel0_tayfine_df(df z, df& J0, df& Yh) {
+  const int k = min((int)(8.f * z.hi), kTayFine - 1);
+  const df d = df_add_fast(z, df{-(0.0625f + 0.125f * (float)k), 0.f});
+  const float4* t = c_tayfine_df[k];
+  const float4 a = __ldg(&t[0]), b = __ldg(&t[1]), c = __ldg(&t[2]), e = __ldg(&t[3]), f = __ldg(&t[4]),
+               g = __ldg(&t[5]), h = __ldg(&t[6]);
+  J0 = tayfine_eval(a, df{b.x, b.y}, df{b.z, b.w}, df{c.x, c.y}, df{c.z, c.w}, df{e.x, e.y}, d);
+  Yh = tayfine_eval(f, df{g.x, g.y}, df{g.z, g.w}, df{h.x, h.y}, df{h.z, h.w}, df{e.z, e.w}, d);
+}
+
+// Entry E = (amp (beta cos - sin), amp cos) at z >= 20; p = l v - 1/8 turn; ang: the angle table (shared memory).
+__device__ __forceinline__ float4 hankel_far_df(const PairTurns& pr, unsigned long long p, const float4* ang, df iv,
+                                                df rs, df beta, bool near) {
+  const df w = df_mul(pr.iu, iv);
+  const float sh = __fmul_rn(w.hi, w.hi), sl = fmaf(2.f * w.hi, w.lo, fmaf(w.hi, w.hi, -sh));
+  // g = s (25/48 - s rho)
+  constexpr df kG = df_const(25.0 / 48.0);
+  float rho = fmaf(sh, 109818.0144f, -4218.12863f);
+  rho = fmaf(sh, rho, 187.743036f);
+  rho = fmaf(sh, rho, -13.1045092f);
+  rho = fmaf(sh, rho, 1.67656250f);
+  const float gc = fmaf(-sh, rho, kG.lo);
+  const float gh = __fmul_rn(sh, kG.hi), gl = fmaf(sh, gc, fmaf(sl, kG.hi, fmaf(sh, kG.hi, -gh)));
+  // phi = -w/8 + (w/8) g = -q + (ah + al)
+  const float qh = 0.125f * w.hi, ql = 0.125f * w.lo;
+  const float ah = __fmul_rn(qh, gh), al = fmaf(ql, gh, fmaf(qh, gl, fmaf(qh, gh, -ah)));
+  // both high parts join the phase as integers of 2^-31 turns (|.| < 2^22: rounded by the FP32 add of 1.5 2^23)
+  constexpr double kTurn = 6.28318530717958647692 / 4294967296.0;    // 2^-32 turns in radians
+  constexpr df kT = df_const(kTurn), kT2 = df_const(2.0 * kTurn);
+  constexpr float kPerRad = (float)(0.5 / kTurn), kMagic = 12582912.f;
+  const float m1 = fmaf(qh, -kPerRad, kMagic), m2 = fmaf(ah, kPerRad, kMagic);
+  const float f1 = __fsub_rn(m1, kMagic), f2 = __fsub_rn(m2, kMagic);
+  const int n = (int)(__float_as_uint(m1) + __float_as_uint(m2) - 2u * 0x4B400000u) * 2;
+  float res = __fadd_rn(fmaf(f1, -kT2.hi, -qh), fmaf(f2, -kT2.hi, ah));
+  res = __fadd_rn(res, fmaf(-__fadd_rn(f1, f2), kT2.lo, __fsub_rn(al, ql)));
+  const unsigned hi = (unsigned)(p >> 32) + (unsigned)n;
+  const unsigned idx = (hi + 0x400000u) >> 23;
+  // integers below 2^22 and 2^23 to float by an exponent and a subtraction (the conversion unit is slower)
+  const float fr = __fsub_rn(__uint_as_float(0x4B400000u + (hi - (idx << 23))), kMagic);
+  const float fl = __fsub_rn(__uint_as_float(0x4B000000u | ((unsigned)p >> 9)), 8388608.f);
+  constexpr float kLow = (float)(kTurn / 8388608.0);
+  const float xh = __fmul_rn(fr, kT.hi);
+  float xl = fmaf(fr, kT.lo, fmaf(fr, kT.hi, -xh));
+  xl = __fadd_rn(fmaf(fl, kLow, xl), res);
+  // sin x = xh + sx, cos x - 1 = ch + cl
+  const float uh = __fmul_rn(xh, xh), ul = fmaf(2.f * xh, xl, fmaf(xh, xh, -uh));
+  const float ch = -0.5f * uh;
+  const float sx = fmaf(xh, __fmul_rn(uh, fmaf(uh, 1.f / 120.f, -1.f / 6.f)), fmaf(xl, ch, xl));
+  const float cl = fmaf(__fmul_rn(uh, uh), 1.f / 24.f, -0.5f * ul);
+  const float4 t = ang[idx & (kAngles - 1)];
+  // cos, sin of the sum: the corrections C ch -+ S x are small against the table value
+  df co, si;
+  {
+    const float A = __fmul_rn(t.z, xh), B = __fmul_rn(t.x, ch);
+    const float Ae = fmaf(t.w, xh, fmaf(t.z, sx, fmaf(t.z, xh, -A)));
+    const float Be = fmaf(t.y, ch, fmaf(t.x, cl, fmaf(t.x, ch, -B)));
+    float dh, dl;
+    quick_two_sum(-A, B, dh, dl);
+    quick_two_sum(t.x, dh, co.hi, co.lo);
+    co.lo = __fadd_rn(__fadd_rn(co.lo, t.y), __fadd_rn(dl, __fsub_rn(Be, Ae)));
+  }
+  {
+    const float A = __fmul_rn(t.x, xh), B = __fmul_rn(t.z, ch);
+    const float Ae = fmaf(t.y, xh, fmaf(t.x, sx, fmaf(t.x, xh, -A)));
+    const float Be = fmaf(t.w, ch, fmaf(t.z, cl, fmaf(t.z, ch, -B)));
+    float dh, dl;
+    quick_two_sum(A, B, dh, dl);
+    quick_two_sum(t.z, dh, si.hi, si.lo);
+    si.lo = __fadd_rn(__fadd_rn(si.lo, t.w), __fadd_rn(dl, __fadd_rn(Be, Ae)));
+  }
+  // amplitude: amp (1 - mu), mu = s/16 - s^2 kappa
+  float kap = fmaf(sh, -93.7731580f, 5.82897780f);
+  kap = fmaf(sh, kap, -0.542836961f);
+  kap = fmaf(sh, kap, 0.103515624f);
+  const float mh = 0.0625f * sh, ml = fmaf(-__fmul_rn(sh, sh), kap, 0.0625f * sl);
+  const df a0 = df_mulq(pr.aw, rs);
+  const float b = __fmul_rn(a0.hi, mh), be = fmaf(a0.lo, mh, fmaf(a0.hi, ml, fmaf(a0.hi, mh, -b)));
+  df amp;
+  quick_two_sum(a0.hi, -b, amp.hi, amp.lo);
+  amp.lo = __fadd_rn(amp.lo, __fsub_rn(a0.lo, be));
+  const df im = df_mulq(amp, co);
+  const df mr = near ? df_dot2(df_neg(beta), co, df{1.f, 0.f}, si) : si;     // -(beta cos - sin)
+  const df re = df_mulq(amp, mr);
+  return make_float4(-re.hi, -re.lo, im.hi, im.lo);
+}
+
+// Entry at z < 20: re = -(w/4) [((2/pi) Lz - beta) J0 + Yhat0], im = (w/4) J0 with Lz = ln(z/2) + gamma.
+__device__ __forceinline__ float4 hankel_near_df(df z, df Lz, df beta, bool near, df qw) {
+  constexpr df k2Pi = df_const(0.63661977236758134307553505349005745);
+  df J0, Yh;
+  bessel0_tayfine_df(z, J0, Yh);
+  df a = df_mul(Lz, k2Pi);
+  if (near) a = df_sub(a, beta);
+  const df re = df_mul(qw, df_dot2(a, J0, df{1.f, 0.f}, Yh));
+  const df im = df_mul(qw, J0);
+  return make_float4(-re.hi, -re.lo, im.hi, im.lo);
+}
+
+// Fills the tables above on the current device.
+inline cudaError_t init_hankel_df() {
+  static float4 ang[kAngles], lg[128], tf[kTayFine][7];
+  auto hi = [](double v) { return (float)v; };
+  auto lo = [](double v) { return (float)(v - (double)(float)v); };
+  for (int k = 0; k < kAngles; ++k) {
+    // the first octant's values, moved by symmetry, so that multiples of a quarter turn are exact
+    const int q = k / 128, r = k % 128;
+    const double a = 2.0 * 3.14159265358979323846 * (r <= 64 ? r : 128 - r) / 512.0;
+    const double c0 = r <= 64 ? std::cos(a) : std::sin(a), s0 = r <= 64 ? std::sin(a) : std::cos(a);
+    const double c = q == 0 ? c0 : q == 1 ? -s0 : q == 2 ? -c0 : s0, s = q == 0 ? s0 : q == 1 ? c0 : q == 2 ? -s0 : -c0;
+    ang[k] = make_float4(hi(c), lo(c), hi(s), lo(s));
+  }
+  for (int k = 0; k < 128; ++k) {
+    const double c = 1.0 + (k + 0.5) / 128.0, rc = std::nearbyint(512.0 / c) / 512.0, l = -std::log(rc);
+    lg[k] = make_float4((float)rc, hi(l), lo(l), 0.f);
+  }
+  double src[2][kTaylorIntervals][kTaylorDegree + 1];
+  cudaError_t e = cudaMemcpyFromSymbol(src[0], kTaylorJ0, sizeof src[0]);
+  if (e == cudaSuccess) e = cudaMemcpyFromSymbol(src[1], kTaylorYh, sizeof src[1]);
+  if (e != cudaSuccess) return e;
+  for (int k = 0; k < kTayFine; ++k) {
+    const double shift = (0.0625 + 0.125 * k) - (0.25 + 0.5 * (k / 4));
+    double c[2][9];
+    for (int f = 0; f < 2; ++f)
+      for (int n = 0; n <= 8; ++n) {      // c_n = sum_m binom(m, n) a_m shift^(m - n)
+        double v = 0.0, binom = 1.0, pw = 1.0;
+        for (int m = n; m <= kTaylorDegree; ++m) {
+          v += binom * src[f][k / 4][m] * pw;
+          binom = binom * (m + 1) / (m + 1 - n);
+          pw *= shift;
+        }
+        c[f][n] = v;
+      }
+    const double *j = c[0], *y = c[1];
+    tf[k][0] = make_float4(hi(j[8]), hi(j[7]), hi(j[6]), hi(j[5]));
+    tf[k][1] = make_float4(hi(j[4]), lo(j[4]), hi(j[3]), lo(j[3]));
+    tf[k][2] = make_float4(hi(j[2]), lo(j[2]), hi(j[1]), lo(j[1]));
+    tf[k][3] = make_float4(hi(j[0]), lo(j[0]), hi(y[0]), lo(y[0]));
+    tf[k][4] = make_float4(hi(y[8]), hi(y[7]), hi(y[6]), hi(y[5]));
+    tf[k][5] = make_float4(hi(y[4]), lo(y[4]), hi(y[3]), lo(y[3]));
+    tf[k][6] = make_float4(hi(y[2]), lo(y[2]), hi(y[1]), lo(y[1]));
+  }
+  if ((e = cudaMemcpyToSymbol(c_angle_df, ang, sizeof ang)) != cudaSuccess) return e;
+  if ((e = cudaMemcpyToSymbol(c_log_df, lg, sizeof lg)) != cudaSuccess) return e;
+  return cudaMemcpyToSymbol(c_tayfine_df, tf, sizeof tf);
+}
+
+}  // namespace fthms

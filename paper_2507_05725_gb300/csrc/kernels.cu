@@ -16,11 +16,13 @@
 //                  memory, with a radix-2 FFT
 //   traces         u_M(z, t) at the output times (eq. mult-scatt-int)
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 
 #include "bessel.cuh"
 #include "cplx.cuh"
 #include "df64.cuh"
+#include "hankel_df.cuh"
 #include "kernels.h"
 #include "lu_common.cuh"
 
@@ -51,7 +53,8 @@ cudaError_t init_constants() {
       td[0][k][n] = make_float2(a, (float)(tj[k][n] - (double)a));
       td[1][k][n] = make_float2(c, (float)(ty[k][n] - (double)c));
     }
-  return cudaMemcpyToSymbol(c_taylor_df, td, sizeof td);
+  e = cudaMemcpyToSymbol(c_taylor_df, td, sizeof td);
+  return e == cudaSuccess ? init_hankel_df() : e;
 }
 
 namespace {
@@ -99,6 +102,21 @@ __global__ void k_freq_tw(DevJob J) {
   double2 sy = cmul(e1, e2);
   J.syn_tw[idx] = make_double2(wl * sy.x, wl * sy.y);
   J.fwd_tw[idx] = make_double2(J.dt * c, J.dt * s);
+}
+
+// Per-frequency constants of the double-float Hankel entries (mixed forms).
+__global__ void k_freq_df(DevJob J) {
+  const int l = blockIdx.x * blockDim.x + threadIdx.x;
+  if (l >= J.L) return;
+  const double x = l > 0 ? (double)l : 1.0, ln = log(x);
+  const df a = df_from(2.0 * kPiD * x), b = df_from(0.5 * kInvPi / x), c = df_from(rsqrt(x)),
+           d = df_from(ln + 1.7219455507509330);      // ln pi + gamma
+  FreqDf f;
+  f.a = make_float4(a.hi, a.lo, b.hi, b.lo);
+  f.b = make_float4(c.hi, c.lo, d.hi, d.lo);
+  f.lnl = ln;
+  f.pad = 0.0;
+  J.freq_df[l] = f;
 }
 
 // Cosine sums F(m) = sum_{n=1}^{N-1} cos(n m pi/N)/n, m = 0..N, of the self log weights
@@ -825,61 +843,77 @@ __device__ __forceinline__ void store_entry(const DevJob& J, double2* p, double2
 }
 constexpr int kAsmBand = 64;   // frequencies per assembly task (matches the planner's band cap)
 
-// Near-rule product-integration weights of the rows of one task at N source nodes (block-wide, all
-// threads call): Wn[r * N + i] = (lambda_0 + 2 sum_n lambda_n T_n(t_i)) / N for the near rows r, with
-// lambda_n(t*) = int log|t* - s| T_n(s)/sqrt(1-s^2) ds for |t*| > 1, = -pi zeta^n / n (n >= 1); the sum
-// stops where |zeta|^n < 1e-18 (the omitted terms are below 1e-17 of the weights).  ctab: 4N doubles,
-// lam: kAsmRows x N doubles of shared memory; Wn may be shared or global memory.
-__device__ void near_weights_block(const CrossTgt* tg, int nrows, int N, double* ctab, double* lam, double* Wn) {
-  __shared__ int s_nlam[kAsmRows];
-  for (int r = threadIdx.x; r < 4 * N; r += blockDim.x) ctab[r] = cospi((double)r / (2.0 * N));
-  if (threadIdx.x < nrows && tg[threadIdx.x].near) {
-    const double ts = tg[threadIdx.x].tstar;
-    const double rt = sqrt(fma(ts, ts, -1.0));
-    const double zeta = ts > 0 ? ts - rt : ts + rt;
-    double* lr = lam + threadIdx.x * N;
-    lr[0] = kPiD * log(0.5 * (fabs(ts) + rt));
-    double pw = 1.0;
-    int n = 1;
-    for (; n < N; ++n) {
-      pw *= zeta;
-      if (fabs(pw) < 1e-18) break;
-      lr[n] = -kPiD * pw / n;
+// Near-rule corrections of the rows of one task at N source nodes (block-wide, all threads call), in FP64:
+// beta[r * N + i] = -(2/pi)(W_i/w - ln|t* - t_i|) for the near rows r, with the product-integration weights
+// W_i = (lambda_0 + 2 sum_{n<N} lambda_n T_n(t_i)) / N, lambda_n(t*) = int log|t* - s| T_n(s)/sqrt(1-s^2) ds for
+// |t*| > 1, = -pi zeta^n / n (n >= 1).  The whole series sums to ln|t* - t_i| (beta is its tail from n = N on), so a row
+// with |zeta|^N < 1e-18 has beta = 0 and is marked by +0.0 at every node without any sum (an exact zero of the formula
+// would come out as -0.0): of the near rows only those next to the arc's ends keep the N-term sums and the
+// logarithms.  12-arc cavity, table of all rows: 13.9 -> 1.9 ms.  tn: the nodes t_i; ctab: 4N doubles, lam: kAsmRows x N
+// doubles of shared memory; beta may be shared or global memory.
+__device__ void near_beta_block(const CrossTgt* tg, int nrows, int N, const double* __restrict__ tn, double* ctab,
+                                double* lam, double* beta) {
+  __shared__ int s_full[kAsmRows], s_any;
+  if (threadIdx.x == 0) s_any = 0;
+  __syncthreads();
+  if (threadIdx.x < nrows) {
+    int full = 0;
+    if (tg[threadIdx.x].near) {
+      const double ts = tg[threadIdx.x].tstar;
+      const double rt = sqrt(fma(ts, ts, -1.0));
+      const double zeta = ts > 0 ? ts - rt : ts + rt;
+      if (!(N * log(fabs(zeta)) < -41.4465)) {            // |zeta|^N >= 1e-18 (or not a number)
+        full = 1;
+        s_any = 1;
+        double* lr = lam + threadIdx.x * N;
+        lr[0] = kPiD * log(0.5 * (fabs(ts) + rt));
+        double pw = 1.0;
+        for (int n = 1; n < N; ++n) {
+          pw *= zeta;
+          lr[n] = -kPiD * pw / n;
+        }
+      }
     }
-    s_nlam[threadIdx.x] = n;
+    s_full[threadIdx.x] = full;
   }
   __syncthreads();
+  if (s_any) {
+    for (int r = threadIdx.x; r < 4 * N; r += blockDim.x) ctab[r] = cospi((double)r / (2.0 * N));
+    __syncthreads();
+  }
   for (int e = threadIdx.x; e < nrows * N; e += blockDim.x) {
-    int r = e / N, i = e % N;
+    const int r = e / N, i = e % N;
     if (!tg[r].near) continue;
-    const double* lr = lam + r * N;
-    const int step = 2 * i + 1, mod = 4 * N, nlam = s_nlam[r];
-    double acc = 0.0;
-    int ph = 0;
-    for (int n = 1; n < nlam; ++n) {
-      ph += step;
-      if (ph >= mod) ph -= mod;
-      acc = fma(lr[n], ctab[ph], acc);
+    double v = 0.0;
+    if (s_full[r]) {
+      const double* lr = lam + r * N;
+      const int step = 2 * i + 1, mod = 4 * N;
+      double acc = 0.0;
+      int ph = 0;
+      for (int n = 1; n < N; ++n) {
+        ph += step;
+        if (ph >= mod) ph -= mod;
+        acc = fma(lr[n], ctab[ph], acc);
+      }
+      v = -kTwoOverPi * fma(lr[0] + 2.0 * acc, kInvPi, -log(fabs(tg[r].tstar - tn[i])));
     }
-    Wn[r * N + i] = (lr[0] + 2.0 * acc) / N;
+    beta[r * N + i] = v;
   }
   __syncthreads();
 }
 
 // Quantities of one (target row, source node) pair shared by every frequency of a band.  Every entry,
 // near or far, is E = (alpha J0 - (w/4) Y, (w/4) J0) with Y = Yhat0 below z = 20 and Y0 above;
-// alpha = A0 + A1 ln l below 20 and beta w/4 above.
-//   far rule:  A0 = -(w/(2 pi)) (ln(hR/2) + gamma),  beta = 0;
-//   near rule: the log-singular part K1 ln|t* - s| is integrated with the weights wn instead of w,
-//              so A0 = -(wn + w (ln(hR/2) + gamma - ln|t* - t_i|))/(2 pi) and
-//              beta = -(2/pi)(wn/w - ln|t* - t_i|).
+// alpha = A0 + A1 ln l below 20, A0 = -(w/(2 pi)) (ln(hR/2) + gamma) + beta w/4, and beta w/4 above.  beta = 0 for
+// the far rule; for the near rule the log-singular part K1 ln|t* - s| is integrated with the weights W_i instead
+// of w, which adds beta (near_beta_block).
 struct PairSetup {
   double R, hR, inv_u, A0, beta;
   int lsw;     // first frequency index with z = l h R >= 20
 };
 
-__device__ __forceinline__ PairSetup pair_setup(const DevJob& J, const CrossTgt& t, double xi, double yi, double ti,
-                                                double wn, int l0, double w, double invw, double inv_h) {
+__device__ __forceinline__ PairSetup pair_setup(const DevJob& J, const CrossTgt& t, double xi, double yi, double beta,
+                                                int l0, double w, double inv_h) {
   PairSetup s;
   const double dx = t.x - xi, dy = t.y - yi;
   const double R2 = fma(dx, dx, dy * dy);
@@ -890,15 +924,8 @@ __device__ __forceinline__ PairSetup pair_setup(const DevJob& J, const CrossTgt&
   s.inv_u = rinv * inv_h;                        // 1 / (h R)
   s.lsw = max(l0, (int)ceil(fmin(kBesselLarge * s.inv_u, 1.0e9)));
   s.A0 = 0.0;
-  s.beta = 0.0;
-  double lt = 0.0;
-  if (t.near) {
-    lt = log(fabs(t.tstar - ti));
-    s.beta = -kTwoOverPi * fma(wn, invw, -lt);
-  } else {
-    wn = 0.0;
-  }
-  if (s.lsw > l0) s.A0 = -0.5 * kInvPi * fma(w, log(0.5 * s.hR) + kEulerGamma - lt, wn);
+  s.beta = beta;
+  if (s.lsw > l0) s.A0 = w * fma(-0.5 * kInvPi, log(0.5 * s.hR) + kEulerGamma, 0.25 * beta);
   return s;
 }
 
@@ -974,7 +1001,7 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
   const CrossTgt* tg = J.tgts + pr.tgt_off + task.row0;
   double* ctab = sha;                                // 4N: cospi(r/(2N))
   double* lam = sha + 4 * N;                         // kAsmRows x N
-  double* Wn = kNear ? lam + kAsmRows * N : sha;     // kAsmRows x N near weights (near launch only)
+  double* Wn = kNear ? lam + kAsmRows * N : sha;     // kAsmRows x N near corrections beta (near launch only)
   __shared__ int any_near;
   if (threadIdx.x == 0) {
     int a = 0;
@@ -983,8 +1010,8 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
   }
   __syncthreads();
   if ((any_near != 0) != kNear) return;
-  if (kNear) near_weights_block(tg, task.nrows, N, ctab, lam, Wn);
-  const double w = kPiD / N, qw = 0.25 * w, invw = N * kInvPi;
+  if (kNear) near_beta_block(tg, task.nrows, N, J.node_t + pn.off, ctab, lam, Wn);
+  const double w = kPiD / N, qw = 0.25 * w;
   const double A1 = -0.5 * kInvPi * w;          // coefficient of ln l below z = 20
   const double camp = kSqrtTwoOverPi * qw;      // sqrt(2/pi) w/4
   const double inv_h = 1.0 / J.h;
@@ -1017,8 +1044,8 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
   for (int e = threadIdx.x; e < task.nrows * N; e += blockDim.x) {
     const int r = e % task.nrows, i = e / task.nrows;
     const CrossTgt t = tg[r];
-    const PairSetup ps = pair_setup(J, t, J.node_x[pn.off + i], J.node_y[pn.off + i], J.node_t[pn.off + i],
-                                    kNear && t.near ? Wn[r * N + i] : 0.0, task.l0, w, invw, inv_h);
+    const PairSetup ps = pair_setup(J, t, J.node_x[pn.off + i], J.node_y[pn.off + i],
+                                    kNear && t.near ? Wn[r * N + i] : 0.0, task.l0, w, inv_h);
     double2* Ep = J.E + (long long)i * ld + task.row0 + r;
     const int lend = min(ps.lsw, task.l1 + 1);
     if (J.mixed && !J.fp64keep) {
@@ -1091,7 +1118,7 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Cross rows evaluated every step (cross_mode 1), nothing stored.  Near weights first, once per job,
+// Cross rows evaluated every step (cross_mode 1), nothing stored.  Near corrections beta first, once per job,
 // into a table (one slab of nrows x N per assembly task with near rows).
 __global__ void __launch_bounds__(kAsmThreads) k_near_weights(DevJob J) {
   const long long off = J.wn_off[blockIdx.x];
@@ -1099,7 +1126,7 @@ __global__ void __launch_bounds__(kAsmThreads) k_near_weights(DevJob J) {
   extern __shared__ double shn[];
   const CrossAsm task = J.asms[blockIdx.x];
   const CrossTgt* tg = J.tgts + J.pairs[task.pair].tgt_off + task.row0;
-  near_weights_block(tg, task.nrows, task.N, shn, shn + 4 * task.N, J.wn + off);
+  near_beta_block(tg, task.nrows, task.N, J.node_t + J.panels[task.panel].off, shn, shn + 4 * task.N, J.wn + off);
 }
 
 // One CTA per (assembly task, band of at most otf_band(Q) frequencies): thread (row r, source group g)
@@ -1132,7 +1159,7 @@ __global__ void __launch_bounds__(kAsmThreads) k_cross_otf(DevJob J) {
   double2* mine = sho + threadIdx.x;                  // slot e at mine[e * kAsmThreads]
   for (int e = 0; e < Q * B; ++e) mine[e * kAsmThreads] = make_double2(0.0, 0.0);
   __syncthreads();
-  const double w = kPiD / N, qw = 0.25 * w, invw = N * kInvPi;
+  const double w = kPiD / N, qw = 0.25 * w;
   const double A1 = -0.5 * kInvPi * w;
   const double camp = kSqrtTwoOverPi * qw;
   const double inv_h = 1.0 / J.h;
@@ -1141,8 +1168,8 @@ __global__ void __launch_bounds__(kAsmThreads) k_cross_otf(DevJob J) {
     const CrossTgt t = tg[r];
     const SysDesc* sj = J.sys + (long long)pr.j * (J.L - 1) + (ot.l0 - 1);   // systems (j, l0..l1)
     for (int i = g; i < N; i += G) {
-      const PairSetup ps = pair_setup(J, t, J.node_x[pn.off + i], J.node_y[pn.off + i], J.node_t[pn.off + i],
-                                      t.near ? Wn[r * N + i] : 0.0, ot.l0, w, invw, inv_h);
+      const PairSetup ps = pair_setup(J, t, J.node_x[pn.off + i], J.node_y[pn.off + i],
+                                      t.near ? Wn[r * N + i] : 0.0, ot.l0, w, inv_h);
       AsymState as{};
       bool started = false;
       for (int b = 0; b < nl; ++b) {
@@ -1174,224 +1201,141 @@ __global__ void __launch_bounds__(kAsmThreads) k_cross_otf(DevJob J) {
   }
 }
 
-// Mixed forms, cross rows evaluated every step in double-float (on the FP32 pipe).  One CTA per (assembly
-// task of kAsmRows target rows, band of at most kOtfBandDf frequencies), kOtfDfThreads threads, sources in
-// tiles of kOtfDfSrc:
-//  1. thread (row r, source i of the tile): the pair's FP64 set-up once (pair_setup), then the entries of
-//     every frequency of the band -- below z = 20 the Taylor form (double-float; FP64 rounded to double-float
-//     in the FP64-kept form), above it Hankel's expansion with its phase advanced by the double-float
-//     rotation e^{i h R} (re-seeded every 16 steps), exactly as the mixed stored-row assembly -- into shared
-//     memory; the tile's double-float densities phi(omega_l) are staged beside them;
-//  2. thread (row, frequency): sum over the tile's sources of entry x density for every window, with
-//     compensated double-float accumulation in source order (deterministic), carried across the tiles.
-// The per-row sums go to the per-row results that k_cross_reduce adds per target in block order.
-constexpr int kOtfDfSrc = 16;
-constexpr int kOtfDfThreads = kAsmRows * kOtfDfSrc;   // 128
-constexpr int kOtfDfPitch = kOtfBandDf + 1;           // float4 per shared-memory row (odd: no bank conflicts)
+// Mixed forms, cross rows evaluated every step in double-float (on the FP32 pipe).  One CTA of kAsmRows warps per
+// (assembly task of kAsmRows target rows, band of at most kOtfBandDf frequencies): warp = target row, lane = source
+// node (s0 + lane, so node coordinates and densities load coalesced and the near rule is warp-uniform), frequencies
+// in register blocks of otf_regs(Q).  A lane sets its pair up in turns (PairTurns), evaluates each entry and multiplies
+// it straight into its own compensated double-float sums, one per (frequency, window); the 32 lanes' sums are added
+// once per block of frequencies.  Entries never leave registers.  An earlier form wrote them to shared memory and
+// summed with one thread per (row, frequency): at bands of one or two frequencies (N grows with every step of omega)
+// 8 to 16 of its 128 threads worked, and each pair paid two sine/cosine series; 12-arc cavity, 5.7e8 pairs x 5 steps,
+// four windows: 501 -> 91 ms; 6 arcs at N = 1024, two windows:
+// 499 -> 335 ms.  Bound by FP32 issue (~125 instructions an entry and 48 a window).
+// kKeep64 (the FP64-kept form): entries below z = 20 from the FP64 Taylor form.
+constexpr int kOtfThreads = 32 * kAsmRows;
+__host__ __device__ constexpr int otf_regs(int Q) { return Q == 1 ? 8 : Q == 2 ? 4 : 1; }
+// blocks per SM: 16 warps of 128 registers, or 24 of 80 where the few sums leave room (measured per Q)
+constexpr int otf_blocks(int Q) { return Q <= 2 ? 2 : 3; }
 
-// sin and cos of theta >= 0 (FP64, up to ~2e4) as double-float: theta reduced by n pi/2 in FP64 (pi/2 as the
-// sum of two doubles), the remainder's double-float Taylor series, the quadrant n mod 4.
-__device__ __forceinline__ void df_sincos_reduced(double theta, df& s, df& c) {
-  constexpr double kPio2Hi = 1.57079632679489661923, kPio2Lo = 6.123233995736766e-17;
-  const double n = rint(theta * kTwoOverPi);
-  const double r = fma(-n, kPio2Lo, fma(-n, kPio2Hi, theta));
-  df sr, cr;
-  df_sincos_taylor(df_from(r), sr, cr);
-  switch (((long long)n) & 3) {
-    case 0: s = sr; c = cr; break;
-    case 1: s = cr; c = df_neg(sr); break;
-    case 2: s = df_neg(sr); c = df_neg(cr); break;
-    default: s = df_neg(cr); c = sr; break;
+// V double-float sums of a warp's lanes added over the lanes (V a power of two <= 32): each halving step keeps one
+// half of the values and hands the other to the partner lane, so lane e << s (s = log2(32/V)) ends with sum e.
+template <int V>
+__device__ __forceinline__ void df_warp_sums(dfacc (&a)[V], int lane) {
+  int w = 16;
+#pragma unroll
+  for (int n = V / 2; n >= 1; n >>= 1, w >>= 1) {
+    const bool up = (lane & w) != 0;
+#pragma unroll
+    for (int e = 0; e < n; ++e) {
+      const dfacc lo = a[e], hi = a[e + n];
+      const float gh = up ? lo.hi : hi.hi, gl = up ? lo.lo : hi.lo;
+      a[e] = up ? hi : lo;
+      a[e].add(__shfl_xor_sync(0xffffffffu, gh, w), __shfl_xor_sync(0xffffffffu, gl, w));
+    }
+  }
+  for (; w >= 1; w >>= 1) {
+    const float gh = a[0].hi, gl = a[0].lo;
+    a[0].add(__shfl_xor_sync(0xffffffffu, gh, w), __shfl_xor_sync(0xffffffffu, gl, w));
   }
 }
 
-// The per-pair quantities of pair_setup on the FP32 pipe (mixed forms, cross rows every step): the distance
-// R from the FP64 coordinate differences by a double-float square root, 1/(hR) and the amplitude
-// sqrt(2/(pi hR)) w/4 in double-float; FP64 only for the differences, the logarithms of the near rule and
-// of the Taylor range (present in the low-frequency bands only) and R itself for the phase reductions.
-struct PairDf {
-  df R, invu, A0, beta, ampw;
-  double R64;
-  float hR;
-  int lsw;
-};
-
-__device__ __forceinline__ PairDf pair_setup_df(const DevJob& J, const CrossTgt& t, double xi, double yi, double ti,
-                                                double wn, int l0, double w, double invw, df h_d, df camp_d) {
-  PairDf p;
-  const double dx = t.x - xi, dy = t.y - yi;
-  p.R = df_sqrt(df_from(fma(dx, dx, dy * dy)));
-  p.R64 = (double)p.R.hi + (double)p.R.lo;
-  const df hR = df_mul(h_d, p.R);
-  p.hR = hR.hi;
-  p.invu = df_div(df{1.f, 0.f}, hR);
-  p.lsw = max(l0, (int)ceilf(fminf((float)kBesselLarge * p.invu.hi, 1.0e9f)));
-  double lt = 0.0, beta = 0.0, A0 = 0.0;
-  if (t.near) {
-    lt = log(fabs(t.tstar - ti));
-    beta = -kTwoOverPi * fma(wn, invw, -lt);
-  } else {
-    wn = 0.0;
-  }
-  if (p.lsw > l0) A0 = -0.5 * kInvPi * fma(w, log(0.5 * J.h * p.R64) + kEulerGamma - lt, wn);
-  p.A0 = df_from(A0);
-  p.beta = df_from(beta);
-  p.ampw = df_mul(df_rsqrt(hR), camp_d);
-  return p;
-}
-
-// Double-float state of Hankel's expansion along a band (the mixed stored-row assembly's recurrence).
-struct AsymDf {
-  df cx, sx, cu, su, ampw, invu, beta;
-  int since, kmax;
-};
-
-__device__ __forceinline__ AsymDf asym_df_start(const PairDf& p, double lh_first, double h) {
-  AsymDf a;
-  a.ampw = p.ampw;
-  a.invu = p.invu;
-  a.beta = p.beta;
-  a.kmax = hankel_terms((float)(lh_first * p.R64));
-  if (p.hR <= 1.0f) df_sincos_taylor(df_from(h * p.R64), a.su, a.cu);
-  else df_sincos_reduced(h * p.R64, a.su, a.cu);
-  a.cx = a.sx = df{0.f, 0.f};
-  a.since = 16;
-  return a;
-}
-
-__device__ __forceinline__ float4 asym_df_entry(AsymDf& a, double lhR, df invl, df rsql) {
-  if (a.since >= 16) {
-    df_phase_seed(lhR, a.cx, a.sx);
-    a.since = 0;
-  }
-  const df wz = df_mul(a.invu, invl);
-  const df w2 = df_neg(df_mul(wz, wz));
-  df P, Qa;
-  hankel_pq_df(a.kmax, w2, P, Qa);
-  Qa = df_mul(Qa, wz);
-  const df amp = df_mul(a.ampw, rsql);
-  const df t1 = df_dot2(P, a.cx, Qa, a.sx);
-  const df t2 = df_dot2(P, a.sx, df_neg(Qa), a.cx);
-  const df re = df_mul(amp, df_dot2(a.beta, t1, df{-1.f, 0.f}, t2));
-  const df im = df_mul(amp, t1);
-  const df cn = df_dot2(a.cx, a.cu, df_neg(a.sx), a.su);
-  a.sx = df_dot2(a.sx, a.cu, a.cx, a.su);
-  a.cx = cn;
-  ++a.since;
-  return make_float4(re.hi, re.lo, im.hi, im.lo);
-}
-
-template <int Q>
-__global__ void __launch_bounds__(kOtfDfThreads) k_cross_otf_df(DevJob J) {
-  constexpr int B = kOtfBandDf;
-  extern __shared__ __align__(16) unsigned char sho_raw[];
-  // entries [row][source][band] and densities [window][source][band], rows of kOtfDfPitch float4: a warp
-  // of phase 2 (one row or window, 32 frequencies) reads 32 consecutive float4, a warp of phase 1 writes
-  // with a 33-float4 stride (both at the minimum of 4 shared-memory wavefronts)
-  float4* Et = reinterpret_cast<float4*>(sho_raw);                 // [kAsmRows * kOtfDfSrc][kOtfDfPitch]
-  float4* Ps = Et + kAsmRows * kOtfDfSrc * kOtfDfPitch;            // [Q * kOtfDfSrc][kOtfDfPitch]
-  __shared__ double tb[4][B];                                       // 1/l, 1/sqrt(l), ln l, l h
-  __shared__ df tbd[4][B];                                          // the same as double-float
+template <int Q, bool kKeep64>
+__global__ void __launch_bounds__(kOtfThreads, otf_blocks(Q)) k_cross_otf_df(DevJob J) {
+  constexpr int B = kOtfBandDf, NB = otf_regs(Q);
+  constexpr int V = NB * (Q == 3 ? 4 : Q) * 2;                      // sums per warp, a power of two
+  __shared__ float4 ang[kAngles];
+  __shared__ FreqDf fr[B];
   __shared__ long long vo[B];                                       // density offsets of the band's systems
-  const CrossOtf ot = J.otf_tasks[blockIdx.x];
+  __shared__ df s_qw, s_camp4;                                      // w/4, w/(4 pi), one thread's FP64
+  // blocks in a strided order: the low-frequency tasks (FP64 Taylor range of the FP64-kept form) are neighbours in
+  // the list and spread over the launch, so the FP64 pipe works beside the other blocks' FP32
+  const long long nt = J.n_otf, stride = J.otf_stride;
+  const CrossOtf ot = J.otf_tasks[(int)((long long)blockIdx.x * stride % nt)];
   const CrossAsm task = J.asms[ot.task];
   const PairDesc pr = J.pairs[task.pair];
   const int N = task.N, nl = ot.l1 - ot.l0 + 1;
   const Panel pn = J.panels[task.panel];
-  const CrossTgt* tg = J.tgts + pr.tgt_off + task.row0;
   const long long woff = J.wn_off[ot.task];
-  const double* Wn = woff >= 0 ? J.wn + woff : nullptr;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, r = tid >> 5;
+  for (int k = tid; k < kAngles; k += kOtfThreads) ang[k] = c_angle_df[k];
   if (tid < nl) {
-    const int l = ot.l0 + tid;
-    tb[0][tid] = 1.0 / l;
-    tb[1][tid] = rsqrt((double)l);
-    tb[2][tid] = log((double)l);
-    tb[3][tid] = l * J.h;
-    for (int k = 0; k < 4; ++k) tbd[k][tid] = df_from(tb[k][tid]);
-    vo[tid] = J.sys[(long long)pr.j * (J.L - 1) + (l - 1)].vec_off;
+    fr[tid] = J.freq_df[ot.l0 + tid];
+    vo[tid] = J.sys[(long long)pr.j * (J.L - 1) + (ot.l0 + tid - 1)].vec_off;
+  }
+  if (tid == kOtfThreads - 1) {
+    const double w4 = 0.25 * kPiD / N;
+    s_qw = df_from(w4);
+    s_camp4 = df_from(w4 * kInvPi);
   }
   __syncthreads();
-  const double w = kPiD / N, qw = 0.25 * w, invw = N * kInvPi;
-  const double A1 = -0.5 * kInvPi * w;
-  const double camp = kSqrtTwoOverPi * qw;
-  const double inv_h = 1.0 / J.h;
-  const df A1_d = df_from(A1), qw_d = df_from(qw), h_d = df_from(J.h), camp_d = df_from(camp);
-  // phase-2 accumulators: thread owns (row, band) pairs p = tid, tid + kOtfDfThreads (row = p / B)
-  constexpr int kPairs = kAsmRows * B / kOtfDfThreads;
-  dfacc acc_re[kPairs][Q], acc_im[kPairs][Q];
-  const int r1 = tid / kOtfDfSrc, i1 = tid % kOtfDfSrc;            // phase-1 pair
-  for (int s0 = 0; s0 < N; s0 += kOtfDfSrc) {
-    const int i = s0 + i1;
-    float4* Ep = Et + (r1 * kOtfDfSrc + i1) * kOtfDfPitch;          // + b
-    if (r1 < task.nrows && i < N) {
-      const CrossTgt t = tg[r1];
-      const double xi = J.node_x[pn.off + i], yi = J.node_y[pn.off + i], ti = J.node_t[pn.off + i];
-      const double wni = t.near ? Wn[r1 * N + i] : 0.0;
-      const PairDf pd = pair_setup_df(J, t, xi, yi, ti, wni, ot.l0, w, invw, h_d, camp_d);
-      const int lend = min(pd.lsw, ot.l1 + 1);
-      if (lend > ot.l0) {                                           // z < 20: Taylor form
-        PairSetup ps{};
-        if (J.fp64keep) ps = pair_setup(J, t, xi, yi, ti, wni, ot.l0, w, invw, inv_h);
-        for (int l = ot.l0; l < lend; ++l) {
-          const int b = l - ot.l0;
-          float4 e;
-          if (J.fp64keep) {
-            e = df_split2(taylor_entry(ps, tb[3][b], tb[2][b], A1, qw));
+  if (r >= task.nrows) return;
+  const CrossTgt t = J.tgts[pr.tgt_off + task.row0 + r];
+  const double* __restrict__ bt = t.near ? J.wn + woff + (long long)r * N : nullptr;
+  const bool near = bt && __double_as_longlong(__ldg(bt)) != 0;     // (+0.0: beta vanishes on the whole row)
+  const double w = kKeep64 ? kPiD / N : 0.0, turns = J.h * (0.5 * kInvPi);
+  const df qw = s_qw, camp4 = s_camp4;
+  const double* __restrict__ nx = J.node_x + pn.off;
+  const double* __restrict__ ny = J.node_y + pn.off;
+#pragma unroll 1
+  for (int b0 = 0; b0 < nl; b0 += NB) {
+    const int nb = min(NB, nl - b0);
+    dfacc acc[V];
+    // T one step ahead: its chain of dependent FP64 operations runs beside the current pair's entries
+    auto turns_at = [&](int i) {
+      const double dx = t.x - __ldg(&nx[i]), dy = t.y - __ldg(&ny[i]);
+      return turns * dist_f64(fma(dx, dx, dy * dy));
+    };
+    double Tn = turns_at(min(lane, N - 1));
+#pragma unroll 1
+    for (int i = lane; i < N; i += 32) {
+      const double T = Tn;
+      if (i - lane + 32 < N) Tn = turns_at(min(i + 32, N - 1));
+      const PairTurns pt = pair_turns(T, camp4);
+      double beta64 = 0.0;
+      df beta{0.f, 0.f};
+      if (near) {
+        beta64 = __ldg(&bt[i]);
+        beta = df_split_bits(beta64);
+      }
+      df lnT{0.f, 0.f};
+      double A0 = 0.0;
+      if (pt.T.hi * fr[b0].a.x < (float)kBesselLarge) {             // the block's first entry is below z = 20
+        if (kKeep64) A0 = w * fma(-0.5 * kInvPi, log(T) + 1.7219455507509330, 0.25 * beta64);   // + ln pi + gamma
+        else lnT = df_log(pt.T);
+      }
+      unsigned long long ph = pt.v * (unsigned long long)(ot.l0 + b0) - (1ull << 61);
+#pragma unroll
+      for (int k = 0; k < NB; ++k) {
+        if (k < nb) {
+          const FreqDf& f = fr[b0 + k];
+          float4 pv[Q], e;
+#pragma unroll
+          for (int q = 0; q < Q; ++q) pv[q] = __ldg(&J.phi_df[vo[b0 + k] + i + (long long)q * N]);
+          if (pt.T.hi * f.a.x < (float)kBesselLarge) {
+            if (kKeep64) {
+              double J0, Yh;
+              bessel0_taylor(T * ((2.0 * kPiD) * (double)(ot.l0 + b0 + k)), J0, Yh);
+              const double alpha = fma(-0.5 * kInvPi * w, f.lnl, A0);
+              e = df_split2(make_double2(fma(alpha, J0, -0.25 * w * Yh), 0.25 * w * J0));
+            } else {
+              e = hankel_near_df(df_mul(pt.T, df{f.a.x, f.a.y}), df_add_fast(lnT, df{f.b.z, f.b.w}), beta, near, qw);
+            }
           } else {
-            df J0, Yh;
-            bessel0_taylor_df(df_mul(tbd[3][b], pd.R), J0, Yh);
-            const df alpha = df_add_fast(df_mul(A1_d, tbd[2][b]), pd.A0);
-            const df re = df_dot2(alpha, J0, df_neg(qw_d), Yh);
-            const df im = df_mul(qw_d, J0);
-            e = make_float4(re.hi, re.lo, im.hi, im.lo);
+            e = hankel_far_df(pt, ph, ang, df{f.a.z, f.a.w}, df{f.b.x, f.b.y}, beta, near);
           }
-          Ep[b] = e;
-        }
-      }
-      if (lend <= ot.l1) {
-        AsymDf as = asym_df_start(pd, tb[3][lend - ot.l0], J.h);
-        for (int l = lend; l <= ot.l1; ++l) {
-          const int b = l - ot.l0;
-          Ep[b] = asym_df_entry(as, tb[3][b] * pd.R64, tbd[0][b], tbd[1][b]);
-        }
-      }
-    } else {
-      for (int b = 0; b < nl; ++b) Ep[b] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    // the tile's densities phi_q(omega_l)[s0 .. s0 + kOtfDfSrc) (zero past N)
-    for (int e = tid; e < nl * Q * kOtfDfSrc; e += kOtfDfThreads) {
-      const int ii = e % kOtfDfSrc, q = (e / kOtfDfSrc) % Q, b = e / (kOtfDfSrc * Q);
-      Ps[(q * kOtfDfSrc + ii) * kOtfDfPitch + b] =
-          s0 + ii < N ? J.phi_df[vo[b] + (long long)q * N + s0 + ii] : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    __syncthreads();
 #pragma unroll
-    for (int k = 0; k < kPairs; ++k) {
-      const int p = tid + k * kOtfDfThreads, r = p / B, b = p % B;
-      if (b < nl) {
-        const float4* Er = Et + r * kOtfDfSrc * kOtfDfPitch + b;
-        const float4* Pb = Ps + b;
-#pragma unroll 4
-        for (int ii = 0; ii < kOtfDfSrc; ++ii) {
-          const float4 e = Er[ii * kOtfDfPitch];
-#pragma unroll
-          for (int q = 0; q < Q; ++q) cdf_mac(acc_re[k][q], acc_im[k][q], e, Pb[(q * kOtfDfSrc + ii) * kOtfDfPitch]);
+          for (int q = 0; q < Q; ++q) cdf_mac(acc[(k * Q + q) * 2], acc[(k * Q + q) * 2 + 1], e, pv[q]);
         }
+        ph += pt.v;
       }
     }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int k = 0; k < kPairs; ++k) {
-    const int p = tid + k * kOtfDfThreads, r = p / B, b = p % B;
-    if (b < nl && r < task.nrows) {
-      const long long row = J.otf_res_off[(long long)task.pair * J.L + ot.l0 + b] + task.row0 + r;
-#pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        const df a = acc_re[k][q].value(), c = acc_im[k][q].value();
-        J.apply_res[row * Q + q] = make_double2((double)a.hi + (double)a.lo, (double)c.hi + (double)c.lo);
-      }
+    df_warp_sums<V>(acc, lane);
+    constexpr int kShift = V == 32 ? 0 : V == 16 ? 1 : V == 8 ? 2 : V == 4 ? 3 : 4;
+    const int e = lane >> kShift, k = e / (2 * Q), q = (e / 2) % Q;
+    if ((lane & ((1 << kShift) - 1)) == 0 && k < nb) {
+      const df v = acc[0].value();
+      const long long row = J.otf_res_off[(long long)task.pair * J.L + ot.l0 + b0 + k] + task.row0 + r;
+      reinterpret_cast<double*>(J.apply_res)[(row * Q + q) * 2 + (e & 1)] = (double)v.hi + (double)v.lo;
     }
   }
 }
@@ -2561,6 +2505,10 @@ cudaError_t launch_tables(const DevJob& J, cudaStream_t st, int* launches) {
   k_fft_tw<<<cdiv(J.K / 2, 256), 256, 0, st>>>(J.fft_tw, J.fft_tw_df, J.K);
   k_freq_tw<<<cdiv((long long)J.Q * J.L, 256), 256, 0, st>>>(J);
   *launches += 2;
+  if (J.freq_df) {
+    k_freq_df<<<cdiv(J.L, 128), 128, 0, st>>>(J);
+    *launches += 1;
+  }
   if (J.n_rlogN > 0) {
     cudaError_t e = launch_tables_rlog_only(J, st, launches);
     if (e != cudaSuccess) return e;
@@ -2882,10 +2830,8 @@ static cudaError_t launch_cross_otf_q(const DevJob& J, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   if (J.n_otf > 0) {
     if (J.mixed) {
-      const size_t sh = (size_t)kOtfDfPitch * (kAsmRows + Q) * kOtfDfSrc * sizeof(float4);
-      e = cudaFuncSetAttribute(k_cross_otf_df<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
-      if (e != cudaSuccess) return e;
-      k_cross_otf_df<Q><<<J.n_otf, kOtfDfThreads, sh, st>>>(J);
+      if (J.fp64keep) k_cross_otf_df<Q, true><<<J.n_otf, kOtfThreads, 0, st>>>(J);
+      else k_cross_otf_df<Q, false><<<J.n_otf, kOtfThreads, 0, st>>>(J);
     } else {
       const size_t sh = (size_t)kAsmThreads * Q * B * sizeof(double2);
       k_cross_otf<Q><<<J.n_otf, kAsmThreads, sh, st>>>(J);

@@ -6,6 +6,9 @@
 
 namespace fthms {
 
+struct FreqDf;   // hankel_df.cuh
+constexpr size_t kFreqDfBytes = 48;
+
 // Device-side view of one job: every pointer is device memory owned by the job.
 struct DevJob {
   int P, L, Q, K, NT, M, n_obs, n_tout, nsys, n_act, n_grp, n_asm, n_tiles, n_rlogN, n_restr;
@@ -65,8 +68,10 @@ struct DevJob {
   // cross-assembly block, per time-transform block and per restriction block
   int shape_solve, shape_asm, shape_time, shape_restr;
   const CrossOtf* otf_tasks;
-  const long long* wn_off;   // per assembly task: near weights offset or -1
-  double* wn;                // near weights, nrows x N per assembly task with near rows
+  long long otf_stride;      // coprime to n_otf: launch order of the tasks
+  const long long* wn_off;   // per assembly task: offset of its near corrections or -1
+  double* wn;                // near corrections beta, nrows x N per assembly task with near rows
+  FreqDf* freq_df;           // [L] constants of the double-float Hankel entries (mixed forms)
   const long long* otf_res_off;
   const int* tpanel;
   const long long* tr_off;

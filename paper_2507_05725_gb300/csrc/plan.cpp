@@ -635,7 +635,8 @@ int build_plan(const fthms_curve* curves, int ncurves, const fthms_arc* arcs, in
     }
     // Near weights once per job (they depend on the target and N only); tasks of at most
     // otf_band(Q) frequencies each.
-    const int band = p.opt.precision >= 1 ? kOtfBandDf : otf_band(p.Q);
+    // (a mixed job that may fall back to FP64 keeps to the FP64 kernel's shorter bands)
+    const int band = p.opt.precision >= 1 && !p.opt.refine_fallback ? kOtfBandDf : otf_band(p.Q);
     p.wn_off.assign(p.asms.size(), -1);
     for (size_t a = 0; a < p.asms.size(); ++a) {
       const CrossAsm& t = p.asms[a];

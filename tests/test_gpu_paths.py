@@ -112,3 +112,26 @@ def test_point_source_rows(F, ctx, case):
         return
     job = F.Job(ctx, p).run().wait()
     assert _rel(job, ref, p) < 1e-11
+
+
+@pytest.mark.parametrize("Q", [1, 2, 3, 4])
+@pytest.mark.parametrize("N,precision", [(31, 1), (33, 2), (0, 1), (0, 2)])
+def test_every_step_rows_at_warp_and_band_edges(F, ctx, Q, N, precision):
+    """Double-float cross rows evaluated every step (a warp per target row, 32 sources at a time, blocks of 1 to 8
+    frequencies) against the FP64 form, stored rows: N around the warp width and bands of one to many equal-N
+    frequencies, near rows on two curves.  1e-10: the mixed forms' bar."""
+    p = wl.random_small(7, n_curves=2, n_arcs_per_curve=3, L=52, M=2, Q=Q, N_fixed=N, W=14.0, H=4.0, n_period=512)
+    ref = F.Job(ctx, p).run().wait()
+    p = copy.deepcopy(p)
+    p["options"]["cross_mode"] = 1
+    p["options"]["refine_max"] = 8
+    job = F.Job(ctx, p, precision=precision).run().wait()
+    num = den = 0.0
+    for j in range(6):
+        for q in range(Q):
+            a, b = F.fthms_densities(ref.req, j, 2, q), F.fthms_densities(job.req, j, 2, q)
+            num += float(np.sum((a - b) ** 2))
+            den += float(np.sum(a ** 2))
+    assert math.sqrt(num / den) < 1e-10
+    t = ref.traces()
+    assert np.max(np.abs(job.traces() - t)) < 1e-10 * np.max(np.abs(t))
