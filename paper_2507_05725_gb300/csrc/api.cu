@@ -390,12 +390,9 @@ fthms_status upload_job(fthms_req* r) {
   TRY(dev_alloc(r, (size_t)std::max(1, p.n_obs * p.Q * p.L), &J.Vobs));
   TRY(dev_alloc(r, (size_t)std::max(1, p.n_obs * p.n_tout), &J.traces));
   TRY(dev_alloc(r, (size_t)p.K / 2, &J.fft_tw));
-  J.freq_df = nullptr;
-  if (J.mixed) {
-    unsigned char* fd = nullptr;
-    TRY(dev_alloc(r, (size_t)p.L * kFreqDfBytes, &fd));
-    J.freq_df = reinterpret_cast<FreqDf*>(fd);
-  }
+  unsigned char* fd = nullptr;
+  TRY(dev_alloc(r, (size_t)p.L * kFreqDfBytes, &fd));
+  J.freq_df = reinterpret_cast<FreqDf*>(fd);
   J.fft_tw_df = nullptr;
   if (J.mixed) TRY(dev_alloc(r, (size_t)p.K / 2, &J.fft_tw_df));
   TRY(dev_alloc(r, (size_t)p.Q * p.L, &J.syn_tw));

@@ -5,16 +5,17 @@
 //            so they lie below 2^-26 of the sum);
 //   z >= 20: modulus and phase, H0^(1)(z) = sqrt(2/(pi z)) m(w) e^{i(z - pi/4 + phi(w))}.  The phase z/(2 pi) = l T mod 1
 //            is an exact 64-bit integer multiple of T's fraction, so no recurrence, no re-seeding and no FP64
-//            reduction: -w/8 and its cubic correction join it as integers, the top 9 bits pick (cos, sin) from a
-//            table of 512 angles and the rest (|x| <= pi/512) needs three Taylor terms.
+//            reduction: -w/8 and its cubic correction join it as integers, the top 10 bits pick (cos, sin) from
+//            a table of 1024 angles and the rest (|x| <= pi/1024) needs three Taylor terms.
 //            phi = -(w/8)(1 - s (25/48 - s rho(s))), m = 1 - s/16 + s^2 kappa(s), s = w^2 (the leading terms of
 //            DLMF 10.18.17-18), rho and kappa polynomials fitted to the exact modulus and phase on s <= 1/400 at 60
-//            digits (their fit errors enter below 2^-54 and 2^-47 of the result).
+//            digits (their fit errors enter below 2^-52 of the result).
 // About 125 FP32-pipe instructions an entry above z = 20 against ~225 of the rotated P + iQ recurrence this
 // replaces, and the set-up per pair needs no sine or cosine, so short bands cost no more per entry than long ones.
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "bessel.cuh"
@@ -23,19 +24,29 @@
 
 namespace fthms {
 
-constexpr int kAngles = 512;            // (cos, sin)(2 pi k/512)
+constexpr int kAngles = 1024;           // (cos, sin)(2 pi k/1024)
 constexpr int kTayFine = 160;           // Taylor intervals of width 1/8 on [0, 20)
 __device__ float4 c_angle_df[kAngles];          // cos hi, lo, sin hi, lo
 __device__ float4 c_tayfine_df[kTayFine][7];    // J0: c8..c5 | c4 c3 | c2 c1 (pairs) | c0, Yhat0: see tayfine_pack
 __device__ float4 c_log_df[128];                // reciprocal rc (9 bits) of the 128th's centre, -ln rc (hi, lo)
 
-// Per-frequency constants as double-float (two float4 a frequency, then ln l in FP64): 2 pi l, 1/(2 pi l);
-// 1/sqrt(l), ln l + ln pi + gamma (so that ln(z/2) + gamma = ln T + it).
+// Per-frequency constants: 2 pi l, 1/(2 pi l); 1/sqrt(l), ln l + ln pi + gamma (so that ln(z/2) + gamma = ln T + it).
 struct FreqDf {
   float4 a, b;
-  double lnl, pad;
+  double lnz, rs;             // ln l + ln pi + gamma and 1/sqrt(l) in FP64
 };
 static_assert(sizeof(FreqDf) == kFreqDfBytes, "size of the per-frequency constants");
+
+__device__ __forceinline__ FreqDf make_freq(int l) {
+  const double x = l > 0 ? (double)l : 1.0;
+  FreqDf f;
+  f.lnz = log(x) + 1.7219455507509330;      // ln pi + gamma
+  f.rs = rsqrt(x);
+  const df a = df_from(6.28318530717958647692 * x), b = df_from(0.5 * kInvPi / x), c = df_from(f.rs), d = df_from(f.lnz);
+  f.a = make_float4(a.hi, a.lo, b.hi, b.lo);
+  f.b = make_float4(c.hi, c.lo, d.hi, d.lo);
+  return f;
+}
 
 // One pair: everything that its frequencies share.
 struct PairTurns {
@@ -162,19 +173,38 @@ __device__ __forceinline__ void bessel0_tayfine_df(df z, df& J0, df& Yh) {
   Yh = tayfine_eval(f, df{g.x, g.y}, df{g.z, g.w}, df{h.x, h.y}, df{h.z, h.w}, df{e.z, e.w}, d);
 }
 
-// Entry E = (amp (beta cos - sin), amp cos) at z >= 20; p = l v - 1/8 turn; ang: the angle table (shared memory).
-__device__ __forceinline__ float4 hankel_far_df(const PairTurns& pr, unsigned long long p, const float4* ang, df iv,
-                                                df rs, df beta, bool near) {
-  const df w = df_mul(pr.iu, iv);
+// Angle and modulus at z >= 20: the table index, the residual angle x = xh + ... as sin x = xh + sx and
+// cos x - 1 = ch + cl, and 1 - m = mh + ml; p = l v - 1/8 turn.  kFine keeps the second-order terms in double-float
+// too (rho(0), kappa(0) as pairs): phase and modulus to 2^-52 instead of 2^-45 near z = 20.
+struct FarAngle {
+  unsigned idx;
+  float xh, sx, ch, cl, mh, ml;
+};
+template <bool kFine>
+__device__ __forceinline__ FarAngle far_angle(df iu, unsigned long long p, df iv) {
+  FarAngle r;
+  const df w = df_mul(iu, iv);
   const float sh = __fmul_rn(w.hi, w.hi), sl = fmaf(2.f * w.hi, w.lo, fmaf(w.hi, w.hi, -sh));
   // g = s (25/48 - s rho)
-  constexpr df kG = df_const(25.0 / 48.0);
+  constexpr df kG = df_const(25.0 / 48.0), kR = df_const(1.67656249910766316), kK = df_const(0.103515624983438744);
   float rho = fmaf(sh, 109818.0144f, -4218.12863f);
   rho = fmaf(sh, rho, 187.743036f);
   rho = fmaf(sh, rho, -13.1045092f);
-  rho = fmaf(sh, rho, 1.67656250f);
-  const float gc = fmaf(-sh, rho, kG.lo);
-  const float gh = __fmul_rn(sh, kG.hi), gl = fmaf(sh, gc, fmaf(sl, kG.hi, fmaf(sh, kG.hi, -gh)));
+  float gh, gl;
+  if (kFine) {
+    const float th = __fmul_rn(sh, kR.hi);                      // s rho(0)
+    const float tl = fmaf(sh, fmaf(sh, rho, kR.lo), fmaf(sl, kR.hi, fmaf(sh, kR.hi, -th)));
+    df c;
+    quick_two_sum(kG.hi, -th, c.hi, c.lo);
+    c.lo = __fadd_rn(c.lo, __fsub_rn(kG.lo, tl));
+    const df g = df_mul(df{sh, sl}, c);
+    gh = g.hi;
+    gl = g.lo;
+  } else {
+    const float gc = fmaf(-sh, fmaf(sh, rho, kR.hi), kG.lo);
+    gh = __fmul_rn(sh, kG.hi);
+    gl = fmaf(sh, gc, fmaf(sl, kG.hi, fmaf(sh, kG.hi, -gh)));
+  }
   // phi = -w/8 + (w/8) g = -q + (ah + al)
   const float qh = 0.125f * w.hi, ql = 0.125f * w.lo;
   const float ah = __fmul_rn(qh, gh), al = fmaf(ql, gh, fmaf(qh, gl, fmaf(qh, gh, -ah)));
@@ -188,47 +218,61 @@ __device__ __forceinline__ float4 hankel_far_df(const PairTurns& pr, unsigned lo
   float res = __fadd_rn(fmaf(f1, -kT2.hi, -qh), fmaf(f2, -kT2.hi, ah));
   res = __fadd_rn(res, fmaf(-__fadd_rn(f1, f2), kT2.lo, __fsub_rn(al, ql)));
   const unsigned hi = (unsigned)(p >> 32) + (unsigned)n;
-  const unsigned idx = (hi + 0x400000u) >> 23;
-  // integers below 2^22 and 2^23 to float by an exponent and a subtraction (the conversion unit is slower)
-  const float fr = __fsub_rn(__uint_as_float(0x4B400000u + (hi - (idx << 23))), kMagic);
+  r.idx = ((hi + 0x200000u) >> 22);
+  // integers below 2^21 and 2^23 to float by an exponent and a subtraction (the conversion unit is slower)
+  const float fr = __fsub_rn(__uint_as_float(0x4B400000u + (hi - (r.idx << 22))), kMagic);
   const float fl = __fsub_rn(__uint_as_float(0x4B000000u | ((unsigned)p >> 9)), 8388608.f);
   constexpr float kLow = (float)(kTurn / 8388608.0);
+  r.idx &= kAngles - 1;
   const float xh = __fmul_rn(fr, kT.hi);
   float xl = fmaf(fr, kT.lo, fmaf(fr, kT.hi, -xh));
   xl = __fadd_rn(fmaf(fl, kLow, xl), res);
-  // sin x = xh + sx, cos x - 1 = ch + cl
   const float uh = __fmul_rn(xh, xh), ul = fmaf(2.f * xh, xl, fmaf(xh, xh, -uh));
-  const float ch = -0.5f * uh;
-  const float sx = fmaf(xh, __fmul_rn(uh, fmaf(uh, 1.f / 120.f, -1.f / 6.f)), fmaf(xl, ch, xl));
-  const float cl = fmaf(__fmul_rn(uh, uh), 1.f / 24.f, -0.5f * ul);
-  const float4 t = ang[idx & (kAngles - 1)];
-  // cos, sin of the sum: the corrections C ch -+ S x are small against the table value
+  r.xh = xh;
+  r.ch = -0.5f * uh;
+  r.sx = fmaf(xh, __fmul_rn(uh, fmaf(uh, 1.f / 120.f, -1.f / 6.f)), fmaf(xl, r.ch, xl));
+  r.cl = fmaf(__fmul_rn(uh, uh), 1.f / 24.f, -0.5f * ul);
+  float kap = fmaf(sh, 2366.77002f, -105.650777f);
+  kap = fmaf(sh, kap, 5.84762562f);
+  kap = fmaf(sh, kap, -0.542846348f);
+  r.mh = 0.0625f * sh;
+  if (kFine) {
+    const float t = __fmul_rn(sh, sh), tl = fmaf(2.f * sh, sl, fmaf(sh, sh, -t));
+    const float kh = __fmul_rn(t, kK.hi);
+    const float kl = fmaf(t, fmaf(sh, kap, kK.lo), fmaf(tl, kK.hi, fmaf(t, kK.hi, -kh)));
+    quick_two_sum(r.mh, -kh, r.mh, r.ml);
+    r.ml = __fadd_rn(r.ml, fmaf(0.0625f, sl, -kl));
+  } else {
+    r.ml = fmaf(-__fmul_rn(sh, sh), fmaf(sh, kap, kK.hi), 0.0625f * sl);
+  }
+  return r;
+}
+
+// cos or sin of (table angle + x) minus the table value, as an unrenormalised pair: a ch -+ b x, with (a, b) the
+// table's value and its partner.
+__device__ __forceinline__ df angle_step(float ah, float al, float bh, float bl, const FarAngle& f) {
+  const float A = __fmul_rn(bh, f.xh), B = __fmul_rn(ah, f.ch);
+  const float Ae = fmaf(bl, f.xh, fmaf(bh, f.sx, fmaf(bh, f.xh, -A)));
+  const float Be = fmaf(al, f.ch, fmaf(ah, f.cl, fmaf(ah, f.ch, -B)));
+  df d;
+  quick_two_sum(A, B, d.hi, d.lo);
+  d.lo = __fadd_rn(d.lo, __fadd_rn(Ae, Be));
+  return d;
+}
+
+// Entry E = (amp (beta cos - sin), amp cos) at z >= 20; ang: the angle table (shared memory).
+__device__ __forceinline__ float4 hankel_far_df(const PairTurns& pr, unsigned long long p, const float4* ang, df iv,
+                                                df rs, df beta, bool near) {
+  const FarAngle f = far_angle<false>(pr.iu, p, iv);
+  const float4 t = ang[f.idx];
+  const df dc = angle_step(t.x, t.y, -t.z, -t.w, f), ds = angle_step(t.z, t.w, t.x, t.y, f);
   df co, si;
-  {
-    const float A = __fmul_rn(t.z, xh), B = __fmul_rn(t.x, ch);
-    const float Ae = fmaf(t.w, xh, fmaf(t.z, sx, fmaf(t.z, xh, -A)));
-    const float Be = fmaf(t.y, ch, fmaf(t.x, cl, fmaf(t.x, ch, -B)));
-    float dh, dl;
-    quick_two_sum(-A, B, dh, dl);
-    quick_two_sum(t.x, dh, co.hi, co.lo);
-    co.lo = __fadd_rn(__fadd_rn(co.lo, t.y), __fadd_rn(dl, __fsub_rn(Be, Ae)));
-  }
-  {
-    const float A = __fmul_rn(t.x, xh), B = __fmul_rn(t.z, ch);
-    const float Ae = fmaf(t.y, xh, fmaf(t.x, sx, fmaf(t.x, xh, -A)));
-    const float Be = fmaf(t.w, ch, fmaf(t.z, cl, fmaf(t.z, ch, -B)));
-    float dh, dl;
-    quick_two_sum(A, B, dh, dl);
-    quick_two_sum(t.z, dh, si.hi, si.lo);
-    si.lo = __fadd_rn(__fadd_rn(si.lo, t.w), __fadd_rn(dl, __fadd_rn(Be, Ae)));
-  }
-  // amplitude: amp (1 - mu), mu = s/16 - s^2 kappa
-  float kap = fmaf(sh, -93.7731580f, 5.82897780f);
-  kap = fmaf(sh, kap, -0.542836961f);
-  kap = fmaf(sh, kap, 0.103515624f);
-  const float mh = 0.0625f * sh, ml = fmaf(-__fmul_rn(sh, sh), kap, 0.0625f * sl);
-  const df a0 = df_mulq(pr.aw, rs);
-  const float b = __fmul_rn(a0.hi, mh), be = fmaf(a0.lo, mh, fmaf(a0.hi, ml, fmaf(a0.hi, mh, -b)));
+  quick_two_sum(t.x, dc.hi, co.hi, co.lo);
+  co.lo = __fadd_rn(__fadd_rn(co.lo, t.y), dc.lo);
+  quick_two_sum(t.z, ds.hi, si.hi, si.lo);
+  si.lo = __fadd_rn(__fadd_rn(si.lo, t.w), ds.lo);
+  const df a0 = df_mulq(pr.aw, rs);                             // amp (1 - mu)
+  const float b = __fmul_rn(a0.hi, f.mh), be = fmaf(a0.lo, f.mh, fmaf(a0.hi, f.ml, fmaf(a0.hi, f.mh, -b)));
   df amp;
   quick_two_sum(a0.hi, -b, amp.hi, amp.lo);
   amp.lo = __fadd_rn(amp.lo, __fsub_rn(a0.lo, be));
@@ -250,6 +294,120 @@ __device__ __forceinline__ float4 hankel_near_df(df z, df Lz, df beta, bool near
   return make_float4(-re.hi, -re.lo, im.hi, im.lo);
 }
 
+// ---- FP64 entries with the FP64 pipe (two lanes a clock and SM) kept for the last additions --------------------
+// Only what reaches the result's leading bits needs FP64: the table values and the final sums and products.  The
+// corrections to a table value are small -- the angle step below 2^-8, the Taylor terms beyond the constant below
+// 2^-6 -- so double-float corrections (2^-46 relative and better) leave the result at FP64's own rounding.  9 FP64
+// instructions an entry against 25 to 45 of the plain FP64 series and rotated recurrence.
+constexpr int kTay64 = 408;             // Taylor intervals of 1/128 turn on [0, 20/(2 pi))
+struct Tay64 {                          // n = 7..5 in FP32, 4..1 double-float (in turns), 0 in FP64
+  float4 hi, c43, c21;
+  double c0, pad;
+};
+__device__ double2 c_angle_f64[kAngles];
+__device__ Tay64 c_tay64[kTay64 + 1][2];        // J0, Yhat0
+__device__ double2 c_log_f64[1024];             // reciprocal (12 bits) of the 1024th's centre, -ln of it
+
+struct AngleTab {                       // shared-memory copy
+  float4 d[kAngles];
+  double2 f[kAngles];
+};
+__device__ __forceinline__ void load_angles(AngleTab& t, bool f64) {
+  for (int k = threadIdx.x; k < kAngles; k += blockDim.x) {
+    t.d[k] = c_angle_df[k];
+    if (f64) t.f[k] = c_angle_f64[k];
+  }
+}
+
+// ln x for a normal x > 0 (-inf at 0): x = 2^e m, r = m rc - 1 exact in one FMA (|r| < 2^-10), ln(1 + r) - r in double-
+// float.  Five FP64 operations.
+__device__ __forceinline__ double log_f64(double x) {
+  const int h = __double2hiint(x);
+  const int ex = ((h >> 20) & 0x7FF) - 1023;
+  const double m = __hiloint2double((h & 0xFFFFF) | 0x3FF00000, __double2loint(x));
+  const double2 tb = __ldg(&c_log_f64[(h >> 10) & 1023]);
+  const double r = fma(m, tb.x, -1.0);
+  const df rd = df_split_bits(r);
+  const float u = __fmul_rn(rd.hi, rd.hi), ul = fmaf(2.f * rd.hi, rd.lo, fmaf(rd.hi, rd.hi, -u));
+  const float c = __fmul_rn(__fmul_rn(u, rd.hi), fmaf(rd.hi, fmaf(rd.hi, 0.2f, -0.25f), 1.f / 3.f));
+  const double q = f2d_bits(-0.5f * u) + f2d_bits(fmaf(-0.5f, ul, c));
+  const double v = (fma((double)ex, 0.69314718055994530941723212145817657, tb.y) + r) + q;
+  return x > 0.0 ? v : __longlong_as_double(0xFFF0000000000000ll);
+}
+
+struct PairF64 {
+  unsigned long long v;   // fraction of T in 2^-64 turns
+  unsigned long long v62; // T in 2^-62 turns (below 4 turns; for z < 20)
+  double T, aw;           // turns, (w/(4 pi)) / sqrt(T)
+  df iu;                  // 1/T
+  float th;
+};
+__device__ __forceinline__ PairF64 pair_f64(double T, double camp4) {
+  PairF64 p;
+  p.T = T;
+  p.v = turn_fraction(T);
+  p.v62 = turn_fraction(0.25 * T);                     // (exact scaling)
+  const df t = df_split_bits(T);
+  p.th = t.hi;
+  const float y = rsqrtf(t.hi);
+  const float q = __fmul_rn(y, y), qe = fmaf(y, y, -q);
+  const float a = __fmul_rn(t.hi, q);
+  const float ae = fmaf(t.lo, q, fmaf(t.hi, qe, fmaf(t.hi, q, -a)));
+  const float e = __fsub_rn(__fsub_rn(1.f, a), ae);
+  df r;
+  quick_two_sum(y, __fmul_rn(y, __fmul_rn(e, fmaf(0.375f, e, 0.5f))), r.hi, r.lo);
+  p.iu = df_mul(r, r);
+  const double s = f2d_bits(r.hi) + f2d_bits(r.lo);    // one Newton step on the pair: 2^-46 -> FP64
+  p.aw = camp4 * fma(fma(-T * s, s, 1.0), 0.5 * s, s);
+  return p;
+}
+
+// z >= 20; p = l v - 1/8 turn, rs = 1/sqrt(l).
+__device__ __forceinline__ double2 hankel_far_f64(const PairF64& pr, unsigned long long p, const AngleTab& ang, df iv,
+                                                  double rs, double beta, bool near) {
+  const FarAngle f = far_angle<true>(pr.iu, p, iv);
+  const float4 t = ang.d[f.idx];
+  const double2 t64 = ang.f[f.idx];
+  const df dc = angle_step(t.x, t.y, -t.z, -t.w, f), ds = angle_step(t.z, t.w, t.x, t.y, f);
+  const double co = t64.x + (f2d_bits(dc.hi) + f2d_bits(dc.lo)), si = t64.y + (f2d_bits(ds.hi) + f2d_bits(ds.lo));
+  const double a0 = pr.aw * rs;
+  const double amp = fma(-a0, f2d_bits(f.mh) + f2d_bits(f.ml), a0);
+  return make_double2(amp * (near ? fma(beta, co, -si) : -si), amp * co);
+}
+
+// J0 and Yhat0 at z = 2 pi u / 2^62 < 20 (u = l v62): interval and offset are bits of u.
+__device__ __forceinline__ double tay64_eval(const Tay64* __restrict__ tab, df d) {
+  const float4 h = __ldg(&tab->hi), a = __ldg(&tab->c43), b = __ldg(&tab->c21);
+  const double c0 = __ldg(&tab->c0);
+  const float q = fmaf(fmaf(h.x, d.hi, h.y), d.hi, h.z);
+  df s = df_add_fast(df{__fmul_rn(q, d.hi), 0.f}, df{a.x, a.y});
+  s = df_add_fast(df_mul(s, d), df{a.z, a.w});
+  s = df_add_fast(df_mul(s, d), df{b.x, b.y});
+  s = df_add_fast(df_mul(s, d), df{b.z, b.w});
+  s = df_mulq(s, d);
+  return c0 + (f2d_bits(s.hi) + f2d_bits(s.lo));
+}
+__device__ __forceinline__ void bessel0_f64(unsigned long long u, double& J0, double& Yh) {
+  const int k = min((int)(u >> 55), kTay64);
+  const long long rem = (long long)(u - ((unsigned long long)k << 55)) - (1ll << 54);
+  df d;                                                 // in turns: |d| <= 2^-8
+  quick_two_sum((float)(int)(rem >> 32) * 0x1p-30f, (float)((unsigned)rem >> 8) * 0x1p-54f, d.hi, d.lo);
+  J0 = tay64_eval(&c_tay64[k][0], d);
+  Yh = tay64_eval(&c_tay64[k][1], d);
+}
+
+// Entry at z < 20, the sum of hankel_near_df in FP64; L = ln(z/2) + gamma.
+__device__ __forceinline__ double2 hankel_near_f64(unsigned long long u, double L, double beta, bool near, double qw) {
+  double J0, Yh;
+  bessel0_f64(u, J0, Yh);
+  const double a = near ? fma(kTwoOverPi, L, -beta) : kTwoOverPi * L;
+  return make_double2(-qw * fma(a, J0, Yh), qw * J0);
+}
+__device__ __forceinline__ float4 split2_bits(double2 v) {
+  const df a = df_split_bits(v.x), b = df_split_bits(v.y);
+  return make_float4(a.hi, a.lo, b.hi, b.lo);
+}
+
 // Fills the tables above on the current device.
 inline cudaError_t init_hankel_df() {
   static float4 ang[kAngles], lg[128], tf[kTayFine][7];
@@ -257,9 +415,9 @@ inline cudaError_t init_hankel_df() {
   auto lo = [](double v) { return (float)(v - (double)(float)v); };
   for (int k = 0; k < kAngles; ++k) {
     // the first octant's values, moved by symmetry, so that multiples of a quarter turn are exact
-    const int q = k / 128, r = k % 128;
-    const double a = 2.0 * 3.14159265358979323846 * (r <= 64 ? r : 128 - r) / 512.0;
-    const double c0 = r <= 64 ? std::cos(a) : std::sin(a), s0 = r <= 64 ? std::sin(a) : std::cos(a);
+    const int q = 4 * k / kAngles, r = k % (kAngles / 4), h = kAngles / 8;
+    const double a = 2.0 * 3.14159265358979323846 * (r <= h ? r : 2 * h - r) / kAngles;
+    const double c0 = r <= h ? std::cos(a) : std::sin(a), s0 = r <= h ? std::sin(a) : std::cos(a);
     const double c = q == 0 ? c0 : q == 1 ? -s0 : q == 2 ? -c0 : s0, s = q == 0 ? s0 : q == 1 ? c0 : q == 2 ? -s0 : -c0;
     ang[k] = make_float4(hi(c), lo(c), hi(s), lo(s));
   }
@@ -293,6 +451,46 @@ inline cudaError_t init_hankel_df() {
     tf[k][5] = make_float4(hi(y[4]), lo(y[4]), hi(y[3]), lo(y[3]));
     tf[k][6] = make_float4(hi(y[2]), lo(y[2]), hi(y[1]), lo(y[1]));
   }
+  static double2 ang64[kAngles], lg64[1024];
+  static Tay64 t64[kTay64 + 1][2];
+  for (int k = 0; k < kAngles; ++k) {
+    const int q = 4 * k / kAngles, r = k % (kAngles / 4), h = kAngles / 8;
+    const double a = 2.0 * 3.14159265358979323846 * (r <= h ? r : 2 * h - r) / kAngles;
+    const double c0 = r <= h ? std::cos(a) : std::sin(a), s0 = r <= h ? std::sin(a) : std::cos(a);
+    ang64[k] = make_double2(q == 0 ? c0 : q == 1 ? -s0 : q == 2 ? -c0 : s0, q == 0 ? s0 : q == 1 ? c0 : q == 2 ? -s0 : -c0);
+  }
+  for (int k = 0; k < 1024; ++k) {
+    const double rc = std::nearbyint(4096.0 / (1.0 + (k + 0.5) / 1024.0)) / 4096.0;
+    lg64[k] = make_double2(rc, -std::log(rc));
+  }
+  const double tau = 6.28318530717958647692;
+  for (int k = 0; k <= kTay64; ++k) {
+    const double z = tau * (k + 0.5) / 128.0;
+    const int K = std::min((int)(2.0 * z), kTaylorIntervals - 1);
+    const long double shift = (long double)tau * (k + 0.5L) / 128.0L + 2.4492935982947064e-16L * (k + 0.5L) / 128.0L -
+                              (0.25L + 0.5L * K);          // (2 pi as the sum of two doubles)
+    for (int f = 0; f < 2; ++f) {
+      double c[8];
+      long double sc = 1.0L;
+      for (int n = 0; n <= 7; ++n, sc *= tau) {
+        long double v = 0.0L, binom = 1.0L, pw = 1.0L;
+        for (int m = n; m <= kTaylorDegree; ++m) {
+          v += binom * src[f][K][m] * pw;
+          binom = binom * (m + 1) / (m + 1 - n);
+          pw *= shift;
+        }
+        c[n] = (double)(v * sc);
+      }
+      t64[k][f].hi = make_float4((float)c[7], (float)c[6], (float)c[5], 0.f);
+      t64[k][f].c43 = make_float4(hi(c[4]), lo(c[4]), hi(c[3]), lo(c[3]));
+      t64[k][f].c21 = make_float4(hi(c[2]), lo(c[2]), hi(c[1]), lo(c[1]));
+      t64[k][f].c0 = c[0];
+      t64[k][f].pad = 0.0;
+    }
+  }
+  if ((e = cudaMemcpyToSymbol(c_angle_f64, ang64, sizeof ang64)) != cudaSuccess) return e;
+  if ((e = cudaMemcpyToSymbol(c_log_f64, lg64, sizeof lg64)) != cudaSuccess) return e;
+  if ((e = cudaMemcpyToSymbol(c_tay64, t64, sizeof t64)) != cudaSuccess) return e;
   if ((e = cudaMemcpyToSymbol(c_angle_df, ang, sizeof ang)) != cudaSuccess) return e;
   if ((e = cudaMemcpyToSymbol(c_log_df, lg, sizeof lg)) != cudaSuccess) return e;
   return cudaMemcpyToSymbol(c_tayfine_df, tf, sizeof tf);

@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <type_traits>
 
 #include "bessel.cuh"
 #include "cplx.cuh"
@@ -32,29 +33,9 @@ cudaError_t init_constants() {
   double ha[20];
   ha[0] = 1.0;
   for (int k = 1; k < 20; ++k) ha[k] = ha[k - 1] * (double)((2 * k - 1) * (2 * k - 1)) / (8.0 * k);
-  float2 hd[20];
-  for (int k = 0; k < 20; ++k) {
-    const float h = (float)ha[k];
-    hd[k] = make_float2(h, (float)(ha[k] - (double)h));
-  }
   cudaError_t e = cudaMemcpyToSymbol(c_hank_a, ha, sizeof ha);
   if (e != cudaSuccess) return e;
-  e = cudaMemcpyToSymbol(c_hank_df, hd, sizeof hd);
-  if (e != cudaSuccess) return e;
-  static double tj[kTaylorIntervals][kTaylorDegree + 1], ty[kTaylorIntervals][kTaylorDegree + 1];
-  static float2 td[2][kTaylorIntervals][kTaylorDegree + 1];
-  e = cudaMemcpyFromSymbol(tj, kTaylorJ0, sizeof tj);
-  if (e != cudaSuccess) return e;
-  e = cudaMemcpyFromSymbol(ty, kTaylorYh, sizeof ty);
-  if (e != cudaSuccess) return e;
-  for (int k = 0; k < kTaylorIntervals; ++k)
-    for (int n = 0; n <= kTaylorDegree; ++n) {
-      const float a = (float)tj[k][n], c = (float)ty[k][n];
-      td[0][k][n] = make_float2(a, (float)(tj[k][n] - (double)a));
-      td[1][k][n] = make_float2(c, (float)(ty[k][n] - (double)c));
-    }
-  e = cudaMemcpyToSymbol(c_taylor_df, td, sizeof td);
-  return e == cudaSuccess ? init_hankel_df() : e;
+  return init_hankel_df();
 }
 
 namespace {
@@ -104,19 +85,10 @@ __global__ void k_freq_tw(DevJob J) {
   J.fwd_tw[idx] = make_double2(J.dt * c, J.dt * s);
 }
 
-// Per-frequency constants of the double-float Hankel entries (mixed forms).
+// Per-frequency constants of the Hankel entries.
 __global__ void k_freq_df(DevJob J) {
   const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= J.L) return;
-  const double x = l > 0 ? (double)l : 1.0, ln = log(x);
-  const df a = df_from(2.0 * kPiD * x), b = df_from(0.5 * kInvPi / x), c = df_from(rsqrt(x)),
-           d = df_from(ln + 1.7219455507509330);      // ln pi + gamma
-  FreqDf f;
-  f.a = make_float4(a.hi, a.lo, b.hi, b.lo);
-  f.b = make_float4(c.hi, c.lo, d.hi, d.lo);
-  f.lnl = ln;
-  f.pad = 0.0;
-  J.freq_df[l] = f;
+  if (l < J.L) J.freq_df[l] = make_freq(l);
 }
 
 // Cosine sums F(m) = sum_{n=1}^{N-1} cos(n m pi/N)/n, m = 0..N, of the self log weights
@@ -232,30 +204,6 @@ __global__ void k_restr(DevJob J) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Self assembly: A_ic = K1(t_i,t_c) Rlog_ic + K2(t_i,t_c) pi/N, symmetric in (i, c), for a band of
-// consecutive frequencies sharing N (nodes, log table, |t - s| and its logarithm are shared).
-// cos(theta - pi/4) and sin(theta - pi/4) as double-float pairs for a phase theta >= 0 given in FP64 (up
-// to ~2e4): theta is reduced by n pi/2 in FP64 (pi/2 as the sum of two doubles, each product inside an
-// FMA), the remainder |r| <= pi/4 is rounded to double-float (~3e-15 absolute) and its sine and cosine
-// come from the double-float Taylor series; the quadrant n mod 4 permutes them.
-__device__ __forceinline__ void df_phase_seed(double theta, df& cx, df& sx) {
-  constexpr double kPio2Hi = 1.57079632679489661923, kPio2Lo = 6.123233995736766e-17;   // pi/2 = Hi + Lo
-  const double n = rint(theta * kTwoOverPi);
-  const double r = fma(-n, kPio2Lo, fma(-n, kPio2Hi, theta));
-  df sr, cr;
-  df_sincos_taylor(df_from(r), sr, cr);
-  df s, c;
-  switch (((long long)n) & 3) {
-    case 0: s = sr; c = cr; break;
-    case 1: s = cr; c = df_neg(sr); break;
-    case 2: s = df_neg(sr); c = df_neg(cr); break;
-    default: s = df_neg(cr); c = sr; break;
-  }
-  constexpr df kSqrtHalfD = df_const(0.70710678118654752440084436210484904);
-  cx = df_mul(df_add(c, s), kSqrtHalfD);      // cos(theta - pi/4)
-  sx = df_mul(df_sub(s, c), kSqrtHalfD);      // sin(theta - pi/4)
-}
-
 // A self-matrix entry: FP64, or (mixed form) the double-float pair the refinement reads plus its FP32
 // rounding for the FP32 factorisation -- what a separate split of the FP64 matrix would give -- or (the
 // FP64-kept form) the FP64 value the FP64 residual reads plus its FP32 rounding.
@@ -276,78 +224,23 @@ __device__ __forceinline__ void store_self(const DevJob& J, long long off, doubl
   }
 }
 
-// P and Q/w of the Hankel asymptotics (kmax + 1 terms each) by Horner's rule in w2 = -1/z^2 in
-// double-float.  With |w2| <= 1/400 (z >= 20) the level-k term is below 2^(-8.6 k) of the sum, so the
-// levels k >= 3 need only FP32 (22 bits) and the outer three double-float, where each product stays
-// far below the coefficient it is added to (no cancellation).
-__device__ __forceinline__ void hankel_pq_df(int kmax, df w2, df& P, df& Qa) {
-  int k;
-  if (kmax >= 3) {
-    const float w2f = w2.hi;
-    float pf = c_hank_df[2 * kmax].x, qf = c_hank_df[2 * kmax + 1].x;
-    for (k = kmax - 1; k >= 3; --k) {
-      pf = fmaf(pf, w2f, c_hank_df[2 * k].x);
-      qf = fmaf(qf, w2f, c_hank_df[2 * k + 1].x);
-    }
-    P = df{pf, 0.f};
-    Qa = df{qf, 0.f};
-    k = 2;
-  } else {
-    const float2 cp = c_hank_df[2 * kmax], cq = c_hank_df[2 * kmax + 1];
-    P = df{cp.x, cp.y};
-    Qa = df{cq.x, cq.y};
-    k = kmax - 1;
-  }
-  for (; k >= 0; --k) {
-    const float2 cp = c_hank_df[2 * k], cq = c_hank_df[2 * k + 1];
-    P = df_add_fast(df_mul(P, w2), df{cp.x, cp.y});
-    Qa = df_add_fast(df_mul(Qa, w2), df{cq.x, cq.y});
-  }
-}
-
-// J0 and Yhat0 for 0 <= z < 20 in double-float (mixed form): the piecewise Taylor expansions of
-// bessel0_taylor with double-float coefficients, products and sums.
-__device__ __forceinline__ void bessel0_taylor_df(df z, df& J0, df& Yh) {
-  const int k = min((int)(2.f * z.hi), kTaylorIntervals - 1);
-  const df d = df_add_fast(z, df{-(0.25f + 0.5f * (float)k), 0.f});
-  const float2* cj = c_taylor_df[0][k];
-  const float2* cy = c_taylor_df[1][k];
-  float2 c = __ldg(&cj[kTaylorDegree]);
-  df j{c.x, c.y};
-  c = __ldg(&cy[kTaylorDegree]);
-  df y{c.x, c.y};
-#pragma unroll
-  for (int n = kTaylorDegree - 1; n >= 0; --n) {
-    c = __ldg(&cj[n]);
-    j = df_add_fast(df_mul(j, d), df{c.x, c.y});
-    c = __ldg(&cy[n]);
-    y = df_add_fast(df_mul(y, d), df{c.x, c.y});
-  }
-  J0 = j;
-  Yh = y;
-}
-
+// Self assembly: A_ic = K1(t_i,t_c) Rlog_ic + K2(t_i,t_c) pi/N, symmetric in (i, c), for a band of consecutive
+// frequencies sharing N (nodes, log weights, |t - s| and its logarithm are shared).  With K1 = -J0/(2 pi) an
+// off-diagonal entry is the near rule's E = amp (beta cos - sin, cos) with beta = (2/pi)(ln|t_i - t_c| - Rlog_ic/w),
+// below and above z = 20 alike (hankel_df.cuh).  kDf: double-float entries for the mixed form's systems that keep
+// double-float matrices; else FP64 entries, bound by the FP64 pipe at 9 of its instructions an entry and ~30 a pair
+// (the series and rotated recurrence before took 25 to 45 an entry): 6 arcs x 384 frequencies, N = 512: 24.6 -> 11.8 ms
+// with the row bounds.
+template <bool kDf>
 __global__ void __launch_bounds__(256) k_assemble_self(DevJob J) {
   const SelfTile tile = J.tiles[blockIdx.x];
   const SysDesc s0 = J.sys[tile.sys];
   const int N = s0.N, nb = tile.nsys;
-  // Mixed form: double-float assembly and storage, except for the systems that keep FP64 (sys_f64).
-  const bool f64 = J.mixed && sys_f64(J, N);
-  const bool df_asm = J.mixed && !f64;
-  __shared__ double lnl[kSelfBand], invl[kSelfBand], rsql[kSelfBand];
-  __shared__ df invl_d[kSelfBand], rsql_d[kSelfBand], lnl_d[kSelfBand], lh_d[kSelfBand];   // mixed form
-  if (threadIdx.x < nb) {
-    const double l = (double)(s0.l + threadIdx.x);
-    lnl[threadIdx.x] = log(l);
-    invl[threadIdx.x] = 1.0 / l;
-    rsql[threadIdx.x] = rsqrt(l);
-    if (J.mixed) {
-      invl_d[threadIdx.x] = df_from(invl[threadIdx.x]);
-      rsql_d[threadIdx.x] = df_from(rsql[threadIdx.x]);
-      lnl_d[threadIdx.x] = df_from(lnl[threadIdx.x]);
-      lh_d[threadIdx.x] = df_from(l * J.h);
-    }
-  }
+  if (kDf == (!J.mixed || sys_f64(J, N))) return;       // the other launch's systems
+  __shared__ AngleTab ang;
+  __shared__ FreqDf fr[kSelfBand];
+  load_angles(ang, !kDf);
+  if (threadIdx.x < nb) fr[threadIdx.x] = J.freq_df ? J.freq_df[s0.l + threadIdx.x] : make_freq(s0.l + threadIdx.x);
   __syncthreads();
   const int i = tile.ti * kSelfTile + (threadIdx.x % kSelfTile);
   const int c = tile.tl * kSelfTile + (threadIdx.x / kSelfTile);
@@ -355,145 +248,51 @@ __global__ void __launch_bounds__(256) k_assemble_self(DevJob J) {
   if (tile.ti == tile.tl && i > c) return;
   const Panel pn = J.panels[s0.panel];
   const double rl = rlog_at(J.rlog + s0.rlog_off, N, i, c);
-  const double w = kPiD / N;
+  const double w = kPiD / N, qw = 0.25 * w;
   const long long e1 = (long long)c * N + i, e2 = (long long)i * N + c;
+  long long mo = s0.mat_off;                            // the band's matrices follow one another
+  const long long nn = (long long)N * N;
   if (i == c) {
-    const double K1 = -0.5 * kInvPi;
-    const double lsp = log(0.5 * J.h * J.node_sp[pn.off + i]);
-    for (int b = 0; b < nb; ++b) {
-      const double re = -0.5 * kInvPi * (kEulerGamma + lnl[b] + lsp);
-      store_self(J, J.sys[tile.sys + b].mat_off + e1, make_double2(fma(K1, rl, re * w), 0.25 * w), f64);
-    }
+    // limit t -> s: K2 = i/4 - (1/(2 pi)) [gamma + ln(kappa |x'|/2)]
+    const double lsp = log(0.5 * J.h * J.node_sp[pn.off + i]) - 1.1447298858494002;   // - ln pi (part of lnz)
+    for (int b = 0; b < nb; ++b, mo += nn)
+      store_self(J, mo + e1, make_double2(-0.5 * kInvPi * fma(w, fr[b].lnz + lsp, rl), qw), !kDf && J.mixed);
     return;
   }
   const double dx = J.node_x[pn.off + i] - J.node_x[pn.off + c];
   const double dy = J.node_y[pn.off + i] - J.node_y[pn.off + c];
-  const double R = sqrt(fma(dx, dx, dy * dy));
-  const double dts = fabs(J.node_t[pn.off + i] - J.node_t[pn.off + c]);
-  const double hR = J.h * R;
-  // A = K1 Rlog + K2 w with K1 = -J0/(2 pi):
-  //   z < 20:  K2 = (i/4) J0 - (J0/(2 pi)) [ln l + ln(hR/(2|t-s|)) + gamma] - Yhat0/4
-  //   z >= 20: K2 = (i/4) J0 - Y0/4 + (J0/(2 pi)) ln|t-s|
-  // so Re A = J0 * alpha - (w/4) Y, with alpha depending on the entry (and on ln l below 20).
-  const double lratio = log(hR / (2.0 * dts)) + kEulerGamma;
-  const double alpha_a = -0.5 * kInvPi * (rl - w * log(dts));          // z >= 20
-  const double qw = 0.25 * w;
-  const double inv_u = 1.0 / hR, amp_u = sqrt(kTwoOverPi * inv_u);
-  const int lsw = max(s0.l, (int)ceil(kBesselLarge * inv_u));         // first l with z >= 20
-  const int lend = s0.l + nb;
-  const double zmin = (lsw * J.h) * R;
-  const int kmax = hankel_terms((float)zmin);
-  if (df_asm) {
-    // Mixed form, z < 20: the Taylor range in double-float, alpha = aw ln l + a0.
-    const df R_d = df_from(R), qw_d = df_from(qw), aw_d = df_from(-0.5 * kInvPi * w),
-             a0_d = df_from(-0.5 * kInvPi * fma(w, lratio, rl));
-    for (int l = s0.l; l < min(lsw, lend); ++l) {
-      const int b = l - s0.l;
-      df J0, Yh;
-      bessel0_taylor_df(df_mul(lh_d[b], R_d), J0, Yh);
-      const df alpha = df_add_fast(df_mul(aw_d, lnl_d[b]), a0_d);
-      const df re = df_dot2(alpha, J0, df_neg(qw_d), Yh);
-      const df im = df_mul(qw_d, J0);
-      const long long mo = J.sys[tile.sys + b].mat_off;
-      const float4 d = make_float4(re.hi, re.lo, im.hi, im.lo);
-      const float2 f = make_float2(re.hi, im.hi);
+  const double T = (J.h * (0.5 * kInvPi)) * dist_f64(fma(dx, dx, dy * dy));
+  const double beta = kTwoOverPi * (log_f64(fabs(J.node_t[pn.off + i] - J.node_t[pn.off + c])) - rl * (N * kInvPi));
+  if (kDf) {
+    const PairTurns pt = pair_turns(T, df_from(qw * kInvPi));
+    const df bd = df_split_bits(beta), qd = df_from(qw);
+    df lnT{0.f, 0.f};
+    if (pt.T.hi * fr[0].a.x < (float)kBesselLarge) lnT = df_log(pt.T);
+    unsigned long long ph = pt.v * (unsigned long long)s0.l - (1ull << 61);
+    for (int b = 0; b < nb; ++b, mo += nn, ph += pt.v) {
+      const FreqDf& f = fr[b];
+      const float4 d = pt.T.hi * f.a.x < (float)kBesselLarge
+                           ? hankel_near_df(df_mul(pt.T, df{f.a.x, f.a.y}), df_add_fast(lnT, df{f.b.z, f.b.w}), bd, true, qd)
+                           : hankel_far_df(pt, ph, ang.d, df{f.a.z, f.a.w}, df{f.b.x, f.b.y}, bd, true);
+      const float2 h = make_float2(d.x, d.z);
       reinterpret_cast<float4*>(J.A)[mo + e1] = d;
       reinterpret_cast<float4*>(J.A)[mo + e2] = d;
-      J.LU32[mo + e1] = f;
-      J.LU32[mo + e2] = f;
+      J.LU32[mo + e1] = h;
+      J.LU32[mo + e2] = h;
     }
   } else {
-    for (int l = s0.l; l < min(lsw, lend); ++l) {
-      const int b = l - s0.l;
-      const double z = (l * J.h) * R;
-      double J0, Yh;
-      bessel0_taylor(z, J0, Yh);
-      const double alpha = -0.5 * kInvPi * fma(w, lnl[b] + lratio, rl);
-      const double2 v = make_double2(fma(alpha, J0, -qw * Yh), qw * J0);
-      const long long mo = J.sys[tile.sys + b].mat_off;
-      store_self(J, mo + e1, v, f64);
-      store_self(J, mo + e2, v, f64);
+    const PairF64 pt = pair_f64(T, qw * kInvPi);
+    double lnT = 0.0;
+    if (pt.th * fr[0].a.x < (float)kBesselLarge) lnT = log_f64(T);
+    unsigned long long ph = pt.v * (unsigned long long)s0.l - (1ull << 61), u = pt.v62 * (unsigned long long)s0.l;
+    for (int b = 0; b < nb; ++b, mo += nn, ph += pt.v, u += pt.v62) {
+      const FreqDf& f = fr[b];
+      const double2 v = pt.th * f.a.x < (float)kBesselLarge
+                            ? hankel_near_f64(u, lnT + f.lnz, beta, true, qw)
+                            : hankel_far_f64(pt, ph, ang, df{f.a.z, f.a.w}, f.rs, beta, true);
+      store_self(J, mo + e1, v, J.mixed);
+      store_self(J, mo + e2, v, J.mixed);
     }
-  }
-  if (df_asm && lsw < lend) {
-    // Mixed form: the recurrence above z = 20 in double-float on the FP32 pipe (about 48 bits), stored
-    // as the pair and its FP32 rounding; FP64 only for the seeds.  (The FP64-kept form assembles the
-    // whole self matrix in FP64, as the plain form does.)
-    const df ampu_d = df_from(amp_u), invu_d = df_from(inv_u), alpha_d = df_from(alpha_a), qw_d = df_from(qw);
-    df cu_d, su_d;
-    if (hR <= 1.0) {
-      df_sincos_taylor(df_from(hR), su_d, cu_d);
-    } else {
-      double su, cu;
-      sincos(hR, &su, &cu);
-      su_d = df_from(su);
-      cu_d = df_from(cu);
-    }
-    df cx_d{0.f, 0.f}, sx_d{0.f, 0.f};
-    int since_d = 16;
-    for (int l = lsw; l < lend; ++l) {
-      const int b = l - s0.l;
-      if (since_d >= 16) {
-        df_phase_seed((l * J.h) * R, cx_d, sx_d);
-        since_d = 0;
-      }
-      const df wz = df_mul(invu_d, invl_d[b]);
-      const df w2 = df_neg(df_mul(wz, wz));
-      df P, Qa;
-      hankel_pq_df(kmax, w2, P, Qa);
-      Qa = df_mul(Qa, wz);
-      const df amp = df_mul(ampu_d, rsql_d[b]);
-      const df J0 = df_mul(amp, df_dot2(P, cx_d, Qa, sx_d));
-      const df Y0 = df_mul(amp, df_dot2(P, sx_d, df_neg(Qa), cx_d));
-      const df re = df_dot2(alpha_d, J0, df_neg(qw_d), Y0);
-      const df im = df_mul(qw_d, J0);
-      const long long mo = J.sys[tile.sys + b].mat_off;
-      const float4 d = make_float4(re.hi, re.lo, im.hi, im.lo);
-      const float2 f = make_float2(re.hi, im.hi);
-      reinterpret_cast<float4*>(J.A)[mo + e1] = d;
-      reinterpret_cast<float4*>(J.A)[mo + e2] = d;
-      J.LU32[mo + e1] = f;
-      J.LU32[mo + e2] = f;
-      const df cn = df_dot2(cx_d, cu_d, df_neg(sx_d), su_d);   // rotation by e^{i h R}
-      sx_d = df_dot2(sx_d, cu_d, cx_d, su_d);
-      cx_d = cn;
-      ++since_d;
-    }
-    return;
-  }
-  double su, cu;
-  if (hR <= 1.0) sincos_taylor(hR, su, cu);
-  else sincos(hR, &su, &cu);
-  double cx = 0.0, sx = 0.0;
-  int since = 16;
-  for (int l = lsw; l < lend; ++l) {
-    const int b = l - s0.l;
-    if (since >= 16) {
-      double sn, cs;
-      sincos((l * J.h) * R, &sn, &cs);
-      cx = (cs + sn) * kSqrtHalf;
-      sx = (sn - cs) * kSqrtHalf;
-      since = 0;
-    }
-    const double wz = inv_u * invl[b];
-    const double w2 = -wz * wz;
-    double P = c_hank_a[2 * kmax], Qa = c_hank_a[2 * kmax + 1];
-    for (int k = kmax - 1; k >= 0; --k) {
-      P = fma(P, w2, c_hank_a[2 * k]);
-      Qa = fma(Qa, w2, c_hank_a[2 * k + 1]);
-    }
-    Qa *= wz;
-    const double amp = amp_u * rsql[b];
-    const double J0 = amp * fma(P, cx, Qa * sx);
-    const double Y0 = amp * fma(P, sx, -Qa * cx);
-    const double2 v = make_double2(fma(alpha_a, J0, -qw * Y0), qw * J0);
-    const long long mo = J.sys[tile.sys + b].mat_off;
-    store_self(J, mo + e1, v, f64);
-    store_self(J, mo + e2, v, f64);
-    const double cn = fma(cx, cu, -sx * su);
-    sx = fma(sx, cu, cx * su);
-    cx = cn;
-    ++since;
   }
 }
 
@@ -836,11 +635,6 @@ constexpr int kAsmThreads = 128;   // small blocks: an 8-row task leaves a short
 constexpr int kAsmMaxThreads = 256;   // largest cross-assembly block a tuned launch may use
 constexpr int kAsmRows = 8;
 
-// A stored cross entry: FP64, or double-float (float4, same 16 bytes) in the mixed-precision form.
-__device__ __forceinline__ void store_entry(const DevJob& J, double2* p, double2 v) {
-  if (J.mixed) *reinterpret_cast<float4*>(p) = df_split2(v);
-  else *p = v;
-}
 constexpr int kAsmBand = 64;   // frequencies per assembly task (matches the planner's band cap)
 
 // Near-rule corrections of the rows of one task at N source nodes (block-wide, all threads call), in FP64:
@@ -849,8 +643,8 @@ constexpr int kAsmBand = 64;   // frequencies per assembly task (matches the pla
 // |t*| > 1, = -pi zeta^n / n (n >= 1).  The whole series sums to ln|t* - t_i| (beta is its tail from n = N on), so a row
 // with |zeta|^N < 1e-18 has beta = 0 and is marked by +0.0 at every node without any sum (an exact zero of the formula
 // would come out as -0.0): of the near rows only those next to the arc's ends keep the N-term sums and the
-// logarithms.  12-arc cavity, table of all rows: 13.9 -> 1.9 ms.  tn: the nodes t_i; ctab: 4N doubles, lam: kAsmRows x N
-// doubles of shared memory; beta may be shared or global memory.
+// logarithms.  12-arc cavity, table of all rows: 13.9 -> 1.9 ms.  tn: the nodes t_i; ctab: 2N + 1 doubles, lam:
+// kAsmRows x N doubles of shared memory; beta may be shared or global memory.
 __device__ void near_beta_block(const CrossTgt* tg, int nrows, int N, const double* __restrict__ tn, double* ctab,
                                 double* lam, double* beta) {
   __shared__ int s_full[kAsmRows], s_any;
@@ -878,7 +672,7 @@ __device__ void near_beta_block(const CrossTgt* tg, int nrows, int N, const doub
   }
   __syncthreads();
   if (s_any) {
-    for (int r = threadIdx.x; r < 4 * N; r += blockDim.x) ctab[r] = cospi((double)r / (2.0 * N));
+    for (int r = threadIdx.x; r <= 2 * N; r += blockDim.x) ctab[r] = cospi((double)r / (2.0 * N));
     __syncthreads();
   }
   for (int e = threadIdx.x; e < nrows * N; e += blockDim.x) {
@@ -893,7 +687,7 @@ __device__ void near_beta_block(const CrossTgt* tg, int nrows, int N, const doub
       for (int n = 1; n < N; ++n) {
         ph += step;
         if (ph >= mod) ph -= mod;
-        acc = fma(lr[n], ctab[ph], acc);
+        acc = fma(lr[n], ctab[ph <= 2 * N ? ph : mod - ph], acc);
       }
       v = -kTwoOverPi * fma(lr[0] + 2.0 * acc, kInvPi, -log(fabs(tg[r].tstar - tn[i])));
     }
@@ -988,20 +782,27 @@ __device__ __forceinline__ double2 asym_entry(AsymState& a, const PairSetup& s, 
   return make_double2(amp * fma(s.beta, t1, -t2), amp * t1);
 }
 
-// kNear: the launch over the tasks with near rows (shared memory for their product-integration weights);
-// otherwise over the far-only tasks, which need only the band tables (more CTAs per SM).  Each launch skips
-// the other kind of task.
-template <bool kNear>
+// kNear: the launch over the tasks with near rows (shared memory for their corrections); otherwise over the far-only
+// tasks, which need only the tables (more CTAs per SM).  Each launch skips the other kind of task.  kForm: 0 the FP64
+// form, 1 the mixed form (double-float entries), 2 the FP64-kept form (double-float, FP64 below z = 20).  A thread
+// owns (row, source) pairs and walks the band's frequencies.  Bound by the FP64 pipe in form 0 (9 instructions an entry,
+// ~25 a pair; 8 obstacle arcs, 4.8e8 entries: 33.2 -> 11.7 ms), by FP32 issue in forms 1 and 2 (~130 instructions;
+// 10.7 -> 4.2 ms; N = 512 with 2.6e9 entries: 29.3 -> 14.1 ms).
+constexpr int kFormF64 = 0, kFormMixed = 1, kFormKeep = 2;
+template <bool kNear, int kForm>
 __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
-  extern __shared__ double sha[];
+  extern __shared__ __align__(16) double sha[];
   const CrossAsm task = J.asms[blockIdx.x];
   const PairDesc pr = J.pairs[task.pair];
   const int N = task.N;
   const Panel pn = J.panels[task.panel];
   const CrossTgt* tg = J.tgts + pr.tgt_off + task.row0;
-  double* ctab = sha;                                // 4N: cospi(r/(2N))
-  double* lam = sha + 4 * N;                         // kAsmRows x N
-  double* Wn = kNear ? lam + kAsmRows * N : sha;     // kAsmRows x N near corrections beta (near launch only)
+  const int nl = task.l1 - task.l0 + 1;
+  FreqDf* fr = reinterpret_cast<FreqDf*>(sha);       // kAsmBand
+  double* bt = sha + kAsmBand * (sizeof(FreqDf) / sizeof(double));   // near launch: kAsmRows x N corrections,
+  double* lam = bt + kAsmRows * N;                   // kAsmRows x N and
+  double* ctab = lam + kAsmRows * N;                 // 2N + 1 doubles of near_beta_block
+  __shared__ AngleTab ang;
   __shared__ int any_near;
   if (threadIdx.x == 0) {
     int a = 0;
@@ -1010,109 +811,61 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
   }
   __syncthreads();
   if ((any_near != 0) != kNear) return;
-  if (kNear) near_beta_block(tg, task.nrows, N, J.node_t + pn.off, ctab, lam, Wn);
-  const double w = kPiD / N, qw = 0.25 * w;
-  const double A1 = -0.5 * kInvPi * w;          // coefficient of ln l below z = 20
-  const double camp = kSqrtTwoOverPi * qw;      // sqrt(2/pi) w/4
-  const double inv_h = 1.0 / J.h;
-  const int ld = pr.nrows;   // blocks are stored source-major: E[i * nrows + row]
-  const int nl = task.l1 - task.l0 + 1;
-  // per-band tables: 1/l, 1/sqrt(l), ln l and omega_l = l h
-  double* invl = kNear ? Wn + kAsmRows * N : sha;    // <= kAsmBand each
-  double* rsql = invl + kAsmBand;
-  double* lnl = rsql + kAsmBand;
-  double* lh = lnl + kAsmBand;
-  df* invl_d = reinterpret_cast<df*>(lh + kAsmBand);      // the same as double-float (mixed form)
-  df* rsql_d = invl_d + kAsmBand;
-  df* lnl_d = rsql_d + kAsmBand;
-  df* lh_d = lnl_d + kAsmBand;
-  for (int b = threadIdx.x; b < nl; b += blockDim.x) {
-    const int l = task.l0 + b;
-    invl[b] = 1.0 / l;
-    rsql[b] = rsqrt((double)l);
-    lnl[b] = log((double)l);
-    lh[b] = l * J.h;
-    if (J.mixed) {
-      invl_d[b] = df_from(invl[b]);
-      rsql_d[b] = df_from(rsql[b]);
-      lnl_d[b] = df_from(lnl[b]);
-      lh_d[b] = df_from(lh[b]);
-    }
-  }
+  load_angles(ang, kForm == kFormF64);
+  for (int b = threadIdx.x; b < nl; b += blockDim.x) fr[b] = J.freq_df[task.l0 + b];
+  if (kNear) near_beta_block(tg, task.nrows, N, J.node_t + pn.off, ctab, lam, bt);
   __syncthreads();
-  const long long* eo = J.e_off + (long long)task.pair * J.L;
+  const double qw = 0.25 * kPiD / N, camp4 = qw * kInvPi, turns = J.h * (0.5 * kInvPi);
+  const df qd = df_from(qw), cd = df_from(camp4);
+  const int ld = pr.nrows;   // blocks are stored source-major: E[i * nrows + row]
+  const long long* eo = J.e_off + (long long)task.pair * J.L + task.l0;
   for (int e = threadIdx.x; e < task.nrows * N; e += blockDim.x) {
     const int r = e % task.nrows, i = e / task.nrows;
     const CrossTgt t = tg[r];
-    const PairSetup ps = pair_setup(J, t, J.node_x[pn.off + i], J.node_y[pn.off + i],
-                                    kNear && t.near ? Wn[r * N + i] : 0.0, task.l0, w, inv_h);
+    const double dx = t.x - J.node_x[pn.off + i], dy = t.y - J.node_y[pn.off + i];
+    const double T = turns * dist_f64(fma(dx, dx, dy * dy));
+    const double beta = kNear && t.near ? bt[r * N + i] : 0.0;
+    const bool near = kNear && beta != 0.0;
     double2* Ep = J.E + (long long)i * ld + task.row0 + r;
-    const int lend = min(ps.lsw, task.l1 + 1);
-    if (J.mixed && !J.fp64keep) {
-      // Mixed form, z < 20: the Taylor range in double-float, stored as double-float pairs.
-      const df R_d = df_from(ps.R), A0_d = df_from(ps.A0), A1_d = df_from(A1), qw_d = df_from(qw);
-      for (int l = task.l0; l < lend; ++l) {
-        const int b = l - task.l0;
-        df J0, Yh;
-        bessel0_taylor_df(df_mul(lh_d[b], R_d), J0, Yh);
-        const df alpha = df_add_fast(df_mul(A1_d, lnl_d[b]), A0_d);
-        const df re = df_dot2(alpha, J0, df_neg(qw_d), Yh);
-        const df im = df_mul(qw_d, J0);
-        *reinterpret_cast<float4*>(Ep + eo[l]) = make_float4(re.hi, re.lo, im.hi, im.lo);
+    if (kForm == kFormF64) {
+      const PairF64 pt = pair_f64(T, camp4);
+      const double lnT = pt.th * fr[0].a.x < (float)kBesselLarge ? log_f64(T) : 0.0;
+      unsigned long long ph = pt.v * (unsigned long long)task.l0 - (1ull << 61),
+                         u = pt.v62 * (unsigned long long)task.l0;
+      for (int b = 0; b < nl; ++b, ph += pt.v, u += pt.v62) {
+        const FreqDf& f = fr[b];
+        Ep[eo[b]] = pt.th * f.a.x < (float)kBesselLarge
+                        ? hankel_near_f64(u, lnT + f.lnz, beta, near, qw)
+                        : hankel_far_f64(pt, ph, ang, df{f.a.z, f.a.w}, f.rs, beta, near);
       }
     } else {
-      for (int l = task.l0; l < lend; ++l) {
-        const int b = l - task.l0;
-        store_entry(J, Ep + eo[l], taylor_entry(ps, lh[b], lnl[b], A1, qw));
-      }
-    }
-    if (ps.lsw > task.l1) continue;
-    const int lsw = ps.lsw;
-    if (J.mixed) {
-      // Mixed form: the same recurrence in double-float on the FP32 pipe (about 48 bits), stored as
-      // the double-float pairs the mixed-form apply reads; FP64 only for the seeds (the step
-      // rotation e^{i h R} itself is evaluated in double-float).
-      const AsymState as = asym_start(ps, lh[lsw - task.l0], camp, false);
-      const df ampw_d = df_from(as.ampw), invu_d = df_from(ps.inv_u), beta_d = df_from(ps.beta);
-      df cu_d, su_d;
-      if (ps.hR <= 1.0) {
-        df_sincos_taylor(df_from(ps.hR), su_d, cu_d);
-      } else {
-        double su, cu;
-        sincos(ps.hR, &su, &cu);
-        su_d = df_from(su);
-        cu_d = df_from(cu);
-      }
-      df cx_d{0.f, 0.f}, sx_d{0.f, 0.f};
-      int since_d = 16;
-      for (int l = lsw; l <= task.l1; ++l) {
-        const int b = l - task.l0;
-        if (since_d >= 16) {
-          df_phase_seed(lh[b] * ps.R, cx_d, sx_d);
-          since_d = 0;
+      const PairTurns pt = pair_turns(T, cd);
+      const df bd = kNear ? df_split_bits(beta) : df{0.f, 0.f};
+      df lnT{0.f, 0.f};
+      double lnT64 = 0.0;
+      unsigned long long v62 = 0ull;
+      if (pt.T.hi * fr[0].a.x < (float)kBesselLarge) {
+        if (kForm == kFormKeep) {
+          lnT64 = log_f64(T);
+          v62 = turn_fraction(0.25 * T);
+        } else {
+          lnT = df_log(pt.T);
         }
-        const df wz = df_mul(invu_d, invl_d[b]);
-        const df w2 = df_neg(df_mul(wz, wz));
-        df P, Qa;
-        hankel_pq_df(as.kmax, w2, P, Qa);
-        Qa = df_mul(Qa, wz);
-        const df a = df_mul(ampw_d, rsql_d[b]);
-        const df t1 = df_dot2(P, cx_d, Qa, sx_d);
-        const df t2 = df_dot2(P, sx_d, df_neg(Qa), cx_d);
-        const df re = df_mul(a, df_dot2(beta_d, t1, df{-1.f, 0.f}, t2));
-        const df im = df_mul(a, t1);
-        *reinterpret_cast<float4*>(Ep + eo[l]) = make_float4(re.hi, re.lo, im.hi, im.lo);
-        const df cn = df_dot2(cx_d, cu_d, df_neg(sx_d), su_d);   // rotation by e^{i h R}
-        sx_d = df_dot2(sx_d, cu_d, cx_d, su_d);
-        cx_d = cn;
-        ++since_d;
       }
-      continue;
-    }
-    AsymState as = asym_start(ps, lh[lsw - task.l0], camp);
-    for (int l = lsw; l <= task.l1; ++l) {
-      const int b = l - task.l0;
-      store_entry(J, Ep + eo[l], asym_entry(as, ps, lh[b], invl[b], rsql[b]));
+      unsigned long long ph = pt.v * (unsigned long long)task.l0 - (1ull << 61);
+      for (int b = 0; b < nl; ++b, ph += pt.v) {
+        const FreqDf& f = fr[b];
+        float4 d;
+        if (pt.T.hi * f.a.x < (float)kBesselLarge) {
+          if (kForm == kFormKeep)
+            d = split2_bits(hankel_near_f64(v62 * (unsigned long long)(task.l0 + b), lnT64 + f.lnz, beta, near, qw));
+          else
+            d = hankel_near_df(df_mul(pt.T, df{f.a.x, f.a.y}), df_add_fast(lnT, df{f.b.z, f.b.w}), bd, near, qd);
+        } else {
+          d = hankel_far_df(pt, ph, ang.d, df{f.a.z, f.a.w}, df{f.b.x, f.b.y}, bd, near);
+        }
+        *reinterpret_cast<float4*>(Ep + eo[b]) = d;
+      }
     }
   }
 }
@@ -1126,7 +879,8 @@ __global__ void __launch_bounds__(kAsmThreads) k_near_weights(DevJob J) {
   extern __shared__ double shn[];
   const CrossAsm task = J.asms[blockIdx.x];
   const CrossTgt* tg = J.tgts + J.pairs[task.pair].tgt_off + task.row0;
-  near_beta_block(tg, task.nrows, task.N, J.node_t + J.panels[task.panel].off, shn, shn + 4 * task.N, J.wn + off);
+  near_beta_block(tg, task.nrows, task.N, J.node_t + J.panels[task.panel].off, shn,
+                  shn + 2 * task.N + 1, J.wn + off);
 }
 
 // One CTA per (assembly task, band of at most otf_band(Q) frequencies): thread (row r, source group g)
@@ -1211,7 +965,7 @@ __global__ void __launch_bounds__(kAsmThreads) k_cross_otf(DevJob J) {
 // 8 to 16 of its 128 threads worked, and each pair paid two sine/cosine series; 12-arc cavity, 5.7e8 pairs x 5 steps,
 // four windows: 501 -> 91 ms; 6 arcs at N = 1024, two windows:
 // 499 -> 335 ms.  Bound by FP32 issue (~125 instructions an entry and 48 a window).
-// kKeep64 (the FP64-kept form): entries below z = 20 from the FP64 Taylor form.
+// kKeep64 (the FP64-kept form): entries below z = 20 in FP64.
 constexpr int kOtfThreads = 32 * kAsmRows;
 __host__ __device__ constexpr int otf_regs(int Q) { return Q == 1 ? 8 : Q == 2 ? 4 : 1; }
 // blocks per SM: 16 warps of 128 registers, or 24 of 80 where the few sums leave room (measured per Q)
@@ -1272,7 +1026,7 @@ __global__ void __launch_bounds__(kOtfThreads, otf_blocks(Q)) k_cross_otf_df(Dev
   const CrossTgt t = J.tgts[pr.tgt_off + task.row0 + r];
   const double* __restrict__ bt = t.near ? J.wn + woff + (long long)r * N : nullptr;
   const bool near = bt && __double_as_longlong(__ldg(bt)) != 0;     // (+0.0: beta vanishes on the whole row)
-  const double w = kKeep64 ? kPiD / N : 0.0, turns = J.h * (0.5 * kInvPi);
+  const double qw64 = kKeep64 ? 0.25 * kPiD / N : 0.0, turns = J.h * (0.5 * kInvPi);
   const df qw = s_qw, camp4 = s_camp4;
   const double* __restrict__ nx = J.node_x + pn.off;
   const double* __restrict__ ny = J.node_y + pn.off;
@@ -1298,10 +1052,15 @@ __global__ void __launch_bounds__(kOtfThreads, otf_blocks(Q)) k_cross_otf_df(Dev
         beta = df_split_bits(beta64);
       }
       df lnT{0.f, 0.f};
-      double A0 = 0.0;
+      double lnT64 = 0.0;
+      unsigned long long v62 = 0ull;
       if (pt.T.hi * fr[b0].a.x < (float)kBesselLarge) {             // the block's first entry is below z = 20
-        if (kKeep64) A0 = w * fma(-0.5 * kInvPi, log(T) + 1.7219455507509330, 0.25 * beta64);   // + ln pi + gamma
-        else lnT = df_log(pt.T);
+        if (kKeep64) {
+          lnT64 = log_f64(T);
+          v62 = turn_fraction(0.25 * T);
+        } else {
+          lnT = df_log(pt.T);
+        }
       }
       unsigned long long ph = pt.v * (unsigned long long)(ot.l0 + b0) - (1ull << 61);
 #pragma unroll
@@ -1313,10 +1072,7 @@ __global__ void __launch_bounds__(kOtfThreads, otf_blocks(Q)) k_cross_otf_df(Dev
           for (int q = 0; q < Q; ++q) pv[q] = __ldg(&J.phi_df[vo[b0 + k] + i + (long long)q * N]);
           if (pt.T.hi * f.a.x < (float)kBesselLarge) {
             if (kKeep64) {
-              double J0, Yh;
-              bessel0_taylor(T * ((2.0 * kPiD) * (double)(ot.l0 + b0 + k)), J0, Yh);
-              const double alpha = fma(-0.5 * kInvPi * w, f.lnl, A0);
-              e = df_split2(make_double2(fma(alpha, J0, -0.25 * w * Yh), 0.25 * w * J0));
+              e = split2_bits(hankel_near_f64(v62 * (unsigned long long)(ot.l0 + b0 + k), lnT64 + f.lnz, beta64, near, qw64));
             } else {
               e = hankel_near_df(df_mul(pt.T, df{f.a.x, f.a.y}), df_add_fast(lnT, df{f.b.z, f.b.w}), beta, near, qw);
             }
@@ -2504,11 +2260,8 @@ cudaError_t launch_bessel0(const double* z, double* j0, double* y0, double* yh, 
 cudaError_t launch_tables(const DevJob& J, cudaStream_t st, int* launches) {
   k_fft_tw<<<cdiv(J.K / 2, 256), 256, 0, st>>>(J.fft_tw, J.fft_tw_df, J.K);
   k_freq_tw<<<cdiv((long long)J.Q * J.L, 256), 256, 0, st>>>(J);
-  *launches += 2;
-  if (J.freq_df) {
-    k_freq_df<<<cdiv(J.L, 128), 128, 0, st>>>(J);
-    *launches += 1;
-  }
+  k_freq_df<<<cdiv(J.L, 128), 128, 0, st>>>(J);
+  *launches += 3;
   if (J.n_rlogN > 0) {
     cudaError_t e = launch_tables_rlog_only(J, st, launches);
     if (e != cudaSuccess) return e;
@@ -2532,8 +2285,14 @@ cudaError_t launch_tables_rlog_only(const DevJob& J, cudaStream_t st, int* launc
 
 cudaError_t launch_assemble_self(const DevJob& J, cudaStream_t st, int* launches) {
   if (J.n_tiles > 0) {
-    k_assemble_self<<<J.n_tiles, 256, 0, st>>>(J);
-    *launches += 1;
+    if (!J.mixed || J.fp64keep || J.max_n >= J.f64_min_n) {
+      k_assemble_self<false><<<J.n_tiles, 256, 0, st>>>(J);
+      *launches += 1;
+    }
+    if (J.mixed && !J.fp64keep) {
+      k_assemble_self<true><<<J.n_tiles, 256, 0, st>>>(J);
+      *launches += 1;
+    }
   }
   // the row bounds of the FP64 matrices, for the first-pass residual's anchors
   const bool any64 = J.mixed && (J.fp64keep || J.max_n >= J.f64_min_n);
@@ -2605,19 +2364,20 @@ cudaError_t launch_fused_asf(const DevJob& J, int* counter, cudaStream_t st, int
 
 cudaError_t launch_cross_assemble(const DevJob& J, cudaStream_t st, int* launches) {
   if (J.n_asm == 0) return cudaSuccess;
-  // Shared layout of k_cross_assemble, in 8-byte words: ctab 4N, lam kAsmRows N, Wn kAsmRows N, then
-  // band tables invl, rsql, lnl, lh (doubles) and invl_d, rsql_d, lnl_d, lh_d (double-float pairs),
-  // kAsmBand each.
-  // (the far-only launch: the band tables alone)
-  const size_t sh = ((size_t)(4 + 2 * kAsmRows) * J.max_n + 8 * kAsmBand) * sizeof(double);
-  const size_t sh_far = (size_t)8 * kAsmBand * sizeof(double);
+  const size_t sh_far = (size_t)kAsmBand * sizeof(FreqDf);   // (the far-only launch: the band's constants alone)
+  const size_t sh = sh_far + (size_t)((2 * kAsmRows + 2) * J.max_n + 1) * sizeof(double);
   const int nt = J.shape_asm > 0 ? J.shape_asm : kAsmThreads;
-  cudaError_t e = cudaFuncSetAttribute(k_cross_assemble<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
-  if (e != cudaSuccess) return e;
-  k_cross_assemble<true><<<J.n_asm, nt, sh, st>>>(J);
-  k_cross_assemble<false><<<J.n_asm, nt, sh_far, st>>>(J);
+  auto go = [&](auto form) {
+    constexpr int F = decltype(form)::value;
+    cudaError_t e = cudaFuncSetAttribute(k_cross_assemble<true, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+    if (e != cudaSuccess) return e;
+    k_cross_assemble<true, F><<<J.n_asm, nt, sh, st>>>(J);
+    k_cross_assemble<false, F><<<J.n_asm, nt, sh_far, st>>>(J);
+    return cudaGetLastError();
+  };
   *launches += 2;
-  return cudaGetLastError();
+  return !J.mixed ? go(std::integral_constant<int, kFormF64>{}) : J.fp64keep ? go(std::integral_constant<int, kFormKeep>{})
+                                                               : go(std::integral_constant<int, kFormMixed>{});
 }
 
 static size_t time_smem(const DevJob& J) { return (size_t)J.K * sizeof(double2) + (size_t)J.NT * sizeof(double); }
@@ -2814,7 +2574,7 @@ cudaError_t launch_cross_apply(const DevJob& J, cudaStream_t st, int* launches) 
 
 cudaError_t launch_near_weights(const DevJob& J, cudaStream_t st, int* launches) {
   if (J.n_asm == 0) return cudaSuccess;
-  const size_t sh = (size_t)(4 + kAsmRows) * J.max_n * sizeof(double);   // ctab 4N, lam kAsmRows N
+  const size_t sh = (size_t)((2 + kAsmRows) * J.max_n + 1) * sizeof(double);   // ctab 2N + 1, lam kAsmRows N
   cudaError_t e = cudaFuncSetAttribute(k_near_weights, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
   if (e != cudaSuccess) return e;
   k_near_weights<<<J.n_asm, kAsmThreads, sh, st>>>(J);

@@ -135,3 +135,17 @@ def test_every_step_rows_at_warp_and_band_edges(F, ctx, Q, N, precision):
     assert math.sqrt(num / den) < 1e-10
     t = ref.traces()
     assert np.max(np.abs(job.traces() - t)) < 1e-10 * np.max(np.abs(t))
+
+
+@pytest.mark.parametrize("N", [5, 47, 96, 200])
+@pytest.mark.parametrize("kappa", [0.01, 3.0, 19.9, 60.0, 700.0])
+def test_self_matrix_over_the_hankel_ranges(F, N, kappa):
+    """Taylor range, asymptotic range and both in one matrix, nearly closed arc (small |t - s| against R).  1e-13 of the
+    largest entry, the bar of the self-matrix parity test."""
+    curve, arc = wl.star(0.3, 5, 0.4), (0.1, 0.1 + 5.9)
+    A = torch.empty(2 * N * N, dtype=torch.float64, device="cuda")
+    F.fthms_assemble_self(curve, arc, N, kappa, A.data_ptr())
+    got = A.cpu().numpy().reshape(N, N, 2)
+    got = (got[..., 0] + 1j * got[..., 1]).T
+    ref = oker.self_matrix(geo.Arc(0, 0, curve, *arc), N, kappa)
+    assert np.max(np.abs(got - ref)) <= 1e-13 * np.max(np.abs(ref))
