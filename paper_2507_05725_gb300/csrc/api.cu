@@ -285,19 +285,21 @@ fthms_status upload_job(fthms_req* r) {
   J.otf_tasks = nullptr;
   J.wn_off = nullptr;
   J.wn = nullptr;
-  J.otf_res_off = nullptr;
-  if (J.mixed || J.otf) {
-    TRY(dev_upload(r, p.grp_res_off, &J.grp_res_off));
-    TRY(dev_alloc(r, (size_t)std::max(1LL, p.res_total) * p.Q, &J.apply_res));
-  }
-  if (J.mixed && !J.otf) {
+  J.row_off = nullptr;
+  J.e_unit = nullptr;
+  J.phi_unit = nullptr;
+  TRY(dev_upload(r, p.grp_res_off, &J.grp_res_off));
+  TRY(dev_upload(r, p.row_off, &J.row_off));
+  TRY(dev_alloc(r, (size_t)std::max(1LL, p.res_total) * p.Q, &J.apply_res));
+  if (!J.otf) {
     TRY(dev_upload(r, p.slices, &J.slices));
     J.n_slices = (int)p.slices.size();
+    TRY(dev_alloc(r, (size_t)std::max(1LL, p.res_total), &J.e_unit));
+    TRY(dev_alloc(r, p.sys.size() * 4, &J.phi_unit));
   }
   if (J.otf) {
     TRY(dev_upload(r, p.otf, &J.otf_tasks));
     TRY(dev_upload(r, p.wn_off, &J.wn_off));
-    TRY(dev_upload(r, p.otf_res_off, &J.otf_res_off));
     TRY(dev_alloc(r, (size_t)p.wn_total, &J.wn));
     J.n_otf = (int)p.otf.size();
     // launch order: about a golden-section stride, made coprime to the task count
@@ -378,7 +380,7 @@ fthms_status upload_job(fthms_req* r) {
     }
   }
   J.phi_df = nullptr;
-  if (J.mixed) TRY(dev_alloc(r, (size_t)p.vec_total, &J.phi_df));
+  if (J.mixed || !J.otf) TRY(dev_alloc(r, (size_t)p.vec_total, &J.phi_df));
   TRY(dev_alloc(r, (size_t)p.vec_total, &J.phi_sum));
   J.phi_all = nullptr;
   if (p.opt.keep_densities) TRY(dev_alloc(r, (size_t)p.vec_total * p.M, &J.phi_all));

@@ -1,0 +1,78 @@
+// Fixed-point cross rows: entries and densities as 56-bit integers in two 28-bit halves, multiplied and summed exactly by
+// 32 x 32 + 64 -> 64-bit multiply-adds.  GB300 issues 64 of those a clock and SM against 2 FP64 lanes and, with its
+// compensation, the equivalent of 2.7 double-float ones: 12 per complex product instead of 4 FP64 FMAs (256 issue
+// slots' worth) or 48 FP32 instructions, so the matvec runs at the speed of its 16 bytes an entry.  A row shares one power
+// of two (a bound of its entries at that frequency), a density vector one per system and window; the rounding to
+// 2^-56 of that bound is the only one before the final conversion (FP64 sums round at every step).
+#pragma once
+#include <cuda_runtime.h>
+
+namespace fthms {
+
+constexpr int kFixBits = 55;            // |X| < 2^55
+
+// v = (x 2^28 + y) 2^(s - 55) for |v| < 2^s, |x| <= 2^27, |y| <= 2^27, rounded to the last place.
+__device__ __forceinline__ int2 fix_split(long long X) {
+  const int x = (int)((X + (1ll << 27)) >> 28);
+  return make_int2(x, (int)(X - ((long long)x << 28)));
+}
+__device__ __forceinline__ int2 fix_f64(double v, int s) {
+  const unsigned h = (unsigned)__double2hiint(v);
+  const int e = (int)((h >> 20) & 0x7FFu);
+  unsigned long long m = ((unsigned long long)((h & 0xFFFFFu) | 0x100000u) << 32) | (unsigned)__double2loint(v);
+  const int sh = e - 1075 + kFixBits - s;               // <= 2
+  if (e == 0 || sh < -60) m = 0ull;
+  else if (sh >= 0) m <<= min(sh, 8);
+  else m = (m + (1ull << (-sh - 1))) >> -sh;
+  return fix_split((h >> 31) ? -(long long)m : (long long)m);
+}
+// The same for a double-float value (c = 2^(27 - s)).
+__device__ __forceinline__ int2 fix_df(float hi, float lo, float c) {
+  const float y = __fmul_rn(hi, c);                     // exact
+  const int a = __float2int_rn(y);
+  const float t = fmaf(lo, c, __fsub_rn(y, (float)a));  // |t| < 5
+  const float q = rintf(t);
+  return make_int2(a + (int)q, __float2int_rn(__fmul_rn(__fsub_rn(t, q), 268435456.f)));
+}
+
+// One warp: N values of a density vector in fixed point, and their unit.  A vector with a value that is not finite gets
+// the unit NaN, so that every sum it enters is NaN.
+__device__ __forceinline__ void fix_vector(const double2* v, int N, double scale, int4* out, double* unit, int lane) {
+  unsigned m = 0u;
+  for (int i = lane; i < N; i += 32)
+    m = max(m, max((unsigned)__double2hiint(v[i].x) & 0x7FFFFFFFu, (unsigned)__double2hiint(v[i].y) & 0x7FFFFFFFu));
+  m = __reduce_max_sync(0xffffffffu, m);
+  const int e = max((int)(m >> 20), 100);               // (zero or tiny: any unit does)
+  const int s = e - 1022;
+  for (int i = lane; i < N; i += 32) {
+    const int2 a = fix_f64(v[i].x, s), b = fix_f64(v[i].y, s);
+    out[i] = make_int4(a.x, a.y, b.x, b.y);
+  }
+  if (lane == 0)
+    *unit = e >= 0x7FF ? __longlong_as_double(0x7FF8000000000000ll)
+                       : scale * __hiloint2double((e - 1022 - kFixBits + 1023) << 20, 0);
+}
+
+// Exact sum of products (the products of two low halves, below 2^-56 of the bounds' product, are dropped); at most
+// kFixRun products between carries (one adds below 2^55 to either running sum).
+constexpr int kFixRun = 64;
+struct fixacc {
+  long long a = 0, b = 0, c = 0;          // high products, cross products (2^28 below), carries (2^32 above)
+  __device__ __forceinline__ void mac(int x0, int x1, int y0, int y1) {
+    a += (long long)x0 * y0;
+    b += (long long)x0 * y1;
+    b += (long long)x1 * y0;
+  }
+  __device__ __forceinline__ void carry() {
+    a += b >> 28;
+    b &= 0xFFFFFFFll;
+    c += a >> 32;
+    a &= 0xFFFFFFFFll;
+  }
+  __device__ __forceinline__ double value() {           // in units of 2^56
+    carry();
+    return fma((double)c, 4294967296.0, (double)a + 0x1p-28 * (double)b);
+  }
+};
+
+}  // namespace fthms

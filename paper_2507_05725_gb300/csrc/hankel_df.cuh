@@ -308,14 +308,16 @@ __device__ double2 c_angle_f64[kAngles];
 __device__ Tay64 c_tay64[kTay64 + 1][2];        // J0, Yhat0
 __device__ double2 c_log_f64[1024];             // reciprocal (12 bits) of the 1024th's centre, -ln of it
 
-struct AngleTab {                       // shared-memory copy
+template <bool kF64>
+struct AngleTab {                       // shared-memory copy (the FP64 values for FP64 entries only)
   float4 d[kAngles];
-  double2 f[kAngles];
+  double2 f[kF64 ? kAngles : 1];
 };
-__device__ __forceinline__ void load_angles(AngleTab& t, bool f64) {
+template <bool kF64>
+__device__ __forceinline__ void load_angles(AngleTab<kF64>& t) {
   for (int k = threadIdx.x; k < kAngles; k += blockDim.x) {
     t.d[k] = c_angle_df[k];
-    if (f64) t.f[k] = c_angle_f64[k];
+    if (kF64) t.f[k] = c_angle_f64[k];
   }
 }
 
@@ -363,7 +365,7 @@ __device__ __forceinline__ PairF64 pair_f64(double T, double camp4) {
 }
 
 // z >= 20; p = l v - 1/8 turn, rs = 1/sqrt(l).
-__device__ __forceinline__ double2 hankel_far_f64(const PairF64& pr, unsigned long long p, const AngleTab& ang, df iv,
+__device__ __forceinline__ double2 hankel_far_f64(const PairF64& pr, unsigned long long p, const AngleTab<true>& ang, df iv,
                                                   double rs, double beta, bool near) {
   const FarAngle f = far_angle<true>(pr.iu, p, iv);
   const float4 t = ang.d[f.idx];

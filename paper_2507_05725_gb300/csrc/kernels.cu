@@ -23,6 +23,7 @@
 #include "bessel.cuh"
 #include "cplx.cuh"
 #include "df64.cuh"
+#include "fixed.cuh"
 #include "hankel_df.cuh"
 #include "kernels.h"
 #include "lu_common.cuh"
@@ -237,9 +238,9 @@ __global__ void __launch_bounds__(256) k_assemble_self(DevJob J) {
   const SysDesc s0 = J.sys[tile.sys];
   const int N = s0.N, nb = tile.nsys;
   if (kDf == (!J.mixed || sys_f64(J, N))) return;       // the other launch's systems
-  __shared__ AngleTab ang;
+  __shared__ AngleTab<!kDf> ang;
   __shared__ FreqDf fr[kSelfBand];
-  load_angles(ang, !kDf);
+  load_angles(ang);
   if (threadIdx.x < nb) fr[threadIdx.x] = J.freq_df ? J.freq_df[s0.l + threadIdx.x] : make_freq(s0.l + threadIdx.x);
   __syncthreads();
   const int i = tile.ti * kSelfTile + (threadIdx.x % kSelfTile);
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(256) k_assemble_self(DevJob J) {
   const double dy = J.node_y[pn.off + i] - J.node_y[pn.off + c];
   const double T = (J.h * (0.5 * kInvPi)) * dist_f64(fma(dx, dx, dy * dy));
   const double beta = kTwoOverPi * (log_f64(fabs(J.node_t[pn.off + i] - J.node_t[pn.off + c])) - rl * (N * kInvPi));
-  if (kDf) {
+  if constexpr (kDf) {
     const PairTurns pt = pair_turns(T, df_from(qw * kInvPi));
     const df bd = df_split_bits(beta), qd = df_from(qw);
     df lnT{0.f, 0.f};
@@ -530,6 +531,13 @@ __device__ void solve_one(const DevJob& J, int sidx, int m, double2* b, int lane
     sum[e] = m == 1 ? v : cadd(sum[e], v);
     if (all) all[e] = v;
   }
+  if (!J.otf) {
+    __syncwarp();
+#pragma unroll 1
+    for (int q = 0; q < QT; ++q)
+      fix_vector(b + q * N, N, 1.0, reinterpret_cast<int4*>(J.phi_df) + s.vec_off + (long long)q * N,
+                 J.phi_unit + 4ll * sidx + q, lane);
+  }
 }
 
 template <int QT>
@@ -602,6 +610,10 @@ __device__ __noinline__ void fused_solve(const DevJob& J, int sidx, int q, doubl
     J.phi[o + e] = v;
     J.phi_sum[o + e] = v;
     if (all) all[e] = v;
+  }
+  if (!J.otf) {
+    __syncwarp();
+    fix_vector(b, N, 1.0, reinterpret_cast<int4*>(J.phi_df) + o, J.phi_unit + 4ll * sidx + q, lane);
   }
 }
 
@@ -802,8 +814,10 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
   double* bt = sha + kAsmBand * (sizeof(FreqDf) / sizeof(double));   // near launch: kAsmRows x N corrections,
   double* lam = bt + kAsmRows * N;                   // kAsmRows x N and
   double* ctab = lam + kAsmRows * N;                 // 2N + 1 doubles of near_beta_block
-  __shared__ AngleTab ang;
+  __shared__ AngleTab<kForm == kFormF64> ang;
   __shared__ int any_near;
+  __shared__ unsigned s_r2[kAsmRows], s_beta[kAsmRows];   // smallest R^2, largest |beta| of a row (FP32 bits)
+  __shared__ short s_exp[kAsmRows][kAsmBand];             // entries of (row, frequency) stay below 2^s_exp
   if (threadIdx.x == 0) {
     int a = 0;
     for (int r = 0; r < task.nrows; ++r) a |= tg[r].near;
@@ -811,11 +825,40 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
   }
   __syncthreads();
   if ((any_near != 0) != kNear) return;
-  load_angles(ang, kForm == kFormF64);
+  load_angles(ang);
   for (int b = threadIdx.x; b < nl; b += blockDim.x) fr[b] = J.freq_df[task.l0 + b];
+  if (threadIdx.x < kAsmRows) {
+    s_r2[threadIdx.x] = 0x7F7FFFFFu;
+    s_beta[threadIdx.x] = 0u;
+  }
   if (kNear) near_beta_block(tg, task.nrows, N, J.node_t + pn.off, ctab, lam, bt);
   __syncthreads();
   const double qw = 0.25 * kPiD / N, camp4 = qw * kInvPi, turns = J.h * (0.5 * kInvPi);
+  // Fixed-point unit per row and frequency: |E| <= (w/4) |H0(z_min)| (1 + max |beta|), |H0(z)| <= sqrt(2/(pi z)) for
+  // every z > 0 (z |H0|^2 increases to 2/pi), and <= 1.5 - 0.64 ln z below 1.  A row through a node, or with a
+  // coordinate that is not a number, gets the unit NaN, as its entries would be.
+  for (int e = threadIdx.x; e < task.nrows * N; e += blockDim.x) {
+    const int r = e % task.nrows, i = e / task.nrows;
+    const double dx = tg[r].x - J.node_x[pn.off + i], dy = tg[r].y - J.node_y[pn.off + i];
+    const float R2 = (float)fma(dx, dx, dy * dy);
+    atomicMin(&s_r2[r], R2 > 0.f ? __float_as_uint(R2) : 0u);
+    if (kNear && tg[r].near) atomicMax(&s_beta[r], __float_as_uint(fabsf((float)bt[r * N + i])));
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < task.nrows * nl; e += blockDim.x) {
+    const int r = e / nl, b = e % nl;
+    const float T = (float)turns * sqrtf(__uint_as_float(s_r2[r])) * 0.99999f;
+    const float z = T * fr[b].a.x;
+    float hb = sqrtf(0.63661978f / z);
+    if (z < 1.f) hb = fminf(hb, 1.5f - 0.64f * logf(z));
+    const float bound = (float)qw * hb * (1.f + __uint_as_float(s_beta[r])) * 1.0001f;
+    const int s = (int)(__float_as_uint(bound) >> 23) - 126;
+    s_exp[r][b] = (short)s;
+    J.e_unit[J.row_off[(long long)task.pair * J.L + task.l0 + b] + task.row0 + r] =
+        s_r2[r] != 0u && s_r2[r] < 0x7F7FFFFFu && s > -60 && s < 120 ? __uint_as_float((unsigned)(s - kFixBits + 127) << 23)
+                                                                   : __uint_as_float(0x7FFFFFFFu);
+  }
+  __syncthreads();
   const df qd = df_from(qw), cd = df_from(camp4);
   const int ld = pr.nrows;   // blocks are stored source-major: E[i * nrows + row]
   const long long* eo = J.e_off + (long long)task.pair * J.L + task.l0;
@@ -826,17 +869,21 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
     const double T = turns * dist_f64(fma(dx, dx, dy * dy));
     const double beta = kNear && t.near ? bt[r * N + i] : 0.0;
     const bool near = kNear && beta != 0.0;
-    double2* Ep = J.E + (long long)i * ld + task.row0 + r;
-    if (kForm == kFormF64) {
+    int4* Ep = reinterpret_cast<int4*>(J.E) + (long long)i * ld + task.row0 + r;
+    auto put = [&](int b, double2 v) {
+      const int s = s_exp[r][b];
+      const int2 x = fix_f64(v.x, s), y = fix_f64(v.y, s);
+      Ep[eo[b]] = make_int4(x.x, x.y, y.x, y.y);
+    };
+    if constexpr (kForm == kFormF64) {
       const PairF64 pt = pair_f64(T, camp4);
       const double lnT = pt.th * fr[0].a.x < (float)kBesselLarge ? log_f64(T) : 0.0;
       unsigned long long ph = pt.v * (unsigned long long)task.l0 - (1ull << 61),
                          u = pt.v62 * (unsigned long long)task.l0;
       for (int b = 0; b < nl; ++b, ph += pt.v, u += pt.v62) {
         const FreqDf& f = fr[b];
-        Ep[eo[b]] = pt.th * f.a.x < (float)kBesselLarge
-                        ? hankel_near_f64(u, lnT + f.lnz, beta, near, qw)
-                        : hankel_far_f64(pt, ph, ang, df{f.a.z, f.a.w}, f.rs, beta, near);
+        put(b, pt.th * f.a.x < (float)kBesselLarge ? hankel_near_f64(u, lnT + f.lnz, beta, near, qw)
+                                                   : hankel_far_f64(pt, ph, ang, df{f.a.z, f.a.w}, f.rs, beta, near));
       }
     } else {
       const PairTurns pt = pair_turns(T, cd);
@@ -857,14 +904,17 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
         const FreqDf& f = fr[b];
         float4 d;
         if (pt.T.hi * f.a.x < (float)kBesselLarge) {
-          if (kForm == kFormKeep)
-            d = split2_bits(hankel_near_f64(v62 * (unsigned long long)(task.l0 + b), lnT64 + f.lnz, beta, near, qw));
-          else
-            d = hankel_near_df(df_mul(pt.T, df{f.a.x, f.a.y}), df_add_fast(lnT, df{f.b.z, f.b.w}), bd, near, qd);
+          if (kForm == kFormKeep) {
+            put(b, hankel_near_f64(v62 * (unsigned long long)(task.l0 + b), lnT64 + f.lnz, beta, near, qw));
+            continue;
+          }
+          d = hankel_near_df(df_mul(pt.T, df{f.a.x, f.a.y}), df_add_fast(lnT, df{f.b.z, f.b.w}), bd, near, qd);
         } else {
           d = hankel_far_df(pt, ph, ang.d, df{f.a.z, f.a.w}, df{f.b.x, f.b.y}, bd, near);
         }
-        *reinterpret_cast<float4*>(Ep + eo[b]) = d;
+        const float c = __uint_as_float((unsigned)(27 - s_exp[r][b] + 127) << 23);
+        const int2 x = fix_df(d.x, d.y, c), y = fix_df(d.z, d.w, c);
+        Ep[eo[b]] = make_int4(x.x, x.y, y.x, y.y);
       }
     }
   }
@@ -950,7 +1000,7 @@ __global__ void __launch_bounds__(kAsmThreads) k_cross_otf(DevJob J) {
     const int rr = e / (Q * nl), q = (e / nl) % Q, b = e % nl;
     double2 sum = make_double2(0.0, 0.0);
     for (int gg = 0; gg < G; ++gg) sum = cadd(sum, sho[(q * B + b) * kAsmThreads + gg * kAsmRows + rr]);
-    const long long row = J.otf_res_off[(long long)task.pair * J.L + ot.l0 + b] + task.row0 + rr;
+    const long long row = J.row_off[(long long)task.pair * J.L + ot.l0 + b] + task.row0 + rr;
     J.apply_res[row * Q + q] = sum;
   }
 }
@@ -1090,97 +1140,13 @@ __global__ void __launch_bounds__(kOtfThreads, otf_blocks(Q)) k_cross_otf_df(Dev
     const int e = lane >> kShift, k = e / (2 * Q), q = (e / 2) % Q;
     if ((lane & ((1 << kShift) - 1)) == 0 && k < nb) {
       const df v = acc[0].value();
-      const long long row = J.otf_res_off[(long long)task.pair * J.L + ot.l0 + b0 + k] + task.row0 + r;
+      const long long row = J.row_off[(long long)task.pair * J.L + ot.l0 + b0 + k] + task.row0 + r;
       reinterpret_cast<double*>(J.apply_res)[(row * Q + q) * 2 + (e & 1)] = (double)v.hi + (double)v.lo;
     }
   }
 }
 
-// ---------------------------------------------------------------------------------------------
-// Cross apply: W_k(x, q, l) = sum_j sum_i E_{l,k,j}[i, r] phi_j[q, i]; observation sums accumulate.
-// One thread per target row, the rows of all source blocks of the group concatenated so that warps
-// stay full (on this GPU an FP64 instruction costs a full warp slot of the FP64 pipe whatever its
-// active lanes); the source-major blocks make every load coalesced, the densities are shared-memory
-// broadcasts, and the per-row sums are added per target in a fixed block order (deterministic).
-// The window count is a template parameter so that no FMA is issued for absent windows.
 constexpr int kApplyThreads = 256;
-constexpr int kApplyMaxBlk = 64;   // receiving groups have at most P <= 64 source blocks
-
-template <int Q>
-__global__ void __launch_bounds__(kApplyThreads) k_cross_apply(DevJob J) {
-  extern __shared__ double2 shc[];
-  const CrossGrp g = J.grps[blockIdx.x];
-  const int l = g.l;
-  const bool obs = g.k == J.P;
-  const int nout = obs ? J.n_obs : J.panels[J.tpanel[g.k]].N;
-  const int nb = g.blk_end - g.blk_begin;
-  __shared__ int s_row0[kApplyMaxBlk + 1], s_ph0[kApplyMaxBlk + 1];
-  if (threadIdx.x == 0) {
-    int r = 0, p = 0;
-    for (int b = 0; b < nb; ++b) {
-      s_row0[b] = r;
-      s_ph0[b] = p;
-      r += J.blks[g.blk_begin + b].nrows;
-      p += Q * J.blks[g.blk_begin + b].N;
-    }
-    s_row0[nb] = r;
-    s_ph0[nb] = p;
-  }
-  __syncthreads();
-  const int nrow = s_row0[nb];
-  double2* acc = shc;                              // [Q][nout]
-  double2* res = acc + (size_t)Q * J.acc_cap;      // [Q][nrow]
-  double2* ph = res + (size_t)Q * J.row_cap;       // concatenated [Q][N_b] densities
-  for (int e = threadIdx.x; e < Q * nout; e += kApplyThreads) acc[e] = make_double2(0.0, 0.0);
-  for (int b = 0; b < nb; ++b) {
-    const CrossBlk B = J.blks[g.blk_begin + b];
-    const double2* p = J.phi + J.sys[B.sys].vec_off;
-    for (int e = threadIdx.x; e < Q * B.N; e += kApplyThreads) ph[s_ph0[b] + e] = p[e];
-  }
-  __syncthreads();
-  int b = 0;
-  for (int row = threadIdx.x; row < nrow; row += kApplyThreads) {
-    while (row >= s_row0[b + 1]) ++b;
-    const CrossBlk B = J.blks[g.blk_begin + b];
-    const int N = B.N, nr = B.nrows, r = row - s_row0[b];
-    const double2* phb = ph + s_ph0[b];
-    double2 s[Q];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) s[q] = make_double2(0.0, 0.0);
-    const double2* __restrict__ Er = J.E + B.e_off + r;
-#pragma unroll 4
-    for (int i = 0; i < N; ++i) {
-      const double2 ev = __ldg(&Er[(long long)i * nr]);
-#pragma unroll
-      for (int q = 0; q < Q; ++q) s[q] = cfma(ev, phb[q * N + i], s[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < Q; ++q) res[q * nrow + row] = s[q];
-  }
-  __syncthreads();
-  for (int bb = 0; bb < nb; ++bb) {
-    const CrossBlk B = J.blks[g.blk_begin + bb];
-    for (int r = threadIdx.x; r < B.nrows; r += kApplyThreads) {
-      const int out = J.tgts[B.tgt_off + r].out;
-#pragma unroll
-      for (int q = 0; q < Q; ++q) acc[q * nout + out] = cadd(acc[q * nout + out], res[q * nrow + s_row0[bb] + r]);
-    }
-    __syncthreads();
-  }
-  if (obs) {
-    for (int e = threadIdx.x; e < Q * nout; e += kApplyThreads) {
-      int q = e / nout, z = e % nout;
-      double2* v = J.Vobs + ((long long)z * Q + q) * J.L + l;
-      *v = cadd(*v, acc[e]);
-    }
-  } else {
-    const long long base = J.tr_off[g.k];
-    for (int e = threadIdx.x; e < Q * nout; e += kApplyThreads) {
-      int q = e / nout, x = e % nout;
-      J.W[((base + x) * Q + q) * J.L + l] = acc[e];
-    }
-  }
-}
 
 // ---------------------------------------------------------------------------------------------
 // Mixed-precision solve: an FP32 blocked solve with the FP32 factors, then refinement steps, each a
@@ -1611,26 +1577,32 @@ __global__ void __launch_bounds__(32 * kSolveWarps, 3) k_msolve(DevJob J, int m,
   for (int e = lane; e < Q * N; e += 32) {
     double2 v = f64 ? out[e] : df_join2(ph[e]);
     v = make_double2(v.x * scale, v.y * scale);
-    pdf[e] = df_split2(v);
+    if (J.otf) pdf[e] = df_split2(v);
     out[e] = v;
     sum[e] = m == 1 ? v : cadd(sum[e], v);
     if (all) all[e] = v;
   }
+  if (!J.otf) {
+    __syncwarp();
+#pragma unroll 1
+    for (int q = 0; q < QT; ++q)
+      fix_vector(out + q * N, N, 1.0, reinterpret_cast<int4*>(pdf) + (long long)q * N, J.phi_unit + 4ll * sidx + q, lane);
+  }
 }
 
-// Entries of a row per batch of the mixed-form cross apply (even: two alternating accumulator sets).
-__host__ __device__ constexpr int apply_batch(int Q) { return Q == 1 ? 8 : Q == 2 ? 6 : 4; }
+// Cross apply: W_k(x, q, l) = sum_j sum_i E_{l,k,j}[i, r] phi_j[q, i]; observation sums accumulate.  First half: one CTA
+// per slice of kApplySlice rows of a group (the rows of all its source blocks, concatenated), one thread per row, the
+// source-major blocks read coalesced.  Entries and densities are fixed-point (fixed.cuh), the sums exact integers,
+// so one kernel serves every form.  The row's entries stream through a per-thread ring of kApplyStages batches in shared
+// memory (cp.async): batch b + 1 is in flight while batch b is summed, and holds no registers; a thread reads only the
+// slots it filled itself (no barrier).  Bound by HBM (16 bytes an entry): 8 obstacle arcs, 4.8e8 entries, 12 steps: 42.7 (FP64 FMAs) ->
+// 17.2 ms, 0.84 of a copy's rate; the mixed forms' double-float sums took 16.8 (N = 512, two windows: 70 either way).
+// Entries of a row per batch:
+__host__ __device__ constexpr int apply_batch(int Q) { return Q <= 2 ? 8 : 4; }
 constexpr int kApplyStages = 2;   // batches per thread in shared memory: one summed while the next lands
-
-// Cross apply in double-float on the FP32 pipe (mixed form): E and phi as df64, compensated sums.
-// Mixed form, first half: one CTA per slice of kApplySlice rows of a group, one thread per row, the
-// row's double-float sum over its block's sources (E and phi as df64, two compensated sums).  The row's
-// entries stream through a per-thread ring of kApplyStages batches in shared memory (cp.async): batch
-// b + 1 is in flight while batch b is summed, so the loads never wait for the FP32 pipe and hold no
-// registers.  A thread reads only the slots it filled itself (no barrier).
 template <int Q>
-__global__ void __launch_bounds__(kApplySlice, 3) k_cross_rows_df(DevJob J) {
-  extern __shared__ __align__(16) float4 she[];     // [kApplyStages][kB][kApplySlice]
+__global__ void __launch_bounds__(kApplySlice, Q == 1 ? 3 : 2) k_cross_rows(DevJob J) {
+  extern __shared__ __align__(16) int4 she[];     // [kApplyStages][kB][kApplySlice]
   const ApplySlice sl = J.slices[blockIdx.x];
   if ((int)threadIdx.x >= sl.nrows) return;
   const int row = sl.row0 + threadIdx.x;
@@ -1642,16 +1614,27 @@ __global__ void __launch_bounds__(kApplySlice, 3) k_cross_rows_df(DevJob J) {
   }
   const CrossBlk B = J.blks[b];
   const int N = B.N, nr = B.nrows;
-  // the block's double-float densities, the same for every row: one cached load per warp and column
-  const float4* __restrict__ phb = J.phi_df + J.sys[B.sys].vec_off;
-  dfacc sr[Q], si[Q], tr[Q], ti[Q];
-  const float4* __restrict__ Er = reinterpret_cast<const float4*>(J.E + B.e_off) + r;
+  // the block's densities, the same for every row: one cached load per warp and column
+  const int4* __restrict__ phb = reinterpret_cast<const int4*>(J.phi_df) + J.sys[B.sys].vec_off;
+  const int4* __restrict__ Er = reinterpret_cast<const int4*>(J.E + B.e_off) + r;
+  fixacc re[Q], im[Q];
+  auto mac = [&](const int4 e, int i) {
+    const int n0 = -e.z, n1 = -e.w;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int4 p = __ldg(&phb[q * N + i]);
+      re[q].mac(e.x, e.y, p.x, p.y);
+      re[q].mac(n0, n1, p.z, p.w);
+      im[q].mac(e.x, e.y, p.z, p.w);
+      im[q].mac(e.z, e.w, p.x, p.y);
+    }
+  };
   constexpr int kB = apply_batch(Q);
   const int nbat = N / kB;
-  float4* mine = she + threadIdx.x;
+  int4* mine = she + threadIdx.x;
   auto issue = [&](int bi) {
-    float4* dst = mine + (bi % kApplyStages) * kB * kApplySlice;
-    const float4* src = Er + (long long)bi * kB * nr;
+    int4* dst = mine + (bi % kApplyStages) * kB * kApplySlice;
+    const int4* src = Er + (long long)bi * kB * nr;
 #pragma unroll
     for (int k = 0; k < kB; ++k) cp_async16(dst + k * kApplySlice, src + (long long)k * nr);
   };
@@ -1665,44 +1648,29 @@ __global__ void __launch_bounds__(kApplySlice, 3) k_cross_rows_df(DevJob J) {
     if (bi + kApplyStages - 1 < nbat) issue(bi + kApplyStages - 1);
     cp_async_commit();                          // (empty near the end: keeps the group count uniform)
     cp_async_wait<kApplyStages - 1>();          // batch bi has landed
-    const float4* src = mine + (bi % kApplyStages) * kB * kApplySlice;
-    const int i = bi * kB;
+    const int4* src = mine + (bi % kApplyStages) * kB * kApplySlice;
 #pragma unroll
-    for (int k = 0; k < kB; k += 2) {
-      const float4 e0 = src[k * kApplySlice], e1 = src[(k + 1) * kApplySlice];
+    for (int k = 0; k < kB; ++k) mac(src[k * kApplySlice], bi * kB + k);
+    // a source adds two products to either half of a sum: kFixRun products between carries
+    if ((bi + 1) % (kFixRun / 2 / kB) == 0) {
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
-        cdf_mac(sr[q], si[q], e0, __ldg(&phb[q * N + i + k]));
-        cdf_mac(tr[q], ti[q], e1, __ldg(&phb[q * N + i + k + 1]));
+        re[q].carry();
+        im[q].carry();
       }
     }
   }
-  int i = nbat * kB;
-  for (; i + 1 < N; i += 2) {
-    const float4 e0 = __ldg(&Er[(long long)i * nr]);
-    const float4 e1 = __ldg(&Er[(long long)(i + 1) * nr]);
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      cdf_mac(sr[q], si[q], e0, __ldg(&phb[q * N + i]));
-      cdf_mac(tr[q], ti[q], e1, __ldg(&phb[q * N + i + 1]));
-    }
-  }
-  if (i < N) {
-    const float4 e0 = __ldg(&Er[(long long)i * nr]);
-#pragma unroll
-    for (int q = 0; q < Q; ++q) cdf_mac(sr[q], si[q], e0, __ldg(&phb[q * N + i]));
-  }
-  double2* out = J.apply_res + (J.grp_res_off[sl.grp] + row) * Q;
+  for (int i = nbat * kB; i < N; ++i) mac(__ldg(&Er[(long long)i * nr]), i);
+  const long long rr = J.grp_res_off[sl.grp] + row;
+  const double unit = (double)J.e_unit[rr] * 0x1p56;
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
-    sr[q].add(tr[q].hi, tr[q].lo);
-    si[q].add(ti[q].hi, ti[q].lo);
-    const df a = sr[q].value(), c = si[q].value();
-    out[q] = make_double2((double)a.hi + (double)a.lo, (double)c.hi + (double)c.lo);
+    const double u = unit * J.phi_unit[4ll * B.sys + q];
+    J.apply_res[rr * Q + q] = make_double2(re[q].value() * u, im[q].value() * u);
   }
 }
 
-// Mixed form, second half: per group, the row sums of every source block added to their targets in
+// Second half: per group, the row sums of every source block added to their targets in
 // the fixed block order (deterministic), then W (transfer nodes) or the observation spectra.
 template <int Q>
 __global__ void __launch_bounds__(kApplyThreads) k_cross_reduce(DevJob J) {
@@ -2541,34 +2509,27 @@ cudaError_t launch_resid(const DevJob& J, int pass, cudaStream_t st, int* launch
 }
 
 template <int Q>
-static cudaError_t launch_cross_apply_q(const DevJob& J, size_t sh, cudaStream_t st) {
-  if (J.mixed) {
-    // the row kernel's ring of entry batches (the densities come through the L1 cache)
-    const size_t sh_rows = (size_t)kApplyStages * apply_batch(Q) * kApplySlice * sizeof(float4);
-    const size_t sh_red = (size_t)Q * J.acc_cap * sizeof(double2);
-    cudaError_t e = cudaFuncSetAttribute(k_cross_rows_df<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_rows);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_cross_reduce<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_red);
-    if (e != cudaSuccess) return e;
-    if (J.n_slices > 0) k_cross_rows_df<Q><<<J.n_slices, kApplySlice, sh_rows, st>>>(J);
-    k_cross_reduce<Q><<<J.n_grp, kApplyThreads, sh_red, st>>>(J);
-    return cudaGetLastError();
-  }
-  cudaError_t e = cudaFuncSetAttribute(k_cross_apply<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+static cudaError_t launch_cross_apply_q(const DevJob& J, cudaStream_t st) {
+  // the row kernel's ring of entry batches (the densities come through the L1 cache)
+  const size_t sh_rows = (size_t)kApplyStages * apply_batch(Q) * kApplySlice * sizeof(int4);
+  const size_t sh_red = (size_t)Q * J.acc_cap * sizeof(double2);
+  cudaError_t e = cudaFuncSetAttribute(k_cross_rows<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_rows);
   if (e != cudaSuccess) return e;
-  k_cross_apply<Q><<<J.n_grp, kApplyThreads, sh, st>>>(J);
+  e = cudaFuncSetAttribute(k_cross_reduce<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_red);
+  if (e != cudaSuccess) return e;
+  if (J.n_slices > 0) k_cross_rows<Q><<<J.n_slices, kApplySlice, sh_rows, st>>>(J);
+  k_cross_reduce<Q><<<J.n_grp, kApplyThreads, sh_red, st>>>(J);
   return cudaGetLastError();
 }
 
 cudaError_t launch_cross_apply(const DevJob& J, cudaStream_t st, int* launches) {
   if (J.n_grp == 0) return cudaSuccess;
-  size_t sh = (size_t)J.Q * (J.acc_cap + J.row_cap + J.ph_cap) * sizeof(double2);
-  *launches += J.mixed ? 2 : 1;
+  *launches += 2;
   switch (J.Q) {
-    case 1: return launch_cross_apply_q<1>(J, sh, st);
-    case 2: return launch_cross_apply_q<2>(J, sh, st);
-    case 3: return launch_cross_apply_q<3>(J, sh, st);
-    default: return launch_cross_apply_q<4>(J, sh, st);
+    case 1: return launch_cross_apply_q<1>(J, st);
+    case 2: return launch_cross_apply_q<2>(J, st);
+    case 3: return launch_cross_apply_q<3>(J, st);
+    default: return launch_cross_apply_q<4>(J, st);
   }
 }
 

@@ -58,9 +58,9 @@ struct DevJob {
   const CrossAsm* asms;
   const CrossGrp* grps;
   const CrossBlk* blks;
-  const ApplySlice* slices;  // mixed-form apply: row slices of the groups
+  const ApplySlice* slices;  // stored cross rows: row slices of the groups
   const long long* grp_res_off;
-  double2* apply_res;        // [group rows][Q] per-row cross sums (mixed form)
+  double2* apply_res;        // [group rows][Q] per-row cross sums
   int n_slices, slice_ph_cap;
   // cross_mode 1: cross rows evaluated every step (nothing stored)
   int otf, n_otf;
@@ -72,7 +72,9 @@ struct DevJob {
   const long long* wn_off;   // per assembly task: offset of its near corrections or -1
   double* wn;                // near corrections beta, nrows x N per assembly task with near rows
   FreqDf* freq_df;           // [L] constants of the double-float Hankel entries (mixed forms)
-  const long long* otf_res_off;
+  const long long* row_off;  // [pair][L] first row of (pair, l) in the per-row results
+  float* e_unit;             // stored cross rows: unit of a row's fixed-point entries, laid out like the row results
+  double* phi_unit;          // [system][4] unit of a window's fixed-point densities (stored cross rows)
   const int* tpanel;
   const long long* tr_off;
   const double* chi;
@@ -109,13 +111,14 @@ struct DevJob {
   double2* dinv;             // 1 / U_kk
   double2* G;                // data on solve nodes [s][q][i]
   double2* phi;              // current densities
-  float4* phi_df;            // the same as double-float pairs, written by the mixed solve for the apply
+  float4* phi_df;            // the densities for the cross rows: fixed-point int4 (stored rows, every form) or
+                             // double-float pairs (mixed forms, rows evaluated every step)
   double2* phi_sum;
   double2* phi_all;          // [m][...] or null
   double2* W;                // cross fields at transfer nodes [(tr_off+x)*Q+q]*L+l
   double2* Gt;               // transfer-node spectra (same layout)
   double* ginc;              // m = 1 time samples sign chi_k u^i at the active transfer nodes [a][NT]
-  double2* E;                // cross matrices
+  double2* E;                // stored cross rows, fixed-point int4 (16 bytes an entry)
   double2* Vobs;             // [z][q][l]
   double* traces;            // [z][tout]
   double2* fft_tw;           // K/2 twiddles e^{-2 pi i r/K}

@@ -622,17 +622,17 @@ int build_plan(const fthms_curve* curves, int ncurves, const fthms_arc* arcs, in
       l = l1 + 1;
     }
   }
-  if (p.opt.cross_mode == 1) {
-    // Rows of pair (k, j) inside the per-row results of group (k, l), in the groups' block order.
-    p.otf_res_off.assign((size_t)npairs * p.L, -1);
-    for (size_t gi = 0; gi < p.grps.size(); ++gi) {
-      const CrossGrp& g = p.grps[gi];
-      long long r = p.grp_res_off[gi];
-      for (int pi : pairs_of[g.k]) {
-        p.otf_res_off[(size_t)pi * p.L + g.l] = r;
-        r += p.pairs[pi].nrows;
-      }
+  // Rows of pair (k, j) inside the per-row results of group (k, l), in the groups' block order.
+  p.row_off.assign((size_t)npairs * p.L, -1);
+  for (size_t gi = 0; gi < p.grps.size(); ++gi) {
+    const CrossGrp& g = p.grps[gi];
+    long long r = p.grp_res_off[gi];
+    for (int pi : pairs_of[g.k]) {
+      p.row_off[(size_t)pi * p.L + g.l] = r;
+      r += p.pairs[pi].nrows;
     }
+  }
+  if (p.opt.cross_mode == 1) {
     // Near weights once per job (they depend on the target and N only); tasks of at most
     // otf_band(Q) frequencies each.
     // (a mixed job that may fall back to FP64 keeps to the FP64 kernel's shorter bands)
@@ -720,9 +720,14 @@ size_t plan_device_bytes(const Plan& p) {
   b += (size_t)p.n_obs * p.Q * p.L * 16 + (size_t)p.n_obs * p.n_tout * 8;
   b += p.node_t.size() * 32 + p.tgts.size() * sizeof(CrossTgt) + p.blks.size() * sizeof(CrossBlk) +
        p.asms.size() * sizeof(CrossAsm) + p.self_tiles.size() * sizeof(SelfTile) + p.sys.size() * (sizeof(SysDesc) + sizeof(int)) + p.slices.size() * sizeof(ApplySlice) + p.grp_res_off.size() * 8;
-  if (p.opt.precision >= 1 || p.opt.cross_mode == 1) b += (size_t)p.res_total * p.Q * 16;   // per-row cross sums
+  b += (size_t)p.res_total * p.Q * 16 + p.row_off.size() * 8;   // per-row cross sums
+  if (p.opt.cross_mode == 0) {                                  // fixed-point units and densities
+    b += (size_t)p.res_total * 4 + p.sys.size() * 32;
+    if (p.opt.precision == 0) b += (size_t)p.vec_total * 16;
+  }
+  b += (size_t)p.L * 48;
   if (p.opt.cross_mode == 1)
-    b += (size_t)p.wn_total * 8 + p.otf.size() * sizeof(CrossOtf) + p.otf_res_off.size() * 8 + p.wn_off.size() * 8;
+    b += (size_t)p.wn_total * 8 + p.otf.size() * sizeof(CrossOtf) + p.wn_off.size() * 8;
   b += p.win.size() * 8 + (size_t)p.Q * p.L * 32 + (size_t)p.K * (p.opt.precision >= 1 ? 16 : 8) + p.chi.size() * 8;
   return b;
 }

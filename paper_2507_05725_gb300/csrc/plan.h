@@ -76,7 +76,7 @@ struct Plan {
   std::vector<CrossOtf> otf;            // cross_mode 1: on-the-fly tasks
   std::vector<long long> wn_off;         // per assembly task: offset of its near weights (nrows x N), or -1
   long long wn_total = 0;
-  std::vector<long long> otf_res_off;    // [pairs][L]: first row of pair (k, j) in group (k, l)'s result rows
+  std::vector<long long> row_off;    // [pairs][L]: first row of pair (k, j) in group (k, l)'s result rows
   std::vector<CrossAsm> asms;
   std::vector<SelfTile> self_tiles;
 

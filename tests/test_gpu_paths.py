@@ -43,6 +43,20 @@ def _rel(job, ref, problem):
     return math.sqrt(num / den)
 
 
+def _self_reference(curve, arc, N, kappa):
+    """The oracle's self matrix with the log weights' phases k m pi/N reduced in integers (its own carry
+    cos(k arccos t_i) with a rounding error that grows with k, 1e-12 of the largest entry at N = 1024)."""
+    t, n = geo.cheb_nodes(N), np.arange(1, N)
+    arc_ = geo.Arc(0, 0, curve, *arc)
+    cosr = np.cos(np.arange(2 * N) * (np.pi / N))
+    Fm = np.array([np.sum(cosr[(n * m) % (2 * N)] / n) for m in range(2 * N)])
+    i = np.arange(N)
+    rlog = -(np.pi / N) * (math.log(2.0) + Fm[np.abs(i[:, None] - i)] + Fm[i[:, None] + i + 1])
+    X = arc_.point(t)[0]
+    R = np.linalg.norm(X[:, None] - X[None], axis=-1)
+    return oker.self_matrix(arc_, N, kappa) - special.j0(kappa * R) / (2.0 * np.pi) * (rlog - oker.rlog_self(N))
+
+
 @pytest.mark.parametrize("N", [2, 3, 31, 32, 33, 64, 65, 1023, 1024])
 def test_log_weights_at_block_edges(F, N):
     """The cosine sums F(0..N) come in blocks of 32 values; the matrix takes F(|i-l|) and F(i+l+1), folded at N.
@@ -52,17 +66,7 @@ def test_log_weights_at_block_edges(F, N):
     F.fthms_assemble_self(curve, arc, N, kappa, A.data_ptr())
     got = A.cpu().numpy().reshape(N, N, 2)
     got = (got[..., 0] + 1j * got[..., 1]).T
-    # The oracle's own weights carry cos(k arccos t_i) with a rounding error that grows with k (1e-12 of the
-    # largest entry at N = 1024), so they are replaced by the same sums with the phase k m pi/N reduced in integers.
-    t, n = geo.cheb_nodes(N), np.arange(1, N)
-    arc_ = geo.Arc(0, 0, curve, *arc)
-    cosr = np.cos(np.arange(2 * N) * (np.pi / N))
-    Fm = np.array([np.sum(cosr[(n * m) % (2 * N)] / n) for m in range(2 * N)])
-    i = np.arange(N)
-    rlog = -(np.pi / N) * (math.log(2.0) + Fm[np.abs(i[:, None] - i)] + Fm[i[:, None] + i + 1])
-    X = arc_.point(t)[0]
-    R = np.linalg.norm(X[:, None] - X[None], axis=-1)
-    ref = oker.self_matrix(arc_, N, kappa) - special.j0(kappa * R) / (2.0 * np.pi) * (rlog - oker.rlog_self(N))
+    ref = _self_reference(curve, arc, N, kappa)
     assert np.max(np.abs(got - ref)) <= 1e-13 * np.max(np.abs(ref))
 
 
@@ -147,5 +151,44 @@ def test_self_matrix_over_the_hankel_ranges(F, N, kappa):
     F.fthms_assemble_self(curve, arc, N, kappa, A.data_ptr())
     got = A.cpu().numpy().reshape(N, N, 2)
     got = (got[..., 0] + 1j * got[..., 1]).T
-    ref = oker.self_matrix(geo.Arc(0, 0, curve, *arc), N, kappa)
+    ref = _self_reference(curve, arc, N, kappa)
     assert np.max(np.abs(got - ref)) <= 1e-13 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("Q,N", [(1, 31), (1, 129), (2, 32), (2, 67), (3, 64), (4, 65)])
+def test_stored_rows_in_fixed_point(F, ctx, precision, Q, N):
+    """Stored cross rows (56-bit integers, carries every 32 sources, batches of 4 or 8) against rows evaluated every
+    step in FP64: node counts around the batches and carries, an observation point next to the boundary (entries
+    far above the others) and one far away.  1e-11 / 1e-10: the FP64 and mixed bars."""
+    p = wl.random_small(11, n_curves=2, n_arcs_per_curve=3, L=40, M=2, Q=Q, N_fixed=N, W=12.0, H=4.0, n_period=512)
+    p["options"]["obs"] = np.array([[0.0, 1.9], [40.0, -7.0], [9.0, 0.3]])
+    p["options"]["refine_max"] = 8
+    q_ = copy.deepcopy(p)
+    q_["options"]["cross_mode"] = 1
+    ref = F.Job(ctx, q_).run().wait()
+    job = F.Job(ctx, p, precision=precision).run().wait()
+    tol = 1e-11 if precision == 0 else 1e-10
+    num = den = 0.0
+    for j in range(6):
+        for q in range(Q):
+            a, b = F.fthms_densities(ref.req, j, 2, q), F.fthms_densities(job.req, j, 2, q)
+            num += float(np.sum((a - b) ** 2))
+            den += float(np.sum(a ** 2))
+    assert math.sqrt(num / den) < tol
+    t = ref.traces()
+    assert np.all(np.abs(job.traces() - t) <= 10 * tol * np.max(np.abs(t), axis=1, keepdims=True))
+
+
+def test_stored_rows_at_the_largest_node_count(F, ctx):
+    """N = 1427 is the most that stored rows accept: the near tasks' shared memory is full there."""
+    p = wl.random_small(2, n_arcs_per_curve=3, L=4, M=2, N_fixed=1427, W=24.0, H=0.3, n_period=64, kind=1)
+    p["options"]["refine_max"] = 8
+    jobs = []
+    for mode in (0, 1):
+        p["options"]["cross_mode"] = mode
+        jobs.append(F.Job(ctx, p, precision=2).run())
+        F.LIB.fthms_wait(jobs[-1].req, -1)
+    for j in range(3):
+        a, b = (F.fthms_densities(x.req, j, 2, 0) for x in jobs)
+        assert np.linalg.norm(a - b) <= 1e-10 * np.linalg.norm(b)
