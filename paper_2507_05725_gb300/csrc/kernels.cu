@@ -1714,40 +1714,68 @@ __global__ void __launch_bounds__(kApplyThreads) k_cross_reduce(DevJob J) {
 constexpr int kTimeThreads = 256;
 constexpr int kTimeMaxThreads = 512;   // largest time-transform block a tuned launch may use
 
-// In-place radix-2 decimation-in-time FFT, y_r = sum_b X_b e^{-2 pi i b r/K}; input in
-// bit-reversed order.
-__device__ void block_fft(double2* buf, int K, int logK, const double2* __restrict__ tw) {
-  for (int s = 1; s <= logK; ++s) {
-    const int half = 1 << (s - 1);
-    const int tws = K >> s;   // twiddle stride
-    for (int j = threadIdx.x; j < K / 2; j += blockDim.x) {
-      const int pos = j & (half - 1);
-      const int i0 = ((j >> (s - 1)) << s) + pos;
-      const int i1 = i0 + half;
-      const double2 wv = tw[pos * tws];
-      const double2 a = buf[i0];
-      const double2 bb = cmul(buf[i1], wv);
-      buf[i0] = cadd(a, bb);
-      buf[i1] = csub(a, bb);
+// The transforms' complex arithmetic: FP64, or double-float on the FP32 pipe (mixed form; complex values as float4:
+// re.hi, re.lo, im.hi, im.lo).
+struct FftF64 {
+  using T = double2;
+  static __device__ __forceinline__ const T* tw(const DevJob& J) { return J.fft_tw; }
+  static __device__ __forceinline__ T mul(T a, T b) { return cmul(a, b); }
+  static __device__ __forceinline__ T add(T a, T b) { return cadd(a, b); }
+  static __device__ __forceinline__ T sub(T a, T b) { return csub(a, b); }
+  static __device__ __forceinline__ T neg(T a) { return make_double2(-a.x, -a.y); }
+  static __device__ __forceinline__ T conj(T a) { return make_double2(a.x, -a.y); }
+  static __device__ __forceinline__ T times_i(T a) { return make_double2(-a.y, a.x); }
+  static __device__ __forceinline__ T from(double2 a) { return a; }
+  static __device__ __forceinline__ double2 to(T a) { return a; }
+};
+struct FftDf {
+  using T = float4;
+  static __device__ __forceinline__ const T* tw(const DevJob& J) { return J.fft_tw_df; }
+  static __device__ __forceinline__ T mul(T a, T b) { return dfc_mul(a, b); }
+  static __device__ __forceinline__ T add(T a, T b) { return dfc_add(a, b); }
+  static __device__ __forceinline__ T sub(T a, T b) { return dfc_sub(a, b); }
+  static __device__ __forceinline__ T neg(T a) { return make_float4(-a.x, -a.y, -a.z, -a.w); }
+  static __device__ __forceinline__ T conj(T a) { return make_float4(a.x, a.y, -a.z, -a.w); }
+  static __device__ __forceinline__ T times_i(T a) { return make_float4(-a.z, -a.w, a.x, a.y); }
+  static __device__ __forceinline__ T from(double2 a) { return df_split2(a); }
+  static __device__ __forceinline__ double2 to(T a) { return df_join2(a); }
+};
+
+// In-place decimation-in-time FFT of n = 2^logn points, y_r = sum_b X_b e^{-2 pi i b r/n}, input in bit-reversed order,
+// two radix-2 stages at a time (three complex products per four points; a single stage first when logn is odd).
+// tw: e^{-2 pi i r/K}, r < K/2, K a multiple of n.
+template <class O>
+__device__ void block_fft(typename O::T* buf, int logn, const typename O::T* __restrict__ tw, int K) {
+  using T = typename O::T;
+  const int n = 1 << logn;
+  int half = 1;
+  if (logn & 1) {
+    for (int j = threadIdx.x; j < n / 2; j += blockDim.x) {
+      const T a = buf[2 * j], c = buf[2 * j + 1];
+      buf[2 * j] = O::add(a, c);
+      buf[2 * j + 1] = O::sub(a, c);
     }
     __syncthreads();
+    half = 2;
   }
-}
-
-// The same FFT in double-float on the FP32 pipe (mixed form): complex values as float4 (re.hi,
-// re.lo, im.hi, im.lo), twiddles from a double-float table.
-__device__ void block_fft_df(float4* buf, int K, int logK, const float4* __restrict__ tw) {
-  for (int s = 1; s <= logK; ++s) {
-    const int half = 1 << (s - 1);
-    const int tws = K >> s;
-    for (int j = threadIdx.x; j < K / 2; j += blockDim.x) {
-      const int pos = j & (half - 1);
-      const int i0 = ((j >> (s - 1)) << s) + pos;
-      const int i1 = i0 + half;
-      const float4 a = buf[i0];
-      const float4 bb = dfc_mul(buf[i1], tw[pos * tws]);
-      buf[i0] = dfc_add(a, bb);
-      buf[i1] = dfc_sub(a, bb);
+  for (; half < n; half *= 4) {
+    const int ts = K / (4 * half);          // twiddle stride of the second stage
+    for (int j = threadIdx.x; j < n / 4; j += blockDim.x) {
+      const int pos = j & (half - 1), i0 = ((j & ~(half - 1)) << 2) + pos;
+      T* p = buf + i0;
+      const T x0 = p[0];
+      T t1 = p[half], t2 = p[2 * half], t3 = p[3 * half];
+      if (half > 1) {
+        const int k = pos * ts, k3 = 3 * k;
+        t1 = O::mul(t1, tw[2 * k]);
+        t2 = O::mul(t2, tw[k]);
+        t3 = O::mul(t3, k3 < K / 2 ? tw[k3] : O::neg(tw[k3 - K / 2]));
+      }
+      const T y0 = O::add(x0, t1), y1 = O::sub(x0, t1), u = O::add(t2, t3), v = O::times_i(O::sub(t2, t3));
+      p[0] = O::add(y0, u);
+      p[half] = O::sub(y1, v);
+      p[2 * half] = O::sub(y0, u);
+      p[3 * half] = O::add(y1, v);
     }
     __syncthreads();
   }
@@ -1755,47 +1783,94 @@ __device__ void block_fft_df(float4* buf, int K, int logK, const float4* __restr
 
 __device__ __forceinline__ int bitrev(int b, int logK) { return (int)(__brev((unsigned)b) >> (32 - logK)); }
 
-// Transform of the bit-reversed spectrum in buf (FP64, or double-float for DF) and read-back of bin
-// r as FP64.
-template <bool DF>
-__device__ __forceinline__ void fft_in_place(const DevJob& J, double2* buf) {
-  if (DF) block_fft_df(reinterpret_cast<float4*>(buf), J.K, J.logK, J.fft_tw_df);
-  else block_fft(buf, J.K, J.logK, J.fft_tw);
-}
-template <bool DF>
-__device__ __forceinline__ void fft_put(double2* buf, int i, double2 v) {
-  if (DF) reinterpret_cast<float4*>(buf)[i] = df_split2(v);
-  else buf[i] = v;
-}
-template <bool DF>
-__device__ __forceinline__ double2 fft_get(const double2* buf, int i) {
-  if (DF) return df_join2(reinterpret_cast<const float4*>(buf)[i]);
-  return buf[i];
-}
+// Both transforms work on real samples of one period K, so each window takes one complex FFT of K/2 points: even
+// samples in the real part and odd ones in the imaginary part.  FP64 form: bound by the FP64 pipe, about half of the
+// full-length radix-2 transforms' work (4096 samples, two windows, 2 700 nodes: 31.3 -> 14.3 ms a job of 7 steps).
 
-// Windowed slow transforms of g[0..NT) into out[q*L + l] (eq. Fourierk with the exact phase split).
-template <bool DF>
-__device__ void forward_all(const DevJob& J, const double* g, double2* buf, double2* out) {
-  const int K = J.K, NT = J.NT, L = J.L;
+// Windowed slow transforms of g[0..NT) into out[q*L + l] (eq. Fourierk with the exact phase split): with C the FFT of
+// x[2n] + i x[2n+1], bin k of the real sequence is (C_k + C*_{-k})/2 - (i/2) e^{-2 pi i k/K} (C_k - C*_{-k}).
+template <class O>
+__device__ void forward_all(const DevJob& J, const double* g, double2* sbuf, double2* out) {
+  using T = typename O::T;
+  T* buf = reinterpret_cast<T*>(sbuf);
+  const int K = J.K, K2 = K / 2, NT = J.NT, L = J.L;
+  const T* __restrict__ tw = O::tw(J);
   for (int q = 0; q < J.Q; ++q) {
     const double* wq = J.win + (long long)q * NT;
-    for (int b = threadIdx.x; b < K; b += blockDim.x) {
-      double acc = 0.0;
-      for (int n = b; n < NT; n += K) acc = fma(g[n], wq[n], acc);
-      fft_put<DF>(buf, bitrev(b, J.logK), make_double2(acc, 0.0));
+    for (int b = threadIdx.x; b < K2; b += blockDim.x) {
+      double2 acc = make_double2(0.0, 0.0);
+      for (int n = 2 * b; n < NT; n += K) {
+        acc.x = fma(g[n], wq[n], acc.x);
+        if (n + 1 < NT) acc.y = fma(g[n + 1], wq[n + 1], acc.y);
+      }
+      buf[bitrev(b, J.logK - 1)] = O::from(acc);
     }
     __syncthreads();
-    fft_in_place<DF>(J, buf);
+    block_fft<O>(buf, J.logK - 1, tw, K);
     for (int l = threadIdx.x; l < L; l += blockDim.x) {
       double2 v = make_double2(0.0, 0.0);
       if (l > 0) {
-        double2 y = fft_get<DF>(buf, l & (K - 1));
-        v = cmul(J.fwd_tw[q * L + l], make_double2(y.x, -y.y));
+        const int k = l & (K - 1), kk = k & (K2 - 1);
+        const T c = buf[kk], d = O::conj(buf[(K2 - kk) & (K2 - 1)]);
+        const T t = k < K2 ? tw[kk] : O::neg(tw[kk]);
+        const T y = O::sub(O::add(c, d), O::times_i(O::mul(t, O::sub(c, d))));   // twice the bin
+        const double2 yy = O::to(y);
+        v = cmul(J.fwd_tw[q * L + l], make_double2(0.5 * yy.x, -0.5 * yy.y));
       }
       out[q * L + l] = v;
     }
     __syncthreads();
   }
+}
+
+// g[nlo_q + r] += Re sum_l syn_tw[l] W_l e^{-2 pi i l r/K} for one window: with S the spectrum folded to one period,
+// the real part's spectrum is H_b = (S_b + S*_{-b})/2, and the K/2-point FFT of (H_b + H_{b+K/2}) + i e^{-2 pi i b/K}
+// (H_b - H_{b+K/2}) gives the samples in pairs.
+template <class O>
+__device__ void synth_window(const DevJob& J, int q, const double2* __restrict__ Wq, double2* sbuf, double* g) {
+  using T = typename O::T;
+  T* buf = reinterpret_cast<T*>(sbuf);
+  const int K = J.K, K2 = K / 2, L = J.L, NT = J.NT;
+  const T* __restrict__ tw = O::tw(J);
+  const double2* __restrict__ st = J.syn_tw + (long long)q * L;
+  auto fold = [&](int b, double2& s) {        // S_b; l = 0 (the constant) is not solved
+    bool any = false;
+    for (int l = (b == 0 ? K : b); l < L; l += K) {
+      s = any ? cfma(st[l], Wq[l], s) : cmul(st[l], Wq[l]);
+      any = true;
+    }
+    return any;
+  };
+  for (int b = threadIdx.x; b < K2; b += blockDim.x) {
+    // twice H_b and H_{b+K/2}: S_b + S*_{K-b} and S_{b+K/2} + S*_{K/2-b}
+    double2 s0{}, s1{}, s2{}, s3{};
+    bool lo = fold(b, s0), hi = fold(b + K2, s1);
+    if (fold((K - b) & (K - 1), s2)) {
+      s0 = lo ? cadd(s0, make_double2(s2.x, -s2.y)) : make_double2(s2.x, -s2.y);
+      lo = true;
+    }
+    if (fold(K2 - b, s3)) {
+      s1 = hi ? cadd(s1, make_double2(s3.x, -s3.y)) : make_double2(s3.x, -s3.y);
+      hi = true;
+    }
+    T v = O::from(make_double2(0.0, 0.0));
+    if (lo || hi) {
+      const T a = O::from(s0), c = O::from(s1);
+      const T e = !hi ? a : !lo ? c : O::add(a, c), o = !hi ? a : !lo ? O::neg(c) : O::sub(a, c);
+      v = O::add(e, O::times_i(O::mul(tw[b], o)));
+    }
+    buf[bitrev(b, J.logK - 1)] = v;
+  }
+  __syncthreads();
+  block_fft<O>(buf, J.logK - 1, tw, K);
+  const int n0 = J.nlo[q];
+  for (int r = threadIdx.x; r < K2; r += blockDim.x) {
+    const double2 v = O::to(buf[r]);
+    const int n = n0 + 2 * r;
+    if (n < NT) g[n] = fma(0.5, v.x, g[n]);
+    if (n + 1 < NT) g[n + 1] = fma(0.5, v.y, g[n + 1]);
+  }
+  __syncthreads();
 }
 
 // Sampled signal: the degree-7 Lagrange interpolant through the samples i0 .. i0 + 7, i0 = floor(s) - 3,
@@ -2051,12 +2126,12 @@ __global__ void __launch_bounds__(kTimeMaxThreads) k_incident(DevJob J) {
   extern __shared__ double2 sht[];
   const int a = blockIdx.x;
   const int k = J.act_arc[a], x = J.act_idx[a];
-  double2* buf = sht;                               // K
-  double* g = reinterpret_cast<double*>(sht + J.K); // NT
+  double2* buf = sht;                                   // K/2
+  double* g = reinterpret_cast<double*>(sht + J.K / 2); // NT
   const double* src = J.ginc + (long long)a * J.NT;
   for (int n = threadIdx.x; n < J.NT; n += blockDim.x) g[n] = src[n];
   __syncthreads();
-  forward_all<DF>(J, g, buf, J.Gt + (J.tr_off[k] + x) * J.Q * J.L);
+  forward_all<std::conditional_t<DF, FftDf, FftF64>>(J, g, buf, J.Gt + (J.tr_off[k] + x) * J.Q * J.L);
 }
 
 // PART = 0: the whole step at one transfer node (synthesis, -chi_k, windowed forward transforms).  In a
@@ -2067,32 +2142,18 @@ __global__ void __launch_bounds__(kTimeMaxThreads) k_synth_fwd(DevJob J) {
   extern __shared__ double2 sht[];
   const int a = blockIdx.x;
   const int k = J.act_arc[a], x = J.act_idx[a];
-  const int K = J.K, L = J.L, NT = J.NT;
-  double2* buf = sht;
-  double* g = reinterpret_cast<double*>(sht + K);
+  using O = std::conditional_t<DF, FftDf, FftF64>;
+  const int L = J.L, NT = J.NT;
+  double2* buf = sht;                                   // K/2
+  double* g = reinterpret_cast<double*>(sht + J.K / 2); // NT
   const long long base = (J.tr_off[k] + x) * J.Q * L;
   double* gpart = J.ginc + (long long)a * NT;
   if (PART == 2) {
     for (int n = threadIdx.x; n < NT; n += blockDim.x) g[n] = gpart[n];
   } else {
     for (int n = threadIdx.x; n < NT; n += blockDim.x) g[n] = 0.0;
-    for (int q = 0; q < J.Q; ++q) {
-      const double2* Wq = J.W + base + (long long)q * L;
-      const double2* st = J.syn_tw + (long long)q * L;
-      for (int b = threadIdx.x; b < K; b += blockDim.x) {
-        double2 acc = make_double2(0.0, 0.0);
-        for (int l = (b == 0 ? K : b); l < L; l += K) acc = cfma(st[l], Wq[l], acc);
-        fft_put<DF>(buf, bitrev(b, J.logK), acc);
-      }
-      __syncthreads();
-      fft_in_place<DF>(J, buf);
-      const int n0 = J.nlo[q];
-      for (int r = threadIdx.x; r < K; r += blockDim.x) {
-        const int n = n0 + r;
-        if (n < NT) g[n] += fft_get<DF>(buf, r).x;
-      }
-      __syncthreads();
-    }
+    __syncthreads();
+    for (int q = 0; q < J.Q; ++q) synth_window<O>(J, q, J.W + base + (long long)q * L, buf, g);
     if (PART == 1) {
       for (int n = threadIdx.x; n < NT; n += blockDim.x) gpart[n] = g[n];
       return;
@@ -2101,7 +2162,7 @@ __global__ void __launch_bounds__(kTimeMaxThreads) k_synth_fwd(DevJob J) {
   const double mchi = -J.chi[J.tr_off[k] + x];
   for (int n = threadIdx.x; n < NT; n += blockDim.x) g[n] *= mchi;
   __syncthreads();
-  forward_all<DF>(J, g, buf, J.Gt + base);
+  forward_all<O>(J, g, buf, J.Gt + base);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2348,7 +2409,8 @@ cudaError_t launch_cross_assemble(const DevJob& J, cudaStream_t st, int* launche
                                                                : go(std::integral_constant<int, kFormMixed>{});
 }
 
-static size_t time_smem(const DevJob& J) { return (size_t)J.K * sizeof(double2) + (size_t)J.NT * sizeof(double); }
+// one window's K/2 complex points and the samples
+static size_t time_smem(const DevJob& J) { return (size_t)J.K * sizeof(double) + (size_t)J.NT * sizeof(double); }
 
 bool incident_recurrent(const DevJob& J) {
   return J.sig_kind == 0 && J.sig_nt == 0 && J.dt * kIncRun <= 2.0 * J.width;
