@@ -295,8 +295,8 @@ fthms_status upload_job(fthms_req* r) {
     TRY(dev_upload(r, p.slices, &J.slices));
     J.n_slices = (int)p.slices.size();
     TRY(dev_alloc(r, (size_t)std::max(1LL, p.res_total), &J.e_unit));
-    TRY(dev_alloc(r, p.sys.size() * 4, &J.phi_unit));
   }
+  if (J.mixed || !J.otf) TRY(dev_alloc(r, p.sys.size() * 4, &J.phi_unit));
   if (J.otf) {
     TRY(dev_upload(r, p.otf, &J.otf_tasks));
     TRY(dev_upload(r, p.wn_off, &J.wn_off));
@@ -326,13 +326,11 @@ fthms_status upload_job(fthms_req* r) {
   J.dinv32 = nullptr;
   J.rres = nullptr;
   J.rres64 = nullptr;
-  J.dcorr = nullptr;
   J.mdone = nullptr;
   J.mrel = nullptr;
   J.mrho = nullptr;
   J.mscale = nullptr;
-  J.arow = nullptr;
-  J.phistat = nullptr;
+  J.a_unit = nullptr;
   J.f64_min_n = J.fp64keep ? 0 : (J.mixed ? kLuBigMin : 1 << 30);
   J.rchunks = nullptr;
   J.n_rchunks = 0;
@@ -344,13 +342,11 @@ fthms_status upload_job(fthms_req* r) {
     TRY(dev_alloc(r, (size_t)p.piv_total, &J.dinv32));
     TRY(dev_alloc(r, (size_t)p.vec_total, &J.rres));
     TRY(dev_alloc(r, (size_t)p.vec_total, &J.rres64));
-    TRY(dev_alloc(r, (size_t)p.vec_total, &J.dcorr));
     TRY(dev_alloc(r, p.sys.size(), &J.mdone));
     TRY(dev_alloc(r, p.sys.size(), &J.mrel));
     TRY(dev_alloc(r, p.sys.size(), &J.mrho));
     TRY(dev_alloc(r, p.sys.size(), &J.mscale));
-    TRY(dev_alloc(r, (size_t)p.piv_total, &J.arow));
-    TRY(dev_alloc(r, p.sys.size() * 4, &J.phistat));
+    TRY(dev_alloc(r, (size_t)p.piv_total, &J.a_unit));
     TRY(dev_upload(r, p.rchunks, &J.rchunks));
     J.n_rchunks = (int)p.rchunks.size();
   }

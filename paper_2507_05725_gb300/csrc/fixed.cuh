@@ -35,6 +35,13 @@ __device__ __forceinline__ int2 fix_df(float hi, float lo, float c) {
   return make_int2(a + (int)q, __float2int_rn(__fmul_rn(__fsub_rn(t, q), 268435456.f)));
 }
 
+// A float |v| < 2^s (c = 2^(27 - s)).
+__device__ __forceinline__ int2 fix_f32(float v, float c) {
+  const float y = __fmul_rn(v, c);                      // exact
+  const int a = __float2int_rn(y);
+  return make_int2(a, __float2int_rn(__fmul_rn(__fsub_rn(y, (float)a), 268435456.f)));
+}
+
 // One warp: N values of a density vector in fixed point, and their unit.  A vector with a value that is not finite gets
 // the unit NaN, so that every sum it enters is NaN.
 __device__ __forceinline__ void fix_vector(const double2* v, int N, double scale, int4* out, double* unit, int lane) {

@@ -1214,11 +1214,6 @@ constexpr int kRefineCap = 16;          // largest refine_max accepted
 constexpr double kFirstRhoSafety = 10.0;
 constexpr int kResidThreads = 128;
 
-// One thread per row (rows past N recompute the last row and store nothing), all Q windows of the row:
-// r_q = G_q - A phi_q with compensated double-float sums over the columns in order.
-template <int Q>
-__global__ void __launch_bounds__(kResidThreads) k_mresid(DevJob J);
-
 // Asynchronous 16-byte copies global -> shared (bypassing L1), for streams whose loads would otherwise
 // occupy registers until they land.
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
@@ -1231,219 +1226,157 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(kPending) : "memory");
 }
 
-// Per row of the systems that keep FP64, upper bounds of the 1-norm and the 2-norm of the row's 2N real
-// components (|Re a_ij|, |Im a_ij|) in FP32, once per job after the assembly: each |a| bounded from above by
-// its 23 leading fraction bits times (1 + 2^-22), the sums of 2N such floats (or their squares) by (1 + 2^-10)
-// for their roundings (2N 2^-24 < 2^-10), the square root by (1 + 2^-20).  The first-pass residual sizes the
-// anchors of its FP32-pipe sums from them.
-__device__ __forceinline__ float abs_bound_f32(double a) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFull;
-  const int e = (int)(u >> 52);
-  if (e >= 1023 + 127) return __uint_as_float(0x7F800000u);   // beyond FP32 (or not finite): +inf
-  if (e < 1023 - 126) return 0x1p-126f;                       // below FP32's normal range
-  const unsigned frac23 = (unsigned)(u >> 29) & 0x7FFFFFu;
-  return __fmul_rn(__uint_as_float(((unsigned)(e - 1023 + 127) << 23) | frac23), 1.f + 0x1p-22f);
-}
-__global__ void __launch_bounds__(kResidThreads) k_arow_norms(DevJob J) {
-  const int chunk = blockIdx.x * (kResidThreads / 32) + (threadIdx.x >> 5);
-  if (chunk >= J.n_rchunks) return;
-  const ResidChunk c = J.rchunks[chunk];
-  const SysDesc s = J.sys[c.sys];
-  const int N = s.N;
-  if (!sys_f64(J, N)) return;
-  const int i = c.row0 + (threadIdx.x & 31);
-  if (i >= N) return;
-  const double2* __restrict__ A64 = J.A + s.mat_off;
-  float n1 = 0.f, n2 = 0.f;
-#pragma unroll 4
-  for (int j = 0; j < N; ++j) {
-    const double2 a = __ldg(&A64[(long long)j * N + i]);
-    const float br = abs_bound_f32(a.x), bi = abs_bound_f32(a.y);
-    n1 = __fadd_rn(n1, __fadd_rn(br, bi));
-    n2 = fmaf(br, br, fmaf(bi, bi, n2));
-  }
-  J.arow[s.piv_off + i] =
-      make_float2(__fmul_rn(n1, 1.f + 0x1p-10f), __fmul_rn(__fsqrt_rn(__fmul_rn(n2, 1.f + 0x1p-10f)), 1.f + 0x1p-20f));
-}
-
-// The first-pass residual of the systems that keep FP64 (all in the FP64-kept form), to FP64 accuracy on both
-// arithmetic pipes at once: phi_0 is the FP32 solution (exactly a float), so every product a_ij phi_j can be
-// formed exactly from a three-float split of the FP64 entry.  A warp sums its rows either through FP64 FMAs
-// (acc) or through those products and anchored sums on the FP32 pipe (aacc, anchors sized per window from
-// the smaller of the row's 1-norm times max |phi_0| and its 2-norm times |phi_0|_2); the FP64 pipe, which
-// alone would bound the kernel at 8 DFMA per entry and two windows, and the FP32 pipe then work side by
-// side.  Either way G - A phi_0 comes out with an error of the order of an FP64 accumulation's (about 2^-50
-// of sum_j |a_ij phi_j|).
+// One thread's row of a fixed-point product: sums over N sources of entry (at src + i stride) times the densities
+// den[q N + i] of every window.  The entries stream through the thread's own ring of kStages batches in shared memory
+// (ring + k blockDim.x, cp.async): the next batches are in flight while one is summed and hold no registers; a thread
+// reads only the slots it filled itself (no barrier).  The densities are the same for the whole warp: one cached load
+// per column.
+constexpr int kFixStages = 2;
+__host__ __device__ constexpr int fix_batch(int Q) { return Q <= 2 ? 8 : 4; }   // entries a batch
+constexpr size_t fix_ring_bytes(int Q, int threads) { return (size_t)kFixStages * fix_batch(Q) * threads * sizeof(int4); }
 template <int Q>
-__global__ void __launch_bounds__(kResidThreads) k_mresid64(DevJob J) {
-  const int chunk = blockIdx.x * (kResidThreads / 32) + (threadIdx.x >> 5);
-  if (chunk >= J.n_rchunks) return;
-  const ResidChunk c = J.rchunks[chunk];
-  if (J.mdone[c.sys]) return;
-  const SysDesc s = J.sys[c.sys];
-  const int N = s.N;
-  if (!sys_f64(J, N)) return;                 // double-float systems: k_mresid
-  const int i = c.row0 + (threadIdx.x & 31);
-  const int row = i < N ? i : N - 1;
-  const double2* __restrict__ A64 = J.A + s.mat_off;
-  const double2* __restrict__ ph = J.phi + s.vec_off;       // phi_0 as FP64 (exact)
-  const float2* __restrict__ ph32 = J.dcorr + s.vec_off;    // the same values as floats (pass-0 solve)
-  const double2* __restrict__ G = J.G + s.vec_off;
-  const double isc = 1.0 / J.mscale[c.sys];   // a power of two: exact
-  double2 acc[Q];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const double2 g = G[q * N + row];
-    acc[q] = make_double2(g.x * isc, g.y * isc);
-  }
-  // Anchors of the FP32-pipe sums, per window: every partial sum of |a phi_0| along the row (both the real
-  // and the imaginary part's 2N terms) stays below bnd = min(|a_i|_1 max |phi_0|, |a_i|_2 |phi_0|_2) (Hoelder,
-  // Cauchy-Schwarz; all bounded from above), so below 2^(kh-1) with kh = e + 2 for bnd in [2^e, 2^(e+1)).  A
-  // chunk with a row outside the anchors' range sums in FP64.
-  const float2 an = J.arow[s.piv_off + row];
-  const int km_off = -23 + (32 - __clz(2 * N + 3));       // km = kh - 23 + ceil(log2(T + 4)), T = 2N terms a sum
-  bool anchors_ok = true;
-  aacc sr[Q], si[Q];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const float2 ps = J.phistat[c.sys * 4 + q];
-    const float bnd = __fmul_rn(fminf(__fmul_rn(an.x, ps.x), __fmul_rn(an.y, ps.y)), 1.f + 0x1p-20f);
-    const int be = (int)((__float_as_uint(bnd) >> 23) & 0xFFu) - 127;
-    const int kh = bnd > 0.f ? be + 2 : 0;                 // (bnd = 0: every product is zero)
-    anchors_ok = anchors_ok && (bnd == 0.f || (be >= -40 && be <= 100));
-    sr[q].init(kh, kh + km_off);
-    si[q].init(kh, kh + km_off);
-  }
-  auto col64 = [&](const double2 a, int j) {
-#pragma unroll
-    for (int q = 0; q < Q; ++q) acc[q] = cfms(a, ph[q * N + j], acc[q]);
-  };
-  auto colx = [&](const double2 a, int j) {
-    float r1, r2, r3, i1, i2, i3;
-    split3_f64_bits(a.x, r1, r2, r3);
-    split3_f64_bits(a.y, i1, i2, i3);
+__device__ __forceinline__ void fix_row(const int4* __restrict__ src, long long stride, int N, const int4* __restrict__ den,
+                                        int4* ring, fixacc (&re)[Q], fixacc (&im)[Q]) {
+  constexpr int kB = fix_batch(Q);
+  const int T = blockDim.x, nbat = N / kB;
+  auto mac = [&](const int4 e, int i) {
+    const int n0 = -e.z, n1 = -e.w;
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
-      const float2 x = ph32[q * N + j];
-      sr[q].add_prod(r1, r2, r3, x.x);          // Re a phi = ar phr - ai phi
-      sr[q].add_prod(-i1, -i2, -i3, x.y);
-      si[q].add_prod(r1, r2, r3, x.y);          // Im a phi = ar phi + ai phr
-      si[q].add_prod(i1, i2, i3, x.x);
+      const int4 p = __ldg(&den[q * N + i]);
+      re[q].mac(e.x, e.y, p.x, p.y);
+      im[q].mac(e.x, e.y, p.z, p.w);
+      re[q].mac(n0, n1, p.z, p.w);
+      im[q].mac(e.z, e.w, p.x, p.y);
     }
   };
-  // warps specialise: one of every six 32-row chunks sums in FP64, the rest on the FP32 pipe, so that warps
-  // waiting on the FP64 pipe and warps issuing FP32 work share each SM (measured per job, N = 512: one chunk
-  // in three on the FP64 pipe 91.6 ms, in four 79.9, in six 76.6, in eight 80.6)
-  const bool on_fp32 = (chunk % 6) != 0 && __all_sync(0xffffffffu, anchors_ok);
-  int j0 = 0;
-  if (on_fp32) {
+  auto issue = [&](int bi) {
+    int4* dst = ring + (bi % kFixStages) * kB * T;
+    const int4* s = src + (long long)bi * kB * stride;
+#pragma unroll
+    for (int k = 0; k < kB; ++k) cp_async16(dst + k * T, s + k * stride);
+  };
+#pragma unroll
+  for (int bi = 0; bi < kFixStages - 1; ++bi) {
+    if (bi < nbat) issue(bi);
+    cp_async_commit();
+  }
 #pragma unroll 1
-    for (; j0 + 4 <= N; j0 += 4) {             // four entries of the row loaded before their sums
-      double2 a[4];
+  for (int bi = 0; bi < nbat; ++bi) {
+    if (bi + kFixStages - 1 < nbat) issue(bi + kFixStages - 1);
+    cp_async_commit();                          // (empty near the end: keeps the group count uniform)
+    cp_async_wait<kFixStages - 1>();            // batch bi has landed
+    const int4* s = ring + (bi % kFixStages) * kB * T;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) a[k] = __ldg(&A64[(long long)(j0 + k) * N + row]);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) colx(a[k], j0 + k);
+    for (int k = 0; k < kB; ++k) mac(s[k * T], bi * kB + k);
+    // a source adds two products to either half of a sum: kFixRun products between carries
+    if ((bi + 1) % (kFixRun / 2 / kB) == 0) {
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
-        sr[q].renorm();
-        si[q].renorm();
+        re[q].carry();
+        im[q].carry();
       }
     }
-    for (; j0 < N; ++j0) colx(__ldg(&A64[(long long)j0 * N + row]), j0);
-  } else {
-#pragma unroll 1
-    for (; j0 + 8 <= N; j0 += 8) {
-      double2 a[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) a[k] = __ldg(&A64[(long long)(j0 + k) * N + row]);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) col64(a[k], j0 + k);
-    }
-    for (; j0 < N; ++j0) col64(__ldg(&A64[(long long)j0 * N + row]), j0);
   }
-  if (i < N) {
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const double2 r = make_double2(acc[q].x - sr[q].value(), acc[q].y - si[q].value());
-      J.rres[s.vec_off + q * N + i] = make_float2(__double2float_rn(r.x), __double2float_rn(r.y));
-      J.rres64[s.vec_off + q * N + i] = r;
+  for (int i = nbat * kB; i < N; ++i) mac(__ldg(&src[(long long)i * stride]), i);
+}
+
+// The FP64-kept matrices in fixed point (fixed.cuh) for the refinement, converted in place once per job after the assembly:
+// every entry of row i as a 56-bit integer in units of a power of two just above the row's largest component (rounding
+// below 2^-56 of it; a row with an entry that is not finite gets the unit NaN).  A block stages kRows rows of one
+// system in shared memory, so the matrix is read and written once: bound by HBM.
+constexpr int kFixThreads = 256;
+template <int kRows>
+__global__ void __launch_bounds__(kFixThreads) k_afix(DevJob J) {
+  extern __shared__ __align__(16) double2 shx[];        // [N][kRows]
+  __shared__ unsigned s_max[kRows];
+  const ResidChunk c = J.rchunks[blockIdx.x];
+  const SysDesc s = J.sys[c.sys];
+  const int N = s.N, r = threadIdx.x % kRows, j0 = threadIdx.x / kRows;
+  if (!sys_f64(J, N)) return;
+  double2* A = J.A + s.mat_off;
+  for (int row0 = c.row0; row0 < min(c.row0 + 32, N); row0 += kRows) {
+    if (threadIdx.x < kRows) s_max[threadIdx.x] = 0u;
+    __syncthreads();
+    const bool on = row0 + r < N;
+    if (on) {
+      unsigned m = 0u;
+      for (int j = j0; j < N; j += kFixThreads / kRows) {
+        const double2 v = __ldcs(&A[(long long)j * N + row0 + r]);
+        shx[j * kRows + r] = v;
+        m = max(m, max((unsigned)__double2hiint(v.x) & 0x7FFFFFFFu, (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu));
+      }
+      atomicMax(&s_max[r], m);
     }
+    __syncthreads();
+    if (on) {
+      const int e = max((int)(s_max[r] >> 20) - 1022, -60);         // every |component| < 2^e
+      for (int j = j0; j < N; j += kFixThreads / kRows) {
+        const double2 v = shx[j * kRows + r];
+        const int2 x = fix_f64(v.x, e), y = fix_f64(v.y, e);
+        __stcs(reinterpret_cast<int4*>(A) + (long long)j * N + row0 + r, make_int4(x.x, x.y, y.x, y.y));
+      }
+      if (j0 == 0)
+        J.a_unit[s.piv_off + row0 + r] =
+            e > 60 ? __uint_as_float(0x7FFFFFFFu) : __uint_as_float((unsigned)(e - kFixBits + 127) << 23);
+    }
+    __syncthreads();
   }
 }
 
-// Later passes of the systems that keep FP64: the residual of the previous pass updated with its
-// correction, r <- r - A d, instead of a new FP64 residual G - A phi (the same value: phi grew by d).  The
-// FP64 matrix is split into two floats by integer operations (split_f64_bits) and d is an FP32 vector, so
-// every product is formed to about 2^-47 on the FP32 pipe (FMA two-product) and summed with compensated
-// double-float sums over the columns in order.  The update's error, about 2^-47 |A| |d|, stays far below
-// the FP64 residual's 2^-53 |A| |phi| since the correction d is much smaller than phi; the FP64 pipe does
-// one conversion per row.
+// Refinement residuals of the systems that keep FP64, one thread per row (rows past N recompute the last row and store
+// nothing), all Q windows of the row: pass 1 r = G - A phi_0, later passes r <- r - A d with the last correction (the same value: phi grew by d).
+// Matrix and vector are fixed-point and the sum is exact, rounded once to FP64 and once more in the subtraction -- below
+// an FP64 accumulation's error; all residuals run in units of a power of two of the right-hand side (exact).  Bound by HBM (16
+// bytes an entry); the FP64 and anchored FP32 sums (first pass) and double-float sums (later ones) before, 96 to 225
+// instructions an entry at two windows, were issue-bound: N = 512, 2304 systems, 8 steps: 30.5 + 20.6 -> 15.8 + 16.5 ms.
 template <int Q>
-__global__ void __launch_bounds__(kResidThreads) k_mresid_upd(DevJob J) {
+__global__ void __launch_bounds__(kResidThreads, 4) k_mresid(DevJob J, int pass) {
   const int chunk = blockIdx.x * (kResidThreads / 32) + (threadIdx.x >> 5);
   if (chunk >= J.n_rchunks) return;
   const ResidChunk c = J.rchunks[chunk];
   if (J.mdone[c.sys]) return;
   const SysDesc s = J.sys[c.sys];
   const int N = s.N;
-  if (!sys_f64(J, N)) return;                 // double-float systems: k_mresid
+  if (!sys_f64(J, N)) return;                 // double-float systems: k_mresid_df
   const int i = c.row0 + (threadIdx.x & 31);
   const int row = i < N ? i : N - 1;
-  const double2* __restrict__ A64 = J.A + s.mat_off;
-  const float2* __restrict__ d = J.dcorr + s.vec_off;
-  double2* r64 = J.rres64 + s.vec_off;
-  dfacc re[Q], im[Q];
+  extern __shared__ __align__(16) int4 she[];
+  fixacc re[Q], im[Q];
+  fix_row<Q>(reinterpret_cast<const int4*>(J.A) + s.mat_off + row, N, N, reinterpret_cast<const int4*>(J.phi_df) + s.vec_off,
+             she + threadIdx.x, re, im);
+  if (i >= N) return;
+  const double ua = (double)J.a_unit[s.piv_off + i] * 0x1p56;
+  const double isc = pass == 1 ? 1.0 / J.mscale[c.sys] : 0.0;   // a power of two: exact
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
-    const float4 rd = df_split2(r64[q * N + row]);
-    re[q].add(rd.x, rd.y);
-    im[q].add(rd.z, rd.w);
-  }
-  // r -= a d:  Re -= ar dr - ai di,  Im -= ar di + ai dr; kB matrix entries of the row loaded before their sums
-  constexpr int kB = Q <= 2 ? 8 : 4;
-  auto step = [&](const double2 a, int j) {
-    float arh, arl, aih, ail;
-    split_f64_bits(a.x, arh, arl);
-    split_f64_bits(a.y, aih, ail);
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const float2 dv = d[q * N + j];
-      dfacc_mac1(re[q], -arh, -arl, dv.x);
-      dfacc_mac1(re[q], aih, ail, dv.y);
-      dfacc_mac1(im[q], -arh, -arl, dv.y);
-      dfacc_mac1(im[q], -aih, -ail, dv.x);
+    const long long o = s.vec_off + (long long)q * N + i;
+    double2 r;
+    if (pass == 1) {
+      const double2 g = J.G[o];
+      r = make_double2(g.x * isc, g.y * isc);
+    } else {
+      r = J.rres64[o];
     }
-  };
-  int j0 = 0;
-#pragma unroll 1
-  for (; j0 + kB <= N; j0 += kB) {
-    double2 a[kB];
-#pragma unroll
-    for (int k = 0; k < kB; ++k) a[k] = __ldg(&A64[(long long)(j0 + k) * N + row]);
-#pragma unroll
-    for (int k = 0; k < kB; ++k) step(a[k], j0 + k);
-  }
-  for (; j0 < N; ++j0) step(__ldg(&A64[(long long)j0 * N + row]), j0);
-  if (i < N) {
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const df rr = re[q].value(), ri = im[q].value();
-      J.rres[s.vec_off + q * N + i] = make_float2(rr.hi + rr.lo, ri.hi + ri.lo);
-      r64[q * N + i] = make_double2((double)rr.hi + (double)rr.lo, (double)ri.hi + (double)ri.lo);
-    }
+    const double u = ua * J.phi_unit[4ll * c.sys + q];
+    r.x = fma(-u, re[q].value(), r.x);
+    r.y = fma(-u, im[q].value(), r.y);
+    J.rres64[o] = r;
+    J.rres[o] = make_float2(__double2float_rn(r.x), __double2float_rn(r.y));
   }
 }
 
+// The same for the mixed form's systems that keep double-float matrices: r = G - A phi in compensated double-float sums
+// (one window: HBM-bound already, and no conversion of the matrix).
 template <int Q>
-__global__ void __launch_bounds__(kResidThreads) k_mresid(DevJob J) {
+__global__ void __launch_bounds__(kResidThreads) k_mresid_df(DevJob J) {
   const int chunk = blockIdx.x * (kResidThreads / 32) + (threadIdx.x >> 5);
   if (chunk >= J.n_rchunks) return;
   const ResidChunk c = J.rchunks[chunk];
   if (J.mdone[c.sys]) return;
   const SysDesc s = J.sys[c.sys];
   const int N = s.N;
-  if (sys_f64(J, N)) return;                  // FP64 systems: k_mresid64
+  if (sys_f64(J, N)) return;                  // these: k_mresid
   const int i = c.row0 + (threadIdx.x & 31);
   const int row = i < N ? i : N - 1;
   const float4* __restrict__ Adf = reinterpret_cast<const float4*>(J.A) + s.mat_off;
@@ -1494,6 +1427,23 @@ __global__ void __launch_bounds__(kResidThreads) k_mresid(DevJob J) {
   }
 }
 
+// One warp: the FP32 solution (or correction) b[0..N) of one window in fixed point for the next residual.
+__device__ __forceinline__ void fix_correction(const float2* b, int N, int4* out, double* unit, int lane) {
+  unsigned m = 0u;
+  for (int i = lane; i < N; i += 32)
+    m = max(m, max(__float_as_uint(b[i].x) & 0x7FFFFFFFu, __float_as_uint(b[i].y) & 0x7FFFFFFFu));
+  m = __reduce_max_sync(0xffffffffu, m);
+  const int e = max((int)(m >> 23), 30) - 126;          // every |component| < 2^e (subnormal and tiny: any unit does)
+  const bool bad = m >= 0x7F800000u || e > 120;
+  const float c0 = __uint_as_float((unsigned)(127 - e / 2) << 23), c1 = __uint_as_float((unsigned)(27 - (e - e / 2) + 127) << 23);
+  for (int i = lane; i < N; i += 32) {                  // (scaled in two steps: 2^(27 - e) may leave FP32's range)
+    const int2 x = fix_f32(__fmul_rn(b[i].x, c0), c1), y = fix_f32(__fmul_rn(b[i].y, c0), c1);
+    out[i] = make_int4(x.x, x.y, y.x, y.y);
+  }
+  if (lane == 0)
+    *unit = bad ? __longlong_as_double(0x7FF8000000000000ll) : __hiloint2double((e - kFixBits + 1023) << 20, 0);
+}
+
 // pass 0: solve with FP32 G, store phi as double-float (FP64 in the FP64-kept form, whose residual reads
 // it), mark the system as refining.  pass p >= 1: solve for the correction from the residual, add it in
 // double-float (FP64), and finish the system (FP64 densities, their double-float copy for the cross apply,
@@ -1539,30 +1489,18 @@ __global__ void __launch_bounds__(32 * kSolveWarps, 3) k_msolve(DevJob J, int m,
   __syncwarp();
   tri_solve<float2, QT>(b, N, L32, piv, dinv, lane);
   double2* ph64 = J.phi + s.vec_off;
-  float2* dc = J.dcorr + s.vec_off;
+  auto keep = [&] {                           // b for the next residual
+#pragma unroll 1
+    for (int q = 0; q < QT; ++q)
+      fix_correction(b + q * N, N, reinterpret_cast<int4*>(J.phi_df) + s.vec_off + (long long)q * N,
+                     J.phi_unit + 4ll * sidx + q, lane);
+  };
   if (pass == 0) {
-    if (f64) {
-#pragma unroll
-      for (int q = 0; q < QT; ++q) {
-        float pm = 0.f, p2 = 0.f;
-        for (int e = q * N + lane; e < (q + 1) * N; e += 32) {
-          ph64[e] = make_double2(b[e].x, b[e].y);
-          dc[e] = b[e];                       // phi_0 as floats for the first residual's FP32-pipe columns
-          pm = fmaxf(pm, fmaxf(fabsf(b[e].x), fabsf(b[e].y)));
-          p2 = fmaf(b[e].x, b[e].x, fmaf(b[e].y, b[e].y, p2));
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, o));
-          p2 = __fadd_rn(p2, __shfl_xor_sync(0xffffffffu, p2, o));
-        }
-        // the first residual's anchors: max |component| and an upper bound of the window's 2-norm
-        if (lane == 0)
-          J.phistat[sidx * 4 + q] =
-              make_float2(pm, __fmul_rn(__fsqrt_rn(__fmul_rn(p2, 1.f + 0x1p-10f)), 1.f + 0x1p-20f));
-      }
-    } else {
-      for (int e = lane; e < Q * N; e += 32) ph[e] = make_float4(b[e].x, 0.f, b[e].y, 0.f);
+    for (int e = lane; e < Q * N; e += 32) {
+      if (f64) ph64[e] = make_double2(b[e].x, b[e].y);
+      else ph[e] = make_float4(b[e].x, 0.f, b[e].y, 0.f);
     }
+    if (f64) keep();
     if (lane == 0) J.mdone[sidx] = 0;
     return;
   }
@@ -1570,7 +1508,6 @@ __global__ void __launch_bounds__(32 * kSolveWarps, 3) k_msolve(DevJob J, int m,
   for (int e = lane; e < Q * N; e += 32) {
     const float2 d = b[e];
     if (f64) {
-      dc[e] = d;                              // the next pass updates the residual with it
       double2 p = ph64[e];
       p.x += (double)d.x;
       p.y += (double)d.y;
@@ -1605,6 +1542,7 @@ __global__ void __launch_bounds__(32 * kSolveWarps, 3) k_msolve(DevJob J, int m,
   }
   const double left = rel * rho;
   if (left >= J.refine_tol && pass < J.refine_max) {
+    if (f64) keep();
     if (lane == 0) J.mrel[sidx] = (float)rel;
     return;
   }
@@ -1640,16 +1578,11 @@ __global__ void __launch_bounds__(32 * kSolveWarps, 3) k_msolve(DevJob J, int m,
 // Cross apply: W_k(x, q, l) = sum_j sum_i E_{l,k,j}[i, r] phi_j[q, i]; observation sums accumulate.  First half: one CTA
 // per slice of kApplySlice rows of a group (the rows of all its source blocks, concatenated), one thread per row, the
 // source-major blocks read coalesced.  Entries and densities are fixed-point (fixed.cuh), the sums exact integers,
-// so one kernel serves every form.  The row's entries stream through a per-thread ring of kApplyStages batches in shared
-// memory (cp.async): batch b + 1 is in flight while batch b is summed, and holds no registers; a thread reads only the
-// slots it filled itself (no barrier).  Bound by HBM (16 bytes an entry): 8 obstacle arcs, 4.8e8 entries, 12 steps: 42.7 (FP64 FMAs) ->
+// so one kernel serves every form (fix_row).  Bound by HBM (16 bytes an entry): 8 obstacle arcs, 4.8e8 entries, 12 steps: 42.7 (FP64 FMAs) ->
 // 17.2 ms, 0.84 of a copy's rate; the mixed forms' double-float sums took 16.8 (N = 512, two windows: 70 either way).
-// Entries of a row per batch:
-__host__ __device__ constexpr int apply_batch(int Q) { return Q <= 2 ? 8 : 4; }
-constexpr int kApplyStages = 2;   // batches per thread in shared memory: one summed while the next lands
 template <int Q>
 __global__ void __launch_bounds__(kApplySlice, Q == 1 ? 3 : 2) k_cross_rows(DevJob J) {
-  extern __shared__ __align__(16) int4 she[];     // [kApplyStages][kB][kApplySlice]
+  extern __shared__ __align__(16) int4 she[];
   const ApplySlice sl = J.slices[blockIdx.x];
   if ((int)threadIdx.x >= sl.nrows) return;
   const int row = sl.row0 + threadIdx.x;
@@ -1660,54 +1593,9 @@ __global__ void __launch_bounds__(kApplySlice, Q == 1 ? 3 : 2) k_cross_rows(DevJ
     ++b;
   }
   const CrossBlk B = J.blks[b];
-  const int N = B.N, nr = B.nrows;
-  // the block's densities, the same for every row: one cached load per warp and column
-  const int4* __restrict__ phb = reinterpret_cast<const int4*>(J.phi_df) + J.sys[B.sys].vec_off;
-  const int4* __restrict__ Er = reinterpret_cast<const int4*>(J.E + B.e_off) + r;
   fixacc re[Q], im[Q];
-  auto mac = [&](const int4 e, int i) {
-    const int n0 = -e.z, n1 = -e.w;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const int4 p = __ldg(&phb[q * N + i]);
-      re[q].mac(e.x, e.y, p.x, p.y);
-      re[q].mac(n0, n1, p.z, p.w);
-      im[q].mac(e.x, e.y, p.z, p.w);
-      im[q].mac(e.z, e.w, p.x, p.y);
-    }
-  };
-  constexpr int kB = apply_batch(Q);
-  const int nbat = N / kB;
-  int4* mine = she + threadIdx.x;
-  auto issue = [&](int bi) {
-    int4* dst = mine + (bi % kApplyStages) * kB * kApplySlice;
-    const int4* src = Er + (long long)bi * kB * nr;
-#pragma unroll
-    for (int k = 0; k < kB; ++k) cp_async16(dst + k * kApplySlice, src + (long long)k * nr);
-  };
-#pragma unroll
-  for (int bi = 0; bi < kApplyStages - 1; ++bi) {
-    if (bi < nbat) issue(bi);
-    cp_async_commit();
-  }
-#pragma unroll 1
-  for (int bi = 0; bi < nbat; ++bi) {
-    if (bi + kApplyStages - 1 < nbat) issue(bi + kApplyStages - 1);
-    cp_async_commit();                          // (empty near the end: keeps the group count uniform)
-    cp_async_wait<kApplyStages - 1>();          // batch bi has landed
-    const int4* src = mine + (bi % kApplyStages) * kB * kApplySlice;
-#pragma unroll
-    for (int k = 0; k < kB; ++k) mac(src[k * kApplySlice], bi * kB + k);
-    // a source adds two products to either half of a sum: kFixRun products between carries
-    if ((bi + 1) % (kFixRun / 2 / kB) == 0) {
-#pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        re[q].carry();
-        im[q].carry();
-      }
-    }
-  }
-  for (int i = nbat * kB; i < N; ++i) mac(__ldg(&Er[(long long)i * nr]), i);
+  fix_row<Q>(reinterpret_cast<const int4*>(J.E + B.e_off) + r, B.nrows, B.N,
+             reinterpret_cast<const int4*>(J.phi_df) + J.sys[B.sys].vec_off, she + threadIdx.x, re, im);
   const long long rr = J.grp_res_off[sl.grp] + row;
   const double unit = (double)J.e_unit[rr] * 0x1p56;
 #pragma unroll
@@ -2370,11 +2258,14 @@ cudaError_t launch_assemble_self(const DevJob& J, cudaStream_t st, int* launches
       *launches += 1;
     }
   }
-  // the row bounds of the FP64 matrices, for the first-pass residual's anchors
-  const bool any64 = J.mixed && (J.fp64keep || J.max_n >= J.f64_min_n);
-  const int rgrid = cdiv(J.n_rchunks, kResidThreads / 32);
-  if (any64 && J.arow && rgrid > 0) {
-    k_arow_norms<<<rgrid, kResidThreads, 0, st>>>(J);
+  // the FP64-kept systems' fixed-point matrices (rows staged: 8 while two blocks fit an SM, else 4)
+  if (J.mixed && J.n_rchunks > 0 && (J.fp64keep || J.max_n >= J.f64_min_n)) {
+    const bool wide = J.max_n <= 800;
+    const size_t sh = (size_t)(wide ? 8 : 4) * J.max_n * sizeof(int4);
+    cudaError_t e = cudaFuncSetAttribute(wide ? k_afix<8> : k_afix<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+    if (e != cudaSuccess) return e;
+    if (wide) k_afix<8><<<J.n_rchunks, kFixThreads, sh, st>>>(J);
+    else k_afix<4><<<J.n_rchunks, kFixThreads, sh, st>>>(J);
     *launches += 1;
   }
   return cudaGetLastError();
@@ -2555,18 +2446,22 @@ static cudaError_t launch_msolve_q(const DevJob& J, int m, int pass, cudaStream_
   return cudaGetLastError();
 }
 
-// Mixed forms: the residuals before refinement pass `pass` >= 1: FP64 for the systems that keep FP64 at
-// the first pass, updated with the last correction at later ones (reading of the FP64 residual), double-float
-// for the others.
+// Mixed forms: the residuals before refinement pass `pass` >= 1.
 template <int QT>
 static cudaError_t launch_resid_q(const DevJob& J, int pass, cudaStream_t st, int* launches) {
   const int rgrid = cdiv(J.n_rchunks, kResidThreads / 32);
   if (rgrid == 0) return cudaSuccess;
-  const bool any64 = J.fp64keep || J.max_n >= J.f64_min_n, anydf = !J.fp64keep;
-  if (any64 && pass == 1) k_mresid64<QT><<<rgrid, kResidThreads, 0, st>>>(J);
-  else if (any64) k_mresid_upd<QT><<<rgrid, kResidThreads, 0, st>>>(J);
-  if (anydf) k_mresid<QT><<<rgrid, kResidThreads, 0, st>>>(J);
-  *launches += (int)any64 + (int)anydf;
+  if (J.fp64keep || J.max_n >= J.f64_min_n) {
+    const size_t sh = fix_ring_bytes(QT, kResidThreads);
+    cudaError_t e = cudaFuncSetAttribute(k_mresid<QT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+    if (e != cudaSuccess) return e;
+    k_mresid<QT><<<rgrid, kResidThreads, sh, st>>>(J, pass);
+    *launches += 1;
+  }
+  if (!J.fp64keep) {
+    k_mresid_df<QT><<<rgrid, kResidThreads, 0, st>>>(J);
+    *launches += 1;
+  }
   return cudaGetLastError();
 }
 
@@ -2620,7 +2515,7 @@ cudaError_t launch_resid(const DevJob& J, int pass, cudaStream_t st, int* launch
 template <int Q>
 static cudaError_t launch_cross_apply_q(const DevJob& J, cudaStream_t st) {
   // the row kernel's ring of entry batches (the densities come through the L1 cache)
-  const size_t sh_rows = (size_t)kApplyStages * apply_batch(Q) * kApplySlice * sizeof(int4);
+  const size_t sh_rows = fix_ring_bytes(Q, kApplySlice);
   const size_t sh_red = (size_t)Q * J.acc_cap * sizeof(double2);
   cudaError_t e = cudaFuncSetAttribute(k_cross_rows<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_rows);
   if (e != cudaSuccess) return e;

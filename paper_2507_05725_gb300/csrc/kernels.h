@@ -74,7 +74,7 @@ struct DevJob {
   FreqDf* freq_df;           // [L] constants of the double-float Hankel entries (mixed forms)
   const long long* row_off;  // [pair][L] first row of (pair, l) in the per-row results
   float* e_unit;             // stored cross rows: unit of a row's fixed-point entries, laid out like the row results
-  double* phi_unit;          // [system][4] unit of a window's fixed-point densities (stored cross rows)
+  double* phi_unit;          // [system][4] unit of a window's fixed-point densities (and, mixed forms, corrections)
   const int* tpanel;
   const long long* tr_off;
   const double* chi;
@@ -87,23 +87,20 @@ struct DevJob {
   const double* s_q;         // [Q]
   double H, period;
   // work arrays
-  double2* A;                // LU factors (mixed form: the matrix itself, as double-float)
+  double2* A;                // LU factors (mixed forms: the matrix itself, double-float, or fixed-point int4
+                             // after the assembly for the systems that keep FP64)
   float2* LU32;              // FP32 factors (mixed form)
   float2* dinv32;            // FP32 1 / U_kk (mixed form)
   double* refine_resid;      // [0] max estimated error left, [1] refinement passes, [2] unconverged
                              // (system, step) pairs (64-bit integers in [1], [2]; mixed form)
   float* sys_err;            // per system: max over steps of the estimated relative error left (mixed form)
   float2* rres;              // FP32-rounded refinement residuals, laid out like G (mixed form)
-  double2* rres64;           // FP64-kept systems: the residual the next pass updates, laid out like G
-  float2* dcorr;             // FP64-kept systems: the last FP32 correction, laid out like G
+  double2* rres64;           // the residual the next pass updates, laid out like G (mixed forms)
   int* mdone;                // per system: 1 once its refinement has finished this step (mixed form)
   float* mrel;               // per system: relative size of its last correction (mixed form)
   float* mrho;               // per system: largest contraction factor measured in earlier steps (0: none yet)
   double* mscale;            // per system and step: power of two near max |G|; refinement runs in G / mscale
-  float2* arow;              // FP64-kept systems, per row (once per job): upper bounds of the 1-norm and the 2-norm
-                             // of the row's 2N real components (|Re a_ij|, |Im a_ij|)
-  float2* phistat;           // FP64-kept systems, per system and window (4 slots a system, every step): max |component|
-                             // and an upper bound of the 2-norm of the pass-0 FP32 solution
+  float* a_unit;             // per row: unit of the matrix row's fixed-point entries (systems that keep FP64)
   int f64_min_n;             // mixed forms: systems of at least this N keep FP64 matrices and residuals
   const ResidChunk* rchunks; // 32-row chunks of the systems, largest first (mixed form)
   int n_rchunks;

@@ -706,8 +706,8 @@ size_t plan_device_bytes(const Plan& p) {
   size_t b = 0;
   b += (size_t)p.mat_total * 16;                 // A / LU
   if (p.opt.precision >= 1)                      // FP32 factors, residuals and corrections, refinement state
-    b += (size_t)p.mat_total * 8 + (size_t)p.piv_total * 8 + (size_t)p.vec_total * (8 + 16 + 16 + 8) +
-         p.sys.size() * (24 + 32) + (size_t)p.piv_total * 8 + p.rchunks.size() * sizeof(ResidChunk);
+    b += (size_t)p.mat_total * 8 + (size_t)p.piv_total * 8 + (size_t)p.vec_total * (8 + 16 + 16) +
+         p.sys.size() * (24 + 32) + (size_t)p.piv_total * 4 + p.rchunks.size() * sizeof(ResidChunk);
   b += p.sig_f.size() * 8;                       // samples of a sampled signal
   b += (size_t)p.piv_total * 4;                  // pivots
   b += (size_t)p.rlog_total * 8;                 // cosine sums of the self log weights
@@ -722,8 +722,8 @@ size_t plan_device_bytes(const Plan& p) {
        p.asms.size() * sizeof(CrossAsm) + p.self_tiles.size() * sizeof(SelfTile) + p.sys.size() * (sizeof(SysDesc) + sizeof(int)) + p.slices.size() * sizeof(ApplySlice) + p.grp_res_off.size() * 8;
   b += (size_t)p.res_total * p.Q * 16 + p.row_off.size() * 8;   // per-row cross sums
   if (p.opt.cross_mode == 0) {                                  // fixed-point units and densities
-    b += (size_t)p.res_total * 4 + p.sys.size() * 32;
-    if (p.opt.precision == 0) b += (size_t)p.vec_total * 16;
+    b += (size_t)p.res_total * 4;
+    if (p.opt.precision == 0) b += (size_t)p.vec_total * 16 + p.sys.size() * 32;
   }
   b += (size_t)p.L * 48;
   if (p.opt.cross_mode == 1)
