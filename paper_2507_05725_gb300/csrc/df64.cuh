@@ -332,4 +332,49 @@ struct aacc {
   }
 };
 
+// Two floats in one register pair: one instruction per operation on both (the FP32 pipe's rate is the same, the issue
+// slots are half).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// dfacc for two sums at once; (na, nal) is the negated factor, so that the product's error comes out negated.
+struct dfacc2 {
+  f32x2 hi = 0ull, lo = 0ull;
+  __device__ __forceinline__ void mac(f32x2 ah, f32x2 nah, f32x2 nal, f32x2 bh, f32x2 bl) {
+    const f32x2 p = mul2(ah, bh);
+    f32x2 ne = fma2(nah, bh, p);
+    ne = fma2(nah, bl, ne);
+    ne = fma2(nal, bh, ne);
+    const f32x2 s = add2(hi, p), v = sub2(s, hi);
+    const f32x2 t = add2(sub2(hi, sub2(s, v)), sub2(p, v));
+    hi = s;
+    lo = add2(lo, sub2(t, ne));
+  }
+};
+
 }  // namespace fthms

@@ -1131,6 +1131,7 @@ __global__ void __launch_bounds__(kOtfThreads, otf_blocks(Q)) k_cross_otf_df(Dev
   for (int b0 = 0; b0 < nl; b0 += NB) {
     const int nb = min(NB, nl - b0);
     dfacc acc[V];
+    dfacc2 acc2[NB][Q / 2 > 0 ? Q / 2 : 1][2];      // windows in pairs: (re, im)
     // T one step ahead: its chain of dependent FP64 operations runs beside the current pair's entries
     auto turns_at = [&](int i) {
       const double dx = t.x - __ldg(&nx[i]), dy = t.y - __ldg(&ny[i]);
@@ -1164,9 +1165,12 @@ __global__ void __launch_bounds__(kOtfThreads, otf_blocks(Q)) k_cross_otf_df(Dev
       for (int k = 0; k < NB; ++k) {
         if (k < nb) {
           const FreqDf& f = fr[b0 + k];
+          // densities: windows in pairs (re hi hi lo lo, im hi hi lo lo), an odd last one alone
           float4 pv[Q], e;
+          const float4* __restrict__ pd = J.phi_df + vo[b0 + k];
 #pragma unroll
-          for (int q = 0; q < Q; ++q) pv[q] = __ldg(&J.phi_df[vo[b0 + k] + i + (long long)q * N]);
+          for (int q = 0; q < Q; ++q)
+            pv[q] = __ldg(&pd[q < (Q & ~1) ? (long long)(q & ~1) * N + 2 * i + (q & 1) : (long long)q * N + i]);
           if (pt.T.hi * f.a.x < (float)kBesselLarge) {
             if (kKeep64) {
               e = split2_bits(hankel_near_f64(v62 * (unsigned long long)(ot.l0 + b0 + k), lnT64 + f.lnz, beta64, near, qw64));
@@ -1176,12 +1180,34 @@ __global__ void __launch_bounds__(kOtfThreads, otf_blocks(Q)) k_cross_otf_df(Dev
           } else {
             e = hankel_far_df(pt, ph, ang, df{f.a.z, f.a.w}, df{f.b.x, f.b.y}, beta, near);
           }
+          if constexpr (Q >= 2) {
+            const f32x2 xr = pack2(e.x, e.x), nxr = pack2(-e.x, -e.x), nlr = pack2(-e.y, -e.y), lr = pack2(e.y, e.y);
+            const f32x2 xi = pack2(e.z, e.z), nxi = pack2(-e.z, -e.z), nli = pack2(-e.w, -e.w), li = pack2(e.w, e.w);
 #pragma unroll
-          for (int q = 0; q < Q; ++q) cdf_mac(acc[(k * Q + q) * 2], acc[(k * Q + q) * 2 + 1], e, pv[q]);
+            for (int g = 0; g < Q / 2; ++g) {
+              const float4 a = pv[2 * g], b = pv[2 * g + 1];
+              const f32x2 rh = pack2(a.x, a.y), rl = pack2(a.z, a.w), ih = pack2(b.x, b.y), il = pack2(b.z, b.w);
+              acc2[k][g][0].mac(xr, nxr, nlr, rh, rl);
+              acc2[k][g][0].mac(nxi, xi, li, ih, il);
+              acc2[k][g][1].mac(xr, nxr, nlr, ih, il);
+              acc2[k][g][1].mac(xi, nxi, nli, rh, rl);
+            }
+          }
+          if constexpr (Q & 1) cdf_mac(acc[(k * Q + Q - 1) * 2], acc[(k * Q + Q - 1) * 2 + 1], e, pv[Q - 1]);
         }
         ph += pt.v;
       }
     }
+#pragma unroll
+    for (int k = 0; k < NB; ++k)
+#pragma unroll
+      for (int g = 0; g < Q / 2; ++g)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          dfacc &a = acc[(k * Q + 2 * g) * 2 + c], &b = acc[(k * Q + 2 * g + 1) * 2 + c];
+          unpack2(acc2[k][g][c].hi, a.hi, b.hi);
+          unpack2(acc2[k][g][c].lo, a.lo, b.lo);
+        }
     df_warp_sums<V>(acc, lane);
     constexpr int kShift = V == 32 ? 0 : V == 16 ? 1 : V == 8 ? 2 : V == 4 ? 3 : 4;
     const int e = lane >> kShift, k = e / (2 * Q), q = (e / 2) % Q;
@@ -1562,7 +1588,19 @@ __global__ void __launch_bounds__(32 * kSolveWarps, 3) k_msolve(DevJob J, int m,
   for (int e = lane; e < Q * N; e += 32) {
     double2 v = f64 ? out[e] : df_join2(ph[e]);
     v = make_double2(v.x * scale, v.y * scale);
-    if (J.otf) pdf[e] = df_split2(v);
+    if (J.otf) {                              // windows in pairs, as k_cross_otf_df reads them
+      const float4 d = df_split2(v);
+      const int q = e / N, i = e % N;
+      if (q < (QT & ~1)) {
+        float* p = reinterpret_cast<float*>(pdf + (long long)(q & ~1) * N + 2 * i) + (q & 1);
+        p[0] = d.x;
+        p[2] = d.y;
+        p[4] = d.z;
+        p[6] = d.w;
+      } else {
+        pdf[e] = d;
+      }
+    }
     out[e] = v;
     sum[e] = m == 1 ? v : cadd(sum[e], v);
     if (all) all[e] = v;
