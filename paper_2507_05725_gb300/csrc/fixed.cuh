@@ -42,6 +42,13 @@ __device__ __forceinline__ int2 fix_f32(float v, float c) {
   return make_int2(a, __float2int_rn(__fmul_rn(__fsub_rn(y, (float)a), 268435456.f)));
 }
 
+// (double)t by two FP64 additions (the bits of both halves placed under 2^84 and 2^52).
+__device__ __forceinline__ double ll_to_double(long long t) {
+  const double h = __hiloint2double(0x45300000, (int)(t >> 32) ^ (int)0x80000000u);
+  const double l = __hiloint2double(0x43300000, (int)(unsigned)t);
+  return (h - 19342822341709703277445120.0) + l;        // 2^84 + 2^63 + 2^52
+}
+
 // One warp: N values of a density vector in fixed point, and their unit.  A vector with a value that is not finite gets
 // the unit NaN, so that every sum it enters is NaN.
 __device__ __forceinline__ void fix_vector(const double2* v, int N, double scale, int4* out, double* unit, int lane) {

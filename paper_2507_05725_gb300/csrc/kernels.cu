@@ -352,7 +352,19 @@ constexpr int kPS = kNB + 1;   // padded panel row stride (bank-conflict-free co
 constexpr int kLuThreads = 256;
 
 // C = double2 (plain form: factors J.A in place) or float2 (mixed form: factors J.LU32 in place).  One system
-// by the whole CTA (kLuThreads threads); shl_raw: max(N (kNB + kPS), 2 kSB^2) elements of shared memory.
+// by the whole CTA (kLuThreads threads); shl_raw: lu_smem bytes of shared memory.
+//
+// FP64 trailing update in fixed point (fixed.cuh): A22 -= L21 U12 took 32 FP64 FMAs an entry and panel, the whole FP64
+// pipe (75% of the kernel's time at its rate).  The multipliers are below 2 (partial pivoting on |re| + |im|) and a column
+// of U12 shares one unit, so both become 56-bit integers in the same shared memory, the eight products sum exactly in
+// integers and only the final conversion and subtraction are FP64: 6 instructions an entry and panel.  A thread takes
+// two columns of a row, so that each multiplier is read once for both.  8192 systems of N 48..259: 31.0 -> 16.6 ms.
+template <class C>
+__host__ __device__ constexpr size_t lu_smem(int N) {
+  const size_t panel = (size_t)N * (kNB + kPS) * sizeof(C) + (sizeof(C) == sizeof(double2) ? (size_t)N * sizeof(double) : 0);
+  const size_t finish = (size_t)2 * kSB * kSB * sizeof(C);
+  return panel > finish ? panel : finish;
+}
 template <class C>
 __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
   C* shl = reinterpret_cast<C*>(shl_raw);
@@ -362,6 +374,7 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
   int* piv = J.piv + s.piv_off;
   C* Pn = shl;                       // [N][kPS] panel rows
   C* U = shl + (size_t)N * kPS;      // [kNB][N] U12 rows
+  [[maybe_unused]] double* unit = reinterpret_cast<double*>(U + (size_t)kNB * N);   // FP64: per column of U12
   __shared__ int spiv[kNB];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   for (int k0 = 0; k0 < N; k0 += kNB) {
@@ -406,13 +419,65 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
             for (int c = 0; c < r; ++c) v = cfms(Pn[r * kPS + c], xv[c], v);
             xv[r] = v;
             Ac[r] = v;
-            U[r * N + j] = v;
+            if constexpr (sizeof(C) == sizeof(float2)) U[r * N + j] = v;
           }
+        }
+        if constexpr (sizeof(C) == sizeof(double2)) {   // (w = kNB here: columns remain)
+          unsigned top = 0u;
+#pragma unroll
+          for (int r = 0; r < kNB; ++r)
+            top = max(top, max((unsigned)__double2hiint(xv[r].x) & 0x7FFFFFFFu, (unsigned)__double2hiint(xv[r].y) & 0x7FFFFFFFu));
+          const int e = max((int)(top >> 20), 100) - 1022;
+#pragma unroll
+          for (int r = 0; r < kNB; ++r) {
+            const int2 x = fix_f64(xv[r].x, e), y = fix_f64(xv[r].y, e);
+            reinterpret_cast<int4*>(U)[r * N + j] = make_int4(x.x, x.y, y.x, y.y);
+          }
+          // unit of a product sum: 2^56 2^(1 - 55) 2^(e - 55)
+          unit[j] = e > 1000 ? __longlong_as_double(0x7FF8000000000000ll) : __hiloint2double((e - 53 + 1023) << 20, 0);
         }
       }
       __syncthreads();
       // A22 -= L21 U12.
       const int mr = nr - w;
+      if constexpr (sizeof(C) == sizeof(double2)) {
+        int4* L = reinterpret_cast<int4*>(Pn) + w * kPS;          // multipliers, converted in place
+        const int4* Ui = reinterpret_cast<const int4*>(U);
+        for (int idx = tid; idx < mr * kNB; idx += kLuThreads) {
+          const int o = (idx / kNB) * kPS + idx % kNB;
+          const C v = Pn[w * kPS + o];
+          const int2 x = fix_f64(v.x, 1), y = fix_f64(v.y, 1);
+          L[o] = make_int4(x.x, x.y, y.x, y.y);
+        }
+        __syncthreads();
+        const int np = (nc + 1) / 2;
+        for (int idx = tid; idx < mr * np; idx += kLuThreads) {
+          const int r = idx % mr, j0 = 2 * (idx / mr), j1 = min(j0 + 1, nc - 1);
+          C* a0 = A + (long long)(k0 + w + j0) * N + k0 + w + r;
+          C* a1 = A + (long long)(k0 + w + j1) * N + k0 + w + r;
+          C v0 = *a0, v1 = *a1;
+          fixacc re0, im0, re1, im1;
+#pragma unroll
+          for (int c = 0; c < kNB; ++c) {
+            const int4 l = L[r * kPS + c], p = Ui[c * N + j0], q = Ui[c * N + j1];
+            const int n0 = -l.z, n1 = -l.w;
+            re0.mac(l.x, l.y, p.x, p.y);
+            im0.mac(l.x, l.y, p.z, p.w);
+            re1.mac(l.x, l.y, q.x, q.y);
+            im1.mac(l.x, l.y, q.z, q.w);
+            re0.mac(n0, n1, p.z, p.w);
+            im0.mac(l.z, l.w, p.x, p.y);
+            re1.mac(n0, n1, q.z, q.w);
+            im1.mac(l.z, l.w, q.x, q.y);
+          }
+          auto less = [](double v, double u, const fixacc& s) { return fma(-u, ll_to_double(s.a + (s.b >> 28)), v); };
+          const double u0 = unit[j0], u1 = unit[j1];
+          v0 = make_double2(less(v0.x, u0, re0), less(v0.y, u0, im0));
+          v1 = make_double2(less(v1.x, u1, re1), less(v1.y, u1, im1));
+          *a0 = v0;
+          if (j1 > j0) *a1 = v1;
+        }
+      } else
       for (long long idx = tid; idx < (long long)mr * nc; idx += kLuThreads) {
         int j = (int)(idx / mr), r = (int)(idx % mr);
         C* a = A + (long long)(k0 + w + j) * N + k0 + w + r;
@@ -432,7 +497,7 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
 }
 
 template <class C>
-__global__ void __launch_bounds__(kLuThreads) k_lu(DevJob J) {
+__global__ void __launch_bounds__(kLuThreads, sizeof(C) == sizeof(double2) ? 3 : 1) k_lu(DevJob J) {
   extern __shared__ __align__(16) unsigned char shl_raw[];
   lu_one<C>(J, J.lu_small[blockIdx.x], shl_raw);
 }
@@ -2321,7 +2386,7 @@ cudaError_t launch_lu_small(const DevJob& J, cudaStream_t st, int* launches) {
     if (J.n_lu_small > 0) {
       int small_max = 0;   // systems above kLuBigMin go to the tensor-core path; J.max_n bounds the rest
       small_max = std::min(J.max_n, kLuBigMin - 1);
-      size_t sh = std::max((size_t)small_max * (kNB + kPS), (size_t)2 * kSB * kSB) * sizeof(float2);
+      size_t sh = lu_smem<float2>(small_max);
       cudaError_t e = cudaFuncSetAttribute(k_lu<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
       if (e != cudaSuccess) return e;
       k_lu<float2><<<J.n_lu_small, kLuThreads, sh, st>>>(J);
@@ -2331,7 +2396,7 @@ cudaError_t launch_lu_small(const DevJob& J, cudaStream_t st, int* launches) {
     return cudaSuccess;
   }
   if (J.n_lu_small == 0) return cudaSuccess;
-  size_t sh = std::max((size_t)J.max_n * (kNB + kPS), (size_t)2 * kSB * kSB) * sizeof(double2);
+  size_t sh = lu_smem<double2>(J.max_n);
   cudaError_t e = cudaFuncSetAttribute(k_lu<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
   if (e != cudaSuccess) return e;
   k_lu<double2><<<J.n_lu_small, kLuThreads, sh, st>>>(J);
@@ -2357,7 +2422,7 @@ static cudaError_t launch_fused_q(const DevJob& J, int* counter, size_t sh, cuda
 
 cudaError_t launch_fused_asf(const DevJob& J, int* counter, cudaStream_t st, int* launches) {
   if (J.nsys == 0) return cudaSuccess;
-  const size_t sh = std::max((size_t)J.max_n * (kNB + kPS), (size_t)2 * kSB * kSB) * sizeof(double2);
+  const size_t sh = lu_smem<double2>(J.max_n);
   *launches += 1;
   switch (J.Q) {
     case 1: return launch_fused_q<1>(J, counter, sh, st);
