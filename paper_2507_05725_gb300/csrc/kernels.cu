@@ -346,13 +346,14 @@ __global__ void __launch_bounds__(256) k_assemble_self(DevJob J) {
 
 // ---------------------------------------------------------------------------------------------
 // Blocked right-looking LU with partial pivoting (pivot: max |re| + |im|, first index on ties),
-// one CTA of 256 threads per system, panel width 8 in shared memory, column-major factor in HBM.
+// one CTA of 256 threads (small FP64 systems: 128) per system, panel width 8 in shared memory, column-major factor in HBM.
 constexpr int kNB = 8;
 constexpr int kPS = kNB + 1;   // padded panel row stride (bank-conflict-free column access)
 constexpr int kLuThreads = 256;
+constexpr int kLuNarrow = 135;   // FP64 jobs of systems up to this size: 128 threads (launch_lu says why)
 
 // C = double2 (plain form: factors J.A in place) or float2 (mixed form: factors J.LU32 in place).  One system
-// by the whole CTA (kLuThreads threads); shl_raw: lu_smem bytes of shared memory.
+// by the whole CTA (NT threads); shl_raw: lu_smem bytes of shared memory.
 //
 // FP64 trailing update in fixed point (fixed.cuh): A22 -= L21 U12 took 32 FP64 FMAs an entry and panel, the whole FP64
 // pipe (75% of the kernel's time at its rate).  The multipliers are below 2 (partial pivoting on |re| + |im|) and a column
@@ -365,7 +366,7 @@ __host__ __device__ constexpr size_t lu_smem(int N) {
   const size_t finish = (size_t)2 * kSB * kSB * sizeof(C);
   return panel > finish ? panel : finish;
 }
-template <class C>
+template <class C, int NT>
 __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
   C* shl = reinterpret_cast<C*>(shl_raw);
   const SysDesc s = J.sys[sidx];
@@ -380,7 +381,7 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
   for (int k0 = 0; k0 < N; k0 += kNB) {
     const int w = min(kNB, N - k0);
     const int nr = N - k0;
-    for (int idx = tid; idx < nr * w; idx += kLuThreads) {
+    for (int idx = tid; idx < nr * w; idx += NT) {
       int c = idx / nr, r = idx % nr;
       Pn[r * kPS + c] = A[(long long)(k0 + c) * N + k0 + r];
     }
@@ -392,12 +393,12 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
       if (lane < w) piv[k0 + lane] = k0 + spiv[lane];
     }
     __syncthreads();
-    for (int idx = tid; idx < nr * w; idx += kLuThreads) {
+    for (int idx = tid; idx < nr * w; idx += NT) {
       int c = idx / nr, r = idx % nr;
       A[(long long)(k0 + c) * N + k0 + r] = Pn[r * kPS + c];
     }
     // Row interchanges on the columns outside the panel.
-    for (int col = tid; col < N; col += kLuThreads) {
+    for (int col = tid; col < N; col += NT) {
       if (col >= k0 && col < k0 + w) continue;
       C* Ac = A + (long long)col * N + k0;
       for (int c = 0; c < w; ++c) {
@@ -409,7 +410,7 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
     const int nc = N - k0 - w;
     if (nc > 0) {
       // U12 = L11^{-1} A12 (unit lower triangular solve), one column per thread.
-      for (int j = tid; j < nc; j += kLuThreads) {
+      for (int j = tid; j < nc; j += NT) {
         C* Ac = A + (long long)(k0 + w + j) * N + k0;
         C xv[kNB];
 #pragma unroll
@@ -443,7 +444,7 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
       if constexpr (sizeof(C) == sizeof(double2)) {
         int4* L = reinterpret_cast<int4*>(Pn) + w * kPS;          // multipliers, converted in place
         const int4* Ui = reinterpret_cast<const int4*>(U);
-        for (int idx = tid; idx < mr * kNB; idx += kLuThreads) {
+        for (int idx = tid; idx < mr * kNB; idx += NT) {
           const int o = (idx / kNB) * kPS + idx % kNB;
           const C v = Pn[w * kPS + o];
           const int2 x = fix_f64(v.x, 1), y = fix_f64(v.y, 1);
@@ -451,7 +452,7 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
         }
         __syncthreads();
         const int np = (nc + 1) / 2;
-        for (int idx = tid; idx < mr * np; idx += kLuThreads) {
+        for (int idx = tid; idx < mr * np; idx += NT) {
           const int r = idx % mr, j0 = 2 * (idx / mr), j1 = min(j0 + 1, nc - 1);
           C* a0 = A + (long long)(k0 + w + j0) * N + k0 + w + r;
           C* a1 = A + (long long)(k0 + w + j1) * N + k0 + w + r;
@@ -478,7 +479,7 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
           if (j1 > j0) *a1 = v1;
         }
       } else
-      for (long long idx = tid; idx < (long long)mr * nc; idx += kLuThreads) {
+      for (long long idx = tid; idx < (long long)mr * nc; idx += NT) {
         int j = (int)(idx / mr), r = (int)(idx % mr);
         C* a = A + (long long)(k0 + w + j) * N + k0 + w + r;
         C v = *a;
@@ -490,16 +491,18 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
     }
     __syncthreads();
   }
-  lu_finish<C, kLuThreads>(A, N,
+  lu_finish<C, NT>(A, N,
                            (sizeof(C) == sizeof(double2) ? reinterpret_cast<C*>(J.dinv) : reinterpret_cast<C*>(J.dinv32)) +
                                s.piv_off,
                            shl);
 }
 
-template <class C>
-__global__ void __launch_bounds__(kLuThreads, sizeof(C) == sizeof(double2) ? 3 : 1) k_lu(DevJob J) {
+// Threads per system: the panel's columns are one warp's work, so an FP64 system below about a hundred nodes, whose
+// shared memory lets six share an SM, runs faster on fewer (768 systems of N = 96: 1.73 -> 1.47 ms at 128 threads).
+template <class C, int NT>
+__global__ void __launch_bounds__(NT, sizeof(C) == sizeof(double2) ? 768 / NT : 1) k_lu(DevJob J) {
   extern __shared__ __align__(16) unsigned char shl_raw[];
-  lu_one<C>(J, J.lu_small[blockIdx.x], shl_raw);
+  lu_one<C, NT>(J, J.lu_small[blockIdx.x], shl_raw);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -733,8 +736,9 @@ __device__ __noinline__ void fused_solve(const DevJob& J, int sidx, int q, doubl
 // system.  Each CTA takes the next system from a work counter (systems by decreasing N, so the largest start
 // first and the small ones fill the tail), assembles its matrix, factors it (lu_one) and solves its step-1
 // windows, one warp per window; the counter is reset by the host before the launch.
+constexpr int kFusedThreads = 256;
 template <int QT>
-__global__ void __launch_bounds__(kLuThreads, 2) k_fused_asf(DevJob J, int* counter) {
+__global__ void __launch_bounds__(kFusedThreads, 2) k_fused_asf(DevJob J, int* counter) {
   extern __shared__ __align__(16) unsigned char shf_raw[];
   __shared__ int s_item;
   for (;;) {
@@ -745,7 +749,7 @@ __global__ void __launch_bounds__(kLuThreads, 2) k_fused_asf(DevJob J, int* coun
     const int sidx = J.sys_order[item];
     assemble_one(J, sidx);
     __syncthreads();
-    lu_one<double2>(J, sidx, shf_raw);
+    lu_one<double2, kFusedThreads>(J, sidx, shf_raw);
     __syncthreads();
     const int wid = threadIdx.x >> 5;
     if (wid < QT) fused_solve(J, sidx, wid, reinterpret_cast<double2*>(shf_raw) + (size_t)wid * J.max_n, threadIdx.x & 31);
@@ -2387,21 +2391,28 @@ cudaError_t launch_lu_small(const DevJob& J, cudaStream_t st, int* launches) {
       int small_max = 0;   // systems above kLuBigMin go to the tensor-core path; J.max_n bounds the rest
       small_max = std::min(J.max_n, kLuBigMin - 1);
       size_t sh = lu_smem<float2>(small_max);
-      cudaError_t e = cudaFuncSetAttribute(k_lu<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+      cudaError_t e = cudaFuncSetAttribute(k_lu<float2, kLuThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
       if (e != cudaSuccess) return e;
-      k_lu<float2><<<J.n_lu_small, kLuThreads, sh, st>>>(J);
+      k_lu<float2, kLuThreads><<<J.n_lu_small, kLuThreads, sh, st>>>(J);
       *launches += 1;
       return cudaGetLastError();
     }
     return cudaSuccess;
   }
   if (J.n_lu_small == 0) return cudaSuccess;
-  size_t sh = lu_smem<double2>(J.max_n);
-  cudaError_t e = cudaFuncSetAttribute(k_lu<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
-  if (e != cudaSuccess) return e;
-  k_lu<double2><<<J.n_lu_small, kLuThreads, sh, st>>>(J);
+  const size_t sh = lu_smem<double2>(J.max_n);
+  auto go = [&](auto nt) {
+    constexpr int NT = decltype(nt)::value;
+    cudaError_t e = cudaFuncSetAttribute(k_lu<double2, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+    if (e != cudaSuccess) return e;
+    k_lu<double2, NT><<<J.n_lu_small, NT, sh, st>>>(J);
+    return cudaGetLastError();
+  };
   *launches += 1;
-  return cudaGetLastError();
+  // A small system's panel keeps one warp busy while the others wait, so more and narrower CTAs an SM win; a large
+  // system's trailing update wants the wide one.  768 systems, 128 against 256 threads: N = 64 0.77 / 0.93 ms, N = 96
+  // 1.47 / 1.73, N = 128 2.56 / 2.90, N = 144 4.05 / 3.61, N = 256 15.7 / 13.6 (the factors are the same bit for bit).
+  return J.max_n <= kLuNarrow ? go(std::integral_constant<int, 128>{}) : go(std::integral_constant<int, kLuThreads>{});
 }
 
 template <int QT>
@@ -2411,12 +2422,12 @@ static cudaError_t launch_fused_q(const DevJob& J, int* counter, size_t sh, cuda
   int dev = 0, sms = 0, per_sm = 0;
   e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fused_asf<QT>, kLuThreads, sh);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fused_asf<QT>, kFusedThreads, sh);
   if (e != cudaSuccess) return e;
   const int grid = std::max(1, std::min(J.nsys, sms * std::max(per_sm, 1)));
   e = cudaMemsetAsync(counter, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
-  k_fused_asf<QT><<<grid, kLuThreads, sh, st>>>(J, counter);
+  k_fused_asf<QT><<<grid, kFusedThreads, sh, st>>>(J, counter);
   return cudaGetLastError();
 }
 
