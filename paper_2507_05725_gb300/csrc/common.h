@@ -84,16 +84,9 @@ struct CrossAsm {
   int pad;
 };
 
-// On-the-fly cross task (cross_mode 1): assembly task `task`, restricted to the frequencies l0..l1
-// (at most otf_band(Q) of them: the per-frequency sums of a CTA take 128 x Q x otf_band(Q) complex
-// values of shared memory, at most 32 KB).
+// On-the-fly cross task (cross_mode 1): assembly task `task`, restricted to the frequencies l0..l1 (at most kOtfBand of
+// them, whose constants a CTA keeps in shared memory).
 constexpr int kOtfBand = 16;
-template <int Q> struct OtfBand { static constexpr int value = kOtfBand / Q > 4 ? kOtfBand / Q : 4; };
-inline int otf_band(int Q) { return kOtfBand / Q > 4 ? kOtfBand / Q : 4; }   // host side of OtfBand
-// Mixed forms: the double-float every-step kernel evaluates a (row, source) pair for bands of up to
-// kOtfBandDf frequencies (its per-pair set-up amortised over the band; 16 rather than 32 leaves room for more
-// CTAs per SM).
-constexpr int kOtfBandDf = 16;
 struct CrossOtf {
   int task;
   int l0, l1;

@@ -824,92 +824,6 @@ __device__ void near_beta_block(const CrossTgt* tg, int nrows, int N, const doub
   __syncthreads();
 }
 
-// Quantities of one (target row, source node) pair shared by every frequency of a band.  Every entry,
-// near or far, is E = (alpha J0 - (w/4) Y, (w/4) J0) with Y = Yhat0 below z = 20 and Y0 above;
-// alpha = A0 + A1 ln l below 20, A0 = -(w/(2 pi)) (ln(hR/2) + gamma) + beta w/4, and beta w/4 above.  beta = 0 for
-// the far rule; for the near rule the log-singular part K1 ln|t* - s| is integrated with the weights W_i instead
-// of w, which adds beta (near_beta_block).
-struct PairSetup {
-  double R, hR, inv_u, A0, beta;
-  int lsw;     // first frequency index with z = l h R >= 20
-};
-
-__device__ __forceinline__ PairSetup pair_setup(const DevJob& J, const CrossTgt& t, double xi, double yi, double beta,
-                                                int l0, double w, double inv_h) {
-  PairSetup s;
-  const double dx = t.x - xi, dy = t.y - yi;
-  const double R2 = fma(dx, dx, dy * dy);
-  const double rinv = rsqrt(R2);
-  const double R0 = R2 * rinv;
-  s.R = fma(fma(-R0, R0, R2), 0.5 * rinv, R0);   // one Newton step on sqrt(R2)
-  s.hR = J.h * s.R;
-  s.inv_u = rinv * inv_h;                        // 1 / (h R)
-  s.lsw = max(l0, (int)ceil(fmin(kBesselLarge * s.inv_u, 1.0e9)));
-  s.A0 = 0.0;
-  s.beta = beta;
-  if (s.lsw > l0) s.A0 = w * fma(-0.5 * kInvPi, log(0.5 * s.hR) + kEulerGamma, 0.25 * beta);
-  return s;
-}
-
-// Entry at z = (l h) R < 20 from the Taylor tables (lh = l h, lnl = ln l).
-__device__ __forceinline__ double2 taylor_entry(const PairSetup& s, double lh, double lnl, double A1, double qw) {
-  double J0, Yh;
-  bessel0_taylor(lh * s.R, J0, Yh);
-  const double alpha = fma(A1, lnl, s.A0);
-  return make_double2(fma(alpha, J0, -qw * Yh), qw * J0);
-}
-
-// Above z = 20 the Hankel expansion's phase advances by the fixed rotation e^{i h R} from one frequency
-// to the next (re-seeded by sincos every 16 steps); 1/z = (1/(hR))(1/l) and sqrt(2/(pi z)) =
-// sqrt(2/(pi hR))/sqrt(l); the number of terms follows the first (smallest) z of the run.
-struct AsymState {
-  double cx, sx;   // cos(z - pi/4), sin(z - pi/4) at the current frequency
-  double cu, su;   // the step rotation e^{i h R}
-  double ampw;     // sqrt(2/(pi h R)) w/4
-  int since, kmax;
-};
-
-__device__ __forceinline__ AsymState asym_start(const PairSetup& s, double lh_first, double camp, bool step = true) {
-  AsymState a;
-  a.ampw = rsqrt(s.hR) * camp;
-  a.su = 0.0;
-  a.cu = 1.0;
-  if (step) {
-    if (s.hR <= 1.0) sincos_taylor(s.hR, a.su, a.cu);
-    else sincos(s.hR, &a.su, &a.cu);
-  }
-  a.kmax = hankel_terms((float)(lh_first * s.R));
-  a.cx = a.sx = 0.0;
-  a.since = 16;
-  return a;
-}
-
-__device__ __forceinline__ double2 asym_entry(AsymState& a, const PairSetup& s, double lh, double invl, double rsql) {
-  if (a.since >= 16) {
-    double sn, cs;
-    sincos(lh * s.R, &sn, &cs);
-    a.cx = (cs + sn) * kSqrtHalf;
-    a.sx = (sn - cs) * kSqrtHalf;
-    a.since = 0;
-  }
-  const double wz = s.inv_u * invl;
-  const double w2 = -wz * wz;
-  double P = c_hank_a[2 * a.kmax], Qa = c_hank_a[2 * a.kmax + 1];
-  for (int k = a.kmax - 1; k >= 0; --k) {
-    P = fma(P, w2, c_hank_a[2 * k]);
-    Qa = fma(Qa, w2, c_hank_a[2 * k + 1]);
-  }
-  Qa *= wz;
-  const double amp = a.ampw * rsql;
-  const double t1 = fma(P, a.cx, Qa * a.sx);             // J0 / amp
-  const double t2 = fma(P, a.sx, -Qa * a.cx);            // Y0 / amp
-  const double cn = fma(a.cx, a.cu, -a.sx * a.su);
-  a.sx = fma(a.sx, a.cu, a.cx * a.su);
-  a.cx = cn;
-  ++a.since;
-  return make_double2(amp * fma(s.beta, t1, -t2), amp * t1);
-}
-
 // kNear: the launch over the tasks with near rows (shared memory for their corrections); otherwise over the far-only
 // tasks, which need only the tables (more CTAs per SM).  Each launch skips the other kind of task.  kForm: 0 the FP64
 // form, 1 the mixed form (double-float entries), 2 the FP64-kept form (double-float, FP64 below z = 20).  A thread
@@ -1049,80 +963,101 @@ __global__ void __launch_bounds__(kAsmThreads) k_near_weights(DevJob J) {
                   shn + 2 * task.N + 1, J.wn + off);
 }
 
-// One CTA per (assembly task, band of at most otf_band(Q) frequencies): thread (row r, source group g)
-// evaluates the entries of its sources i = g, g + 16, ... for every frequency of the band exactly as
-// k_cross_assemble does, multiplies them by the densities of the current step and adds them into its
-// own slot of partial sums in shared memory; the 16 partial sums of a row are then added in group
-// order (deterministic) into the per-row results, which k_cross_reduce adds per target in block order.
+constexpr int kOtfThreads = 32 * kAsmRows;
+
+// V sums of a warp's lanes added over the lanes (V a power of two <= 32): each halving step keeps one half of the values
+// and hands the other to the partner lane, so lane e << log2(32/V) ends with sum e.
+template <int V>
+__device__ __forceinline__ void warp_sums(double (&a)[V], int lane) {
+  int w = 16;
+#pragma unroll
+  for (int n = V / 2; n >= 1; n >>= 1, w >>= 1) {
+    const bool up = (lane & w) != 0;
+#pragma unroll
+    for (int e = 0; e < n; ++e) {
+      const double keep = up ? a[e + n] : a[e], give = up ? a[e] : a[e + n];
+      a[e] = keep + __shfl_xor_sync(0xffffffffu, give, w);
+    }
+  }
+  for (; w >= 1; w >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], w);
+}
+
+// FP64 form: one CTA of kAsmRows warps per (assembly task, band of at most kOtfBand frequencies), warp = target row,
+// lane = source node, frequencies in register blocks; each entry (hankel_df.cuh: 9 FP64 instructions) goes straight
+// into the lane's FP64 sums, which are added over the lanes once per block.  Bound by the FP64 pipe; the rotated
+// recurrences summed through shared memory before took 25 to 45 FP64 instructions an entry besides the 4 a window:
+// 8 obstacle arcs, 256 frequencies, 2 steps: 23.3 -> 12.3 ms; 3 arcs of a disk at N = 96, 2 steps: 2.26 -> 0.88 ms.
+__host__ __device__ constexpr int otf64_regs(int Q) { return Q == 1 ? 4 : Q == 2 ? 2 : 1; }
 template <int Q>
-__global__ void __launch_bounds__(kAsmThreads) k_cross_otf(DevJob J) {
-  constexpr int B = OtfBand<Q>::value;
-  constexpr int G = kAsmThreads / kAsmRows;          // source groups
-  extern __shared__ double2 sho[];                    // [Q * B][G * kAsmRows] partial sums: slot-major, so
-                                                      // a warp's read-modify-writes hit consecutive words
-  __shared__ double tb[4][B];                         // 1/l, 1/sqrt(l), ln l, l h
-  const CrossOtf ot = J.otf_tasks[blockIdx.x];
+__global__ void __launch_bounds__(kOtfThreads, 2) k_cross_otf(DevJob J) {
+  constexpr int NB = otf64_regs(Q), V = NB * (Q == 3 ? 4 : Q) * 2;
+  __shared__ AngleTab<true> ang;
+  __shared__ FreqDf fr[kOtfBand];
+  __shared__ long long vo[kOtfBand];
+  const CrossOtf ot = J.otf_tasks[(int)((long long)blockIdx.x * J.otf_stride % J.n_otf)];
   const CrossAsm task = J.asms[ot.task];
   const PairDesc pr = J.pairs[task.pair];
   const int N = task.N, nl = ot.l1 - ot.l0 + 1;
   const Panel pn = J.panels[task.panel];
-  const CrossTgt* tg = J.tgts + pr.tgt_off + task.row0;
   const long long woff = J.wn_off[ot.task];
-  const double* Wn = woff >= 0 ? J.wn + woff : nullptr;
-  if (threadIdx.x < nl) {
-    const int l = ot.l0 + threadIdx.x;
-    tb[0][threadIdx.x] = 1.0 / l;
-    tb[1][threadIdx.x] = rsqrt((double)l);
-    tb[2][threadIdx.x] = log((double)l);
-    tb[3][threadIdx.x] = l * J.h;
+  const int tid = threadIdx.x, lane = tid & 31, r = tid >> 5;
+  load_angles(ang);
+  if (tid < nl) {
+    fr[tid] = J.freq_df[ot.l0 + tid];
+    vo[tid] = J.sys[(long long)pr.j * (J.L - 1) + (ot.l0 + tid - 1)].vec_off;
   }
-  double2* mine = sho + threadIdx.x;                  // slot e at mine[e * kAsmThreads]
-  for (int e = 0; e < Q * B; ++e) mine[e * kAsmThreads] = make_double2(0.0, 0.0);
   __syncthreads();
-  const double w = kPiD / N, qw = 0.25 * w;
-  const double A1 = -0.5 * kInvPi * w;
-  const double camp = kSqrtTwoOverPi * qw;
-  const double inv_h = 1.0 / J.h;
-  const int r = threadIdx.x % kAsmRows, g = threadIdx.x / kAsmRows;
-  if (r < task.nrows) {
-    const CrossTgt t = tg[r];
-    const SysDesc* sj = J.sys + (long long)pr.j * (J.L - 1) + (ot.l0 - 1);   // systems (j, l0..l1)
-    for (int i = g; i < N; i += G) {
-      const PairSetup ps = pair_setup(J, t, J.node_x[pn.off + i], J.node_y[pn.off + i],
-                                      t.near ? Wn[r * N + i] : 0.0, ot.l0, w, inv_h);
-      AsymState as{};
-      bool started = false;
-      for (int b = 0; b < nl; ++b) {
-        const int l = ot.l0 + b;
-        double2 E;
-        if (l < ps.lsw) {
-          E = taylor_entry(ps, tb[3][b], tb[2][b], A1, qw);
-        } else {
-          if (!started) {
-            as = asym_start(ps, tb[3][b], camp);
-            started = true;
-          }
-          E = asym_entry(as, ps, tb[3][b], tb[0][b], tb[1][b]);
-        }
-        const double2* ph = J.phi + sj[b].vec_off + i;
+  if (r >= task.nrows) return;
+  const CrossTgt t = J.tgts[pr.tgt_off + task.row0 + r];
+  const double* __restrict__ bt = t.near ? J.wn + woff + (long long)r * N : nullptr;
+  const bool near = bt && __double_as_longlong(__ldg(bt)) != 0;     // (+0.0: beta vanishes on the whole row)
+  const double qw = 0.25 * kPiD / N, camp4 = qw * kInvPi, turns = J.h * (0.5 * kInvPi);
+  const double* __restrict__ nx = J.node_x + pn.off;
+  const double* __restrict__ ny = J.node_y + pn.off;
+#pragma unroll 1
+  for (int b0 = 0; b0 < nl; b0 += NB) {
+    const int nb = min(NB, nl - b0);
+    double acc[V];                                    // [frequency][window][re, im]
 #pragma unroll
-        for (int q = 0; q < Q; ++q)
-          mine[(q * B + b) * kAsmThreads] = cfma(E, ph[q * N], mine[(q * B + b) * kAsmThreads]);
+    for (int e = 0; e < V; ++e) acc[e] = 0.0;
+#pragma unroll 1
+    for (int i = lane; i < N; i += 32) {
+      const double dx = t.x - __ldg(&nx[i]), dy = t.y - __ldg(&ny[i]);
+      const double T = turns * dist_f64(fma(dx, dx, dy * dy));
+      const PairF64 pt = pair_f64(T, camp4);
+      const double beta = near ? __ldg(&bt[i]) : 0.0;
+      const double lnT = pt.th * fr[b0].a.x < (float)kBesselLarge ? log_f64(T) : 0.0;
+      unsigned long long ph = pt.v * (unsigned long long)(ot.l0 + b0) - (1ull << 61),
+                         u = pt.v62 * (unsigned long long)(ot.l0 + b0);
+#pragma unroll
+      for (int k = 0; k < NB; ++k, ph += pt.v, u += pt.v62) {
+        if (k < nb) {
+          const FreqDf& f = fr[b0 + k];
+          const double2 e = pt.th * f.a.x < (float)kBesselLarge
+                                ? hankel_near_f64(u, lnT + f.lnz, beta, near, qw)
+                                : hankel_far_f64(pt, ph, ang, df{f.a.z, f.a.w}, f.rs, beta, near);
+          const double2* __restrict__ pd = J.phi + vo[b0 + k] + i;
+#pragma unroll
+          for (int q = 0; q < Q; ++q) {
+            const double2 s = cfma(e, pd[(long long)q * N], make_double2(acc[(k * Q + q) * 2], acc[(k * Q + q) * 2 + 1]));
+            acc[(k * Q + q) * 2] = s.x;
+            acc[(k * Q + q) * 2 + 1] = s.y;
+          }
+        }
       }
     }
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < task.nrows * Q * nl; e += kAsmThreads) {
-    const int rr = e / (Q * nl), q = (e / nl) % Q, b = e % nl;
-    double2 sum = make_double2(0.0, 0.0);
-    for (int gg = 0; gg < G; ++gg) sum = cadd(sum, sho[(q * B + b) * kAsmThreads + gg * kAsmRows + rr]);
-    const long long row = J.row_off[(long long)task.pair * J.L + ot.l0 + b] + task.row0 + rr;
-    J.apply_res[row * Q + q] = sum;
+    warp_sums<V>(acc, lane);
+    constexpr int kShift = V == 32 ? 0 : V == 16 ? 1 : V == 8 ? 2 : V == 4 ? 3 : 4;
+    const int e = lane >> kShift, k = e / (2 * Q), q = (e / 2) % Q;
+    if ((lane & ((1 << kShift) - 1)) == 0 && k < nb) {
+      const long long row = J.row_off[(long long)task.pair * J.L + ot.l0 + b0 + k] + task.row0 + r;
+      reinterpret_cast<double*>(J.apply_res)[(row * Q + q) * 2 + (e & 1)] = acc[0];
+    }
   }
 }
 
 // Mixed forms, cross rows evaluated every step in double-float (on the FP32 pipe).  One CTA of kAsmRows warps per
-// (assembly task of kAsmRows target rows, band of at most kOtfBandDf frequencies): warp = target row, lane = source
+// (assembly task of kAsmRows target rows, band of at most kOtfBand frequencies): warp = target row, lane = source
 // node (s0 + lane, so node coordinates and densities load coalesced and the near rule is warp-uniform), frequencies
 // in register blocks of otf_regs(Q).  A lane sets its pair up in turns (PairTurns), evaluates each entry and multiplies
 // it straight into its own compensated double-float sums, one per (frequency, window); the 32 lanes' sums are added
@@ -1132,7 +1067,6 @@ __global__ void __launch_bounds__(kAsmThreads) k_cross_otf(DevJob J) {
 // four windows: 501 -> 91 ms; 6 arcs at N = 1024, two windows:
 // 499 -> 335 ms.  Bound by FP32 issue (~125 instructions an entry and 48 a window).
 // kKeep64 (the FP64-kept form): entries below z = 20 in FP64.
-constexpr int kOtfThreads = 32 * kAsmRows;
 __host__ __device__ constexpr int otf_regs(int Q) { return Q == 1 ? 8 : Q == 2 ? 4 : 1; }
 // blocks per SM: 16 warps of 128 registers, or 24 of 80 where the few sums leave room (measured per Q)
 constexpr int otf_blocks(int Q) { return Q <= 2 ? 2 : 3; }
@@ -1161,7 +1095,7 @@ __device__ __forceinline__ void df_warp_sums(dfacc (&a)[V], int lane) {
 
 template <int Q, bool kKeep64>
 __global__ void __launch_bounds__(kOtfThreads, otf_blocks(Q)) k_cross_otf_df(DevJob J) {
-  constexpr int B = kOtfBandDf, NB = otf_regs(Q);
+  constexpr int B = kOtfBand, NB = otf_regs(Q);
   constexpr int V = NB * (Q == 3 ? 4 : Q) * 2;                      // sums per warp, a power of two
   __shared__ float4 ang[kAngles];
   __shared__ FreqDf fr[B];
@@ -2663,7 +2597,6 @@ cudaError_t launch_near_weights(const DevJob& J, cudaStream_t st, int* launches)
 
 template <int Q>
 static cudaError_t launch_cross_otf_q(const DevJob& J, cudaStream_t st) {
-  constexpr int B = OtfBand<Q>::value;
   const size_t sh_red = (size_t)Q * J.acc_cap * sizeof(double2);
   cudaError_t e = cudaFuncSetAttribute(k_cross_reduce<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_red);
   if (e != cudaSuccess) return e;
@@ -2672,8 +2605,7 @@ static cudaError_t launch_cross_otf_q(const DevJob& J, cudaStream_t st) {
       if (J.fp64keep) k_cross_otf_df<Q, true><<<J.n_otf, kOtfThreads, 0, st>>>(J);
       else k_cross_otf_df<Q, false><<<J.n_otf, kOtfThreads, 0, st>>>(J);
     } else {
-      const size_t sh = (size_t)kAsmThreads * Q * B * sizeof(double2);
-      k_cross_otf<Q><<<J.n_otf, kAsmThreads, sh, st>>>(J);
+      k_cross_otf<Q><<<J.n_otf, kOtfThreads, 0, st>>>(J);
     }
   }
   k_cross_reduce<Q><<<J.n_grp, kApplyThreads, sh_red, st>>>(J);

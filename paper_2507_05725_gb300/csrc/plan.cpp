@@ -633,10 +633,9 @@ int build_plan(const fthms_curve* curves, int ncurves, const fthms_arc* arcs, in
     }
   }
   if (p.opt.cross_mode == 1) {
-    // Near weights once per job (they depend on the target and N only); tasks of at most
-    // otf_band(Q) frequencies each.
-    // (a mixed job that may fall back to FP64 keeps to the FP64 kernel's shorter bands)
-    const int band = p.opt.precision >= 1 && !p.opt.refine_fallback ? kOtfBandDf : otf_band(p.Q);
+    // Near corrections once per job (they depend on the target and N only); tasks of at most kOtfBand frequencies,
+    // which the kernels of every form take (a mixed job may fall back to FP64).
+    const int band = kOtfBand;
     p.wn_off.assign(p.asms.size(), -1);
     for (size_t a = 0; a < p.asms.size(); ++a) {
       const CrossAsm& t = p.asms[a];
