@@ -22,48 +22,6 @@ constexpr double kInvPi = 0.31830988618379067153776752674502872;
 constexpr double kTwoOverPi = 0.63661977236758134307553505349005745;
 constexpr double kSqrtHalf = 0.70710678118654752440084436210484904;
 constexpr double kBesselLarge = 20.0;
-constexpr double kSqrtTwoOverPi = 0.79788456080286535587989211986876373;
-
-// Terms (k = 0..kmax of P, k = 0..kmax of Q/w) of Hankel's expansion needed at z >= 20: the first
-// omitted terms a_{2kmax+2}/z^{2kmax+2} and a_{2kmax+3}/z^{2kmax+3} stay below 2^-54 from these
-// bounds on (below 24.2 the 9-term sum is the one checked against arbitrary-precision values).
-__device__ __forceinline__ int hankel_terms(float z) {
-  return z >= 467.f ? 2 : z >= 135.f ? 3 : z >= 67.7f ? 4 : z >= 44.2f ? 5 : z >= 33.5f ? 6 : z >= 27.7f ? 7
-       : z >= 24.2f ? 8 : 9;
-}
-
-// sin x and cos x for |x| <= 1 from their Taylor series (x^21/21! and x^22/22! < 2e-20 bound the
-// truncation), by Horner's rule in u = x^2 with the coefficients (-1)^k/(2k+1)! and (-1)^k/(2k)!.
-// Used for the per-pair phase step e^{i h R}, whose argument is small.
-__device__ __forceinline__ void sincos_taylor(double x, double& s, double& c) {
-  constexpr double f3 = 6.0, f5 = f3 * 20.0, f7 = f5 * 42.0, f9 = f7 * 72.0, f11 = f9 * 110.0,
-                   f13 = f11 * 156.0, f15 = f13 * 210.0, f17 = f15 * 272.0, f19 = f17 * 342.0;
-  constexpr double f2 = 2.0, f4 = f2 * 12.0, f6 = f4 * 30.0, f8 = f6 * 56.0, f10 = f8 * 90.0,
-                   f12 = f10 * 132.0, f14 = f12 * 182.0, f16 = f14 * 240.0, f18 = f16 * 306.0,
-                   f20 = f18 * 380.0;
-  const double u = x * x;
-  double ps = -1.0 / f19;
-  ps = fma(ps, u, 1.0 / f17);
-  ps = fma(ps, u, -1.0 / f15);
-  ps = fma(ps, u, 1.0 / f13);
-  ps = fma(ps, u, -1.0 / f11);
-  ps = fma(ps, u, 1.0 / f9);
-  ps = fma(ps, u, -1.0 / f7);
-  ps = fma(ps, u, 1.0 / f5);
-  ps = fma(ps, u, -1.0 / f3);
-  s = fma(x * u, ps, x);
-  double pc = 1.0 / f20;
-  pc = fma(pc, u, -1.0 / f18);
-  pc = fma(pc, u, 1.0 / f16);
-  pc = fma(pc, u, -1.0 / f14);
-  pc = fma(pc, u, 1.0 / f12);
-  pc = fma(pc, u, -1.0 / f10);
-  pc = fma(pc, u, 1.0 / f8);
-  pc = fma(pc, u, -1.0 / f6);
-  pc = fma(pc, u, 1.0 / f4);
-  pc = fma(pc, u, -1.0 / f2);
-  c = fma(u, pc, 1.0);
-}
 
 // Hankel coefficients a_k (filled by init_constants(); this header is included by one translation
 // unit only).
@@ -130,29 +88,6 @@ __device__ __forceinline__ Bessel0 bessel0(double z) {
     b.has_yhat = false;
   }
   return b;
-}
-
-// Full kernel Phi = (i/4) H0^(1)(z) = (-Y0/4, J0/4) for z > 0.
-__device__ __forceinline__ double2 phi_kernel(double z) {
-  Bessel0 b = bessel0(z);
-  double y0 = b.has_yhat ? fma(kTwoOverPi * (log(0.5 * z) + kEulerGamma), b.j0, b.y) : b.y;
-  return make_double2(-0.25 * y0, 0.25 * b.j0);
-}
-
-// Log-split pieces at a pair with parameter distance dts = |t - s| > 0 and z = kappa R:
-//   K1 = -J0/(2 pi),  K2 = K - K1 ln|t - s|
-//      = (i/4) J0 - (J0/(2 pi)) [ln(z/(2|t-s|)) + gamma] - Yhat0/4   (z < 20)
-//      = (i/4) J0 - Y0/4 + (J0/(2 pi)) ln|t-s|                       (z >= 20)
-__device__ __forceinline__ void log_split(double z, double dts, double& K1, double2& K2) {
-  Bessel0 b = bessel0(z);
-  K1 = -0.5 * kInvPi * b.j0;
-  double re;
-  if (b.has_yhat) {
-    re = fma(K1, log(z / (2.0 * dts)) + kEulerGamma, -0.25 * b.y);
-  } else {
-    re = fma(-K1, log(dts), -0.25 * b.y);
-  }
-  K2 = make_double2(re, 0.25 * b.j0);
 }
 
 }  // namespace fthms

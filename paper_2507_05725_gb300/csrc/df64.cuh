@@ -202,136 +202,6 @@ __device__ __forceinline__ void cdf_mac(dfacc& re, dfacc& im, float4 a, float4 b
   im.mac(a.z, a.w, b.x, b.y);
 }
 
-}  // namespace fthms
-
-namespace fthms {
-
-// sqrt(a) for a > 0 in double-float: the FP32 root r corrected once by Newton's step with the exact
-// residual a - r^2 (two-product), error about 2^-46.
-__device__ __forceinline__ df df_sqrt(df a) {
-  const float r = sqrtf(a.hi);
-  const float p = __fmul_rn(r, r);
-  const float pe = fmaf(r, r, -p);                    // r^2 = p + pe exactly
-  const float d = __fadd_rn(__fadd_rn(__fsub_rn(a.hi, p), a.lo), -pe);
-  df out;
-  quick_two_sum(r, __fdiv_rn(d, __fmul_rn(2.f, r)), out.hi, out.lo);
-  return out;
-}
-
-// 1 / sqrt(a) for a > 0 in double-float: y = rsqrt(a.hi) refined by one Newton step y (3 - a y^2) / 2
-// with the product in double-float, error about 2^-46.
-__device__ __forceinline__ df df_rsqrt(df a) {
-  const float y = rsqrtf(a.hi);
-  const df y2 = df_mul(df{y, 0.f}, df{y, 0.f});
-  const df e = df_sub(df{1.f, 0.f}, df_mul(a, y2));   // 1 - a y^2, small
-  df out;
-  quick_two_sum(y, __fmul_rn(__fmul_rn(0.5f, y), e.hi), out.hi, out.lo);
-  return out;
-}
-
-
-// a ~ hi + lo for a double a with 2^-60 <= |a| < 2^100 by integer operations only (no FP64 instruction):
-// hi = a truncated to 24 significant bits, lo = the 29 fraction bits below them rounded to 24 bits (one
-// integer-to-float conversion, its exponent then shifted by that of a), so |a - hi - lo| <= 2^-47 |a|.
-// Outside that range (zero included) the FP64 conversions.
-__device__ __forceinline__ void split_f64_bits(double a, float& hi, float& lo) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(a);
-  const unsigned int uh = (unsigned int)(u >> 32), ul = (unsigned int)u;
-  const int e = (int)((uh >> 20) & 0x7FFu);                   // biased FP64 exponent
-  if (e < 1023 - 60 || e > 1023 + 100) {
-    hi = __double2float_rn(a);
-    lo = __double2float_rn(a - (double)hi);
-    return;
-  }
-  const unsigned int sign = uh & 0x80000000u;
-  const unsigned int frac23 = __funnelshift_l(ul, uh, 3) & 0x007FFFFFu;   // the top 23 fraction bits
-  hi = __uint_as_float(sign | ((unsigned int)(e - 1023 + 127) << 23) | frac23);
-  const unsigned int rem = ul & 0x1FFFFFFFu;                  // the 29 fraction bits below: rem 2^(e - 1075)
-  const float r = __uint2float_rn(rem);
-  lo = rem ? __uint_as_float(sign | (__float_as_uint(r) + ((unsigned int)(e - 1075) << 23))) : 0.f;
-}
-
-// acc += a * b for a = ah + al (double-float) and b a float: the exact error of ah b by the FMA
-// two-product, al b added to the low word.
-__device__ __forceinline__ void dfacc_mac1(dfacc& acc, float ah, float al, float b) {
-  const float p = __fmul_rn(ah, b);
-  float e = fmaf(ah, b, -p);
-  e = fmaf(al, b, e);
-  float s, t;
-  two_sum(acc.hi, p, s, t);
-  acc.hi = s;
-  acc.lo = __fadd_rn(acc.lo, __fadd_rn(t, e));
-}
-
-// a = a1 + a2 + a3 exactly for a double a with 2^-60 <= |a| < 2^100, by integer operations only: a1 = a truncated
-// to 24 significant bits, a2 = the next 24 bits, a3 = the last 5 (integers below 2^24 convert to float exactly,
-// then their exponents are shifted by that of a).  Outside that range (zero included; |a| below 2^128) by FP64
-// operations.
-__device__ __forceinline__ void split3_f64_bits(double a, float& a1, float& a2, float& a3) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(a);
-  const unsigned int uh = (unsigned int)(u >> 32), ul = (unsigned int)u;
-  const int e = (int)((uh >> 20) & 0x7FFu);
-  if (e < 1023 - 60 || e > 1023 + 100) {
-    a1 = __double2float_rn(a);
-    const double r = a - (double)a1;
-    a2 = __double2float_rn(r);
-    a3 = __double2float_rn(r - (double)a2);
-    return;
-  }
-  const unsigned int sign = uh & 0x80000000u;
-  a1 = __uint_as_float(sign | ((unsigned int)(e - 1023 + 127) << 23) | (__funnelshift_l(ul, uh, 3) & 0x007FFFFFu));
-  const unsigned int rem = ul & 0x1FFFFFFFu;            // the 29 fraction bits below a1: rem 2^(e - 1075)
-  const unsigned int top = rem >> 5, low = rem & 31u;
-  a2 = top ? __uint_as_float(sign | (__float_as_uint(__uint2float_rn(top)) + ((unsigned int)(e - 1070) << 23))) : 0.f;
-  a3 = low ? __uint_as_float(sign | (__float_as_uint(__uint2float_rn(low)) + ((unsigned int)(e - 1075) << 23))) : 0.f;
-}
-
-// Anchored sums of products a x (a = a1 + a2 + a3 the exact three-float split, x a float) on the FP32 pipe,
-// by error-free extraction against fixed power-of-two anchors (the "ExtractScalar" step of Rump, Ogita and
-// Oishi's accurate summation, 2008).  With every partial sum of |a x| below 2^(kh-1), H starts at
-// 1.5 2^kh and stays in [2^kh, 2^(kh+1)]: t = H + p1 and q = t - H are exact (Sterbenz), and p1 - q is the
-// exact part of p1 below H's ulp (Fast2Sum, |H| >= |p1|).  Those parts, the product errors e1 (FMA
-// two-product) and a2 x go the same way into M, anchored at 1.5 2^km (km = kh - 23 + ceil(log2(T + 4)) for
-// T terms, so M too stays in its binade); a2 x through one FMA (M + a2 x rounded once, then the exact
-// q and the rest a2 x - q rounded once more, ~2^(km-47)).  What falls below M's ulp, and a3 x, are added
-// plainly in l, which renorm() folds back into M.  18 FP32 instructions a product instead of the 34 that
-// exact three-level two-sums take; the error, about 2^-50 of the sum of |a x| (the anchors' scale), is of
-// the order of an FP64 accumulation's.
-struct aacc {
-  float H, M, l, sh, sm;
-  __device__ __forceinline__ void init(int kh, int km) {     // -126 < km < kh < 128
-    H = sh = __uint_as_float(((unsigned)(127 + kh) << 23) | 0x400000u);   // 1.5 2^kh
-    M = sm = __uint_as_float(((unsigned)(127 + km) << 23) | 0x400000u);
-    l = 0.f;
-  }
-  __device__ __forceinline__ void put_m(float v) {      // |v| <= |M| / 2: exact split into M's grid and l
-    const float t = __fadd_rn(M, v);
-    l = __fadd_rn(l, __fsub_rn(v, __fsub_rn(t, M)));
-    M = t;
-  }
-  __device__ __forceinline__ void add_prod(float a1, float a2, float a3, float x) {
-    const float p1 = __fmul_rn(a1, x), e1 = fmaf(a1, x, -p1);
-    const float t = __fadd_rn(H, p1);
-    const float r1 = __fsub_rn(p1, __fsub_rn(t, H));
-    H = t;
-    put_m(r1);
-    put_m(e1);
-    const float u = fmaf(a2, x, M);
-    const float q = __fsub_rn(u, M);
-    l = __fadd_rn(l, fmaf(a2, x, -q));
-    M = u;
-    l = fmaf(a3, x, l);
-  }
-  __device__ __forceinline__ void renorm() {       // l's high part into M (exact), keeping l small
-    const float t = __fadd_rn(M, l);
-    l = __fsub_rn(l, __fsub_rn(t, M));
-    M = t;
-  }
-  __device__ __forceinline__ double value() const {
-    return ((double)__fsub_rn(H, sh) + (double)__fsub_rn(M, sm)) + (double)l;
-  }
-};
-
 // Two floats in one register pair: one instruction per operation on both (the FP32 pipe's rate is the same, the issue
 // slots are half).
 typedef unsigned long long f32x2;

@@ -72,8 +72,8 @@ __device__ __forceinline__ double dist_f64(double R2) {
   return fma(fma(-r, r, R2), hy, r);
 }
 
-// hi + lo ~ a to 2^-47 by integer operations and selects alone (split_f64_bits without its FP64 branch, whose
-// instructions occupy the FP64 pipe even when no lane takes them): below FP32's normal range zero, above it NaN.
+// hi + lo ~ a to 2^-47 by integer operations and selects alone (an FP64 branch for the rare ranges would occupy the
+// FP64 pipe even when no lane takes it: 10 of its slots a pair): below FP32's normal range zero, above it NaN.
 __device__ __forceinline__ df df_split_bits(double a) {
   const unsigned uh = (unsigned)__double2hiint(a), ul = (unsigned)__double2loint(a);
   const int e = (int)((uh >> 20) & 0x7FFu);
