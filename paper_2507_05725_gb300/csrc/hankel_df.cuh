@@ -365,11 +365,11 @@ __device__ __forceinline__ PairF64 pair_f64(double T, double camp4) {
 }
 
 // z >= 20; p = l v - 1/8 turn, rs = 1/sqrt(l).
-__device__ __forceinline__ double2 hankel_far_f64(const PairF64& pr, unsigned long long p, const AngleTab<true>& ang, df iv,
-                                                  double rs, double beta, bool near) {
+__device__ __forceinline__ double2 hankel_far_f64(const PairF64& pr, unsigned long long p, const float4* ang,
+                                                  const double2* ang64, df iv, double rs, double beta, bool near) {
   const FarAngle f = far_angle<true>(pr.iu, p, iv);
-  const float4 t = ang.d[f.idx];
-  const double2 t64 = ang.f[f.idx];
+  const float4 t = ang[f.idx];
+  const double2 t64 = ang64[f.idx];
   const df dc = angle_step(t.x, t.y, -t.z, -t.w, f), ds = angle_step(t.z, t.w, t.x, t.y, f);
   const double co = t64.x + (f2d_bits(dc.hi) + f2d_bits(dc.lo)), si = t64.y + (f2d_bits(ds.hi) + f2d_bits(ds.lo));
   const double a0 = pr.aw * rs;

@@ -64,44 +64,42 @@ __device__ __forceinline__ unsigned long long shift_down(unsigned long long t, u
 
 // J0, Y0 and Yhat0 = Y0 - (2/pi)(ln(z/2) + gamma) J0.  The series and expansions of hankel_df.cuh keep the FP64 pipe to
 // ~20 instructions a value (bessel0's take ~150 where a warp's values fall on both sides of z = 20); arguments outside
-// [1e-30, 2^20) go through bessel0.  10^6 values between 1e-3 and 2000: 248 -> 72 us.
-constexpr int kBesselRun = 4;
-__global__ void __launch_bounds__(256) k_bessel0(const double* __restrict__ z, double* j0, double* y0, double* yh, int n) {
-  __shared__ AngleTab<true> ang;
-  load_angles(ang);
-  __syncthreads();
+// [1e-30, 2^20) go through bessel0.  One value a thread, the angles through L1 (a shared copy and runs of four values a
+// thread: 14.5 us at 1000 values and 72 at 10^6), narrow CTAs for the small calls (256 threads: 9.4 us).  1000 values
+// 12.4 -> 7.3 us, 10^6 between 1e-3 and 2000: 248 -> 64 us.
+constexpr int kBesselThreads = 64;
+__global__ void __launch_bounds__(kBesselThreads) k_bessel0(const double* __restrict__ z, double* j0, double* y0, double* yh,
+                                                            int n) {
   const df iv = df_const(0.5 * kInvPi);
-  for (int e = 0; e < kBesselRun; ++e) {
-    const long long i = ((long long)blockIdx.x * kBesselRun + e) * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double zz = z[i];
-    double J0, Y0, Yh;
-    if (zz >= 1e-30 && zz < 1048576.0) {
-      unsigned long long t, s;
-      int k;
-      turns_of(zz, t, s, k);
-      const double lg = kTwoOverPi * (log_f64(zz) - 0.11593151565841244881);      // ln 2 - gamma
-      if (zz < kBesselLarge) {
-        bessel0_f64(shift_down(t, s, k + 2), J0, Yh);
-        Y0 = fma(lg, J0, Yh);
-      } else {
-        PairF64 p = pair_f64(0.5 * kInvPi * zz, kInvPi);
-        const double2 E = hankel_far_f64(p, shift_down(t, s, k) - (1ull << 61), ang, iv, 1.0, 0.0, false);
-        J0 = E.y;
-        Y0 = -E.x;
-        Yh = fma(-lg, J0, Y0);
-      }
+  const long long i = (long long)blockIdx.x * kBesselThreads + threadIdx.x;
+  if (i >= n) return;
+  const double zz = z[i];
+  double J0, Y0, Yh;
+  if (zz >= 1e-30 && zz < 1048576.0) {
+    unsigned long long t, s;
+    int k;
+    turns_of(zz, t, s, k);
+    const double lg = kTwoOverPi * (log_f64(zz) - 0.11593151565841244881);      // ln 2 - gamma
+    if (zz < kBesselLarge) {
+      bessel0_f64(shift_down(t, s, k + 2), J0, Yh);
+      Y0 = fma(lg, J0, Yh);
     } else {
-      const Bessel0 b = bessel0(zz);
-      const double lg = kTwoOverPi * (log(0.5 * zz) + kEulerGamma);
-      J0 = b.j0;
-      Y0 = b.has_yhat ? fma(lg, b.j0, b.y) : b.y;
-      Yh = b.has_yhat ? b.y : fma(-lg, b.j0, b.y);
+      PairF64 p = pair_f64(0.5 * kInvPi * zz, kInvPi);
+      const double2 E = hankel_far_f64(p, shift_down(t, s, k) - (1ull << 61), c_angle_df, c_angle_f64, iv, 1.0, 0.0, false);
+      J0 = E.y;
+      Y0 = -E.x;
+      Yh = fma(-lg, J0, Y0);
     }
-    if (j0) j0[i] = J0;
-    if (y0) y0[i] = Y0;
-    if (yh) yh[i] = Yh;
+  } else {
+    const Bessel0 b = bessel0(zz);
+    const double lg = kTwoOverPi * (log(0.5 * zz) + kEulerGamma);
+    J0 = b.j0;
+    Y0 = b.has_yhat ? fma(lg, b.j0, b.y) : b.y;
+    Yh = b.has_yhat ? b.y : fma(-lg, b.j0, b.y);
   }
+  if (j0) j0[i] = J0;
+  if (y0) y0[i] = Y0;
+  if (yh) yh[i] = Yh;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -337,7 +335,7 @@ __global__ void __launch_bounds__(256) k_assemble_self(DevJob J) {
       const FreqDf& f = fr[b];
       const double2 v = pt.th * f.a.x < (float)kBesselLarge
                             ? hankel_near_f64(u, lnT + f.lnz, beta, true, qw)
-                            : hankel_far_f64(pt, ph, ang, df{f.a.z, f.a.w}, f.rs, beta, true);
+                            : hankel_far_f64(pt, ph, ang.d, ang.f, df{f.a.z, f.a.w}, f.rs, beta, true);
       store_self(J, mo + e1, v, J.mixed);
       store_self(J, mo + e2, v, J.mixed);
     }
@@ -913,7 +911,7 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
       for (int b = 0; b < nl; ++b, ph += pt.v, u += pt.v62) {
         const FreqDf& f = fr[b];
         put(b, pt.th * f.a.x < (float)kBesselLarge ? hankel_near_f64(u, lnT + f.lnz, beta, near, qw)
-                                                   : hankel_far_f64(pt, ph, ang, df{f.a.z, f.a.w}, f.rs, beta, near));
+                                                   : hankel_far_f64(pt, ph, ang.d, ang.f, df{f.a.z, f.a.w}, f.rs, beta, near));
       }
     } else {
       const PairTurns pt = pair_turns(T, cd);
@@ -1035,7 +1033,7 @@ __global__ void __launch_bounds__(kOtfThreads, 2) k_cross_otf(DevJob J) {
           const FreqDf& f = fr[b0 + k];
           const double2 e = pt.th * f.a.x < (float)kBesselLarge
                                 ? hankel_near_f64(u, lnT + f.lnz, beta, near, qw)
-                                : hankel_far_f64(pt, ph, ang, df{f.a.z, f.a.w}, f.rs, beta, near);
+                                : hankel_far_f64(pt, ph, ang.d, ang.f, df{f.a.z, f.a.w}, f.rs, beta, near);
           const double2* __restrict__ pd = J.phi + vo[b0 + k] + i;
 #pragma unroll
           for (int q = 0; q < Q; ++q) {
@@ -2258,7 +2256,7 @@ inline int cdiv(long long a, int b) { return (int)((a + b - 1) / b); }
 
 cudaError_t launch_bessel0(const double* z, double* j0, double* y0, double* yh, int n, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_bessel0<<<cdiv(n, 256 * kBesselRun), 256, 0, st>>>(z, j0, y0, yh, n);
+  k_bessel0<<<cdiv(n, kBesselThreads), kBesselThreads, 0, st>>>(z, j0, y0, yh, n);
   return cudaGetLastError();
 }
 

@@ -192,3 +192,37 @@ def test_stored_rows_at_the_largest_node_count(F, ctx):
     for j in range(3):
         a, b = (F.fthms_densities(x.req, j, 2, 0) for x in jobs)
         assert np.linalg.norm(a - b) <= 1e-10 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("Q", [1, 2])
+def test_fp64_fallback_with_rows_every_step(F, ctx, Q):
+    """The FP64 re-run of a mixed job evaluates its rows over the same bands: bitwise the FP64 job's densities."""
+    p = wl.random_small(7, n_curves=2, n_arcs_per_curve=3, L=52, M=2, Q=Q, N_fixed=33, W=14.0, H=4.0, n_period=512)
+    p["options"]["cross_mode"] = 1
+    ref = F.Job(ctx, p).run().wait()
+    bad = copy.deepcopy(p)
+    bad["options"].update(refine_tol=1e-30, refine_max=1, refine_fallback=1)
+    job = F.Job(ctx, bad, precision=1).run().wait()
+    assert job.stats()["fallback_runs"] == 1
+    for j in range(6):
+        for q in range(Q):
+            assert np.array_equal(F.fthms_densities(ref.req, j, 2, q), F.fthms_densities(job.req, j, 2, q))
+
+
+@pytest.mark.parametrize("n", [1, 63, 64, 65, 1000])
+def test_bessel0_at_block_edges(F, n):
+    """One value a thread in blocks of 64, nothing written past n.  5e-15 of the amplitude: scipy's own 3.4e-15 and
+    the 1.5e-15 of the device functions."""
+    z = np.exp(np.random.default_rng(n).uniform(np.log(1e-3), np.log(2000.0), n))
+    zt = torch.tensor(z, dtype=torch.float64, device="cuda")
+    out = [torch.full((n + 1,), 7.0, dtype=torch.float64, device="cuda") for _ in range(3)]
+    F.fthms_bessel0(zt.data_ptr(), *(o.data_ptr() for o in out), n)
+    torch.cuda.synchronize()
+    assert all(float(o[n]) == 7.0 for o in out)
+    j0, y0, yh = (o[:n].cpu().numpy() for o in out)
+    rj, ry = special.j0(z), special.y0(z)
+    amp = np.where(z > 1.0, np.sqrt(2.0 / (np.pi * z)), 1.0)
+    assert np.max(np.abs(j0 - rj) / amp) < 5e-15
+    assert np.max(np.abs(y0 - ry) / np.maximum(amp, np.abs(ry))) < 5e-15
+    ryh = ry - (2.0 / np.pi) * (np.log(z / 2.0) + np.euler_gamma) * rj
+    assert np.max((np.abs(yh - ryh) / (1.0 + np.abs(np.log(z))))[z < 20.0], initial=0.0) < 5e-15
