@@ -62,10 +62,6 @@ def _hbm_peak_gbs():
 
 HBM_PEAK_GBS = _hbm_peak_gbs()
 FP64_PEAK_GFLOPS = 152 * 4 * 2.07  # 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz max SM clock
-# Algorithmic FP64 flops of one stored kernel entry: one far-field Hankel step at four asymptotic terms, the
-# most common count at this workload (4 + 4 Horner FMAs, 1/z and 1/z^2, the amplitude, the two components,
-# the phase rotation).
-FLOPS_PER_KERNEL_ENTRY = 34
 
 
 def kernels_hash():
@@ -367,11 +363,11 @@ def stage_rooflines(r, problem, stored_rows):
     hbm = f"peak: measured copy bandwidth ({PEAK_NOTE})"
     fp64 = "peak: FP64 pipe derived from the unit counts and clock: 152 SMs x 4 flop/clk x 2.07 GHz"
     if stored_rows:
-        name = "k_cross_rows_df" if prec >= 1 else "k_cross_apply"
+        name = "k_cross_rows"
         by = 16.0 * st["cross_entries"] * M
         tr = tpu[name] * st["cross_entries"] * M if name in tpu else None
         add("cross_apply", name, "hbm", by, HBM_PEAK_GBS, "GB/s",
-            f"every stored cross entry (16 B) read once per step{', then an ordered per-group reduce (~1% of the stage)' if prec else ''}; {hbm}",
+            f"every stored cross entry (16 B of fixed point) read once per step, then an ordered per-group reduce (~1% of the stage); {hbm}",
             traffic=tr, launches=M)
     if prec >= 1:
         solve_units = sum_n2 * M * (1.0 + passes)
@@ -379,19 +375,18 @@ def stage_rooflines(r, problem, stored_rows):
             f"the FP32 factor (8 B per entry) read once per solve pass, 1 + {passes:.3f} passes per system and step; {hbm}",
             traffic=tpu["k_msolve"] * solve_units if "k_msolve" in tpu else None)
         if prec == 2:
-            add("resid", "k_mresid64", "hbm", 16.0 * sum_n2 * M, HBM_PEAK_GBS, "GB/s",
-                f"first-pass residual to FP64 accuracy: the FP64 matrix (16 B per entry) read once per step; a "
-                f"sixth of the rows on the FP64 pipe (8 DFMA per entry, two windows), the rest in anchored sums of "
-                f"exact products on the FP32 pipe; {hbm}", traffic=tpu["k_mresid64"] * sum_n2 * M if "k_mresid64" in tpu else None)
-            upd_units = sum_n2 * M * max(passes - 1.0, 0.0)
-            add("resid_upd", "k_mresid_upd", "hbm", 16.0 * upd_units, HBM_PEAK_GBS,
-                "GB/s", f"later-pass residual updates: the FP64 matrix (16 B per entry) read once per pass, "
-                        f"{max(passes - 1.0, 0.0):.3f} passes per system and step; {hbm}",
-                traffic=tpu["k_mresid_upd"] * upd_units if "k_mresid_upd" in tpu else None)
-        else:
             add("resid", "k_mresid", "hbm", 16.0 * sum_n2 * M, HBM_PEAK_GBS, "GB/s",
+                f"first-pass residual: the kept matrix in 56-bit fixed point (16 B per entry) read once per step, exact "
+                f"integer sums; {hbm}", traffic=tpu["k_mresid"] * sum_n2 * M if "k_mresid" in tpu else None)
+            upd_units = sum_n2 * M * max(passes - 1.0, 0.0)
+            add("resid_upd", "k_mresid", "hbm", 16.0 * upd_units, HBM_PEAK_GBS,
+                "GB/s", f"later-pass residual updates: the kept matrix (16 B per entry) read once per pass, "
+                        f"{max(passes - 1.0, 0.0):.3f} passes per system and step; {hbm}",
+                traffic=tpu["k_mresid"] * upd_units if "k_mresid" in tpu else None)
+        else:
+            add("resid", "k_mresid_df", "hbm", 16.0 * sum_n2 * M, HBM_PEAK_GBS, "GB/s",
                 f"first-pass double-float residual: the kept matrix (16 B per entry) read once; {hbm}")
-            add("resid_upd", "k_mresid", "hbm", 16.0 * sum_n2 * M * max(passes - 1.0, 0.0), HBM_PEAK_GBS, "GB/s",
+            add("resid_upd", "k_mresid_df", "hbm", 16.0 * sum_n2 * M * max(passes - 1.0, 0.0), HBM_PEAK_GBS, "GB/s",
                 f"later-pass residuals: the kept matrix read once per pass; {hbm}")
         if st.get("lu_tensor_systems", 0) > 0:
             add("lu_update", "k_lu_big_update", "tensor", lu_update_flops(problem, st["lu_tensor_systems"]),
@@ -400,10 +395,6 @@ def stage_rooflines(r, problem, stored_rows):
                 f"per panel); peak: TF32 dense = measured bf16 sustained x 1.1/2.25 ({PEAK_NOTE})")
     else:
         add("solve", "k_solve", "alu", st["solve_flops"], FP64_PEAK_GFLOPS, "GFLOP/s", fp64)
-        add("lu", "k_lu<double2>", "alu", st["lu_flops"], FP64_PEAK_GFLOPS, "GFLOP/s", "(8/3) sum N^3; " + fp64)
-        if stored_rows:
-            add("cross_assemble", "k_cross_assemble", "alu", FLOPS_PER_KERNEL_ENTRY * st["cross_entries"],
-                FP64_PEAK_GFLOPS, "GFLOP/s", "34-flop model of one far-field Hankel step per entry; " + fp64)
     return out
 
 

@@ -10,13 +10,13 @@ c3s: the 12-arc cavity (cross rows evaluated every step), M = 2, precision 1, as
 c4: the mixed-precision configuration (6 arcs of 5 ellipses) at N = 1024 on 64 frequencies of the same grid
     spacing (omega up to 25), M = 2, in the FP64-kept form with tensor-core LU (about 10 GB on the device:
     every kernel's data are far above L2); the launches of interest are k_lu_big_update, k_lu_big_panel,
-    k_mresid64, k_msolve and k_cross_otf_df.
+    k_mresid, k_msolve and k_cross_otf_df.
 c4s: the mixed-precision configuration at N = 512 on 128 frequencies of the same grid spacing (omega up to
     50), M = 2, cross rows evaluated every step, in the FP64-kept form with the bench's tuned shapes
     (tensor-core LU at N = 512): 768 systems, about 5 GB on the device; the launches of interest are k_lu_big_update, k_lu_big_panel,
-    k_msolve, k_mresid64 and k_cross_otf_df.
+    k_msolve, k_mresid and k_cross_otf_df.
 c4r: the same at N = 512 on 16 frequencies (omega up to 6.3), M = 2, stored cross rows (1.75 GB of them, far
-    above L2), FP64-kept form with the tuned shapes: the launch of interest is k_cross_rows_df.
+    above L2), FP64-kept form with the tuned shapes: the launch of interest is k_cross_rows.
 c4-launches: one full-size job of the mixed-precision configuration at N = 512 (1023 frequencies, M = 8,
     the bench's headline workload) in the FP64-kept form with the bench's tuned shapes and the tensor-core
     LU, for a launch list.
