@@ -174,13 +174,13 @@ __device__ __forceinline__ void bessel0_tayfine_df(df z, df& J0, df& Yh) {
 }
 
 // Angle and modulus at z >= 20: the table index, the residual angle x = xh + ... as sin x = xh + sx and
-// cos x - 1 = ch + cl, and 1 - m = mh + ml; p = l v - 1/8 turn.  kFine keeps the second-order terms in double-float
-// too (rho(0), kappa(0) as pairs): phase and modulus to 2^-52 instead of 2^-45 near z = 20.
+// cos x - 1 = ch + cl, and 1 - m = mh + ml; p = l v - 1/8 turn.  The second-order terms stay in
+// double-float (rho(0), kappa(0) as pairs): phase and modulus to 2^-52 near z = 20; in FP32 they reach 2^-45 there, which
+// ill-conditioned precision-1 jobs show (densities 1.2e-11 off instead of 7.4e-12) for 5% of the assembly's time.
 struct FarAngle {
   unsigned idx;
   float xh, sx, ch, cl, mh, ml;
 };
-template <bool kFine>
 __device__ __forceinline__ FarAngle far_angle(df iu, unsigned long long p, df iv) {
   FarAngle r;
   const df w = df_mul(iu, iv);
@@ -190,21 +190,13 @@ __device__ __forceinline__ FarAngle far_angle(df iu, unsigned long long p, df iv
   float rho = fmaf(sh, 109818.0144f, -4218.12863f);
   rho = fmaf(sh, rho, 187.743036f);
   rho = fmaf(sh, rho, -13.1045092f);
-  float gh, gl;
-  if (kFine) {
-    const float th = __fmul_rn(sh, kR.hi);                      // s rho(0)
-    const float tl = fmaf(sh, fmaf(sh, rho, kR.lo), fmaf(sl, kR.hi, fmaf(sh, kR.hi, -th)));
-    df c;
-    quick_two_sum(kG.hi, -th, c.hi, c.lo);
-    c.lo = __fadd_rn(c.lo, __fsub_rn(kG.lo, tl));
-    const df g = df_mul(df{sh, sl}, c);
-    gh = g.hi;
-    gl = g.lo;
-  } else {
-    const float gc = fmaf(-sh, fmaf(sh, rho, kR.hi), kG.lo);
-    gh = __fmul_rn(sh, kG.hi);
-    gl = fmaf(sh, gc, fmaf(sl, kG.hi, fmaf(sh, kG.hi, -gh)));
-  }
+  const float th = __fmul_rn(sh, kR.hi);                        // s rho(0)
+  const float tl = fmaf(sh, fmaf(sh, rho, kR.lo), fmaf(sl, kR.hi, fmaf(sh, kR.hi, -th)));
+  df c;
+  quick_two_sum(kG.hi, -th, c.hi, c.lo);
+  c.lo = __fadd_rn(c.lo, __fsub_rn(kG.lo, tl));
+  const df g = df_mul(df{sh, sl}, c);
+  const float gh = g.hi, gl = g.lo;
   // phi = -w/8 + (w/8) g = -q + (ah + al)
   const float qh = 0.125f * w.hi, ql = 0.125f * w.lo;
   const float ah = __fmul_rn(qh, gh), al = fmaf(ql, gh, fmaf(qh, gl, fmaf(qh, gh, -ah)));
@@ -236,15 +228,11 @@ __device__ __forceinline__ FarAngle far_angle(df iu, unsigned long long p, df iv
   kap = fmaf(sh, kap, 5.84762562f);
   kap = fmaf(sh, kap, -0.542846348f);
   r.mh = 0.0625f * sh;
-  if (kFine) {
-    const float t = __fmul_rn(sh, sh), tl = fmaf(2.f * sh, sl, fmaf(sh, sh, -t));
-    const float kh = __fmul_rn(t, kK.hi);
-    const float kl = fmaf(t, fmaf(sh, kap, kK.lo), fmaf(tl, kK.hi, fmaf(t, kK.hi, -kh)));
-    quick_two_sum(r.mh, -kh, r.mh, r.ml);
-    r.ml = __fadd_rn(r.ml, fmaf(0.0625f, sl, -kl));
-  } else {
-    r.ml = fmaf(-__fmul_rn(sh, sh), fmaf(sh, kap, kK.hi), 0.0625f * sl);
-  }
+  const float t = __fmul_rn(sh, sh), te = fmaf(2.f * sh, sl, fmaf(sh, sh, -t));
+  const float kh = __fmul_rn(t, kK.hi);
+  const float kl = fmaf(t, fmaf(sh, kap, kK.lo), fmaf(te, kK.hi, fmaf(t, kK.hi, -kh)));
+  quick_two_sum(r.mh, -kh, r.mh, r.ml);
+  r.ml = __fadd_rn(r.ml, fmaf(0.0625f, sl, -kl));
   return r;
 }
 
@@ -263,7 +251,7 @@ __device__ __forceinline__ df angle_step(float ah, float al, float bh, float bl,
 // Entry E = (amp (beta cos - sin), amp cos) at z >= 20; ang: the angle table (shared memory).
 __device__ __forceinline__ float4 hankel_far_df(const PairTurns& pr, unsigned long long p, const float4* ang, df iv,
                                                 df rs, df beta, bool near) {
-  const FarAngle f = far_angle<false>(pr.iu, p, iv);
+  const FarAngle f = far_angle(pr.iu, p, iv);
   const float4 t = ang[f.idx];
   const df dc = angle_step(t.x, t.y, -t.z, -t.w, f), ds = angle_step(t.z, t.w, t.x, t.y, f);
   df co, si;
@@ -367,7 +355,7 @@ __device__ __forceinline__ PairF64 pair_f64(double T, double camp4) {
 // z >= 20; p = l v - 1/8 turn, rs = 1/sqrt(l).
 __device__ __forceinline__ double2 hankel_far_f64(const PairF64& pr, unsigned long long p, const float4* ang,
                                                   const double2* ang64, df iv, double rs, double beta, bool near) {
-  const FarAngle f = far_angle<true>(pr.iu, p, iv);
+  const FarAngle f = far_angle(pr.iu, p, iv);
   const float4 t = ang[f.idx];
   const double2 t64 = ang64[f.idx];
   const df dc = angle_step(t.x, t.y, -t.z, -t.w, f), ds = angle_step(t.z, t.w, t.x, t.y, f);

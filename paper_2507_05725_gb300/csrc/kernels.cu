@@ -496,9 +496,10 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
 }
 
 // Threads per system: the panel's columns are one warp's work, so an FP64 system below about a hundred nodes, whose
-// shared memory lets six share an SM, runs faster on fewer (768 systems of N = 96: 1.73 -> 1.47 ms at 128 threads).
+// shared memory lets six share an SM, runs faster on fewer (768 systems of N = 96: 1.73 -> 1.47 ms at 128 threads).  The
+// FP32 form fits 48 registers, five CTAs an SM (8192 systems of N 48..259: three 5.53 ms, four 4.63, five 4.22).
 template <class C, int NT>
-__global__ void __launch_bounds__(NT, sizeof(C) == sizeof(double2) ? 768 / NT : 1) k_lu(DevJob J) {
+__global__ void __launch_bounds__(NT, sizeof(C) == sizeof(double2) ? 768 / NT : 5) k_lu(DevJob J) {
   extern __shared__ __align__(16) unsigned char shl_raw[];
   lu_one<C, NT>(J, J.lu_small[blockIdx.x], shl_raw);
 }
@@ -823,13 +824,12 @@ __device__ void near_beta_block(const CrossTgt* tg, int nrows, int N, const doub
 }
 
 // kNear: the launch over the tasks with near rows (shared memory for their corrections); otherwise over the far-only
-// tasks, which need only the tables (more CTAs per SM).  Each launch skips the other kind of task.  kForm: 0 the FP64
-// form, 1 the mixed form (double-float entries), 2 the FP64-kept form (double-float, FP64 below z = 20).  A thread
-// owns (row, source) pairs and walks the band's frequencies.  Bound by the FP64 pipe in form 0 (9 instructions an entry,
-// ~25 a pair; 8 obstacle arcs, 4.8e8 entries: 33.2 -> 11.7 ms), by FP32 issue in forms 1 and 2 (~130 instructions;
-// 10.7 -> 4.2 ms; N = 512 with 2.6e9 entries: 29.3 -> 14.1 ms).
-constexpr int kFormF64 = 0, kFormMixed = 1, kFormKeep = 2;
-template <bool kNear, int kForm>
+// tasks, which need only the tables (more CTAs per SM).  Each launch skips the other kind of task.  kF64: the FP64 form;
+// else the mixed forms (FP64 below z = 20, double-float above).  A thread owns (row, source) pairs and walks the
+// band's frequencies.  Bound by the FP64 pipe in the FP64 form (9 instructions an entry, ~25 a pair; 8 obstacle arcs,
+// 4.8e8 entries: 34 -> 12.4 ms), by FP32 issue in the mixed forms (~135 instructions; 12 -> 5.3 ms; N = 512 with 2.6e9
+// entries: 29.3 -> 17.1 ms).
+template <bool kNear, bool kF64>
 __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
   extern __shared__ __align__(16) double sha[];
   const CrossAsm task = J.asms[blockIdx.x];
@@ -842,7 +842,7 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
   double* bt = sha + kAsmBand * (sizeof(FreqDf) / sizeof(double));   // near launch: kAsmRows x N corrections,
   double* lam = bt + kAsmRows * N;                   // kAsmRows x N and
   double* ctab = lam + kAsmRows * N;                 // 2N + 1 doubles of near_beta_block
-  __shared__ AngleTab<kForm == kFormF64> ang;
+  __shared__ AngleTab<kF64> ang;
   __shared__ int any_near;
   __shared__ unsigned s_r2[kAsmRows], s_beta[kAsmRows];   // smallest R^2, largest |beta| of a row (FP32 bits)
   __shared__ short s_exp[kAsmRows][kAsmBand];             // entries of (row, frequency) stay below 2^s_exp
@@ -887,7 +887,7 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
                                                                    : __uint_as_float(0x7FFFFFFFu);
   }
   __syncthreads();
-  const df qd = df_from(qw), cd = df_from(camp4);
+  const df cd = df_from(camp4);
   const int ld = pr.nrows;   // blocks are stored source-major: E[i * nrows + row]
   const long long* eo = J.e_off + (long long)task.pair * J.L + task.l0;
   for (int e = threadIdx.x; e < task.nrows * N; e += blockDim.x) {
@@ -903,7 +903,7 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
       const int2 x = fix_f64(v.x, s), y = fix_f64(v.y, s);
       Ep[eo[b]] = make_int4(x.x, x.y, y.x, y.y);
     };
-    if constexpr (kForm == kFormF64) {
+    if constexpr (kF64) {
       const PairF64 pt = pair_f64(T, camp4);
       const double lnT = pt.th * fr[0].a.x < (float)kBesselLarge ? log_f64(T) : 0.0;
       unsigned long long ph = pt.v * (unsigned long long)task.l0 - (1ull << 61),
@@ -916,30 +916,20 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
     } else {
       const PairTurns pt = pair_turns(T, cd);
       const df bd = kNear ? df_split_bits(beta) : df{0.f, 0.f};
-      df lnT{0.f, 0.f};
-      double lnT64 = 0.0;
+      double lnT = 0.0;
       unsigned long long v62 = 0ull;
       if (pt.T.hi * fr[0].a.x < (float)kBesselLarge) {
-        if (kForm == kFormKeep) {
-          lnT64 = log_f64(T);
-          v62 = turn_fraction(0.25 * T);
-        } else {
-          lnT = df_log(pt.T);
-        }
+        lnT = log_f64(T);
+        v62 = turn_fraction(0.25 * T);
       }
       unsigned long long ph = pt.v * (unsigned long long)task.l0 - (1ull << 61);
       for (int b = 0; b < nl; ++b, ph += pt.v) {
         const FreqDf& f = fr[b];
-        float4 d;
         if (pt.T.hi * f.a.x < (float)kBesselLarge) {
-          if (kForm == kFormKeep) {
-            put(b, hankel_near_f64(v62 * (unsigned long long)(task.l0 + b), lnT64 + f.lnz, beta, near, qw));
-            continue;
-          }
-          d = hankel_near_df(df_mul(pt.T, df{f.a.x, f.a.y}), df_add_fast(lnT, df{f.b.z, f.b.w}), bd, near, qd);
-        } else {
-          d = hankel_far_df(pt, ph, ang.d, df{f.a.z, f.a.w}, df{f.b.x, f.b.y}, bd, near);
+          put(b, hankel_near_f64(v62 * (unsigned long long)(task.l0 + b), lnT + f.lnz, beta, near, qw));
+          continue;
         }
+        const float4 d = hankel_far_df(pt, ph, ang.d, df{f.a.z, f.a.w}, df{f.b.x, f.b.y}, bd, near);
         const float c = __uint_as_float((unsigned)(27 - s_exp[r][b] + 127) << 23);
         const int2 x = fix_df(d.x, d.y, c), y = fix_df(d.z, d.w, c);
         Ep[eo[b]] = make_int4(x.x, x.y, y.x, y.y);
@@ -2381,7 +2371,7 @@ cudaError_t launch_cross_assemble(const DevJob& J, cudaStream_t st, int* launche
   const size_t sh = sh_far + (size_t)((2 * kAsmRows + 2) * J.max_n + 1) * sizeof(double);
   const int nt = J.shape_asm > 0 ? J.shape_asm : kAsmThreads;
   auto go = [&](auto form) {
-    constexpr int F = decltype(form)::value;
+    constexpr bool F = decltype(form)::value;
     cudaError_t e = cudaFuncSetAttribute(k_cross_assemble<true, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
     if (e != cudaSuccess) return e;
     k_cross_assemble<true, F><<<J.n_asm, nt, sh, st>>>(J);
@@ -2389,8 +2379,7 @@ cudaError_t launch_cross_assemble(const DevJob& J, cudaStream_t st, int* launche
     return cudaGetLastError();
   };
   *launches += 2;
-  return !J.mixed ? go(std::integral_constant<int, kFormF64>{}) : J.fp64keep ? go(std::integral_constant<int, kFormKeep>{})
-                                                               : go(std::integral_constant<int, kFormMixed>{});
+  return J.mixed ? go(std::false_type{}) : go(std::true_type{});
 }
 
 // one window's K/2 complex points and the samples
