@@ -10,7 +10,7 @@
 //            phi = -(w/8)(1 - s (25/48 - s rho(s))), m = 1 - s/16 + s^2 kappa(s), s = w^2 (the leading terms of
 //            DLMF 10.18.17-18), rho and kappa polynomials fitted to the exact modulus and phase on s <= 1/400 at 60
 //            digits (their fit errors enter below 2^-52 of the result).
-// About 125 FP32-pipe instructions an entry above z = 20 against ~225 of the rotated P + iQ recurrence this
+// About 135 FP32-pipe instructions an entry above z = 20 against ~225 of the rotated P + iQ recurrence this
 // replaces, and the set-up per pair needs no sine or cosine, so short bands cost no more per entry than long ones.
 #pragma once
 #include <cuda_runtime.h>

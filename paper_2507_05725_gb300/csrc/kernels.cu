@@ -1052,8 +1052,8 @@ __global__ void __launch_bounds__(kOtfThreads, 2) k_cross_otf(DevJob J) {
 // once per block of frequencies.  Entries never leave registers.  An earlier form wrote them to shared memory and
 // summed with one thread per (row, frequency): at bands of one or two frequencies (N grows with every step of omega)
 // 8 to 16 of its 128 threads worked, and each pair paid two sine/cosine series; 12-arc cavity, 5.7e8 pairs x 5 steps,
-// four windows: 501 -> 91 ms; 6 arcs at N = 1024, two windows:
-// 499 -> 335 ms.  Bound by FP32 issue (~125 instructions an entry and 48 a window).
+// four windows: 501 -> 89 ms; 6 arcs at N = 1024, two windows: 499 -> 329 ms.  Bound by FP32 issue (~135 instructions
+// an entry and 24 to 48 a window).
 // kKeep64 (the FP64-kept form): entries below z = 20 in FP64.
 __host__ __device__ constexpr int otf_regs(int Q) { return Q == 1 ? 8 : Q == 2 ? 4 : 1; }
 // blocks per SM: 16 warps of 128 registers, or 24 of 80 where the few sums leave room (measured per Q)
