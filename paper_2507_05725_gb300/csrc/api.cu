@@ -730,6 +730,14 @@ static fthms_status wait_run(fthms_req* req, int timeout_ms) {
   }
 }
 
+// Why a mixed-form job cannot run again in FP64 (nullptr: it can).
+static const char* no_fallback(const fthms_req* req) {
+  if (req->plan.ranks > 1) return "a frequency-partitioned job never falls back alone: its ranks would stop meeting in the all-reduce";
+  if (req->plan.maxN > kLuSmallMax) return "a system exceeds the FP64 form's N <= 800";
+  if (!req->plain_apply_fits) return "the stored cross rows exceed its apply";
+  return nullptr;
+}
+
 // After a finished run of a mixed-form job: read how many (system, step) refinements stayed above
 // refine_tol; with refine_fallback the whole job runs again in FP64 (every stage, on the job's stream).
 static fthms_status check_convergence(fthms_req* req) {
@@ -754,8 +762,8 @@ static fthms_status check_convergence(fthms_req* req) {
                      cudaMemcpyDeviceToHost, req->stream));
   CK(cudaStreamSynchronize(req->stream));
   if (bad == 0) return FTHMS_OK;
-  // (a frequency-partitioned job never falls back alone: its ranks would stop meeting in the all-reduce)
-  if (req->plan.opt.refine_fallback && req->plain_apply_fits && req->plan.ranks <= 1) {
+  const char* why_not = no_fallback(req);
+  if (req->plan.opt.refine_fallback && !why_not) {
     req->J.mixed = 0;
     req->J.fp64keep = 0;
     if (req->graph) {                  // the captured graph holds the mixed-form kernels
@@ -768,10 +776,11 @@ static fthms_status check_convergence(fthms_req* req) {
     req->conv_checked = true;
     return FTHMS_OK;
   }
-  char buf[200];
+  char buf[320];
+  const bool asked = req->plan.opt.refine_fallback && why_not;
   snprintf(buf, sizeof buf, "fthms_wait: %llu (system, step) refinements stayed above refine_tol = %.3g after %d "
-           "passes%s", bad, req->plan.opt.refine_tol, req->plan.opt.refine_max,
-           req->plan.opt.refine_fallback ? " (no FP64 fallback: the stored cross rows exceed its apply)" : "");
+           "passes%s%s%s", bad, req->plan.opt.refine_tol, req->plan.opt.refine_max, asked ? " (no FP64 fallback: " : "",
+           asked ? why_not : "", asked ? ")" : "");
   req->conv_status = FTHMS_ENOCONV;
   req->conv_msg = buf;
   g_last_error = buf;

@@ -499,9 +499,9 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
 // shared memory lets six share an SM, runs faster on fewer (768 systems of N = 96: 1.73 -> 1.47 ms at 128 threads).  The
 // FP32 form fits 48 registers, five CTAs an SM (8192 systems of N 48..259: three 5.53 ms, four 4.63, five 4.22).
 template <class C, int NT>
-__global__ void __launch_bounds__(NT, sizeof(C) == sizeof(double2) ? 768 / NT : 5) k_lu(DevJob J) {
+__global__ void __launch_bounds__(NT, sizeof(C) == sizeof(double2) ? 768 / NT : 5) k_lu(DevJob J, const int* __restrict__ list) {
   extern __shared__ __align__(16) unsigned char shl_raw[];
-  lu_one<C, NT>(J, J.lu_small[blockIdx.x], shl_raw);
+  lu_one<C, NT>(J, list[blockIdx.x], shl_raw);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2315,19 +2315,20 @@ cudaError_t launch_lu_small(const DevJob& J, cudaStream_t st, int* launches) {
       size_t sh = lu_smem<float2>(small_max);
       cudaError_t e = cudaFuncSetAttribute(k_lu<float2, kLuThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
       if (e != cudaSuccess) return e;
-      k_lu<float2, kLuThreads><<<J.n_lu_small, kLuThreads, sh, st>>>(J);
+      k_lu<float2, kLuThreads><<<J.n_lu_small, kLuThreads, sh, st>>>(J, J.lu_small);
       *launches += 1;
       return cudaGetLastError();
     }
     return cudaSuccess;
   }
-  if (J.n_lu_small == 0) return cudaSuccess;
+  // FP64: every system, whatever the split of the mixed form (a job that falls back keeps its split)
+  if (J.nsys == 0) return cudaSuccess;
   const size_t sh = lu_smem<double2>(J.max_n);
   auto go = [&](auto nt) {
     constexpr int NT = decltype(nt)::value;
     cudaError_t e = cudaFuncSetAttribute(k_lu<double2, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
     if (e != cudaSuccess) return e;
-    k_lu<double2, NT><<<J.n_lu_small, NT, sh, st>>>(J);
+    k_lu<double2, NT><<<J.nsys, NT, sh, st>>>(J, J.sys_order);
     return cudaGetLastError();
   };
   *launches += 1;

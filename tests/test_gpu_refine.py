@@ -114,6 +114,47 @@ def test_fp64_fallback_replaces_unconverged_results(F, ctx):
     job.release()
 
 
+@pytest.mark.parametrize("precision,otf", [(1, 0), (2, 0), (1, 1)])
+def test_fp64_fallback_factors_the_systems_of_the_tensor_core_lu(F, ctx, precision, otf):
+    """The FP64 re-run factors every system, also those that the mixed run gave to the tensor-core LU (launch shape:
+    N >= 256): bitwise the FP64 job, whether all systems (N = 300) or some of them (N above and below 256) took it; a
+    second run of the same job, and one after the shapes are set again, give the same."""
+    for fixed in (300, 0):
+        p = wl.random_small(5, n_curves=1, n_arcs_per_curve=3, L=6, M=2, N_fixed=fixed, W=30.0, H=0.5, n_period=64)
+        if not fixed:
+            p["options"].update(N_ppw=5.0, N_off=40)
+        p["options"]["cross_mode"] = otf
+        ref = F.Job(ctx, p).run().wait()
+        N = [d.size for d in ref.densities(0, 2, 0).values()]
+        assert max(N) >= 256 and max(N) <= 800 and (fixed or min(N) < 256)
+        bad = copy.deepcopy(p)
+        bad["options"].update(refine_tol=1e-30, refine_max=1, refine_fallback=1, shapes=[0, 0, 0, 0, 256])
+        job = F.Job(ctx, bad, precision=precision).run().wait()
+        for again in range(3):
+            assert job.stats()["fallback_runs"] == 1
+            assert np.array_equal(job.traces(), ref.traces())
+            for j in range(3):
+                assert np.array_equal(F.fthms_densities(ref.req, j, 2, 0), F.fthms_densities(job.req, j, 2, 0))
+            if again == 1:
+                F.fthms_set_shapes(job.req, [0, 0, 0, 0, 256])
+            job.run().wait()
+        ref.release()
+        job.release()
+
+
+def test_no_fp64_fallback_above_its_largest_system(F, ctx):
+    """A mixed job with systems above N = 800, which the FP64 form does not take: FTHMS_ENOCONV names the reason, and
+    the mixed results stay readable."""
+    p = wl.random_small(2, n_arcs_per_curve=3, L=4, M=1, N_fixed=801, W=24.0, H=0.3, n_period=64, kind=1)
+    p["options"].update(refine_tol=1e-30, refine_max=1, refine_fallback=1)
+    job = F.Job(ctx, p, precision=2).run()
+    with pytest.raises(F.FthmsError) as e:
+        job.wait()
+    assert e.value.status == F.FTHMS_ENOCONV and "800" in str(e.value)
+    assert job.stats()["fallback_runs"] == 0 and np.all(np.isfinite(F.fthms_densities(job.req, 0, 1, 0)))
+    job.release()
+
+
 def test_tighter_refinement_tolerance_is_met(F, ctx):
     """refine_tol = 1e-14 with up to 6 passes: more passes per system, every estimate below the target and
     the densities closer to the FP64 oracle than the default form's bar."""
