@@ -9,22 +9,27 @@
 
 namespace fthms {
 
-constexpr int kFixBits = 55;            // |X| < 2^55
+// v = (x 2^kLow + y) 2^(s - kFixBits) for |v| < 2^s, |x| and |y| <= 2^(kLow - 1), rounded to the last place.
+__host__ __device__ constexpr int fix_bits(int low) { return 2 * low - 1; }   // |X| < 2^fix_bits
+constexpr int kFixLow = 28;             // cross rows and refinement residuals (sums of any length, with carries)
+constexpr int kFixBits = fix_bits(kFixLow);
+constexpr int kLuLow = 30;              // LU updates (sums of eight products)
 
-// v = (x 2^28 + y) 2^(s - 55) for |v| < 2^s, |x| <= 2^27, |y| <= 2^27, rounded to the last place.
+template <int kLow = kFixLow>
 __device__ __forceinline__ int2 fix_split(long long X) {
-  const int x = (int)((X + (1ll << 27)) >> 28);
-  return make_int2(x, (int)(X - ((long long)x << 28)));
+  const int x = (int)((X + (1ll << (kLow - 1))) >> kLow);
+  return make_int2(x, (int)(X - ((long long)x << kLow)));
 }
+template <int kLow = kFixLow>
 __device__ __forceinline__ int2 fix_f64(double v, int s) {
   const unsigned h = (unsigned)__double2hiint(v);
   const int e = (int)((h >> 20) & 0x7FFu);
   unsigned long long m = ((unsigned long long)((h & 0xFFFFFu) | 0x100000u) << 32) | (unsigned)__double2loint(v);
-  const int sh = e - 1075 + kFixBits - s;               // <= 2
+  const int sh = e - 1075 + fix_bits(kLow) - s;         // <= fix_bits - 53
   if (e == 0 || sh < -60) m = 0ull;
   else if (sh >= 0) m <<= min(sh, 8);
   else m = (m + (1ull << (-sh - 1))) >> -sh;
-  return fix_split((h >> 31) ? -(long long)m : (long long)m);
+  return fix_split<kLow>((h >> 31) ? -(long long)m : (long long)m);
 }
 // The same for a double-float value (c = 2^(27 - s)).
 __device__ __forceinline__ int2 fix_df(float hi, float lo, float c) {
@@ -67,26 +72,38 @@ __device__ __forceinline__ void fix_vector(const double2* v, int N, double scale
                        : scale * __hiloint2double((e - 1022 - kFixBits + 1023) << 20, 0);
 }
 
-// Exact sum of products (the products of two low halves, below 2^-56 of the bounds' product, are dropped); at most
-// kFixRun products between carries (one adds below 2^55 to either running sum).
+// Sum of products, exact but for the products of two low halves (below 2^-kFixBits of the bounds' product each), which are
+// dropped; at most kFixRun products between carries (one adds below 2^55 to either running sum).
 constexpr int kFixRun = 64;
-struct fixacc {
-  long long a = 0, b = 0, c = 0;          // high products, cross products (2^28 below), carries (2^32 above)
+template <int kLow>
+struct fixacc_low {
+  long long a = 0, b = 0, c = 0;          // high products, cross products (2^kLow below), carries (2^32 above)
   __device__ __forceinline__ void mac(int x0, int x1, int y0, int y1) {
     a += (long long)x0 * y0;
     b += (long long)x0 * y1;
     b += (long long)x1 * y0;
   }
   __device__ __forceinline__ void carry() {
-    a += b >> 28;
-    b &= 0xFFFFFFFll;
+    a += b >> kLow;
+    b &= (1ll << kLow) - 1;
     c += a >> 32;
     a &= 0xFFFFFFFFll;
   }
-  __device__ __forceinline__ double value() {           // in units of 2^56
+  __device__ __forceinline__ double value() {           // in units of 2^(2 kLow)
     carry();
-    return fma((double)c, 4294967296.0, (double)a + 0x1p-28 * (double)b);
+    return fma((double)c, 4294967296.0, (double)a + (1.0 / (1ll << kLow)) * (double)b);
   }
+  // A short sum without carries, to the nearest of the same units.  (Cut instead of rounded, every panel of a
+  // factorisation moves an entry the same way: 2e-14 of the matrix at N = 400 where FP64 gives 3.5e-15.)
+  __device__ __forceinline__ long long nearest() const { return a + ((b + (1ll << (kLow - 1))) >> kLow); }
 };
+using fixacc = fixacc_low<kFixLow>;
+
+// LU updates: multipliers below 2 and a column of U12 below 2^e, eight complex products a sum.  |l| <= sqrt(2) (partial
+// pivoting on |re| + |im|), so with 2^29 for either half's bound a sum stays below 8 x 3 x 2^58 < 2^63 and needs no
+// carry.  The unit of a sum: 2^(2 kLuLow) 2^(1 - bits) 2^(e - bits); NaN for a column that is not finite.
+__device__ __forceinline__ double lu_unit(int e) {
+  return e > 1000 ? __longlong_as_double(0x7FF8000000000000ll) : __hiloint2double((e + 3 - 2 * kLuLow + 1023) << 20, 0);
+}
 
 }  // namespace fthms

@@ -355,9 +355,12 @@ constexpr int kLuNarrow = 135;   // FP64 jobs of systems up to this size: 128 th
 //
 // FP64 trailing update in fixed point (fixed.cuh): A22 -= L21 U12 took 32 FP64 FMAs an entry and panel, the whole FP64
 // pipe (75% of the kernel's time at its rate).  The multipliers are below 2 (partial pivoting on |re| + |im|) and a column
-// of U12 shares one unit, so both become 56-bit integers in the same shared memory, the eight products sum exactly in
-// integers and only the final conversion and subtraction are FP64: 6 instructions an entry and panel.  A thread takes
-// two columns of a row, so that each multiplier is read once for both.  8192 systems of N 48..259: 31.0 -> 16.6 ms.
+// of U12 shares one unit, so both become 60-bit integers in the same shared memory and the eight products sum in
+// integers (low x low halves dropped), rounded once to 2^-57 of the column's largest entry; only the final conversion
+// and subtraction are FP64: 6 instructions an entry and panel.  One FP64 rounding a panel in place of sixteen: |LU - PA|
+// over |A| at N = 400 2.7e-16 against 9.3e-16 of the FMAs (oracle's self matrices), entry by entry 3.9e-16 against 1.3e-15
+// of |L||U|.  A thread takes two columns of a row, so that each multiplier is read once for both.  8192 systems of N
+// 48..259: 31.0 -> 16.6 ms.
 template <class C>
 __host__ __device__ constexpr size_t lu_smem(int N) {
   const size_t panel = (size_t)N * (kNB + kPS) * sizeof(C) + (sizeof(C) == sizeof(double2) ? (size_t)N * sizeof(double) : 0);
@@ -429,11 +432,10 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
           const int e = max((int)(top >> 20), 100) - 1022;
 #pragma unroll
           for (int r = 0; r < kNB; ++r) {
-            const int2 x = fix_f64(xv[r].x, e), y = fix_f64(xv[r].y, e);
+            const int2 x = fix_f64<kLuLow>(xv[r].x, e), y = fix_f64<kLuLow>(xv[r].y, e);
             reinterpret_cast<int4*>(U)[r * N + j] = make_int4(x.x, x.y, y.x, y.y);
           }
-          // unit of a product sum: 2^56 2^(1 - 55) 2^(e - 55)
-          unit[j] = e > 1000 ? __longlong_as_double(0x7FF8000000000000ll) : __hiloint2double((e - 53 + 1023) << 20, 0);
+          unit[j] = lu_unit(e);
         }
       }
       __syncthreads();
@@ -445,7 +447,7 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
         for (int idx = tid; idx < mr * kNB; idx += NT) {
           const int o = (idx / kNB) * kPS + idx % kNB;
           const C v = Pn[w * kPS + o];
-          const int2 x = fix_f64(v.x, 1), y = fix_f64(v.y, 1);
+          const int2 x = fix_f64<kLuLow>(v.x, 1), y = fix_f64<kLuLow>(v.y, 1);
           L[o] = make_int4(x.x, x.y, y.x, y.y);
         }
         __syncthreads();
@@ -455,7 +457,7 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
           C* a0 = A + (long long)(k0 + w + j0) * N + k0 + w + r;
           C* a1 = A + (long long)(k0 + w + j1) * N + k0 + w + r;
           C v0 = *a0, v1 = *a1;
-          fixacc re0, im0, re1, im1;
+          fixacc_low<kLuLow> re0, im0, re1, im1;
 #pragma unroll
           for (int c = 0; c < kNB; ++c) {
             const int4 l = L[r * kPS + c], p = Ui[c * N + j0], q = Ui[c * N + j1];
@@ -469,7 +471,7 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
             re1.mac(n0, n1, q.z, q.w);
             im1.mac(l.z, l.w, q.x, q.y);
           }
-          auto less = [](double v, double u, const fixacc& s) { return fma(-u, ll_to_double(s.a + (s.b >> 28)), v); };
+          auto less = [](double v, double u, const fixacc_low<kLuLow>& s) { return fma(-u, ll_to_double(s.nearest()), v); };
           const double u0 = unit[j0], u1 = unit[j1];
           v0 = make_double2(less(v0.x, u0, re0), less(v0.y, u0, im0));
           v1 = make_double2(less(v1.x, u1, re1), less(v1.y, u1, im1));

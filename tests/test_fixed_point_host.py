@@ -1,0 +1,168 @@
+"""The kernels' fixed-point arithmetic (csrc/fixed.cuh, csrc/cplx.cuh) compiled for the host and compared with the FP64
+arithmetic whose place it takes, both against quadruple precision."""
+import ctypes as ct
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import workloads as wl
+from oracle import geometry as geo
+from oracle import kernels as oker
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2507_05725_gb300", "csrc")
+
+SOURCE = r"""
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <utility>
+#include <vector>
+
+// the device intrinsics that the headers use
+static long long bits(double v) { long long u; std::memcpy(&u, &v, 8); return u; }
+static double dbl(long long u) { double v; std::memcpy(&v, &u, 8); return v; }
+static int __double2hiint(double v) { return (int)(bits(v) >> 32); }
+static int __double2loint(double v) { return (int)bits(v); }
+static double __hiloint2double(int h, int l) { return dbl(((long long)h << 32) | (unsigned)l); }
+static double __longlong_as_double(long long u) { return dbl(u); }
+static float __fmul_rn(float a, float b) { return a * b; }
+static float __fsub_rn(float a, float b) { return a - b; }
+static int __float2int_rn(float a) { return (int)std::nearbyintf(a); }
+static unsigned __reduce_max_sync(unsigned, unsigned m) { return m; }
+using std::max;
+using std::min;
+#include "cplx.cuh"
+#include "fixed.cuh"
+using namespace fthms;
+#ifdef __SIZEOF_FLOAT128__
+using quad = __float128;
+#else
+using quad = long double;   // (128 bits where there is no __float128)
+#endif
+
+// One factorisation as the one-CTA kernel makes it: panels of 8 columns in FP64 with partial pivoting, and the trailing
+// updates by FP64 FMAs (fixed = 0) or in fixed point.
+extern "C" void lu(double2* A, int* perm, int N, int fixed) {
+  auto at = [&](int r, int c) -> double2& { return A[(size_t)c * N + r]; };
+  for (int i = 0; i < N; ++i) perm[i] = i;
+  for (int k0 = 0; k0 < N; k0 += 8) {
+    const int w = min(8, N - k0), k1 = k0 + w;
+    for (int k = k0; k < k1; ++k) {
+      int p = k;
+      auto size = [&](int r) { return std::fabs(at(r, k).x) + std::fabs(at(r, k).y); };
+      for (int r = k + 1; r < N; ++r) if (size(r) > size(p)) p = r;
+      if (p != k) {
+        for (int j = 0; j < N; ++j) std::swap(at(k, j), at(p, j));
+        std::swap(perm[k], perm[p]);
+      }
+      const double2 inv = crecip(at(k, k));
+      for (int r = k + 1; r < N; ++r) {
+        const double2 l = at(r, k) = cmul(at(r, k), inv);
+        for (int c = k + 1; c < k1; ++c) at(r, c) = cfms(l, at(k, c), at(r, c));
+      }
+    }
+    std::vector<int4> L((size_t)8 * (N - k1));
+    for (int r = k1; r < N; ++r)
+      for (int c = 0; c < 8; ++c) {
+        const int2 x = fix_f64<kLuLow>(at(r, k0 + c).x, 1), y = fix_f64<kLuLow>(at(r, k0 + c).y, 1);
+        L[(size_t)8 * (r - k1) + c] = make_int4(x.x, x.y, y.x, y.y);
+      }
+    for (int j = k1; j < N; ++j) {
+      unsigned top = 0u;
+      for (int r = k0; r < k1; ++r) {
+        for (int c = k0; c < r; ++c) at(r, j) = cfms(at(r, c), at(c, j), at(r, j));
+        top = max(top, max(__double2hiint(at(r, j).x) & 0x7FFFFFFFu, __double2hiint(at(r, j).y) & 0x7FFFFFFFu));
+      }
+      const int e = max((int)(top >> 20), 100) - 1022;
+      int4 U[8];
+      for (int c = 0; c < 8; ++c) {
+        const int2 x = fix_f64<kLuLow>(at(k0 + c, j).x, e), y = fix_f64<kLuLow>(at(k0 + c, j).y, e);
+        U[c] = make_int4(x.x, x.y, y.x, y.y);
+      }
+      for (int r = k1; r < N; ++r) {
+        double2& v = at(r, j);
+        if (!fixed) {
+          for (int c = k0; c < k1; ++c) v = cfms(at(r, c), at(c, j), v);
+          continue;
+        }
+        fixacc_low<kLuLow> re, im;
+        for (int c = 0; c < 8; ++c) {
+          const int4 l = L[(size_t)8 * (r - k1) + c], p = U[c];
+          re.mac(l.x, l.y, p.x, p.y);
+          im.mac(l.x, l.y, p.z, p.w);
+          re.mac(-l.z, -l.w, p.z, p.w);
+          im.mac(l.z, l.w, p.x, p.y);
+        }
+        v.x = fma(-lu_unit(e), ll_to_double(re.nearest()), v.x);
+        v.y = fma(-lu_unit(e), ll_to_double(im.nearest()), v.y);
+      }
+    }
+  }
+}
+
+// P A - L U: Frobenius norm over |A|'s, largest entry over |L||U|'s, and the mean (re, im) over the mean |a|.
+extern "C" void lu_error(const double2* A, const double2* F, const int* perm, int N, double* out) {
+  double num = 0, den = 0, big = 0, re = 0, im = 0, sum = 0;
+  for (int j = 0; j < N; ++j)
+    for (int i = 0; i < N; ++i) {
+      quad x = 0, y = 0;
+      double size = 0;
+      for (int k = 0; k <= min(i, j); ++k) {
+        const double2 l = k == i ? make_double2(1, 0) : F[(size_t)k * N + i], u = F[(size_t)j * N + k];
+        x += (quad)l.x * u.x - (quad)l.y * u.y;
+        y += (quad)l.x * u.y + (quad)l.y * u.x;
+        size += std::hypot(l.x, l.y) * std::hypot(u.x, u.y);
+      }
+      const double2 a = A[(size_t)j * N + perm[i]];
+      const double dx = (double)(x - a.x), dy = (double)(y - a.y);
+      num += dx * dx + dy * dy;
+      den += a.x * a.x + a.y * a.y;
+      big = max(big, std::hypot(dx, dy) / size);
+      re += dx;
+      im += dy;
+      sum += std::hypot(a.x, a.y);
+    }
+  out[0] = std::sqrt(num / den);
+  out[1] = big;
+  out[2] = re / sum;
+  out[3] = im / sum;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("fixed")
+    src, so = d / "fixed.cpp", d / "fixed.so"
+    src.write_text(SOURCE)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-w", "-shared", "-fPIC", "-I", CSRC, "-I",
+                    os.path.join(cuda, "include"), str(src), "-o", str(so)], check=True)
+    return ct.CDLL(str(so))
+
+
+def _ptr(a):
+    return ct.c_void_p(a.ctypes.data)
+
+
+@pytest.mark.parametrize("N,kappa", [(17, 5.0), (48, 12.0), (136, 3.0), (136, 34.0), (259, 65.0)])
+def test_lu_updates_are_no_less_accurate_than_fp64(lib, N, kappa):
+    """Trailing updates of the FP64 LU on the oracle's self matrices.  One rounding to the column's unit and one FP64
+    rounding a panel take the place of sixteen FP64 roundings and the panels are the same, so the error may not exceed that
+    of the FMAs: in norm, entry by entry (a quarter more: a maximum over N^2 values), and without a direction (the
+    rounding is to the nearest: the mean error stays below a tenth of the error's own size)."""
+    A = np.asfortranarray(oker.self_matrix(geo.Arc(0, 0, wl.kite(0.1, 0.2), -1.3, 1.1), N, kappa).astype(complex))
+    err = []
+    for fixed in (0, 1):
+        F, perm, out = A.copy(order="F"), np.zeros(N, np.int32), np.zeros(4)
+        lib.lu(_ptr(F), _ptr(perm), N, fixed)
+        lib.lu_error(_ptr(A), _ptr(F), _ptr(perm), N, _ptr(out))
+        err.append(out)
+    fma, fix = err
+    assert fix[0] <= fma[0]
+    assert fix[1] <= 1.25 * fma[1]
+    assert max(abs(fix[2]), abs(fix[3])) <= 0.1 * fix[0]
