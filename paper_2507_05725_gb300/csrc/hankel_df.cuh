@@ -19,6 +19,7 @@
 #include <cmath>
 
 #include "bessel.cuh"
+#include "bits64.cuh"
 #include "df64.cuh"
 #include "kernels.h"
 
@@ -48,29 +49,12 @@ __device__ __forceinline__ FreqDf make_freq(int l) {
   return f;
 }
 
-// One pair: everything that its frequencies share.
+// One pair: everything that its frequencies share.  T = h R/(2 pi) carries no unit and lies in FP32's range (a pair below
+// 2^-126 turns is taken as z = 0 with the logarithm's FP64 value in the FP64 forms, above 2^127 it gives NaN).
 struct PairTurns {
   unsigned long long v;   // fraction of T in units of 2^-64 turns
   df T, iu, aw;           // T, 1/T, (w/(4 pi)) / sqrt(T)
 };
-
-__device__ __forceinline__ double f2d_bits(float f) {       // exact for normal f (zero gives 2^-127-ish)
-  const unsigned u = __float_as_uint(f);
-  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
-}
-__device__ __forceinline__ float d2f_trunc(double d) {      // a non-negative double in FP32's normal range, truncated
-  return __uint_as_float((((unsigned)__double2hiint(d) - 0x38000000u) << 3) | ((unsigned)__double2loint(d) >> 29));
-}
-
-// Distance in FP64 without the library's square root: the FP32 reciprocal root and two Newton steps on r^2 = R2
-// (relative error 2^-22 -> 2^-45 -> below 2^-53).
-__device__ __forceinline__ double dist_f64(double R2) {
-  const float y = rsqrtf(d2f_trunc(R2));
-  const double yd = f2d_bits(y), hy = f2d_bits(0.5f * y);
-  double r = R2 * yd;
-  r = fma(fma(-r, r, R2), hy, r);
-  return fma(fma(-r, r, R2), hy, r);
-}
 
 // hi + lo ~ a to 2^-47 by integer operations and selects alone (an FP64 branch for the rare ranges would occupy the
 // FP64 pipe even when no lane takes it: 10 of its slots a pair): below FP32's normal range zero, above it NaN.

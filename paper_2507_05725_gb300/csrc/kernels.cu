@@ -846,7 +846,7 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
   double* ctab = lam + kAsmRows * N;                 // 2N + 1 doubles of near_beta_block
   __shared__ AngleTab<kF64> ang;
   __shared__ int any_near;
-  __shared__ unsigned s_r2[kAsmRows], s_beta[kAsmRows];   // smallest R^2, largest |beta| of a row (FP32 bits)
+  __shared__ unsigned s_r2[kAsmRows], s_beta[kAsmRows];   // smallest R^2 (FP64 high word), largest |beta| of a row (FP32 bits)
   __shared__ short s_exp[kAsmRows][kAsmBand];             // entries of (row, frequency) stay below 2^s_exp
   if (threadIdx.x == 0) {
     int a = 0;
@@ -858,7 +858,7 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
   load_angles(ang);
   for (int b = threadIdx.x; b < nl; b += blockDim.x) fr[b] = J.freq_df[task.l0 + b];
   if (threadIdx.x < kAsmRows) {
-    s_r2[threadIdx.x] = 0x7F7FFFFFu;
+    s_r2[threadIdx.x] = 0x7FF00000u;
     s_beta[threadIdx.x] = 0u;
   }
   if (kNear) near_beta_block(tg, task.nrows, N, J.node_t + pn.off, ctab, lam, bt);
@@ -866,27 +866,27 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
   const double qw = 0.25 * kPiD / N, camp4 = qw * kInvPi, turns = J.h * (0.5 * kInvPi);
   // Fixed-point unit per row and frequency: |E| <= (w/4) |H0(z_min)| (1 + max |beta|), |H0(z)| <= sqrt(2/(pi z)) for
   // every z > 0 (z |H0|^2 increases to 2/pi), and <= 1.5 - 0.64 ln z below 1.  A row through a node, or with a
-  // coordinate that is not a number, gets the unit NaN, as its entries would be.
+  // distance that is not finite, gets the unit NaN, as its entries would be.
   for (int e = threadIdx.x; e < task.nrows * N; e += blockDim.x) {
     const int r = e % task.nrows, i = e / task.nrows;
     const double dx = tg[r].x - J.node_x[pn.off + i], dy = tg[r].y - J.node_y[pn.off + i];
-    const float R2 = (float)fma(dx, dx, dy * dy);
-    atomicMin(&s_r2[r], R2 > 0.f ? __float_as_uint(R2) : 0u);
+    const unsigned h = (unsigned)__double2hiint(fma(dx, dx, dy * dy));
+    atomicMin(&s_r2[r], h - 0x100000u < 0x7FE00000u ? h : 0u);      // normal and finite
     if (kNear && tg[r].near) atomicMax(&s_beta[r], __float_as_uint(fabsf((float)bt[r * N + i])));
   }
   __syncthreads();
   for (int e = threadIdx.x; e < task.nrows * nl; e += blockDim.x) {
     const int r = e / nl, b = e % nl;
-    const float T = (float)turns * sqrtf(__uint_as_float(s_r2[r])) * 0.99999f;
-    const float z = T * fr[b].a.x;
+    const double T = turns * dist_f64(__hiloint2double((int)s_r2[r], 0));
+    const float z = (float)T * fr[b].a.x * 0.99999f;
     float hb = sqrtf(0.63661978f / z);
-    if (z < 1.f) hb = fminf(hb, 1.5f - 0.64f * logf(z));
+    if (z < 1.f) hb = fminf(hb, 1.5f - 0.64f * ((float)(log_f64(T) + fr[b].lnz) + 0.1159f));   // (ln z, ln 2 - gamma)
     const float bound = (float)qw * hb * (1.f + __uint_as_float(s_beta[r])) * 1.0001f;
-    const int s = (int)(__float_as_uint(bound) >> 23) - 126;
+    const int s = max((int)(__float_as_uint(bound) >> 23) - 126, -64);
     s_exp[r][b] = (short)s;
     J.e_unit[J.row_off[(long long)task.pair * J.L + task.l0 + b] + task.row0 + r] =
-        s_r2[r] != 0u && s_r2[r] < 0x7F7FFFFFu && s > -60 && s < 120 ? __uint_as_float((unsigned)(s - kFixBits + 127) << 23)
-                                                                   : __uint_as_float(0x7FFFFFFFu);
+        s_r2[r] != 0u && z < 3e38f && s < 120 ? __uint_as_float((unsigned)(s - kFixBits + 127) << 23)
+                                              : __uint_as_float(0x7FFFFFFFu);
   }
   __syncthreads();
   const df cd = df_from(camp4);

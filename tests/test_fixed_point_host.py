@@ -1,5 +1,5 @@
-"""The kernels' fixed-point arithmetic (csrc/fixed.cuh, csrc/cplx.cuh) compiled for the host and compared with the FP64
-arithmetic whose place it takes, both against quadruple precision."""
+"""The kernels' fixed-point and bit arithmetic (csrc/fixed.cuh, csrc/bits64.cuh) compiled for the host and compared with the
+FP64 arithmetic whose place it takes, both against a higher precision."""
 import ctypes as ct
 import os
 import subprocess
@@ -31,10 +31,14 @@ static double __hiloint2double(int h, int l) { return dbl(((long long)h << 32) |
 static double __longlong_as_double(long long u) { return dbl(u); }
 static float __fmul_rn(float a, float b) { return a * b; }
 static float __fsub_rn(float a, float b) { return a - b; }
+static unsigned __float_as_uint(float v) { unsigned u; std::memcpy(&u, &v, 4); return u; }
+static float __uint_as_float(unsigned u) { float v; std::memcpy(&v, &u, 4); return v; }
+static float rsqrtf(float v) { return 1.f / std::sqrt(v); }
 static int __float2int_rn(float a) { return (int)std::nearbyintf(a); }
 static unsigned __reduce_max_sync(unsigned, unsigned m) { return m; }
 using std::max;
 using std::min;
+#include "bits64.cuh"
 #include "cplx.cuh"
 #include "fixed.cuh"
 using namespace fthms;
@@ -43,6 +47,10 @@ using quad = __float128;
 #else
 using quad = long double;   // (128 bits where there is no __float128)
 #endif
+
+extern "C" void dist(const double* R2, double* r, int n) {
+  for (int i = 0; i < n; ++i) r[i] = dist_f64(R2[i]);
+}
 
 // One factorisation as the one-CTA kernel makes it: panels of 8 columns in FP64 with partial pivoting, and the trailing
 // updates by FP64 FMAs (fixed = 0) or in fixed point.
@@ -166,3 +174,18 @@ def test_lu_updates_are_no_less_accurate_than_fp64(lib, N, kappa):
     assert fix[0] <= fma[0]
     assert fix[1] <= 1.25 * fma[1]
     assert max(abs(fix[2]), abs(fix[3])) <= 0.1 * fix[0]
+
+
+def test_distances_in_any_unit_of_length(lib):
+    """dist_f64 over the whole range of R^2: two Newton steps leave less than half a unit in the last place, the last
+    rounding adds half of one (2^-52 together); zero stays zero, and what is not a finite number gives none."""
+    rng = np.random.default_rng(3)
+    R2 = np.concatenate([np.exp2(rng.uniform(-1021.0, 1023.0, 20000)), np.exp2(rng.uniform(-60.0, 60.0, 5000)),
+                         np.exp2(np.arange(-1022.0, 1024.0)), np.nextafter(np.exp2(np.arange(-1021.0, 1024.0)), 0.0), [0.0]])
+    r = np.full_like(R2, np.nan)
+    lib.dist(_ptr(R2), _ptr(r), R2.size)
+    want = np.sqrt(R2.astype(np.longdouble))
+    assert np.all(np.abs(r - want) <= want * 2.0 ** -52)
+    bad, out = np.array([np.inf, np.nan, -1.0]), np.zeros(3)
+    lib.dist(_ptr(bad), _ptr(out), 3)
+    assert not np.any(np.isfinite(out[:2]))

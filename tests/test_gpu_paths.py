@@ -226,3 +226,48 @@ def test_bessel0_at_block_edges(F, n):
     assert np.max(np.abs(y0 - ry) / np.maximum(amp, np.abs(ry))) < 5e-15
     ryh = ry - (2.0 / np.pi) * (np.log(z / 2.0) + np.euler_gamma) * rj
     assert np.max((np.abs(yh - ryh) / (1.0 + np.abs(np.log(z))))[z < 20.0], initial=0.0) < 5e-15
+
+
+def _in_units(p, s):
+    """The same problem with lengths and times in units 1/s (s a power of two, so that every product is exact); the
+    amplitude goes the other way, which keeps amplitude x time, the densities' unit."""
+    p = copy.deepcopy(p)
+    for c in p["curves"]:
+        for k in ("ax", "bx", "ay", "by"):
+            c[k] = [s * v for v in c[k]]
+    g, o = p["signal"], p["options"]
+    g.update(z0=[s * v for v in g["z0"]], carrier=g["carrier"] / s, centre=g["centre"] * s, width=g["width"] * s,
+             amp=g["amp"] / s)
+    o.update(W=o["W"] / s, H=o["H"] * s, obs=s * o["obs"], tout0=s * o["tout0"], dtout=s * o["dtout"])
+    return p
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("bits", [-70, 70])
+def test_results_do_not_depend_on_the_unit_of_length(F, ctx, precision, mode, bits):
+    """Distances of 1e-21 and 1e21 (their squares leave FP32's range) with wavelengths to match: bit for bit the result
+    in units of one, near and far rows, below and above z = 20."""
+    p = wl.random_small(7, n_curves=2, n_arcs_per_curve=3, L=40, M=2, Q=2, W=14.0, H=4.0, n_period=512, kind=0)
+    p["options"]["cross_mode"] = mode
+    p["options"]["refine_max"] = 8
+    s = 2.0 ** bits
+    a, b = (F.Job(ctx, x, precision=precision).run().wait() for x in (p, _in_units(p, s)))
+    assert np.array_equal(a.traces(), s * b.traces()) and np.max(np.abs(a.traces())) > 0.0
+    for j in range(6):
+        for q in range(2):
+            assert np.array_equal(F.fthms_densities(a.req, j, 2, q), F.fthms_densities(b.req, j, 2, q))
+
+
+@pytest.mark.parametrize("bits", [-480, -320, -80, 80, 480])
+def test_self_matrix_does_not_depend_on_the_unit_of_length(F, bits):
+    curve, arc, N, kappa, s = wl.star(0.3, 5, 0.4), (0.1, 2.2), 47, 19.9, 2.0 ** bits
+    scaled = {k: [s * v for v in c] for k, c in curve.items()}
+    out = []
+    for c, k in ((curve, kappa), (scaled, kappa / s)):
+        for call in (F.fthms_assemble_self, F.fthms_assemble_self_noalloc):
+            A = torch.zeros(2 * N * N, dtype=torch.float64, device="cuda")
+            call(c, arc, N, k, A.data_ptr())
+            torch.cuda.synchronize()
+            out.append(A.cpu())
+    assert torch.equal(out[0], out[2]) and torch.equal(out[1], out[3]) and bool(torch.all(torch.isfinite(out[0])))
