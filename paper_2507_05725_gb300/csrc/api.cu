@@ -52,7 +52,7 @@ fthms_status ensure_device(int dev) {
   CK(cudaSetDevice(dev));
   std::lock_guard<std::mutex> lk(g_init_mu);
   if (dev >= 0 && dev < 64 && !g_init_done[dev]) {
-    CK(init_constants());
+    CK(init_constants(dev));
     // Job memory comes from the device's stream-ordered pool (cudaMallocAsync); keep what released
     // jobs free there for the next job instead of returning it to the driver at every synchronisation
     // (a per-process pool attribute; the HBM budget still admits jobs by its own accounting).

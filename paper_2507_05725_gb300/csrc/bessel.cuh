@@ -23,7 +23,7 @@ constexpr double kTwoOverPi = 0.63661977236758134307553505349005745;
 constexpr double kSqrtHalf = 0.70710678118654752440084436210484904;
 constexpr double kBesselLarge = 20.0;
 
-// Hankel coefficients a_k (filled by init_constants(); this header is included by one translation
+// Hankel coefficients a_k (filled by init_tables(); this header is included by one translation
 // unit only).
 __constant__ double c_hank_a[20];
 

@@ -17,6 +17,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 
 #include "bessel.cuh"
 #include "bits64.cuh"
@@ -382,8 +383,18 @@ __device__ __forceinline__ float4 split2_bits(double2 v) {
   return make_float4(a.hi, a.lo, b.hi, b.lo);
 }
 
-// Fills the tables above on the current device.
-inline cudaError_t init_hankel_df() {
+// Fills the tables above and bessel.cuh's on device dev (current), once: the first caller of any thread computes and
+// uploads them while the others wait, and returns when they are on the device (a stream of the caller's own does not wait
+// for the copies by itself).
+inline cudaError_t init_tables(int dev) {
+  static std::mutex mu;
+  static bool done[64];
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lk(mu);
+  if (done[dev]) return cudaSuccess;
+  double ha[20];
+  ha[0] = 1.0;
+  for (int k = 1; k < 20; ++k) ha[k] = ha[k - 1] * (double)((2 * k - 1) * (2 * k - 1)) / (8.0 * k);
   static float4 ang[kAngles], lg[128], tf[kTayFine][7];
   auto hi = [](double v) { return (float)v; };
   auto lo = [](double v) { return (float)(v - (double)(float)v); };
@@ -467,7 +478,11 @@ inline cudaError_t init_hankel_df() {
   if ((e = cudaMemcpyToSymbol(c_tay64, t64, sizeof t64)) != cudaSuccess) return e;
   if ((e = cudaMemcpyToSymbol(c_angle_df, ang, sizeof ang)) != cudaSuccess) return e;
   if ((e = cudaMemcpyToSymbol(c_log_df, lg, sizeof lg)) != cudaSuccess) return e;
-  return cudaMemcpyToSymbol(c_tayfine_df, tf, sizeof tf);
+  if ((e = cudaMemcpyToSymbol(c_tayfine_df, tf, sizeof tf)) != cudaSuccess) return e;
+  if ((e = cudaMemcpyToSymbol(c_hank_a, ha, sizeof ha)) != cudaSuccess) return e;
+  if ((e = cudaStreamSynchronize(nullptr)) != cudaSuccess) return e;
+  done[dev] = true;
+  return cudaSuccess;
 }
 
 }  // namespace fthms

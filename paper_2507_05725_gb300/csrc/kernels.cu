@@ -30,14 +30,7 @@
 
 namespace fthms {
 
-cudaError_t init_constants() {
-  double ha[20];
-  ha[0] = 1.0;
-  for (int k = 1; k < 20; ++k) ha[k] = ha[k - 1] * (double)((2 * k - 1) * (2 * k - 1)) / (8.0 * k);
-  cudaError_t e = cudaMemcpyToSymbol(c_hank_a, ha, sizeof ha);
-  if (e != cudaSuccess) return e;
-  return init_hankel_df();
-}
+cudaError_t init_constants(int dev) { return init_tables(dev); }
 
 namespace {
 

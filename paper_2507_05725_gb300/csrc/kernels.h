@@ -125,7 +125,7 @@ struct DevJob {
   long long vec_total;
 };
 
-cudaError_t init_constants();
+cudaError_t init_constants(int dev);
 
 // Sets the calling thread's message returned by fthms_last_error() (defined with the C ABI).
 void set_last_error(const char* msg);

@@ -46,7 +46,7 @@ fthms_status scratch_address(int dev, unsigned char** out) {
     void* p = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_scratch);
     if (e != cudaSuccess) return cuda_msg(e, "cudaGetSymbolAddress(no-alloc scratch)");
-    e = init_constants();
+    e = init_constants(dev);
     if (e != cudaSuccess) return cuda_msg(e, "init_constants");
     g_scratch_dev[dev] = static_cast<unsigned char*>(p);
   }

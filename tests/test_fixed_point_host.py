@@ -13,7 +13,7 @@ from oracle import kernels as oker
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2507_05725_gb300", "csrc")
 
-SOURCE = r"""
+SHIM = r"""
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -30,14 +30,26 @@ static int __double2loint(double v) { return (int)bits(v); }
 static double __hiloint2double(int h, int l) { return dbl(((long long)h << 32) | (unsigned)l); }
 static double __longlong_as_double(long long u) { return dbl(u); }
 static float __fmul_rn(float a, float b) { return a * b; }
+static float __fadd_rn(float a, float b) { return a + b; }
+static float __fdiv_rn(float a, float b) { return a / b; }
+static double rsqrt(double v) { return 1.0 / std::sqrt(v); }
+static long long __double_as_longlong(double v) { return bits(v); }
 static float __fsub_rn(float a, float b) { return a - b; }
 static unsigned __float_as_uint(float v) { unsigned u; std::memcpy(&u, &v, 4); return u; }
 static float __uint_as_float(unsigned u) { float v; std::memcpy(&v, &u, 4); return v; }
 static float rsqrtf(float v) { return 1.f / std::sqrt(v); }
+static float __double2float_rn(double v) { return (float)v; }
+static float __uint2float_rn(unsigned v) { return (float)v; }
+static unsigned __funnelshift_l(unsigned l, unsigned h, int k) { return (unsigned)(((((unsigned long long)h) << 32 | l) << k) >> 32); }
+template <class T> static T __ldg(const T* p) { return *p; }
+static uint3 threadIdx, blockDim;
 static int __float2int_rn(float a) { return (int)std::nearbyintf(a); }
 static unsigned __reduce_max_sync(unsigned, unsigned m) { return m; }
 using std::max;
 using std::min;
+"""
+
+SOURCE = SHIM + r"""
 #include "bits64.cuh"
 #include "cplx.cuh"
 #include "fixed.cuh"
@@ -142,15 +154,69 @@ extern "C" void lu_error(const double2* A, const double2* F, const int* perm, in
 """
 
 
+TABLES = SHIM + r"""
+#include <atomic>
+#include <thread>
+#include <unistd.h>
+
+#include "hankel_df.cuh"
+
+// A runtime that takes its time and counts the copies under way.
+static std::atomic<int> inside, most, to_device, waits;
+static void slow() {
+  const int n = ++inside;
+  for (int m = most; n > m && !most.compare_exchange_weak(m, n);) {}
+  usleep(2000);
+  --inside;
+}
+extern "C" cudaError_t cudaMemcpyToSymbol(const void* d, const void* s, size_t n, size_t, cudaMemcpyKind) {
+  slow();
+  ++to_device;
+  std::memcpy(const_cast<void*>(d), s, n);
+  return cudaSuccess;
+}
+extern "C" cudaError_t cudaMemcpyFromSymbol(void* d, const void* s, size_t n, size_t, cudaMemcpyKind) {
+  slow();
+  std::memcpy(d, s, n);
+  return cudaSuccess;
+}
+extern "C" cudaError_t cudaStreamSynchronize(cudaStream_t) { ++waits; return cudaSuccess; }
+
+// Four threads' first calls on a device, then a call on another one: copies at once, copies and waits after each part,
+// tables missing when a thread's call returned.
+extern "C" void first_calls(int* out) {
+  std::atomic<int> missing{0};
+  std::vector<std::thread> t;
+  for (int k = 0; k < 4; ++k)
+    t.emplace_back([&] {
+      if (fthms::init_tables(3) != cudaSuccess || fthms::c_hank_a[0] != 1.0 || fthms::c_angle_f64[0].x != 1.0 || waits == 0) ++missing;
+    });
+  for (auto& x : t) x.join();
+  out[0] = most;
+  out[1] = to_device;
+  out[2] = missing;
+  const int bad = fthms::init_tables(4) != cudaSuccess || fthms::init_tables(4) != cudaSuccess ||
+                  fthms::init_tables(-1) == cudaSuccess || fthms::init_tables(64) == cudaSuccess;
+  out[3] = to_device;
+  out[4] = bad;
+  out[5] = waits;
+}
+"""
+
+
+def _compile(tmp_path_factory, name, source):
+    d = tmp_path_factory.mktemp(name)
+    src, so = d / f"{name}.cpp", d / f"{name}.so"
+    src.write_text(source)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-w", "-pthread", "-shared", "-fPIC", "-Wl,-Bsymbolic",
+                    "-I", CSRC, "-I", os.path.join(cuda, "include"), str(src), "-o", str(so)], check=True)
+    return ct.CDLL(str(so))
+
+
 @pytest.fixture(scope="module")
 def lib(tmp_path_factory):
-    d = tmp_path_factory.mktemp("fixed")
-    src, so = d / "fixed.cpp", d / "fixed.so"
-    src.write_text(SOURCE)
-    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
-    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-w", "-shared", "-fPIC", "-I", CSRC, "-I",
-                    os.path.join(cuda, "include"), str(src), "-o", str(so)], check=True)
-    return ct.CDLL(str(so))
+    return _compile(tmp_path_factory, "fixed", SOURCE)
 
 
 def _ptr(a):
@@ -189,3 +255,13 @@ def test_distances_in_any_unit_of_length(lib):
     bad, out = np.array([np.inf, np.nan, -1.0]), np.zeros(3)
     lib.dist(_ptr(bad), _ptr(out), 3)
     assert not np.any(np.isfinite(out[:2]))
+
+
+def test_tables_are_filled_once_whoever_calls_first(tmp_path_factory):
+    """The tables of a device are computed and uploaded by one thread while the others' first calls wait for them, once
+    per device, and the upload is waited for."""
+    out = (ct.c_int * 6)()
+    _compile(tmp_path_factory, "tables", TABLES).first_calls(out)
+    at_once, copies, missing, copies2, bad, waits = out
+    assert at_once == 1 and missing == 0 and bad == 0
+    assert copies > 0 and copies2 == 2 * copies and waits == 2
