@@ -31,7 +31,7 @@ __constant__ double c_hank_a[20];
 // are entire), 13 terms each, coefficients from gen_bessel_taylor.py (mpmath).  Every lane runs the
 // same instruction stream (two 12-step Horner chains), whatever its interval.
 __device__ __forceinline__ void bessel0_taylor(double z, double& J0, double& Yh) {
-  const int k = min((int)(2.0 * z), kTaylorIntervals - 1);
+  const int k = min(max((int)(2.0 * z), 0), kTaylorIntervals - 1);   // (a negative z stays inside the table)
   const double d = z - fma(0.5, (double)k, 0.25);
   const double* cj = kTaylorJ0[k];
   const double* cy = kTaylorYh[k];

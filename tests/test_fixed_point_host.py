@@ -50,6 +50,16 @@ using std::min;
 """
 
 SOURCE = SHIM + r"""
+// (bessel.cuh reads its tables through this: the addresses are recorded, not read)
+static const double *g_low, *g_high;
+static double watched(const double* p) {
+  g_low = g_low ? min(g_low, p) : p;
+  g_high = max(g_high, p);
+  return 1.0;
+}
+#define __ldg watched
+#include "bessel.cuh"
+#undef __ldg
 #include "bits64.cuh"
 #include "cplx.cuh"
 #include "fixed.cuh"
@@ -62,6 +72,14 @@ using quad = long double;   // (128 bits where there is no __float128)
 
 extern "C" void dist(const double* R2, double* r, int n) {
   for (int i = 0; i < n; ++i) r[i] = dist_f64(R2[i]);
+}
+
+// Whether bessel0(z) reads inside its two tables (or nothing).
+extern "C" int taylor_reads_inside(double z) {
+  const double *a = &kTaylorJ0[0][0], *b = &kTaylorYh[0][0];
+  g_low = g_high = nullptr;
+  bessel0(z);
+  return !g_low || (g_low >= min(a, b) && g_high < max(a, b) + sizeof kTaylorJ0 / sizeof(double));
 }
 
 // One factorisation as the one-CTA kernel makes it: panels of 8 columns in FP64 with partial pivoting, and the trailing
@@ -265,3 +283,11 @@ def test_tables_are_filled_once_whoever_calls_first(tmp_path_factory):
     at_once, copies, missing, copies2, bad, waits = out
     assert at_once == 1 and missing == 0 and bad == 0
     assert copies > 0 and copies2 == 2 * copies and waits == 2
+
+
+@pytest.mark.parametrize("z", [0.0, 19.999, -0.3, -0.6, -7.0, -1e9, -np.inf, np.inf, np.nan])
+def test_bessel_tables_are_read_inside_whatever_the_argument(lib, z):
+    """fthms_bessel0 asks for z > 0, but an argument on the device cannot be refused: it must not lead outside the
+    tables."""
+    lib.taylor_reads_inside.argtypes = [ct.c_double]
+    assert lib.taylor_reads_inside(z)
