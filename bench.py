@@ -376,7 +376,7 @@ def stage_rooflines(r, problem, stored_rows):
             traffic=tpu["k_msolve"] * solve_units if "k_msolve" in tpu else None)
         if prec == 2:
             add("resid", "k_mresid", "hbm", 16.0 * sum_n2 * M, HBM_PEAK_GBS, "GB/s",
-                f"first-pass residual: the kept matrix in 56-bit fixed point (16 B per entry) read once per step, exact "
+                f"first-pass residual: the kept matrix in 60-bit fixed point (16 B per entry) read once per step, exact "
                 f"integer sums; {hbm}", traffic=tpu["k_mresid"] * sum_n2 * M if "k_mresid" in tpu else None)
             upd_units = sum_n2 * M * max(passes - 1.0, 0.0)
             add("resid_upd", "k_mresid", "hbm", 16.0 * upd_units, HBM_PEAK_GBS,

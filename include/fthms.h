@@ -113,13 +113,13 @@ typedef struct {
  *              of the time transforms, the restriction and the sums of cross rows evaluated every step
  *              in double-float on the FP32 pipe; diagonal self entries, the stored cross entries at
  *              z < 20, node distances, transform folds and phase factors stay FP64, phases are exact integers of turns, and stored cross rows
- *              (every precision) are 56-bit fixed point with exact sums.  The refinement solves the
+ *              (every precision) are 58-bit fixed point with exact sums.  The refinement solves the
  *              double-float matrix exactly; its rounding (~2^-47 of an entry) still reaches the
  *              densities through the matrix's conditioning, so the systems with N > 800 (factored with
  *              tensor-core updates, conditioning growing with N) keep matrices and residuals as in form 2.
  *              N > 800 (up to 2048): FP32 LU with tcgen05 (3xTF32) trailing updates, precisions 1 and 2.  2 = the mixed form
  *              with FP64 kept where accuracy is decided: the self matrices assembled in FP64 (the FP32
- *              factor is their rounding) and kept in 56-bit fixed point, a unit per row, with exact
+ *              factor is their rounding) and kept in 60-bit fixed point, a unit per row, with exact
  *              refinement residuals rounded to FP64, the z < 20 entries of rows evaluated every step, and
  *              the FFT butterflies of the time transforms (everything else as in 1).  Others -> ENOTIMPL.
  *  keep_densities : 1 keeps phi_{j,m,q}(omega_l) of every step for fthms_densities; 0 keeps only

@@ -450,7 +450,7 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
           C* a0 = A + (long long)(k0 + w + j0) * N + k0 + w + r;
           C* a1 = A + (long long)(k0 + w + j1) * N + k0 + w + r;
           C v0 = *a0, v1 = *a1;
-          fixacc_low<kLuLow> re0, im0, re1, im1;
+          fixacc<kLuLow> re0, im0, re1, im1;
 #pragma unroll
           for (int c = 0; c < kNB; ++c) {
             const int4 l = L[r * kPS + c], p = Ui[c * N + j0], q = Ui[c * N + j1];
@@ -464,7 +464,7 @@ __device__ void lu_one(const DevJob& J, int sidx, unsigned char* shl_raw) {
             re1.mac(n0, n1, q.z, q.w);
             im1.mac(l.z, l.w, q.x, q.y);
           }
-          auto less = [](double v, double u, const fixacc_low<kLuLow>& s) { return fma(-u, ll_to_double(s.nearest()), v); };
+          auto less = [](double v, double u, const fixacc<kLuLow>& s) { return fma(-u, ll_to_double(s.nearest()), v); };
           const double u0 = unit[j0], u1 = unit[j1];
           v0 = make_double2(less(v0.x, u0, re0), less(v0.y, u0, im0));
           v1 = make_double2(less(v1.x, u1, re1), less(v1.y, u1, im1));
@@ -878,7 +878,7 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
     const int s = max((int)(__float_as_uint(bound) >> 23) - 126, -64);
     s_exp[r][b] = (short)s;
     J.e_unit[J.row_off[(long long)task.pair * J.L + task.l0 + b] + task.row0 + r] =
-        s_r2[r] != 0u && z < 3e38f && s < 120 ? __uint_as_float((unsigned)(s - kFixBits + 127) << 23)
+        s_r2[r] != 0u && z < 3e38f && s < 120 ? __uint_as_float((unsigned)(s - fix_bits(kRowLow) + 127) << 23)
                                               : __uint_as_float(0x7FFFFFFFu);
   }
   __syncthreads();
@@ -895,7 +895,7 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
     int4* Ep = reinterpret_cast<int4*>(J.E) + (long long)i * ld + task.row0 + r;
     auto put = [&](int b, double2 v) {
       const int s = s_exp[r][b];
-      const int2 x = fix_f64(v.x, s), y = fix_f64(v.y, s);
+      const int2 x = fix_f64<kRowLow>(v.x, s), y = fix_f64<kRowLow>(v.y, s);
       Ep[eo[b]] = make_int4(x.x, x.y, y.x, y.y);
     };
     if constexpr (kF64) {
@@ -925,8 +925,8 @@ __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
           continue;
         }
         const float4 d = hankel_far_df(pt, ph, ang.d, df{f.a.z, f.a.w}, df{f.b.x, f.b.y}, bd, near);
-        const float c = __uint_as_float((unsigned)(27 - s_exp[r][b] + 127) << 23);
-        const int2 x = fix_df(d.x, d.y, c), y = fix_df(d.z, d.w, c);
+        const float c = __uint_as_float((unsigned)(kRowLow - 1 - s_exp[r][b] + 127) << 23);
+        const int2 x = fix_df<kRowLow>(d.x, d.y, c), y = fix_df<kRowLow>(d.z, d.w, c);
         Ep[eo[b]] = make_int4(x.x, x.y, y.x, y.y);
       }
     }
@@ -1246,9 +1246,9 @@ __device__ __forceinline__ void cp_async_wait() {
 constexpr int kFixStages = 2;
 __host__ __device__ constexpr int fix_batch(int Q) { return Q <= 2 ? 8 : 4; }   // entries a batch
 constexpr size_t fix_ring_bytes(int Q, int threads) { return (size_t)kFixStages * fix_batch(Q) * threads * sizeof(int4); }
-template <int Q>
+template <int Q, int kLow>
 __device__ __forceinline__ void fix_row(const int4* __restrict__ src, long long stride, int N, const int4* __restrict__ den,
-                                        int4* ring, fixacc (&re)[Q], fixacc (&im)[Q]) {
+                                        int4* ring, fixacc<kLow> (&re)[Q], fixacc<kLow> (&im)[Q]) {
   constexpr int kB = fix_batch(Q);
   const int T = blockDim.x, nbat = N / kB;
   auto mac = [&](const int4 e, int i) {
@@ -1281,8 +1281,8 @@ __device__ __forceinline__ void fix_row(const int4* __restrict__ src, long long 
     const int4* s = ring + (bi % kFixStages) * kB * T;
 #pragma unroll
     for (int k = 0; k < kB; ++k) mac(s[k * T], bi * kB + k);
-    // a source adds two products to either half of a sum: kFixRun products between carries
-    if ((bi + 1) % (kFixRun / 2 / kB) == 0) {
+    // a source adds two products to a sum
+    if ((bi + 1) % (fix_run(kLow) / 2 / kB) == 0) {
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
         re[q].carry();
@@ -1294,8 +1294,8 @@ __device__ __forceinline__ void fix_row(const int4* __restrict__ src, long long 
 }
 
 // The FP64-kept matrices in fixed point (fixed.cuh) for the refinement, converted in place once per job after the assembly:
-// every entry of row i as a 56-bit integer in units of a power of two just above the row's largest component (rounding
-// below 2^-56 of it; a row with an entry that is not finite gets the unit NaN).  A block stages kRows rows of one
+// every entry of row i as a 60-bit integer in units of a power of two just above the row's largest component (rounding
+// below 2^-60 of it; a row with an entry that is not finite gets the unit NaN).  A block stages kRows rows of one
 // system in shared memory, so the matrix is read and written once: bound by HBM.
 constexpr int kFixThreads = 256;
 template <int kRows>
@@ -1325,12 +1325,12 @@ __global__ void __launch_bounds__(kFixThreads) k_afix(DevJob J) {
       const int e = max((int)(s_max[r] >> 20) - 1022, -60);         // every |component| < 2^e
       for (int j = j0; j < N; j += kFixThreads / kRows) {
         const double2 v = shx[j * kRows + r];
-        const int2 x = fix_f64(v.x, e), y = fix_f64(v.y, e);
+        const int2 x = fix_f64<kMatLow>(v.x, e), y = fix_f64<kMatLow>(v.y, e);
         __stcs(reinterpret_cast<int4*>(A) + (long long)j * N + row0 + r, make_int4(x.x, x.y, y.x, y.y));
       }
       if (j0 == 0)
         J.a_unit[s.piv_off + row0 + r] =
-            e > 60 ? __uint_as_float(0x7FFFFFFFu) : __uint_as_float((unsigned)(e - kFixBits + 127) << 23);
+            e > 60 ? __uint_as_float(0x7FFFFFFFu) : __uint_as_float((unsigned)(e - fix_bits(kMatLow) + 127) << 23);
     }
     __syncthreads();
   }
@@ -1354,11 +1354,11 @@ __global__ void __launch_bounds__(kResidThreads, 4) k_mresid(DevJob J, int pass)
   const int i = c.row0 + (threadIdx.x & 31);
   const int row = i < N ? i : N - 1;
   extern __shared__ __align__(16) int4 she[];
-  fixacc re[Q], im[Q];
-  fix_row<Q>(reinterpret_cast<const int4*>(J.A) + s.mat_off + row, N, N, reinterpret_cast<const int4*>(J.phi_df) + s.vec_off,
+  fixacc<kMatLow> re[Q], im[Q];
+  fix_row<Q, kMatLow>(reinterpret_cast<const int4*>(J.A) + s.mat_off + row, N, N, reinterpret_cast<const int4*>(J.phi_df) + s.vec_off,
              she + threadIdx.x, re, im);
   if (i >= N) return;
-  const double ua = (double)J.a_unit[s.piv_off + i] * 0x1p56;
+  const double ua = (double)J.a_unit[s.piv_off + i] * (double)(1ll << 2 * kMatLow);
   const double isc = pass == 1 ? 1.0 / J.mscale[c.sys] : 0.0;   // a power of two: exact
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
@@ -1447,13 +1447,13 @@ __device__ __forceinline__ void fix_correction(const float2* b, int N, int4* out
   m = __reduce_max_sync(0xffffffffu, m);
   const int e = max((int)(m >> 23), 30) - 126;          // every |component| < 2^e (subnormal and tiny: any unit does)
   const bool bad = m >= 0x7F800000u || e > 120;
-  const float c0 = __uint_as_float((unsigned)(127 - e / 2) << 23), c1 = __uint_as_float((unsigned)(27 - (e - e / 2) + 127) << 23);
-  for (int i = lane; i < N; i += 32) {                  // (scaled in two steps: 2^(27 - e) may leave FP32's range)
-    const int2 x = fix_f32(__fmul_rn(b[i].x, c0), c1), y = fix_f32(__fmul_rn(b[i].y, c0), c1);
+  const float c0 = __uint_as_float((unsigned)(127 - e / 2) << 23), c1 = __uint_as_float((unsigned)(kMatLow - 1 - (e - e / 2) + 127) << 23);
+  for (int i = lane; i < N; i += 32) {                  // (scaled in two steps: 2^(29 - e) may leave FP32's range)
+    const int2 x = fix_f32<kMatLow>(__fmul_rn(b[i].x, c0), c1), y = fix_f32<kMatLow>(__fmul_rn(b[i].y, c0), c1);
     out[i] = make_int4(x.x, x.y, y.x, y.y);
   }
   if (lane == 0)
-    *unit = bad ? __longlong_as_double(0x7FF8000000000000ll) : __hiloint2double((e - kFixBits + 1023) << 20, 0);
+    *unit = bad ? __longlong_as_double(0x7FF8000000000000ll) : __hiloint2double((e - fix_bits(kMatLow) + 1023) << 20, 0);
 }
 
 // pass 0: solve with FP32 G, store phi as double-float (FP64 in the FP64-kept form, whose residual reads
@@ -1617,11 +1617,11 @@ __global__ void __launch_bounds__(kApplySlice, Q == 1 ? 3 : 2) k_cross_rows(DevJ
     ++b;
   }
   const CrossBlk B = J.blks[b];
-  fixacc re[Q], im[Q];
-  fix_row<Q>(reinterpret_cast<const int4*>(J.E + B.e_off) + r, B.nrows, B.N,
+  fixacc<kRowLow> re[Q], im[Q];
+  fix_row<Q, kRowLow>(reinterpret_cast<const int4*>(J.E + B.e_off) + r, B.nrows, B.N,
              reinterpret_cast<const int4*>(J.phi_df) + J.sys[B.sys].vec_off, she + threadIdx.x, re, im);
   const long long rr = J.grp_res_off[sl.grp] + row;
-  const double unit = (double)J.e_unit[rr] * 0x1p56;
+  const double unit = (double)J.e_unit[rr] * (double)(1ll << 2 * kRowLow);
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     const double u = unit * J.phi_unit[4ll * B.sys + q];

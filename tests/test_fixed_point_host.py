@@ -6,6 +6,7 @@ import subprocess
 
 import numpy as np
 import pytest
+from scipy import special
 
 import workloads as wl
 from oracle import geometry as geo
@@ -127,7 +128,7 @@ extern "C" void lu(double2* A, int* perm, int N, int fixed) {
           for (int c = k0; c < k1; ++c) v = cfms(at(r, c), at(c, j), v);
           continue;
         }
-        fixacc_low<kLuLow> re, im;
+        fixacc<kLuLow> re, im;
         for (int c = 0; c < 8; ++c) {
           const int4 l = L[(size_t)8 * (r - k1) + c], p = U[c];
           re.mac(l.x, l.y, p.x, p.y);
@@ -140,6 +141,80 @@ extern "C" void lu(double2* A, int* perm, int N, int fixed) {
       }
     }
   }
+}
+
+// Sums over N sources with the row kernels' carries; X, Y: [N][2] values as integers of fix_bits(low) bits.  Returns how many
+// of the two sums differ from the exact sums of the products kept.
+template <int kLow>
+static int exact_sums(const long long* X, const long long* Y, int N) {
+  fixacc<kLow> re, im;
+  __int128 er = 0, ei = 0;
+  auto kept = [](int2 a, int2 b) { return ((__int128)a.x * b.x << kLow) + (__int128)a.x * b.y + (__int128)a.y * b.x; };
+  for (int i = 0; i < N; ++i) {
+    const int2 a = fix_split<kLow>(X[2 * i]), b = fix_split<kLow>(X[2 * i + 1]);
+    const int2 c = fix_split<kLow>(Y[2 * i]), d = fix_split<kLow>(Y[2 * i + 1]), n = make_int2(-b.x, -b.y);
+    re.mac(a.x, a.y, c.x, c.y);
+    im.mac(a.x, a.y, d.x, d.y);
+    re.mac(n.x, n.y, d.x, d.y);
+    im.mac(b.x, b.y, c.x, c.y);
+    er += kept(a, c) + kept(n, d);
+    ei += kept(a, d) + kept(b, c);
+    if ((i + 1) % (fix_run(kLow) / 2) == 0) {
+      re.carry();
+      im.carry();
+    }
+  }
+  auto same = [](fixacc<kLow>& s, __int128 want) {
+    s.carry();
+    return (((((__int128)s.c) << 32) + s.a) << kLow) + s.b == want;
+  };
+  return !same(re, er) + !same(im, ei);
+}
+extern "C" int sums_differ(const long long* X, const long long* Y, int N, int low) {
+  return low == kRowLow ? exact_sums<kRowLow>(X, Y, N) : exact_sums<kMatLow>(X, Y, N);
+}
+extern "C" int lows(int* out) { out[0] = kRowLow; out[1] = kMatLow; return 0; }
+
+// R rows of N entries (bounds 2^s[r]) times p (bound 2^sp): errors of FP64 FMAs and of the fixed-point sums over sum |E||p|.
+extern "C" void row_errors(const double2* E, const int* s, const double2* p, int sp, int R, int N, double* out) {
+  for (int r = 0; r < R; ++r, E += N) {
+    quad x = 0, y = 0;
+    double2 f = make_double2(0, 0);
+    fixacc<kRowLow> re, im;
+    double size = 0;
+    for (int i = 0; i < N; ++i) {
+      const double2 e = E[i], v = p[i];
+      x += (quad)e.x * v.x - (quad)e.y * v.y;
+      y += (quad)e.x * v.y + (quad)e.y * v.x;
+      f = cfma(e, v, f);
+      size += std::hypot(e.x, e.y) * std::hypot(v.x, v.y);
+      const int2 a = fix_f64<kRowLow>(e.x, s[r]), b = fix_f64<kRowLow>(e.y, s[r]);
+      const int2 c = fix_f64<kRowLow>(v.x, sp), d = fix_f64<kRowLow>(v.y, sp);
+      re.mac(a.x, a.y, c.x, c.y);
+      im.mac(a.x, a.y, d.x, d.y);
+      re.mac(-b.x, -b.y, d.x, d.y);
+      im.mac(b.x, b.y, c.x, c.y);
+      if ((i + 1) % (fix_run(kRowLow) / 2) == 0) {
+        re.carry();
+        im.carry();
+      }
+    }
+    const double u = std::ldexp(1.0, 2 * kRowLow + s[r] + sp - 2 * fix_bits(kRowLow));
+    out[2 * r] = std::hypot((double)(x - f.x), (double)(y - f.y)) / size;
+    out[2 * r + 1] = std::hypot((double)(x - (quad)(re.value() * u)), (double)(y - (quad)(im.value() * u))) / size;
+  }
+}
+
+// Root mean square over a row (bound 2^e) of the matrices' fixed-point rounding.
+extern "C" double kept_error(const double* v, int n, int e) {
+  double sum = 0;
+  for (int i = 0; i < n; ++i) {
+    const int2 x = fix_f64<kMatLow>(v[i], e);
+    const quad w = ((quad)((long long)x.x << kMatLow) + x.y) * std::ldexp(1.0, e - fix_bits(kMatLow));
+    const double d = (double)(w - v[i]);
+    sum += d * d;
+  }
+  return std::sqrt(sum / n);
 }
 
 // P A - L U: Frobenius norm over |A|'s, largest entry over |L||U|'s, and the mean (re, im) over the mean |a|.
@@ -291,3 +366,80 @@ def test_bessel_tables_are_read_inside_whatever_the_argument(lib, z):
     tables."""
     lib.taylor_reads_inside.argtypes = [ct.c_double]
     assert lib.taylor_reads_inside(z)
+
+
+@pytest.mark.parametrize("which", [0, 1])
+def test_sums_are_exact_up_to_the_largest_values(lib, which):
+    """Sums of 2 048 sources with a carry after each run, at the largest values either half can hold (every sign), random
+    ones, and mixtures: no overflow, nothing lost."""
+    low = (ct.c_int * 2)()
+    lib.lows(low)
+    low = low[which]
+    top, half = 1 << (2 * low - 1), 1 << (low - 1)
+    edge = [top, -top, top - half, half - top, top - half - 1, half - 1, -half, 0, 1, -1]
+    rng = np.random.default_rng(low)
+    N = 2048
+    sets = [np.full(2 * N, v, np.int64) for v in edge]
+    for a in edge:
+        for b in edge:
+            sets.append(np.array([a, b] * N, np.int64))
+    sets += [rng.integers(-top, top, 2 * N, endpoint=True) for _ in range(4)] + [rng.choice(np.array(edge), 2 * N) for _ in range(8)]
+    for X in sets:
+        for Y in sets[::3]:
+            assert lib.sums_differ(_ptr(np.ascontiguousarray(X)), _ptr(np.ascontiguousarray(Y)), N, low) == 0
+
+
+def _near_beta(ts, N):
+    """-(2/pi)(W_i/w - ln|t* - t_i|) of the near rule for a target continued to t*."""
+    t, n = geo.cheb_nodes(N), np.arange(1, N)
+    rt = np.sqrt(ts * ts - 1.0)
+    zeta = ts - rt if ts > 0 else ts + rt
+    W = (np.pi * np.log(0.5 * (abs(ts) + rt)) + 2.0 * np.cos(np.outer(np.arccos(t), n)) @ (-np.pi * zeta ** n / n)) / N
+    return -(2.0 / np.pi) * (W * N / np.pi - np.log(np.abs(ts - t)))
+
+
+@pytest.mark.parametrize("N", [33, 96, 259, 800])
+@pytest.mark.parametrize("rate", [0.02, 0.15, 0.3])
+def test_stored_row_sums_are_no_less_accurate_than_fp64(lib, N, rate):
+    """Rows of cross entries (next to the arc's ends with their near corrections, and far ones) times a density, sums in
+    fixed point against FP64 FMAs over the same FP64 entries.  N roundings of the running sum become one rounding a value
+    of 2^-58 of the bound, so the error may not be larger: root mean square over the near and over the far rows, and the
+    largest."""
+    rng = np.random.default_rng(N)
+    kappa, curve, w = rate * N, wl.kite(0.1, 0.2), np.pi / N
+    X = geo.Arc(0, 0, curve, -1.3, 1.1).point(geo.cheb_nodes(N))[0]
+    ts = rng.choice([-1.0, 1.0], 40) * (1.0 + np.exp(rng.uniform(np.log(1e-4), np.log(2.0), 40)))
+    th, k = -0.1 + 1.2 * ts, np.arange(3)[:, None]
+    near = np.stack([np.dot(curve[a], np.cos(k * th)) + np.dot(curve[b], np.sin(k * th)) for a, b in (("ax", "bx"), ("ay", "by"))], 1)
+    tg = np.concatenate([near, rng.uniform(-8.0, 8.0, (40, 2))])
+    beta = np.concatenate([np.array([_near_beta(t, N) for t in ts]), np.zeros((40, N))])
+    z = kappa * np.linalg.norm(tg[:, None] - X[None], axis=-1)
+    J = special.j0(z)
+    E = np.ascontiguousarray(0.25 * w * (beta * J - special.y0(z) + 1j * J))
+    zm = z.min(1)
+    h0 = np.where(zm < 1.0, np.minimum(np.sqrt(0.6367 / zm), 1.5 - 0.64 * np.log(zm)), np.sqrt(0.6367 / zm))
+    s = (np.floor(np.log2(0.25 * w * h0 * (1.0 + np.abs(beta).max(1)))) + 1).astype(np.int32)      # the kernel's row bound
+    assert np.all(np.abs(E).max(1) < np.exp2(s))
+    p = np.exp(1j * kappa * X[:, 0]) * (1.0 + 0.3 * np.polynomial.chebyshev.chebval(geo.cheb_nodes(N), rng.normal(size=12) + 1j * rng.normal(size=12)))
+    sp = int(np.floor(np.log2(max(np.abs(p.real).max(), np.abs(p.imag).max())))) + 1
+    out = np.zeros((80, 2))
+    lib.row_errors(_ptr(E), _ptr(s), _ptr(p), sp, 80, N, _ptr(out))
+    for rows in (out[:40], out[40:]):
+        fma, fix = np.sqrt(np.mean(rows ** 2, 0))
+        assert fix <= fma and rows[:, 1].max() <= rows[:, 0].max()
+
+
+@pytest.mark.parametrize("N,kappa", [(96, 20.0), (259, 65.0), (512, 150.0), (1024, 150.0)])
+def test_kept_matrices_hold_what_fp64_holds(lib, N, kappa):
+    """The refinement's matrices: their fixed-point rounding against the half unit in the last place that every FP64 entry
+    carries from its own computation.  A row's entries lie up to 2^6 below its largest, which 60 bits (2^-60 of it) cover:
+    below a half of it in the root mean square."""
+    lib.kept_error.restype = ct.c_double
+    A = oker.self_matrix(geo.Arc(0, 0, wl.kite(0.1, 0.2), -1.3, 1.1), N, kappa)
+    kept = own = 0.0
+    for row in A:
+        v = np.ascontiguousarray(np.stack([row.real, row.imag], 1)).ravel()
+        e = int(np.floor(np.log2(np.abs(v).max()))) + 1
+        kept += lib.kept_error(_ptr(v), v.size, e) ** 2
+        own += float(np.mean(np.spacing(np.abs(v)) ** 2)) / 12.0
+    assert np.sqrt(kept) <= 0.5 * np.sqrt(own)
