@@ -102,8 +102,8 @@ typedef struct {
  *  Q, H      : 1 <= Q <= 4 time windows sqcap_q(t) = sqcap(t - s_q), s_q = 1.5 (q-1) H (Section 5).
  *  n_period  : internal time samples per period 2 pi/h of the frequency grid (power of two,
  *              16..16384); dt = 2 pi/(h n_period), t_n = -H + n dt covering [-H, s_Q + H].  The time
- *              kernels keep one period and these N_T samples of a node in shared memory:
- *              16 n_period + 8 N_T <= 232448 bytes, else EINVAL.
+ *              kernels work on a node's N_T samples and its transform in shared memory:
+ *              16 n_period + 8 N_T <= 232448 bytes (a whole period of complex values), else EINVAL.
  *  obs_xy    : n_obs observation points (x, y), host array of 2*n_obs doubles.
  *  n_tout, tout0, dtout : output times tout0 + k dtout of the traces u_M(z, t) (eq. mult-scatt-int).
  *  precision : 0 = FP64 throughout.  1 = mixed form: FP32 LU factors; solutions refined against the
@@ -126,8 +126,10 @@ typedef struct {
  *              the sum over m.
  *  cross_mode: 0 = the cross-arc and observation rows of eq. FDsolk-interior are assembled once per job,
  *              stored in device memory and applied every step (fast while they fit: 16 bytes per
- *              entry).  1 = they are evaluated again in every step and summed at once, nothing stored
- *              (for jobs whose cross rows do not fit, e.g. many arcs on one curve at high frequency).
+ *              entry; precision 0: 16 Q (targets + rows + summed nodes) <= 232448 for every receiver and
+ *              frequency, else EINVAL, and a mixed job above it has no FP64 fallback).  1 = they are evaluated
+ *              again in every step and summed at once, nothing stored (for jobs whose cross rows do not fit,
+ *              e.g. many arcs on one curve at high frequency).
  *              Both modes give the same densities to rounding.  Others -> EINVAL.
  *  refine_tol, refine_max : mixed forms: a system stops refining once the estimated relative error left
  *              is below refine_tol (0 = 1e-12), after at most refine_max passes (0 = 3; at most 16).  The

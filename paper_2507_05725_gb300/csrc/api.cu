@@ -113,7 +113,7 @@ struct fthms_req {
   fthms_status conv_status = FTHMS_OK;
   std::string conv_msg;
   int fallback_runs = 0;           // runs repeated in FP64 after a refinement that did not converge
-  bool plain_apply_fits = true;    // the FP64 stored-row apply fits shared memory (FP64 fallback possible)
+  bool fp64_rows_fit = true;       // stored cross rows within the FP64 form's limit (fthms_options.cross_mode)
   int lu_min = kLuBigMin;          // smallest N factored with tensor-core updates (mixed forms)
   fthms_allreduce_fn allreduce = nullptr;   // sum across the ranks of a frequency-partitioned job
   void* allreduce_user = nullptr;
@@ -214,23 +214,26 @@ fthms_status upload_job(fthms_req* r) {
   J.max_nmax = 0;
   for (int k = 0; k < p.P; ++k) J.max_nmax = std::max(J.max_nmax, p.Nmax[k]);
   J.acc_cap = std::max(J.max_nmax, p.n_obs);
-  J.row_cap = 0;
-  J.ph_cap = 0;
+  int rows_max = 0, nodes_max = 0;
   for (const CrossGrp& g : p.grps) {
-    int rows = 0, nsum = 0;
+    int rows = 0, nodes = 0;
     for (int b = g.blk_begin; b < g.blk_end; ++b) {
       rows += p.blks[b].nrows;
-      nsum += p.blks[b].N;
+      nodes += p.blks[b].N;
     }
-    J.row_cap = std::max(J.row_cap, rows);
-    J.ph_cap = std::max(J.ph_cap, nsum);
+    rows_max = std::max(rows_max, rows);
+    nodes_max = std::max(nodes_max, nodes);
   }
-  // The FP64 stored-row apply keeps a whole group in shared memory (the mixed form works in row slices).
-  r->plain_apply_fits = p.opt.cross_mode != 0 ||
-                        (size_t)J.Q * (J.acc_cap + J.row_cap + J.ph_cap) * 16 <= (size_t)227 * 1024;
-  if (p.opt.precision == 0 && !r->plain_apply_fits)
-    return fail(FTHMS_EINVAL, "fthms_prepare: the stored cross rows of one (arc, frequency) group do not fit the "
-                              "apply's shared memory; use cross_mode 1");
+  // The FP64 form's documented limit on stored rows.  (No kernel needs it any more: the apply works in row slices in
+  // every form.  It stands so that the same jobs are taken and refused.)
+  const size_t group_bytes = (size_t)16 * J.Q * (J.acc_cap + rows_max + nodes_max);
+  r->fp64_rows_fit = p.opt.cross_mode != 0 || group_bytes <= (size_t)227 * 1024;
+  if (p.opt.precision == 0 && !r->fp64_rows_fit) {
+    char buf[240];
+    snprintf(buf, sizeof buf, "fthms_prepare: FP64 stored cross rows take 16 Q (targets + rows + summed nodes) <= 232448 for every "
+             "(arc, frequency) group, this job has %zu; use cross_mode 1", group_bytes);
+    return fail(FTHMS_EINVAL, buf);
+  }
   J.h = p.h; J.dt = p.dt; J.sign = p.sig.sign;
   J.sig_kind = p.sig.kind;
   J.z0x = p.sig.z0[0]; J.z0y = p.sig.z0[1];
@@ -276,7 +279,6 @@ fthms_status upload_job(fthms_req* r) {
   TRY(dev_upload(r, p.grps, &J.grps));
   TRY(dev_upload(r, p.blks, &J.blks));
   J.n_slices = 0;
-  J.slice_ph_cap = p.slice_ph_cap;
   J.slices = nullptr;
   J.grp_res_off = nullptr;
   J.apply_res = nullptr;
@@ -734,7 +736,7 @@ static fthms_status wait_run(fthms_req* req, int timeout_ms) {
 static const char* no_fallback(const fthms_req* req) {
   if (req->plan.ranks > 1) return "a frequency-partitioned job never falls back alone: its ranks would stop meeting in the all-reduce";
   if (req->plan.maxN > kLuSmallMax) return "a system exceeds the FP64 form's N <= 800";
-  if (!req->plain_apply_fits) return "the stored cross rows exceed its apply";
+  if (!req->fp64_rows_fit) return "the stored cross rows exceed the FP64 form's limit";
   return nullptr;
 }
 

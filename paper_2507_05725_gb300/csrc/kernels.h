@@ -13,7 +13,6 @@ constexpr size_t kFreqDfBytes = 48;
 struct DevJob {
   int P, L, Q, K, NT, M, n_obs, n_tout, nsys, n_act, n_grp, n_asm, n_tiles, n_rlogN, n_restr;
   int logK, max_nmax, max_n, acc_cap;
-  int row_cap, ph_cap;           // max rows and max sum of source N over the cross groups
   int mixed;                     // 1: mixed-precision form (FP32 LU + double-float refinement/apply)
   int fp64keep;                  // mixed form with FP64 kept for the small-argument Hankel series, the
                                  // refinement residuals and the FFT butterflies (precision 2)
@@ -61,7 +60,7 @@ struct DevJob {
   const ApplySlice* slices;  // stored cross rows: row slices of the groups
   const long long* grp_res_off;
   double2* apply_res;        // [group rows][Q] per-row cross sums
-  int n_slices, slice_ph_cap;
+  int n_slices;
   // cross_mode 1: cross rows evaluated every step (nothing stored)
   int otf, n_otf;
   // launch shapes chosen by fthms_autotune (0 = built-in default): warps per solve block, threads per

@@ -298,11 +298,11 @@ int build_plan(const fthms_curve* curves, int ncurves, const fthms_arc* arcs, in
     err = "internal time grid longer than 65536 samples";
     return FTHMS_EINVAL;
   }
-  // The time kernels hold one period (n_period complex values) and the internal samples (NT doubles) of a
-  // transfer node in shared memory.
+  // The time kernels hold half a period of complex values (8 n_period bytes) and the internal samples (NT doubles) of a
+  // transfer node in shared memory; the documented limit counts a whole period.
   if ((size_t)p.K * 16 + (size_t)p.NT * 8 > (size_t)227 * 1024) {
-    snprintf(buf, sizeof buf, "n_period (%d) and the internal time samples (%d) need %zu bytes of shared memory; "
-             "at most 232448 (lower n_period, H or Q)", p.K, p.NT, (size_t)p.K * 16 + (size_t)p.NT * 8);
+    snprintf(buf, sizeof buf, "n_period (%d) and the internal time samples (%d) exceed the time kernels' shared memory limit: "
+             "16 n_period + 8 samples = %zu, at most 232448 (lower n_period, H or Q)", p.K, p.NT, (size_t)p.K * 16 + (size_t)p.NT * 8);
     err = buf;
     return FTHMS_EINVAL;
   }
@@ -555,7 +555,7 @@ int build_plan(const fthms_curve* curves, int ncurves, const fthms_arc* arcs, in
       g.blk_end = (int)p.blks.size();
       if (g.blk_end > g.blk_begin) p.grps.push_back(g);
     }
-  // Row slices for the mixed-form apply: kApplySlice consecutive rows of a group per CTA.
+  // Row slices of the stored-row apply: kApplySlice consecutive rows of a group per CTA.
   p.grp_res_off.resize(p.grps.size());
   for (size_t gi = 0; gi < p.grps.size(); ++gi) {
     const CrossGrp& g = p.grps[gi];
@@ -563,28 +563,10 @@ int build_plan(const fthms_curve* curves, int ncurves, const fthms_arc* arcs, in
     int rows = 0;
     for (int b = g.blk_begin; b < g.blk_end; ++b) rows += p.blks[b].nrows;
     p.res_total += rows;
-    // A slice ends early at a block boundary when the densities it stages (Q x summed N) would
-    // exceed kSliceDensities complex values (196 KB of shared memory).
-    const int kSliceDensities = 12288;
     int b = g.blk_begin, rb = 0;              // block containing row0 and its first row
-    for (int row0 = 0; row0 < rows;) {
+    for (int row0 = 0; row0 < rows; row0 += kApplySlice) {
       while (row0 >= rb + p.blks[b].nrows) rb += p.blks[b++].nrows;
-      int end = std::min(row0 + kApplySlice, rows);
-      ApplySlice sl{(int)gi, row0, 0, b, b, rb};
-      int nsum = p.blks[b].N, re = rb + p.blks[b].nrows;
-      while (re < end) {
-        if ((nsum + p.blks[sl.b1 + 1].N) * p.Q > kSliceDensities) {
-          end = re;
-          break;
-        }
-        ++sl.b1;
-        nsum += p.blks[sl.b1].N;
-        re += p.blks[sl.b1].nrows;
-      }
-      sl.nrows = end - row0;
-      p.slice_ph_cap = std::max(p.slice_ph_cap, nsum);
-      p.slices.push_back(sl);
-      row0 = end;
+      p.slices.push_back(ApplySlice{(int)gi, row0, std::min(kApplySlice, rows - row0), b, rb});
     }
   }
   // Stored cross rows: the assembly keeps 4N + 2 kAsmRows N doubles and its band tables in shared memory.

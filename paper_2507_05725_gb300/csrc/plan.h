@@ -72,7 +72,6 @@ struct Plan {
   std::vector<ResidChunk> rchunks;      // 32-row chunks of the systems, largest first (mixed-form residuals)
   std::vector<long long> grp_res_off;    // first row of each group in the per-row result buffer
   long long res_total = 0;               // rows over all groups
-  int slice_ph_cap = 0;                  // max over slices of the summed N of the blocks it overlaps
   std::vector<CrossOtf> otf;            // cross_mode 1: on-the-fly tasks
   std::vector<long long> wn_off;         // per assembly task: offset of its near weights (nrows x N), or -1
   long long wn_total = 0;

@@ -271,3 +271,29 @@ def test_self_matrix_does_not_depend_on_the_unit_of_length(F, bits):
             torch.cuda.synchronize()
             out.append(A.cpu())
     assert torch.equal(out[0], out[2]) and torch.equal(out[1], out[3]) and bool(torch.all(torch.isfinite(out[0])))
+
+
+def test_stored_rows_of_many_large_sources(F, ctx):
+    """A slice of rows over more sources than the FP64 form's limit counts (six arcs of 800 nodes, four windows): the mixed
+    form takes it, the FP64 form and the fallback name the limit."""
+    p = wl.random_small(7, n_curves=2, n_arcs_per_curve=3, L=3, M=2, Q=4, N_fixed=800, W=14.0, H=0.2, n_period=64, kind=1)
+    p["options"]["refine_max"] = 8
+    jobs = []
+    for mode in (0, 1):
+        p["options"]["cross_mode"] = mode
+        jobs.append(F.Job(ctx, p, precision=2).run())
+        F.LIB.fthms_wait(jobs[-1].req, -1)
+    for j in range(6):
+        for q in range(4):
+            a, b = (F.fthms_densities(x.req, j, 2, q) for x in jobs)
+            assert np.linalg.norm(a - b) <= 1e-10 * np.linalg.norm(b)
+    t, u = (x.traces() for x in jobs)
+    assert np.max(np.abs(t - u)) <= 1e-10 * np.max(np.abs(u)) and np.max(np.abs(u)) > 0.0
+    p["options"].update(cross_mode=0, refine_tol=1e-30, refine_max=1, refine_fallback=1)
+    with pytest.raises(F.FthmsError) as e:
+        F.Job(ctx, p, precision=0)
+    assert e.value.status == F.FTHMS_EINVAL and "232448" in str(e.value)
+    job = F.Job(ctx, p, precision=2).run()
+    with pytest.raises(F.FthmsError) as e:
+        job.wait()
+    assert e.value.status == F.FTHMS_ENOCONV and "limit" in str(e.value)
