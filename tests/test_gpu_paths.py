@@ -297,3 +297,40 @@ def test_stored_rows_of_many_large_sources(F, ctx):
     with pytest.raises(F.FthmsError) as e:
         job.wait()
     assert e.value.status == F.FTHMS_ENOCONV and "limit" in str(e.value)
+
+
+@pytest.mark.parametrize("N,L,signal,interpolated", [
+    (72, 41, {}, True),
+    (24, 41, {}, False),                                                          # few nodes
+    (72, 41, dict(z0=[1.004, 0.0]), False),                                       # source next to an arc
+    (160, 41, dict(z0=[1.2, 0.1], carrier=14.0, width=0.6, centre=3.0), False),   # samples and basis outgrow their memory
+    (160, 97, dict(z0=[1.2, 0.1], carrier=14.0, width=0.6, centre=3.0), True),    # distances 0.2 to 2.2, high carrier
+    (72, 97, dict(z0=[6.0, 1.0], carrier=14.0, width=0.6, centre=0.5), True)])    # distances 5.1 to 7.1
+def test_point_source_rule(F, ctx, N, L, signal, interpolated):
+    """Which jobs interpolate the incident field in the distance (two launches more: basis and product), and its accuracy
+    where the distances differ most and the signal oscillates fastest.  1e-11: the FP64 bar."""
+    p = wl.config1(L=L, M=1, N=N)
+    p["options"].update(H=7.5 if signal.get("centre") == 0.5 else 4.0, n_period=256 if L < 50 else 512, W=16.0 if N < 100 else 24.0)
+    p["signal"].update(signal)
+    job = F.Job(ctx, p)
+    F.fthms_profile(job.req, True)
+    job.run().wait()
+    assert F.fthms_stage_times(job.req)["incident"][1] == (4 if interpolated else 2)
+    assert _rel(job, run_oracle(p), p) < 1e-11
+
+
+@pytest.mark.parametrize("N", [8, 33, 96, 135])
+def test_lu_thread_counts_give_the_same_factors(F, ctx, N):
+    """FP64 jobs of systems up to 135 nodes factor with 128 threads a system, others with 256: the densities of small arcs are
+    the same bit for bit with and without a large obstacle in the job (step 1 does not couple them)."""
+    p = wl.random_small(9, n_arcs_per_curve=3, L=24, M=1, W=14.0, H=4.0, n_period=512, kind=1)
+    p["curves"] = [wl.circle(1.0)]
+    p["options"].update(N_min=N, N_off=0, N_ppw=N / (14.0 * 2.7))
+    q = copy.deepcopy(p)
+    q["curves"].append(wl.circle(20.0 if N < 33 else 3.0 if N > 60 else 6.0, 30.0, 0.0))
+    q["arcs"] = q["arcs"] + [(1, a, b) for _, a, b in q["arcs"]]
+    small, mixed = (F.Job(ctx, x).run().wait() for x in (p, q))
+    assert {v.size for v in small.densities(0, 1, 0).values()} == {N}
+    assert 135 < max(v.size for v in mixed.densities(3, 1, 0).values()) <= 800
+    for j in range(3):
+        assert np.array_equal(F.fthms_densities(small.req, j, 1, 0), F.fthms_densities(mixed.req, j, 1, 0))
