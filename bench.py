@@ -62,6 +62,7 @@ def _hbm_peak_gbs():
 
 HBM_PEAK_GBS = _hbm_peak_gbs()
 FP64_PEAK_GFLOPS = 152 * 4 * 2.07  # 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz max SM clock
+INT_MAD_PEAK = 152 * 64 * 2.07     # 152 SMs x 64 integer multiply-adds (32 x 32 + 64) a clock
 
 
 def kernels_hash():
@@ -356,7 +357,8 @@ def stage_rooflines(r, problem, stored_rows):
         out[stage] = {"kernel": kernel, "bound": bound, "achieved": ach, "peak": peak, "unit": unit,
                       "frac": ach / peak, "traffic": traffic, "ms_per_job": ms, "launches_per_job": launches,
                       "ms_per_launch": ms / max(launches, 1),
-                      ("algorithmic_flops_per_launch" if unit.endswith("FLOP/s") else "algorithmic_bytes_per_launch"):
+                      ("algorithmic_flops_per_launch" if unit.endswith("FLOP/s") else
+                       "algorithmic_bytes_per_launch" if unit.endswith("B/s") else "algorithmic_ops_per_launch"):
                           amount / max(launches, 1),
                       "note": note}
 
@@ -395,6 +397,13 @@ def stage_rooflines(r, problem, stored_rows):
                 f"per panel); peak: TF32 dense = measured bf16 sustained x 1.1/2.25 ({PEAK_NOTE})")
     else:
         add("solve", "k_solve", "alu", st["solve_flops"], FP64_PEAK_GFLOPS, "GFLOP/s", fp64)
+        add("lu", "k_lu<double2>", "alu", 1.5 * st["lu_flops"], INT_MAD_PEAK, "Gmad/s",
+            "sum N^3 / 3 complex products of the trailing updates, 12 integer multiply-adds (32 x 32 + 64) each; peak: 152 SMs x "
+            "64 a clock x 2.07 GHz; what bounds it is the panels' chain and FP64")
+        if stored_rows:
+            add("cross_assemble", "k_cross_assemble", "alu", 9.0 * st["cross_entries"], FP64_PEAK_GFLOPS / 2.0, "Ginstr/s",
+                "9 FP64 instructions an entry (the ~25 of a pair, shared by its band, come on top); peak: the FP64 pipe's "
+                "152 SMs x 2 a clock x 2.07 GHz")
     return out
 
 
@@ -604,7 +613,7 @@ def ours(args):
             forms["c2_plain_fp64_fused"] = dict(
                 summary(f2), value=solves_of(c2) / (f2["ms"] / 1e3), workload=WORKLOAD_NAMES["c2"],
                 note="batching form: assembly, LU and step-1 solve of every system in one persistent launch "
-                     "(fthms_use_fused), against c2_plain_fp64's staged launches of the same FP64 kernels",
+                     "(fthms_use_fused), against c2_plain_fp64's staged launches (its assembly evaluates the entries in plain FP64)",
                 fused_ms_per_job=f2["stages"].get("fused", (0.0, 0))[0] if f2["stages"] else None,
                 staged_ms_per_job=sum(p2["stages"][k][0] for k in ("assemble_self", "lu")) + p2["stages"]["solve"][0]
                 / c2["options"]["M"] if p2["stages"] else None)
@@ -631,11 +640,12 @@ def ours(args):
                 "warmup": args.warmup, "ms_per_step": head["ms"], "higher_is_better": True, "scaling": "weak",
                 "vs_baseline": None,
                 "dtype": ({1: "f32 factors (tensor-core 3xTF32 updates above N = 800) + double-float (2 x f32) "
-                              "assembly, refinement, FFT butterflies, restriction and cross apply; f64 set-up, "
-                              "folds and outputs",
-                           2: "f32 factors + f64 self matrices and refinement residuals, f64 small-argument Hankel "
-                              "series and FFT butterflies; double-float far-field recurrence, restriction and cross "
-                              "apply"}[head["precision"]] if mixed else "f64"),
+                              "assembly, refinement, FFT butterflies and restriction; stored cross rows in 58-bit "
+                              "fixed point with exact sums; f64 set-up, folds and outputs",
+                           2: "f32 factors + self matrices assembled in f64 and kept in 60-bit fixed point, refinement "
+                              "residuals exact sums rounded to f64; stored cross rows in 58-bit fixed point with exact "
+                              "sums, their entries f64 below z = 20 and double-float above; f64 FFT butterflies; "
+                              "double-float restriction"}[head["precision"]] if mixed else "f64"),
                 "data": "synthetic",
                 "config": {"workload": wname, "solves_per_step": solves, "systems_per_step": P * (o["L"] - 1),
                            "form": (("mixed" if head["precision"] == 1 else "fp64-kept mixed") +

@@ -106,19 +106,26 @@ typedef struct {
  *              16 n_period + 8 N_T <= 232448 bytes (a whole period of complex values), else EINVAL.
  *  obs_xy    : n_obs observation points (x, y), host array of 2*n_obs doubles.
  *  n_tout, tout0, dtout : output times tout0 + k dtout of the traces u_M(z, t) (eq. mult-scatt-int).
- *  precision : 0 = FP64 throughout.  1 = mixed form: FP32 LU factors; solutions refined against the
- *              matrix kept as double-float (two floats, ~48 bits) until the relative error estimated
- *              to remain (last correction x estimated contraction factor) is below refine_tol, at most
- *              refine_max steps; self and cross entries, the refinement residuals, the FFT butterflies
- *              of the time transforms, the restriction and the sums of cross rows evaluated every step
- *              in double-float on the FP32 pipe; diagonal self entries, the stored cross entries at
- *              z < 20, node distances, transform folds and phase factors stay FP64, phases are exact integers of turns, and stored cross rows
- *              (every precision) are 58-bit fixed point with exact sums.  The refinement solves the
- *              double-float matrix exactly; its rounding (~2^-47 of an entry) still reaches the
+ *  precision : 0 = the FP64 form: matrices, factors, densities, transforms and results are FP64.  Inside
+ *              it three steps use other arithmetic, with errors against higher precision no larger than
+ *              plain FP64's: the Hankel functions add corrections evaluated in double-float or less (they
+ *              lie below 2^-6 of the value) to FP64 table values; the LU's trailing updates are 60-bit
+ *              fixed point, one rounding per panel of 8 columns to 2^-57 of a column's largest entry; and
+ *              stored cross rows and the densities they meet are 58-bit fixed point, in units of a bound
+ *              of the row and of the largest density of the (system, window), with exact sums (every
+ *              precision).
+ *              1 = mixed form: FP32 LU factors; solutions refined against the matrix kept as double-float
+ *              (two floats, ~48 bits) until the relative error estimated to remain (last correction x
+ *              estimated contraction factor) is below refine_tol, at most refine_max steps; self and cross
+ *              entries, the refinement residuals, the FFT butterflies of the time transforms, the
+ *              restriction and the sums of cross rows evaluated every step in double-float on the FP32
+ *              pipe; diagonal self entries, the stored cross entries at z < 20, node distances, transform
+ *              folds and phase factors stay FP64, phases are exact integers of turns.  The refinement
+ *              solves the double-float matrix exactly; its rounding (~2^-47 of an entry) still reaches the
  *              densities through the matrix's conditioning, so the systems with N > 800 (factored with
  *              tensor-core updates, conditioning growing with N) keep matrices and residuals as in form 2.
- *              N > 800 (up to 2048): FP32 LU with tcgen05 (3xTF32) trailing updates, precisions 1 and 2.  2 = the mixed form
- *              with FP64 kept where accuracy is decided: the self matrices assembled in FP64 (the FP32
+ *              N > 800 (up to 2048): FP32 LU with tcgen05 (3xTF32) trailing updates, precisions 1 and 2.
+ *              2 = the mixed form with FP64 kept where accuracy is decided: the self matrices assembled in FP64 (the FP32
  *              factor is their rounding) and kept in 60-bit fixed point, a unit per row, with exact
  *              refinement residuals rounded to FP64, the z < 20 entries of rows evaluated every step, and
  *              the FFT butterflies of the time transforms (everything else as in 1).  Others -> ENOTIMPL.

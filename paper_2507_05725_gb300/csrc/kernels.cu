@@ -1,4 +1,4 @@
-// CUDA kernels (sm_103a, FP64) of the FTH-MS open-arc hot path.
+// CUDA kernels (sm_103a) of the FTH-MS open-arc hot path.
 //
 // Stages (one job):
 //   tables         FFT twiddles, recentring phases, self log-weight tables, restriction tables
@@ -13,7 +13,7 @@
 //     cross_apply  W_k = sum_{j != k, masked} S_j[phi_j] (eq. vtilde) and the observation sum
 //     synth_fwd    recentred inverse transform (eq. TDsol), g = -chi_k w (eq. criterion_int2),
 //                  windowed slow transform (eq. Fourierk) -- one CTA per transfer node, in shared
-//                  memory, with a radix-2 FFT
+//                  memory, with a half-length FFT per window
 //   traces         u_M(z, t) at the output times (eq. mult-scatt-int)
 #include <algorithm>
 #include <cmath>
@@ -245,7 +245,7 @@ __global__ void k_restr(DevJob J) {
 // ---------------------------------------------------------------------------------------------
 // A self-matrix entry: FP64, or (mixed form) the double-float pair the refinement reads plus its FP32
 // rounding for the FP32 factorisation -- what a separate split of the FP64 matrix would give -- or (the
-// FP64-kept form) the FP64 value the FP64 residual reads plus its FP32 rounding.
+// FP64-kept form) the FP64 value, which k_afix turns into fixed point for the residual, plus its FP32 rounding.
 // Mixed forms: systems that keep FP64 matrices and residuals (all in the FP64-kept form; N >= f64_min_n in
 // the mixed form, whose large systems' conditioning would amplify a double-float matrix's rounding).
 __device__ __forceinline__ bool sys_f64(const DevJob& J, int N) { return J.fp64keep || N >= J.f64_min_n; }
@@ -267,7 +267,7 @@ __device__ __forceinline__ void store_self(const DevJob& J, long long off, doubl
 // frequencies sharing N (nodes, log weights, |t - s| and its logarithm are shared).  With K1 = -J0/(2 pi) an
 // off-diagonal entry is the near rule's E = amp (beta cos - sin, cos) with beta = (2/pi)(ln|t_i - t_c| - Rlog_ic/w),
 // below and above z = 20 alike (hankel_df.cuh).  kDf: double-float entries for the mixed form's systems that keep
-// double-float matrices; else FP64 entries, bound by the FP64 pipe at 9 of its instructions an entry and ~30 a pair
+// double-float matrices; else FP64 entries, bound by the FP64 pipe (84% busy) at 9 of its instructions an entry and ~30 a pair
 // (the series and rotated recurrence before took 25 to 45 an entry): 6 arcs x 384 frequencies, N = 512: 24.6 -> 11.8 ms
 // with the row bounds.
 template <bool kDf>
@@ -353,7 +353,8 @@ constexpr int kLuNarrow = 135;   // FP64 jobs of systems up to this size: 128 th
 // and subtraction are FP64: 6 instructions an entry and panel.  One FP64 rounding a panel in place of sixteen: |LU - PA|
 // over |A| at N = 400 2.7e-16 against 9.3e-16 of the FMAs (oracle's self matrices), entry by entry 3.9e-16 against 1.3e-15
 // of |L||U|.  A thread takes two columns of a row, so that each multiplier is read once for both.  8192 systems of N
-// 48..259: 31.0 -> 16.6 ms.
+// 48..259: 31.0 -> 16.6 ms; the FP64 pipe is still 73% busy (panels, U12, the conversions), and warps wait at the
+// panels' barriers.
 template <class C>
 __host__ __device__ constexpr size_t lu_smem(int N) {
   const size_t panel = (size_t)N * (kNB + kPS) * sizeof(C) + (sizeof(C) == sizeof(double2) ? (size_t)N * sizeof(double) : 0);
@@ -659,9 +660,10 @@ __global__ void __launch_bounds__(32 * kSolveWarps) k_solve(DevJob J, int m) {
 }
 
 // The FP64 self matrix of one system (plain form) by one CTA: every entry of the upper triangle (diagonal
-// included) evaluated for the system's own frequency and stored at both mirror positions -- the same
-// log-split rule, Taylor range below z = 20 and Hankel asymptotics above as k_assemble_self, without its
-// sharing of the per-pair terms across a band of frequencies.
+// included) evaluated for the system's own frequency and stored at both mirror positions -- the log-split rule of
+// k_assemble_self with other arithmetic: all in FP64, Taylor series below z = 20 and Hankel's asymptotic series above
+// (bessel.cuh) instead of hankel_df.cuh's, and nothing shared across a band of frequencies.  The two matrices agree to
+// FP64's rounding, not bit for bit.
 __device__ void assemble_one(const DevJob& J, int sidx) {
   const SysDesc s = J.sys[sidx];
   const int N = s.N;
@@ -821,9 +823,10 @@ __device__ void near_beta_block(const CrossTgt* tg, int nrows, int N, const doub
 // kNear: the launch over the tasks with near rows (shared memory for their corrections); otherwise over the far-only
 // tasks, which need only the tables (more CTAs per SM).  Each launch skips the other kind of task.  kF64: the FP64 form;
 // else the mixed forms (FP64 below z = 20, double-float above).  A thread owns (row, source) pairs and walks the
-// band's frequencies.  Bound by the FP64 pipe in the FP64 form (9 instructions an entry, ~25 a pair; 8 obstacle arcs,
-// 4.8e8 entries: 34 -> 12.4 ms), by FP32 issue in the mixed forms (~135 instructions; 12 -> 5.3 ms; N = 512 with 2.6e9
-// entries: 29.3 -> 17.1 ms).
+// band's frequencies.  Bound by the FP64 pipe in the FP64 form (84% busy: 9 instructions an entry, ~25 a pair, which a
+// band of about five frequencies shares on the obstacles; 8 arcs, 4.8e8 entries: 34 -> 12.4 ms); in the mixed forms by
+// issue (68%, ~135 FP32 instructions an entry) and the FP64 of the pairs and of the entries below z = 20 (60%) together
+// (12 -> 5.3 ms; N = 512 with 2.6e9 entries: 29.3 -> 17.1 ms).
 template <bool kNear, bool kF64>
 __global__ void __launch_bounds__(kAsmMaxThreads) k_cross_assemble(DevJob J) {
   extern __shared__ __align__(16) double sha[];
@@ -1047,8 +1050,10 @@ __global__ void __launch_bounds__(kOtfThreads, 2) k_cross_otf(DevJob J) {
 // once per block of frequencies.  Entries never leave registers.  An earlier form wrote them to shared memory and
 // summed with one thread per (row, frequency): at bands of one or two frequencies (N grows with every step of omega)
 // 8 to 16 of its 128 threads worked, and each pair paid two sine/cosine series; 12-arc cavity, 5.7e8 pairs x 5 steps,
-// four windows: 501 -> 89 ms; 6 arcs at N = 1024, two windows: 499 -> 329 ms.  Bound by FP32 issue (~135 instructions
-// an entry and 24 to 48 a window).
+// four windows: 501 -> 89 ms; 6 arcs at N = 1024, two windows: 499 -> 329 ms.  At four windows bound by the FP64
+// pipe (85% busy, issue 59%): a pair's set-up takes ~11 FP64 instructions (differences, distance, scaling), and blocks of
+// one frequency share it with no other entry.  At two windows blocks of four share it: FMA pipe 62%, FP64 45%, issue 68%
+// at two CTAs an SM, no pipe full.  (~135 FP32 instructions an entry and 24 to 48 a window.)
 // kKeep64 (the FP64-kept form): entries below z = 20 in FP64.
 __host__ __device__ constexpr int otf_regs(int Q) { return Q == 1 ? 8 : Q == 2 ? 4 : 1; }
 // blocks per SM: 16 warps of 128 registers, or 24 of 80 where the few sums leave room (measured per Q)
@@ -1209,8 +1214,8 @@ constexpr int kApplyThreads = 256;
 
 // ---------------------------------------------------------------------------------------------
 // Mixed-precision solve: an FP32 blocked solve with the FP32 factors, then refinement steps, each a
-// residual r = G - A phi (A kept as double-float, about 48 bits; the residual in double-float, or in FP64
-// in the FP64-kept form) and an FP32 correction, until the error estimated to remain is below
+// residual r = G - A phi (A kept as double-float, about 48 bits, and the residual too; systems that keep
+// FP64: A in 60-bit fixed point, the residual an exact sum rounded to FP64) and an FP32 correction, until the error estimated to remain is below
 // J.refine_tol, or J.refine_max steps.  Each step shrinks the error by a factor rho (the FP32 solve's
 // relative accuracy), so what remains after a correction of relative size rel is about rho * rel; rho is
 // estimated by the ratio of the last two corrections, or after the first step by kFirstRhoSafety * rel
@@ -1218,8 +1223,8 @@ constexpr int kApplyThreads = 256;
 // right-hand side; the factor covers large systems, where one right-hand side underestimates rho by up
 // to ~10x).  A system still above the tolerance after J.refine_max steps is counted as unconverged.
 // A step is two launches over the
-// systems still refining: k_mresid streams the double-float matrix with one thread per row (many
-// warps in flight per SM), k_msolve runs the triangular solves with one warp per system and little
+// systems still refining: k_mresid (fixed point) or k_mresid_df (double-float) streams the kept matrix with
+// one thread per row (many warps in flight per SM), k_msolve runs the triangular solves with one warp per system and little
 // register state.  Until a system finishes, its densities sit in its phi slots as double-float pairs
 // (16 bytes, the size of the FP64 value written there at the end).
 constexpr int kRefineCap = 16;          // largest refine_max accepted
@@ -1338,9 +1343,9 @@ __global__ void __launch_bounds__(kFixThreads) k_afix(DevJob J) {
 
 // Refinement residuals of the systems that keep FP64, one thread per row (rows past N recompute the last row and store
 // nothing), all Q windows of the row: pass 1 r = G - A phi_0, later passes r <- r - A d with the last correction (the same value: phi grew by d).
-// Matrix and vector are fixed-point and the sum is exact, rounded once to FP64 and once more in the subtraction -- below
-// an FP64 accumulation's error; all residuals run in units of a power of two of the right-hand side (exact).  Bound by HBM (16
-// bytes an entry); the FP64 and anchored FP32 sums (first pass) and double-float sums (later ones) before, 96 to 225
+// Matrix and vector are fixed-point and the sum is exact (low x low halves dropped), rounded once to FP64 and once more in
+// the subtraction -- below an FP64 accumulation's error; all residuals run in units of a power of two of the right-hand side (exact).  Bound by HBM (16
+// bytes an entry, 0.68 of a copy's rate; issue 37%); the FP64 and anchored FP32 sums (first pass) and double-float sums (later ones) before, 96 to 225
 // instructions an entry at two windows, were issue-bound: N = 512, 2304 systems, 8 steps: 30.5 + 20.6 -> 15.8 + 16.5 ms.
 template <int Q>
 __global__ void __launch_bounds__(kResidThreads, 4) k_mresid(DevJob J, int pass) {
@@ -1456,10 +1461,10 @@ __device__ __forceinline__ void fix_correction(const float2* b, int N, int4* out
     *unit = bad ? __longlong_as_double(0x7FF8000000000000ll) : __hiloint2double((e - fix_bits(kMatLow) + 1023) << 20, 0);
 }
 
-// pass 0: solve with FP32 G, store phi as double-float (FP64 in the FP64-kept form, whose residual reads
-// it), mark the system as refining.  pass p >= 1: solve for the correction from the residual, add it in
-// double-float (FP64), and finish the system (FP64 densities, their double-float copy for the cross apply,
-// their running sum, the statistics) once the correction is small enough or p = J.refine_max.
+// pass 0: solve with FP32 G, store phi as double-float (systems that keep FP64: as FP64, and in fixed point for the
+// residual), mark the system as refining.  pass p >= 1: solve for the correction from the residual, add it in
+// double-float (FP64), and finish the system (FP64 densities, their copy for the cross rows, their running sum, the
+// statistics) once the correction is small enough or p = J.refine_max.
 template <int QT>
 __global__ void __launch_bounds__(32 * kSolveWarps, 3) k_msolve(DevJob J, int m, int pass) {
   extern __shared__ __align__(16) unsigned char shm_raw[];

@@ -103,11 +103,11 @@ bool shapes_valid(const int* shapes, bool mixed);
 // Offsets of the device arrays for a plan (bytes are accumulated into plan.device_bytes).
 size_t plan_device_bytes(const Plan& p);
 
-// First-kind nodes of one arc: t_i = cos((2i+1) pi/(2N)), x(t_i), y(t_i), |x'(t_i)|.
 // Chebyshev points in r on [r0, r1] that interpolate the analytic signal's point-source field u^i(r, t) to below
 // rounding, or 0 when no admissible ellipse does (see plan.cpp).
 int incident_points(double r0, double r1, double carrier, double width);
 
+// First-kind nodes of one arc: t_i = cos((2i+1) pi/(2N)), x(t_i), y(t_i), |x'(t_i)|.
 void arc_nodes(const Curve& c, double theta_a, double theta_b, int N, std::vector<double>& t,
                std::vector<double>& x, std::vector<double>& y, std::vector<double>& sp);
 
